@@ -380,19 +380,160 @@ __global__ void __launch_bounds__(kThreads) k_sqdiff_partial(const S* __restrict
     block_sum(acc, partials);
 }
 
-// max over points of |v|_2^2; partials holds 2 * gridDim.x doubles (the
+// max over points of |v|_2^2 in FP64; partials holds 2 * gridDim.x doubles (the
 // first half receives the block maxima, the second half is scratch).
+//
+// Bound: one pass over v (12 B per point, HBM).  The FP64 pipe of this part
+// runs 2 operations per clock and SM, so forming every |v|^2 in FP64 cost ten
+// times the pass (256^3: 336 us; 512^3: 2567 us).  Each point is first
+// formed in FP32 (relative error below 2^-22: three roundings of non-negative
+// terms); only points that can reach the block's largest value so far are
+// formed in FP64, a few per warp.  thr is that value lowered by 2^-20, so a
+// point below it is below the FP64 maximum too; it is raised by a batch's own
+// largest point before the batch is tested, and it stays 0 (every point is
+// formed) until the maximum is normal.  Non-finite points always compare above
+// it (bit patterns of non-negative floats, NaN on top).  The result is the
+// FP64 maximum, bit for bit, and keeps a NaN; maxima are taken on the bit
+// patterns (integers), which order non-negative doubles the same way.
+__device__ __forceinline__ unsigned norm3_bits(float a, float b, float c)
+{
+    return __float_as_uint(fmaf(c, c, fmaf(b, b, a * a)));
+}
+
+__device__ __forceinline__ void norm3_fold(float a, float b, float c, unsigned s, unsigned thr,
+                                           unsigned long long& hi)
+{
+    if (s < thr) return;
+    const double x = a, y = b, z = c;
+    const unsigned long long t =
+        static_cast<unsigned long long>(__double_as_longlong(x * x + y * y + z * z)) & 0x7fffffffffffffffull;
+    hi = t > hi ? t : hi;
+}
+
+__device__ __forceinline__ void norm3_fold4(const float4& a, const float4& b, const float4& c, const uint4& s,
+                                            unsigned thr, unsigned long long& hi)
+{
+    norm3_fold(a.x, b.x, c.x, s.x, thr, hi);
+    norm3_fold(a.y, b.y, c.y, s.y, thr, hi);
+    norm3_fold(a.z, b.z, c.z, s.z, thr, hi);
+    norm3_fold(a.w, b.w, c.w, s.w, thr, hi);
+}
+
+__device__ __forceinline__ uint4 norm3_bits4(const float4& a, const float4& b, const float4& c)
+{
+    return make_uint4(norm3_bits(a.x, b.x, c.x), norm3_bits(a.y, b.y, c.y), norm3_bits(a.z, b.z, c.z),
+                      norm3_bits(a.w, b.w, c.w));
+}
+
+__device__ __forceinline__ unsigned max4(const uint4& s) { return max(max(s.x, s.y), max(s.z, s.w)); }
+
+// Whether any component of the points is non-zero.
+__device__ __forceinline__ bool norm3_any4(const float4& a, const float4& b, const float4& c)
+{
+    return fabsf(a.x) + fabsf(a.y) + fabsf(a.z) + fabsf(a.w) + fabsf(b.x) + fabsf(b.y) + fabsf(b.z) + fabsf(b.w) +
+               fabsf(c.x) + fabsf(c.y) + fabsf(c.z) + fabsf(c.w) !=
+           0.0f;
+}
+
+// The threshold raised by a batch of points of which m is the warp's largest
+// FP32 value.
+__device__ __forceinline__ unsigned norm3_threshold(unsigned m, unsigned thr)
+{
+    const float f = __uint_as_float(m);
+    if (m >= 0x7f800000u || !(f > 1e-30f)) return thr;  // non-finite, or rounding not relative
+    return max(thr, __float_as_uint(f * (1.0f - 9.5367431640625e-07f)));
+}
+
 __global__ void __launch_bounds__(kThreads) k_maxnorm3_partial(const float* __restrict__ v, size_t N,
                                                                 double* __restrict__ partials)
 {
-    double hi = 0.0;
+    __shared__ unsigned bthr;                       // the block's threshold (only ever rises)
+    __shared__ unsigned long long red[kThreads / 32];
+    unsigned long long hi = 0;                      // bits of the FP64 maximum
+    if (threadIdx.x == 0) bthr = 0;
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
     const size_t stride = static_cast<size_t>(gridDim.x) * kThreads;
-    for (size_t i = blockIdx.x * static_cast<size_t>(kThreads) + threadIdx.x; i < N; i += stride) {
-        const double a = v[i], b = v[N + i], c = v[2 * N + i];
-        const double s = a * a + b * b + c * c;
-        hi = max_nan(hi, s);  // a NaN component makes the result NaN
+    const size_t t0 = blockIdx.x * static_cast<size_t>(kThreads) + (threadIdx.x & ~31u);  // uniform in the warp
+    auto raise = [&](unsigned m, unsigned thr) {
+        const unsigned t = norm3_threshold(m, thr);
+        if (t > thr && lane == 0) atomicMax(&bthr, t);
+        return t;
+    };
+    if (aligned16(v) && (N & 3) == 0) {
+        const size_t n4 = N / 4;
+        const float4* v4 = reinterpret_cast<const float4*>(v);
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (size_t base = t0; base < n4; base += 2 * stride) {
+            const size_t i = base + lane, j = i + stride;
+            const bool in = i < n4, jn = j < n4;
+            const float4 a = in ? __ldg(v4 + i) : zero, b = in ? __ldg(v4 + n4 + i) : zero,
+                         c = in ? __ldg(v4 + 2 * n4 + i) : zero;
+            const float4 d = jn ? __ldg(v4 + j) : zero, e = jn ? __ldg(v4 + n4 + j) : zero,
+                         f = jn ? __ldg(v4 + 2 * n4 + j) : zero;
+            unsigned thr = *static_cast<volatile unsigned*>(&bthr);
+            thr = __shfl_sync(0xffffffffu, thr, 0);
+            const uint4 s = norm3_bits4(a, b, c), u = norm3_bits4(d, e, f);
+            const unsigned m = __reduce_max_sync(0xffffffffu, max(max4(s), max4(u)));
+            // FP32 squares of zeros, or of values below 1e-22 or so: only the latter go on
+            if (m == 0u && !__any_sync(0xffffffffu, norm3_any4(a, b, c) || norm3_any4(d, e, f))) continue;
+            if (m >= thr) {
+                thr = raise(m, thr);
+                norm3_fold4(a, b, c, s, thr, hi);
+                norm3_fold4(d, e, f, u, thr, hi);
+            }
+        }
+    } else {
+        for (size_t base = t0; base < N; base += stride) {
+            const size_t i = base + lane;
+            const bool in = i < N;
+            const float a = in ? v[i] : 0.0f, b = in ? v[N + i] : 0.0f, c = in ? v[2 * N + i] : 0.0f;
+            unsigned thr = *static_cast<volatile unsigned*>(&bthr);
+            thr = __shfl_sync(0xffffffffu, thr, 0);
+            const unsigned s = norm3_bits(a, b, c);
+            const unsigned m = __reduce_max_sync(0xffffffffu, s);
+            if (m == 0u && !__any_sync(0xffffffffu, fabsf(a) + fabsf(b) + fabsf(c) != 0.0f)) continue;
+            if (m >= thr) {
+                thr = raise(m, thr);
+                norm3_fold(a, b, c, s, thr, hi);
+            }
+        }
     }
-    block_minmax(hi, hi, partials + gridDim.x, partials);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long t = __shfl_xor_sync(0xffffffffu, hi, o);
+        hi = t > hi ? t : hi;
+    }
+    if (lane == 0) red[threadIdx.x >> 5] = hi;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int w = 1; w < kThreads / 32; ++w) hi = red[w] > hi ? red[w] : hi;
+        partials[blockIdx.x] = __longlong_as_double(static_cast<long long>(hi));
+    }
+}
+
+// Maximum of nb non-negative doubles (bit patterns; NaN on top) into out[0].
+__global__ void __launch_bounds__(kThreads) k_final_max(const double* __restrict__ p, int nb, double* __restrict__ out)
+{
+    __shared__ unsigned long long red[kThreads / 32];
+    unsigned long long hi = 0;
+    for (int i = threadIdx.x; i < nb; i += kThreads) {
+        const unsigned long long t = static_cast<unsigned long long>(__double_as_longlong(p[i])) & 0x7fffffffffffffffull;
+        hi = t > hi ? t : hi;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long t = __shfl_xor_sync(0xffffffffu, hi, o);
+        hi = t > hi ? t : hi;
+    }
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = hi;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int w = 1; w < kThreads / 32; ++w) hi = red[w] > hi ? red[w] : hi;
+        out[0] = __longlong_as_double(static_cast<long long>(hi));
+    }
 }
 
 // Dice counts (Sec. 4.1): both = 0 counts a >= t and b >= t into pa, pb;
@@ -1017,8 +1158,8 @@ void launch_final_sum(const double* partials, int nblocks, double scale, double*
 
 void launch_final_max(const double* partials, int nblocks, double* out, cudaStream_t st)
 {
-    // out[0] receives a throw-away min, out[1] the max
-    k_final_minmax<<<1, kThreads, 0, st>>>(nullptr, partials, nblocks, out);
+    // out[0] is left alone, out[1] receives the maximum
+    k_final_max<<<1, kThreads, 0, st>>>(partials, nblocks, out + 1);
 }
 
 void launch_final_minmax(const double* pmin, const double* pmax, int nblocks, double* out2,
