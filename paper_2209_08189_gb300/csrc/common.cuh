@@ -147,38 +147,6 @@ struct Stencil {
         }
         return r;
     }
-    // Three fields sharing the stencil (f, f + stride, f + 2 stride).
-    __device__ __forceinline__ void eval3(const float* __restrict__ f, uint32_t stride,
-                                          float out[3]) const
-    {
-        constexpr int M = Axis<ORDER>::M;
-        float r0 = 0.0f, r1 = 0.0f, r2 = 0.0f;
-#pragma unroll
-        for (int a = 0; a < M; ++a) {
-            float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f;
-#pragma unroll
-            for (int b = 0; b < M; ++b) {
-                const float* row = f + a1.idx[a] + a2.idx[b];
-                float q0 = 0.0f, q1 = 0.0f, q2 = 0.0f;
-#pragma unroll
-                for (int c = 0; c < M; ++c) {
-                    const int o = a3.idx[c];
-                    q0 = fmaf(a3.w[c], __ldg(row + o), q0);
-                    q1 = fmaf(a3.w[c], __ldg(row + stride + o), q1);
-                    q2 = fmaf(a3.w[c], __ldg(row + 2 * stride + o), q2);
-                }
-                s0 = fmaf(a2.w[b], q0, s0);
-                s1 = fmaf(a2.w[b], q1, s1);
-                s2 = fmaf(a2.w[b], q2, s2);
-            }
-            r0 = fmaf(a1.w[a], s0, r0);
-            r1 = fmaf(a1.w[a], s1, r1);
-            r2 = fmaf(a1.w[a], s2, r2);
-        }
-        out[0] = r0;
-        out[1] = r1;
-        out[2] = r2;
-    }
 };
 
 // Grid coordinates of linear index p.

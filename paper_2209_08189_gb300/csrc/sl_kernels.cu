@@ -72,6 +72,10 @@ __global__ void __launch_bounds__(kTileThreads, CLAIRE_TILE_MIN_BLOCKS)
     for (int c = 0; c < 3; ++c) {
         const float* f = vc + c * N;
         const float ih = c == 0 ? g.ih1 : (c == 1 ? g.ih2 : g.ih3);
+        // weights and offsets are formed anew per component: kept across the
+        // three they do not fit the 64 registers
+#pragma unroll
+        for (int q = 0; q < TILE1; ++q) asm volatile("" : "+f"(u1[q]), "+f"(u2[q]), "+f"(u3[q]));
         if (use_box) {
             tile_load_box<float>(g, f, box, bp, lane, warp);
             cp_async_wait_all();
@@ -306,161 +310,317 @@ __global__ void __launch_bounds__(kThreads) k_convert(const Si* __restrict__ in,
     if (p < n) stf<So>(out + p, ldf<Si>(in + p));
 }
 
-// Deformation map step: u^{j+1} = u^j(X) + (X - x), three components.
-template <int ORDER>
-__global__ void __launch_bounds__(kThreads) k_map_step(Grid g, const float* __restrict__ u_prev,
-                                                        const float* __restrict__ d,
-                                                        float* __restrict__ u)
+// ---- FD8 over 8 x 32 columns ----
+// A CTA owns an 8 x 32 column of (x2, x3) nodes over zlen consecutive x1
+// planes.  Each plane of the column, with the halo of 4 nodes that its
+// differences need in x2 and x3 (periodically wrapped), is staged in shared
+// memory (two buffers, one barrier per plane); every thread keeps the nine
+// values of its own column along x1 in registers, loading one new value per
+// plane.  A plane's values are requested one plane ahead, so their latency
+// overlaps the differences of the plane before.  Each value crosses HBM about
+// once and L2 about 2.5 times, instead of 24 neighbour loads per point and
+// field through L1/L2; the arithmetic is fd8_combine in the same order
+// whatever the split.  Bound: HBM (16 B per point for a gradient or a
+// divergence).  The columns need not divide the grid: nodes past its end are
+// staged from the last wrapped halo node and not written.
+constexpr int kFdRows = 8 + 8, kFdCols = 32 + 8;  // staged plane with its halo of 4
+constexpr int kFdPlane = kFdRows * kFdCols;
+
+// Planes per column: 32 (a quarter of the x1 halo reads of 8 planes) when
+// enough columns remain to fill the chip four times over, else 16, else 8.
+inline int fd_zlen(const Grid& g)
 {
-    const uint32_t p = blockIdx.x * kThreads + threadIdx.x;
-    if (p >= g.N) return;
-    int i, j, k;
-    coords_of(g, p, i, j, k);
-    const size_t N = g.N;
-    const float d1 = __ldg(d + p), d2 = __ldg(d + N + p), d3 = __ldg(d + 2 * N + p);
-    Stencil<ORDER> s;
-    s.build(g, i, j, k, d1, d2, d3);
-    float r[3];
-    s.eval3(u_prev, g.N, r);
-    u[p] = fmaf(d1, g.h1, r[0]);
-    u[N + p] = fmaf(d2, g.h2, r[1]);
-    u[2 * N + p] = fmaf(d3, g.h3, r[2]);
+    const long long cols = static_cast<long long>((g.n3 + 31) / 32) * ((g.n2 + 7) / 8);
+    for (int z = 32; z > 8; z /= 2)
+        if (cols * ((g.n1 + z - 1) / z) >= 4 * 152 * 4) return z;
+    return 8;
 }
 
+inline dim3 fd_grid(const Grid& g, int zlen)
+{
+    return dim3((g.n3 + 31) / 32, (g.n2 + 7) / 8, (g.n1 + zlen - 1) / zlen);
+}
+
+// The nodes a thread stages and owns in the column (bx, by).
+struct FdColumn {
+    int soff[3];   // plane offsets of the up to three halo-plane nodes it stages
+    bool s2;       // whether it stages the third
+    uint32_t col;  // plane offset of its own node (clamped into the grid)
+    bool ok;       // whether its own node exists
+    __device__ __forceinline__ FdColumn(const Grid& g, int bx, int by)
+    {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        const int k = bx * 32 + lane, j = by * 8 + warp;
+        ok = k < g.n3 && j < g.n2;
+        col = static_cast<uint32_t>(min(j, g.n2 - 1)) * g.n3 + min(k, g.n3 - 1);
+        s2 = threadIdx.x + 2 * kThreads < kFdPlane;
+#pragma unroll
+        for (int u = 0; u < 3; ++u) {
+            const int e = min(static_cast<int>(threadIdx.x) + u * kThreads, kFdPlane - 1);
+            const int row = e / kFdCols, c = e - row * kFdCols;
+            // at most n + 3 (the halo of the last node; n2, n3 >= 8 > 4, so one wrap suffices)
+            int gj = min(by * 8 + row - 4, g.n2 + 3);
+            gj = gj < 0 ? gj + g.n2 : (gj >= g.n2 ? gj - g.n2 : gj);
+            int gk = min(bx * 32 + c - 4, g.n3 + 3);
+            gk = gk < 0 ? gk + g.n3 : (gk >= g.n3 ? gk - g.n3 : gk);
+            soff[u] = gj * g.n3 + gk;
+        }
+    }
+};
+
+__device__ __forceinline__ int fd_wrap(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
+
+// x1 queue of one field: the column's values at planes i-4 .. i+4.
 template <class S>
-__global__ void __launch_bounds__(kThreads) k_fd8_grad(Grid g, const S* __restrict__ f,
-                                                        S* __restrict__ out)
+__device__ __forceinline__ void fd_queue_fill(const Grid& g, const S* __restrict__ f, uint32_t col, int i0, float q[9])
 {
-    const uint32_t p = blockIdx.x * kThreads + threadIdx.x;
-    if (p >= g.N) return;
-    int i, j, k;
-    coords_of(g, p, i, j, k);
-    const size_t N = g.N;
-    stf<S>(out + p, fd8_axis<S>(f, p, i, g.n1, g.n23) * g.ih1);
-    stf<S>(out + N + p, fd8_axis<S>(f, p, j, g.n2, g.n3) * g.ih2);
-    stf<S>(out + 2 * N + p, fd8_axis<S>(f, p, k, g.n3, 1) * g.ih3);
+#pragma unroll
+    for (int s = 0; s < 9; ++s) q[s] = ldf<S>(f + static_cast<size_t>(fd_wrap(i0 - 4 + s, g.n1)) * g.n23 + col);
 }
 
-// FD8 gradient on grids whose (x2, x3) planes the 8 x 32 tiles cover exactly:
-// a CTA owns an 8 x 32 column of kFdZ consecutive x1 planes.  Each plane of the
-// tile, with a halo of 4 nodes in x2 and x3 (periodically wrapped), is staged
-// in shared memory (two buffers, one barrier per plane) for the x2 and x3
-// differences; every thread keeps the nine values of its own column along x1
-// in registers for the x1 difference, loading one new plane value per step.
-// Each value then crosses HBM about once and L2 about 2.5 times, instead of
-// the 24 scattered neighbour loads per point of k_fd8_grad; the arithmetic is
-// fd8_combine in the same order, so the results are identical.
-constexpr int kFdZ = 16;                           // x1 planes per CTA
-constexpr int kFdRows = 8 + 8, kFdCols = 32 + 8;   // staged plane with its halo of 4
+__device__ __forceinline__ float fd_queue_diff(const float q[9])
+{
+    float fp[4], fm[4];
+#pragma unroll
+    for (int s = 1; s <= 4; ++s) {
+        fp[s - 1] = q[4 + s];
+        fm[s - 1] = q[4 - s];
+    }
+    return fd8_combine(fp, fm);
+}
 
+__device__ __forceinline__ void fd_queue_push(float q[9], float next)
+{
+#pragma unroll
+    for (int s = 0; s < 8; ++s) q[s] = q[s + 1];
+    q[8] = next;
+}
+
+// Difference at sh[0] along a shared-memory stride.
+template <int STRIDE>
+__device__ __forceinline__ float fd_sh_diff(const float* sh)
+{
+    float fp[4], fm[4];
+#pragma unroll
+    for (int s = 1; s <= 4; ++s) {
+        fp[s - 1] = sh[s * STRIDE];
+        fm[s - 1] = sh[-s * STRIDE];
+    }
+    return fd8_combine(fp, fm);
+}
+
+// FD8 gradient.  256^3 FP32: 71 us; 182 x 218 x 182 FP16, whose grid the
+// columns do not cover: 36.5 us (the per-point kernel: 77 us).
 template <class S>
 __global__ void __launch_bounds__(kThreads) k_fd8_grad_tiled(Grid g, const S* __restrict__ f,
-                                                              S* __restrict__ out)
+                                                              S* __restrict__ out, int zlen)
 {
-    __shared__ float sh[2][kFdRows][kFdCols];
+    __shared__ float sh[2][kFdPlane];
+    const FdColumn t(g, blockIdx.x, blockIdx.y);
+    const int own = (static_cast<int>(threadIdx.x >> 5) + 4) * kFdCols + (threadIdx.x & 31) + 4;
+    const int i0 = blockIdx.z * zlen, i1 = min(i0 + zlen, g.n1);
+    const size_t N = g.N;
+    float q[9];
+    fd_queue_fill<S>(g, f, t.col, i0, q);
+    const S* plane = f + static_cast<size_t>(i0) * g.n23;
+    float p0 = ldf<S>(plane + t.soff[0]), p1 = ldf<S>(plane + t.soff[1]), p2 = t.s2 ? ldf<S>(plane + t.soff[2]) : 0.0f;
+    for (int i = i0; i < i1; ++i) {
+        float* b = sh[(i - i0) & 1];
+        b[threadIdx.x] = p0;
+        b[threadIdx.x + kThreads] = p1;
+        if (t.s2) b[threadIdx.x + 2 * kThreads] = p2;
+        // the next plane's values, requested before the barrier
+        const float qn = ldf<S>(f + static_cast<size_t>(fd_wrap(i + 5, g.n1)) * g.n23 + t.col);
+        if (i + 1 < i1) {
+            plane += g.n23;
+            p0 = ldf<S>(plane + t.soff[0]);
+            p1 = ldf<S>(plane + t.soff[1]);
+            if (t.s2) p2 = ldf<S>(plane + t.soff[2]);
+        }
+        __syncthreads();
+        const float d1 = fd_queue_diff(q), d2 = fd_sh_diff<kFdCols>(b + own), d3 = fd_sh_diff<1>(b + own);
+        if (t.ok) {
+            const size_t p = static_cast<size_t>(i) * g.n23 + t.col;
+            stf<S>(out + p, d1 * g.ih1);
+            stf<S>(out + N + p, d2 * g.ih2);
+            stf<S>(out + 2 * N + p, d3 * g.ih3);
+        }
+        fd_queue_push(q, qn);
+    }
+}
+
+// Divergence of an FP32 vector field, stored as S (256^3: 77 us, the per-point
+// kernel 171 us): x1 differences of v_1 from
+// the register queue, x2 differences of v_2 from a staged plane with the x2
+// halo only (16 rows of 32), x3 differences of v_3 from one with the x3 halo
+// only (8 rows of 40).
+template <class S>
+__global__ void __launch_bounds__(kThreads) k_fd8_div_tiled(Grid g, const float* __restrict__ v,
+                                                             S* __restrict__ out, int zlen)
+{
+    __shared__ float sh2[2][kFdRows * 32], sh3[2][8 * kFdCols];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int k = blockIdx.x * 32 + lane, j = blockIdx.y * 8 + warp;
-    const int i0 = blockIdx.z * kFdZ;
-    const int i1 = min(i0 + kFdZ, g.n1);
-    const size_t N = g.N;
-    // the up to three halo-plane values this thread stages: plane offsets of
-    // the wrapped (x2, x3) nodes (n2, n3 >= 8 > 4, so one wrap suffices)
-    constexpr int kPlane = kFdRows * kFdCols;
-    int soff[3], srow[3], scol[3];
+    const bool ok = k < g.n3 && j < g.n2;
+    const int kc = min(k, g.n3 - 1), jc = min(j, g.n2 - 1);
+    const uint32_t col = static_cast<uint32_t>(jc) * g.n3 + kc;
+    // staged nodes: v_2 at rows warp and warp + 8 of the halo column; v_3 at
+    // elements t and t + 256 (only 320) of the halo rows
+    int o2[2], o3[2];
 #pragma unroll
-    for (int u = 0; u < 3; ++u) {
-        const int e = min(static_cast<int>(threadIdx.x) + u * kThreads, kPlane - 1);
-        srow[u] = e / kFdCols;
-        scol[u] = e - srow[u] * kFdCols;
-        int gj = static_cast<int>(blockIdx.y) * 8 + srow[u] - 4;
-        gj = gj < 0 ? gj + g.n2 : (gj >= g.n2 ? gj - g.n2 : gj);
-        int gk = static_cast<int>(blockIdx.x) * 32 + scol[u] - 4;
-        gk = gk < 0 ? gk + g.n3 : (gk >= g.n3 ? gk - g.n3 : gk);
-        soff[u] = gj * g.n3 + gk;
+    for (int u = 0; u < 2; ++u) {
+        const int gj = fd_wrap(min(static_cast<int>(blockIdx.y) * 8 + warp + 8 * u - 4, g.n2 + 3), g.n2);
+        o2[u] = gj * g.n3 + kc;
+        const int e = min(static_cast<int>(threadIdx.x) + u * kThreads, 8 * kFdCols - 1);
+        const int row = e / kFdCols, c = e - row * kFdCols;
+        const int gk = fd_wrap(min(static_cast<int>(blockIdx.x) * 32 + c - 4, g.n3 + 3), g.n3);
+        o3[u] = min(static_cast<int>(blockIdx.y) * 8 + row, g.n2 - 1) * g.n3 + gk;
     }
-    const bool s2 = threadIdx.x + 2 * kThreads < kPlane;
-    const uint32_t col = static_cast<uint32_t>(j) * g.n3 + k;
-    auto wrap1 = [&](int i) { return i < 0 ? i + g.n1 : (i >= g.n1 ? i - g.n1 : i); };
-    // x1 queue: the column's values at planes i-4 .. i+4
+    const bool s3 = threadIdx.x + kThreads < 8 * kFdCols;
+    const int i0 = blockIdx.z * zlen, i1 = min(i0 + zlen, g.n1);
+    const size_t N = g.N;
     float q[9];
-#pragma unroll
-    for (int s = 0; s < 9; ++s) q[s] = ldf<S>(f + static_cast<size_t>(wrap1(i0 - 4 + s)) * g.n23 + col);
+    fd_queue_fill<float>(g, v, col, i0, q);
+    const float* w2 = v + N + static_cast<size_t>(i0) * g.n23;
+    const float* w3 = v + 2 * N + static_cast<size_t>(i0) * g.n23;
+    float a0 = __ldg(w2 + o2[0]), a1 = __ldg(w2 + o2[1]), c0 = __ldg(w3 + o3[0]), c1 = s3 ? __ldg(w3 + o3[1]) : 0.0f;
     for (int i = i0; i < i1; ++i) {
         const int b = (i - i0) & 1;
-        const S* plane = f + static_cast<size_t>(i) * g.n23;
-        sh[b][srow[0]][scol[0]] = ldf<S>(plane + soff[0]);
-        sh[b][srow[1]][scol[1]] = ldf<S>(plane + soff[1]);
-        if (s2) sh[b][srow[2]][scol[2]] = ldf<S>(plane + soff[2]);
-        // next plane's column value, requested before the barrier
-        const float qn = ldf<S>(f + static_cast<size_t>(wrap1(i + 5)) * g.n23 + col);
+        sh2[b][threadIdx.x] = a0;
+        sh2[b][threadIdx.x + kThreads] = a1;
+        sh3[b][threadIdx.x] = c0;
+        if (s3) sh3[b][threadIdx.x + kThreads] = c1;
+        const float qn = __ldg(v + static_cast<size_t>(fd_wrap(i + 5, g.n1)) * g.n23 + col);
+        if (i + 1 < i1) {
+            w2 += g.n23;
+            w3 += g.n23;
+            a0 = __ldg(w2 + o2[0]);
+            a1 = __ldg(w2 + o2[1]);
+            c0 = __ldg(w3 + o3[0]);
+            if (s3) c1 = __ldg(w3 + o3[1]);
+        }
         __syncthreads();
-        float fp[4], fm[4];
-#pragma unroll
-        for (int s = 1; s <= 4; ++s) {
-            fp[s - 1] = q[4 + s];
-            fm[s - 1] = q[4 - s];
-        }
-        const float d1 = fd8_combine(fp, fm);
-#pragma unroll
-        for (int s = 1; s <= 4; ++s) {
-            fp[s - 1] = sh[b][warp + 4 + s][lane + 4];
-            fm[s - 1] = sh[b][warp + 4 - s][lane + 4];
-        }
-        const float d2 = fd8_combine(fp, fm);
-#pragma unroll
-        for (int s = 1; s <= 4; ++s) {
-            fp[s - 1] = sh[b][warp + 4][lane + 4 + s];
-            fm[s - 1] = sh[b][warp + 4][lane + 4 - s];
-        }
-        const float d3 = fd8_combine(fp, fm);
-        const size_t p = static_cast<size_t>(i) * g.n23 + col;
-        stf<S>(out + p, d1 * g.ih1);
-        stf<S>(out + N + p, d2 * g.ih2);
-        stf<S>(out + 2 * N + p, d3 * g.ih3);
-#pragma unroll
-        for (int s = 0; s < 8; ++s) q[s] = q[s + 1];
-        q[8] = qn;
+        const float d1 = fd_queue_diff(q), d2 = fd_sh_diff<32>(&sh2[b][(warp + 4) * 32 + lane]),
+                    d3 = fd_sh_diff<1>(&sh3[b][warp * kFdCols + lane + 4]);
+        if (ok) stf<S>(out + static_cast<size_t>(i) * g.n23 + col, d1 * g.ih1 + d2 * g.ih2 + d3 * g.ih3);
+        fd_queue_push(q, qn);
     }
 }
 
-// divergence of an FP32 vector field, stored as S
-template <class S>
-__global__ void __launch_bounds__(kThreads) k_fd8_div(Grid g, const float* __restrict__ v,
-                                                       S* __restrict__ out)
+// Order-preserving map between floats (no NaN) and ints, for warp extrema.
+__device__ __forceinline__ int ordered_int(float x)
 {
-    const uint32_t p = blockIdx.x * kThreads + threadIdx.x;
-    if (p >= g.N) return;
-    int i, j, k;
-    coords_of(g, p, i, j, k);
-    const size_t N = g.N;
-    stf<S>(out + p, fd8_axis(v, p, i, g.n1, g.n23) * g.ih1 + fd8_axis(v + N, p, j, g.n2, g.n3) * g.ih2 +
-                        fd8_axis(v + 2 * N, p, k, g.n3, 1) * g.ih3);
+    const int i = __float_as_int(x);
+    return i ^ ((i >> 31) & 0x7fffffff);
 }
+constexpr int kOrderedInf = 0x7f800000;  // +infinity; ~kOrderedInf is -infinity
+__device__ __forceinline__ float ordered_float(int i) { return __int_as_float(i ^ ((i >> 31) & 0x7fffffff)); }
 
 // det(I + grad u) in FP64 with block-wise min / max partials.
-__global__ void __launch_bounds__(kThreads) k_detj_minmax(Grid g, const float* __restrict__ u,
-                                                           double* __restrict__ pmin,
-                                                           double* __restrict__ pmax)
+//
+// Bound: the nine FD8 differences per point.  The FP64 pipe of this part runs
+// 2 operations per clock and SM, so the 30 FP64 operations of every point's
+// determinant were most of the kernel (256^3: 933 us).  Each determinant is
+// first formed in FP32 with an error bound E; only points that may be below
+// the block's smallest or above its largest value so far are formed in FP64.
+// E = 4e-6 m^3, m the largest |entry|: each of the six triple products (at
+// most m^3) carries three entry roundings, two products and up to three sums
+// of relative error 2^-24, together below 6 * 8 * 2^-24 m^3 = 2.9e-6 m^3.
+// A NaN or an overflow fails both comparisons and is formed in FP64.  The
+// extrema are the FP64 ones, bit for bit.  Columns are walked by a fixed
+// number of CTAs (one partial each).  256^3: 328 us.
+__global__ void __launch_bounds__(kThreads) k_detj_minmax(Grid g, const float* __restrict__ u, int zlen, int ncol,
+                                                           double* __restrict__ pmin, double* __restrict__ pmax)
 {
-    double lo = 1e300, hi = -1e300;
+    __shared__ float sh[2][3][kFdPlane];
+    const int own = (static_cast<int>(threadIdx.x >> 5) + 4) * kFdCols + (threadIdx.x & 31) + 4;
+    const int nx = (g.n3 + 31) / 32, ny = (g.n2 + 7) / 8;
     const size_t N = g.N;
-    for (uint32_t p = blockIdx.x * kThreads + threadIdx.x; p < g.N; p += gridDim.x * kThreads) {
-        int i, j, k;
-        coords_of(g, p, i, j, k);
-        double F[3][3];
+    double lo = 1e300, hi = -1e300;
+    __shared__ int blo, bhi;  // the block's bounds of lo and hi (ordered ints)
+    const int lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        blo = kOrderedInf;
+        bhi = ~kOrderedInf;
+    }
+    __syncthreads();
+    int par = 0;
+    for (int cb = blockIdx.x; cb < ncol; cb += gridDim.x) {
+        const int bx = cb % nx, by = (cb / nx) % ny, bz = cb / (nx * ny);
+        const FdColumn t(g, bx, by);
+        const int i0 = bz * zlen, i1 = min(i0 + zlen, g.n1);
+        float q[3][9], p[3][3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            const float* uc = u + c * N;
-            F[c][0] = fd8_axis(uc, p, i, g.n1, g.n23) * g.ih1;
-            F[c][1] = fd8_axis(uc, p, j, g.n2, g.n3) * g.ih2;
-            F[c][2] = fd8_axis(uc, p, k, g.n3, 1) * g.ih3;
-            F[c][c] += 1.0;
+            fd_queue_fill<float>(g, u + c * N, t.col, i0, q[c]);
+            const float* plane = u + c * N + static_cast<size_t>(i0) * g.n23;
+            p[c][0] = __ldg(plane + t.soff[0]);
+            p[c][1] = __ldg(plane + t.soff[1]);
+            p[c][2] = t.s2 ? __ldg(plane + t.soff[2]) : 0.0f;
         }
-        const double det = F[0][0] * (F[1][1] * F[2][2] - F[1][2] * F[2][1]) -
-                           F[0][1] * (F[1][0] * F[2][2] - F[1][2] * F[2][0]) +
-                           F[0][2] * (F[1][0] * F[2][1] - F[1][1] * F[2][0]);
-        lo = min_nan(lo, det);  // a NaN propagates to both extrema
-        hi = max_nan(hi, det);
+        for (int i = i0; i < i1; ++i, par ^= 1) {
+            float qn[3];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                float* b = sh[par][c];
+                b[threadIdx.x] = p[c][0];
+                b[threadIdx.x + kThreads] = p[c][1];
+                if (t.s2) b[threadIdx.x + 2 * kThreads] = p[c][2];
+                qn[c] = __ldg(u + c * N + static_cast<size_t>(fd_wrap(i + 5, g.n1)) * g.n23 + t.col);
+                if (i + 1 < i1) {
+                    const float* plane = u + c * N + static_cast<size_t>(i + 1) * g.n23;
+                    p[c][0] = __ldg(plane + t.soff[0]);
+                    p[c][1] = __ldg(plane + t.soff[1]);
+                    if (t.s2) p[c][2] = __ldg(plane + t.soff[2]);
+                }
+            }
+            __syncthreads();
+            // any value a lane reads here bounds the block's extrema; the warp takes lane 0's
+            float flo = ordered_float(__shfl_sync(0xffffffffu, *static_cast<volatile int*>(&blo), 0)),
+                  fhi = ordered_float(__shfl_sync(0xffffffffu, *static_cast<volatile int*>(&bhi), 0));
+            float e[3][3], f[3][3], m = 0.0f;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                e[c][0] = fd_queue_diff(q[c]) * g.ih1;
+                e[c][1] = fd_sh_diff<kFdCols>(sh[par][c] + own) * g.ih2;
+                e[c][2] = fd_sh_diff<1>(sh[par][c] + own) * g.ih3;
+                fd_queue_push(q[c], qn[c]);
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    f[c][a] = a == c ? 1.0f + e[c][a] : e[c][a];
+                    m = fmaxf(m, fabsf(f[c][a]));
+                }
+            }
+            const float det = f[0][0] * (f[1][1] * f[2][2] - f[1][2] * f[2][1]) -
+                              f[0][1] * (f[1][0] * f[2][2] - f[1][2] * f[2][0]) +
+                              f[0][2] * (f[1][0] * f[2][1] - f[1][1] * f[2][0]);
+            const float E = 4e-6f * m * m * m;
+            const float dlo = det - E, dhi = det + E;
+            // dhi bounds lo from above, dlo bounds hi from below (finite ones only);
+            // the bounds are raised by the plane's own points before it is tested
+            const bool fin = t.ok && fabsf(dlo) < 3e38f && fabsf(dhi) < 3e38f;
+            if (!__any_sync(0xffffffffu, t.ok && !(dlo > flo && dhi < fhi))) continue;  // also NaN
+            flo = fminf(flo, ordered_float(__reduce_min_sync(0xffffffffu, fin ? ordered_int(dhi) : kOrderedInf)));
+            fhi = fmaxf(fhi, ordered_float(__reduce_max_sync(0xffffffffu, fin ? ordered_int(dlo) : ~kOrderedInf)));
+            if (lane == 0) {
+                atomicMin(&blo, ordered_int(flo));
+                atomicMax(&bhi, ordered_int(fhi));
+            }
+            if (t.ok && !(dlo > flo && dhi < fhi)) {
+                double F[3][3];
+#pragma unroll
+                for (int c = 0; c < 3; ++c)
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) F[c][a] = e[c][a];
+#pragma unroll
+                for (int c = 0; c < 3; ++c) F[c][c] += 1.0;
+                const double d = F[0][0] * (F[1][1] * F[2][2] - F[1][2] * F[2][1]) -
+                                 F[0][1] * (F[1][0] * F[2][2] - F[1][2] * F[2][0]) +
+                                 F[0][2] * (F[1][0] * F[2][1] - F[1][1] * F[2][0]);
+                lo = min_nan(lo, d);  // a NaN propagates to both extrema
+                hi = max_nan(hi, d);
+            }
+        }
     }
     block_minmax(lo, hi, pmin, pmax);
 }
@@ -470,16 +630,6 @@ __global__ void __launch_bounds__(kThreads) k_detj_minmax(Grid g, const float* _
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
-
-#define CLAIRE_DISPATCH(order, KERNEL, ...)                                       \
-    do {                                                                          \
-        if ((order) == 3)                                                         \
-            KERNEL<3><<<blocks_for(g.N), kThreads, 0, st>>>(__VA_ARGS__);         \
-        else if ((order) == 4)                                                    \
-            KERNEL<4><<<blocks_for(g.N), kThreads, 0, st>>>(__VA_ARGS__);         \
-        else                                                                      \
-            KERNEL<1><<<blocks_for(g.N), kThreads, 0, st>>>(__VA_ARGS__);         \
-    } while (0)
 
 // tiled gathers: cubic B-spline (order 4) only for FP32 fields
 #define CLAIRE_TILED(order, EPI, fs, d, e)                                        \
@@ -502,31 +652,33 @@ void launch_interp(const Grid& g, int order, const void* f, const float* d, void
     });
 }
 
-template <int ORDER>
+template <int ORDER, bool FULL, bool MAP>
+void launch_fields_tiles(const Grid& g, const float* f, int nf, const float* d, float* out, cudaStream_t st)
+{
+    if (kTiledSmemBytes > 48 * 1024)
+        cudaFuncSetAttribute(k_gather_tiled_fields<ORDER, FULL, MAP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(kTiledSmemBytes));
+    k_gather_tiled_fields<ORDER, FULL, MAP><<<tiled_grid(g), kTileThreads, kTiledSmemBytes, st>>>(g, f, nf, d, out);
+}
+
+template <int ORDER, bool MAP>
 void launch_fields_as(const Grid& g, const float* f, int nf, const float* d, float* out, cudaStream_t st)
 {
-    if (tiles_cover_grid(g)) {
-        if (kTiledSmemBytes > 48 * 1024)
-            cudaFuncSetAttribute(k_gather_tiled_fields<ORDER, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(kTiledSmemBytes));
-        k_gather_tiled_fields<ORDER, true><<<tiled_grid(g), kTileThreads, kTiledSmemBytes, st>>>(g, f, nf, d, out);
-    } else {
-        if (kTiledSmemBytes > 48 * 1024)
-            cudaFuncSetAttribute(k_gather_tiled_fields<ORDER, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(kTiledSmemBytes));
-        k_gather_tiled_fields<ORDER, false><<<tiled_grid(g), kTileThreads, kTiledSmemBytes, st>>>(g, f, nf, d, out);
-    }
+    if (tiles_cover_grid(g))
+        launch_fields_tiles<ORDER, true, MAP>(g, f, nf, d, out, st);
+    else
+        launch_fields_tiles<ORDER, false, MAP>(g, f, nf, d, out, st);
 }
 
 void launch_interp_fields(const Grid& g, int order, const float* f, int nf, const float* d, float* out,
                           cudaStream_t st)
 {
     if (order == 3)
-        launch_fields_as<3>(g, f, nf, d, out, st);
+        launch_fields_as<3, false>(g, f, nf, d, out, st);
     else if (order == 4)
-        launch_fields_as<4>(g, f, nf, d, out, st);
+        launch_fields_as<4, false>(g, f, nf, d, out, st);
     else
-        launch_fields_as<1>(g, f, nf, d, out, st);
+        launch_fields_as<1, false>(g, f, nf, d, out, st);
 }
 
 cudaError_t gather_fallback_tiles(unsigned long long* count, bool reset)
@@ -676,36 +828,37 @@ void launch_from_storage(const void* in, float* out, size_t n, Storage sto, cuda
 void launch_map_step(const Grid& g, int order, const float* u_prev, const float* d, float* u,
                      cudaStream_t st)
 {
-    CLAIRE_DISPATCH(order, k_map_step, g, u_prev, d, u);
+    if (order == 3)
+        launch_fields_as<3, true>(g, u_prev, 3, d, u, st);
+    else if (order == 4)
+        launch_fields_as<4, true>(g, u_prev, 3, d, u, st);
+    else
+        launch_fields_as<1, true>(g, u_prev, 3, d, u, st);
 }
 
 void launch_fd8_grad(const Grid& g, const void* f, void* out, Storage sto, cudaStream_t st)
 {
-    if (g.n3 % 32 == 0 && g.n2 % 8 == 0) {
-        const dim3 grid(g.n3 / 32, g.n2 / 8, (g.n1 + kFdZ - 1) / kFdZ);
-        CLAIRE_STORAGE_DISPATCH(sto, {
-            k_fd8_grad_tiled<SType><<<grid, kThreads, 0, st>>>(g, static_cast<const SType*>(f),
-                                                               static_cast<SType*>(out));
-        });
-        return;
-    }
+    const int z = fd_zlen(g);
     CLAIRE_STORAGE_DISPATCH(sto, {
-        k_fd8_grad<SType><<<blocks_for(g.N), kThreads, 0, st>>>(g, static_cast<const SType*>(f),
-                                                               static_cast<SType*>(out));
+        k_fd8_grad_tiled<SType><<<fd_grid(g, z), kThreads, 0, st>>>(g, static_cast<const SType*>(f),
+                                                                    static_cast<SType*>(out), z);
     });
 }
 
 void launch_fd8_div(const Grid& g, const float* v, void* out, Storage sto, cudaStream_t st)
 {
+    const int z = fd_zlen(g);
     CLAIRE_STORAGE_DISPATCH(sto, {
-        k_fd8_div<SType><<<blocks_for(g.N), kThreads, 0, st>>>(g, v, static_cast<SType*>(out));
+        k_fd8_div_tiled<SType><<<fd_grid(g, z), kThreads, 0, st>>>(g, v, static_cast<SType*>(out), z);
     });
 }
 
 void launch_detj_minmax(const Grid& g, const float* u, double* pmin, double* pmax, int nblocks,
                         cudaStream_t st)
 {
-    k_detj_minmax<<<nblocks, kThreads, 0, st>>>(g, u, pmin, pmax);
+    const int z = fd_zlen(g);
+    const dim3 cols = fd_grid(g, z);
+    k_detj_minmax<<<nblocks, kThreads, 0, st>>>(g, u, z, static_cast<int>(cols.x * cols.y * cols.z), pmin, pmax);
 }
 
 }  // namespace claire
