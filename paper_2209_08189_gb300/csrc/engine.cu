@@ -1836,8 +1836,8 @@ claire_status scatter_transpose(claire_ctx* c, const float* yv, const float* d, 
     CL_LAUNCHED(c);
     {
         KTimer t(c, KK_VJP_SCATTER, (4.0 + 12.0) * c->N, 1.0 * c->N);
-        launch_scatter_fixed(c->grid, c->o.interp, yv, d, v, static_cast<float>(c->dt), mx + 1, c->vjp_acc,
-                             c->stream);
+        CL_CUDA(c, launch_scatter_fixed(c->grid, c->o.interp, yv, d, v, static_cast<float>(c->dt), mx + 1, c->vjp_acc,
+                                        c->stream));
         CL_LAUNCHED(c);
     }
     launch_fixed_to_float(c->vjp_acc, mx + 1, accumulate ? 1 : 0, mult, out, c->N, c->stream);
@@ -1880,7 +1880,6 @@ extern "C" claire_status claire_transport_vjp(claire_ctx* c, const float* v, con
     float* mb = c->r;                // cotangent of the state, two rolling halves
     float* mb2 = c->r + N;
     CL_CUDA(c, cudaMemcpyAsync(mb, gbar, N * sizeof(float), cudaMemcpyDefault, c->stream));
-    CL_CUDA(c, cudaMemsetAsync(dbar, 0, 3 * N * sizeof(float), c->stream));
     CL_TRY(backtrace(c, dv, d, +1));
     float* S = c->vjp_states;
     // states m^1..m^{nt} (all stored), or rolling recomputation from m^0
@@ -1903,7 +1902,7 @@ extern "C" claire_status claire_transport_vjp(claire_ctx* c, const float* v, con
         if (c->o.interp == 4) CL_TRY(bspline_coef(c, mj, 1, &mjc));
         {
             KTimer t(c, KK_VJP_GRAD, 32.0 * N, 1.0 * N);
-            launch_grad_accum(c->grid, c->o.interp, mjc, d, mb, dbar, c->stream);
+            launch_grad_accum(c->grid, c->o.interp, mjc, d, mb, dbar, j == nt - 1, c->stream);
             CL_LAUNCHED(c);
         }
         CL_TRY(scatter_transpose(c, mb, d, nullptr, mb2, false, 1.0f));

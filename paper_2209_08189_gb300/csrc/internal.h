@@ -146,13 +146,14 @@ claire_status ctx_fail(claire_ctx* c, claire_status st, const char* msg);
 void launch_bspline_scale(const Grid& g, cufftComplex* spec, size_t M, int ncomp, cudaStream_t st);
 
 // ---- reverse-mode transport (vjp.cu) ----
-// dbar_c += mbar * d_c I[m](X)   (interpolant gradient at x + d, grid units)
+// dbar_c += mbar * d_c I[m](X)   (interpolant gradient at x + d, grid units);
+// first: dbar is written instead of added to
 void launch_grad_accum(const Grid& g, int order, const float* m, const float* d, const float* mbar, float* dbar,
-                       cudaStream_t st);
+                       bool first, cudaStream_t st);
 // acc += fixed-point(W(x + disp)^T yv), scale from *maxabs = max |yv| (device);
 // disp = d, or -sdt v / h when d is null
-void launch_scatter_fixed(const Grid& g, int order, const float* yv, const float* d, const float* v, float sdt,
-                          const double* maxabs, unsigned long long* acc, cudaStream_t st);
+cudaError_t launch_scatter_fixed(const Grid& g, int order, const float* yv, const float* d, const float* v, float sdt,
+                                 const double* maxabs, unsigned long long* acc, cudaStream_t st);
 // out = mult ((accumulate ? out : 0) + acc / scale); clears acc
 void launch_fixed_to_float(unsigned long long* acc, const double* maxabs, int accumulate, float mult, float* out,
                            size_t n, cudaStream_t st);

@@ -45,7 +45,7 @@ constexpr int TILE1 = CLAIRE_TILE1, TILE2 = CLAIRE_TILE2, TILE3 = 32;
 // CTAs of the tiled gathers (in this translation unit) whose box did not fit
 // and which took the global-memory path; one atomic per such CTA, read by
 // claire_gather_fallback_tiles.
-__device__ unsigned long long g_gather_global_tiles = 0;
+static __device__ unsigned long long g_gather_global_tiles = 0;
 constexpr int kTileThreads = TILE2 * 32;
 constexpr int kBoxCapFloats = CLAIRE_BOX_CAP;
 

@@ -1,0 +1,105 @@
+"""GPU tests of the tiled kernels at the sizes where a tile can go wrong: grids
+that their tiles do not cover, tiles wider than the grid, and boxes that do
+not fit in shared memory."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2209_08189_gb300 import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _ctx(n, **opts):
+    from paper_2209_08189_gb300 import claire
+    return claire.Context(n, 1e-2, 4, stream=torch.cuda.current_stream().cuda_stream, **opts)
+
+
+def _dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a, dtype=np.float32)).cuda()
+
+
+def _rel(a, b):
+    a = a.cpu().numpy().astype(np.float64)
+    return float(np.abs(a - b).max() / np.abs(b).max())
+
+
+@pytest.mark.parametrize("n", [(8, 8, 8), (10, 14, 22), (12, 10, 66), (34, 18, 40), (70, 44, 104)])
+def test_fd8_on_partial_columns(n):
+    """Columns of 8 x 32 nodes past the end of the grid, and halos that wrap
+    onto the column itself; random fields, so every wrong neighbour shows.
+    Tolerance: the oracle parity of the FD8 kernels (FP32 sums of 8 terms)."""
+    rng = np.random.default_rng(3)
+    f, v = rng.standard_normal(n).astype(np.float32), rng.standard_normal((3,) + n).astype(np.float32)
+    ctx = _ctx(n, kernels_only=1)
+    g, d = torch.empty((3,) + n, device="cuda"), torch.empty(n, device="cuda")
+    ctx.fd8_grad(_dev(f), g)
+    ctx.fd8_div(_dev(v), d)
+    ref = oracle.fd8_grad(f.astype(np.float64))
+    for c in range(3):
+        assert _rel(g[c], ref[c]) <= 1e-5
+    assert _rel(d, oracle.fd8_div(v.astype(np.float64))) <= 1e-5
+    ctx.close()
+
+
+@pytest.mark.parametrize("n", [(16, 24, 8), (12, 10, 66), (70, 44, 104)])
+@pytest.mark.parametrize("order", [3, 1, 4])
+def test_detj_on_partial_tiles(n, order):
+    """Map steps and determinant extrema; tolerance of the existing parity test."""
+    v = synth.mode_velocity(n, seed=12, vmax=0.8, kmax=2).astype(np.float32)
+    ctx = _ctx(n, interp=order)
+    lo, hi = ctx.detj(_dev(v))
+    ref = oracle.detj(v.astype(np.float64), oracle.Params(nt=4, order=order))
+    assert abs(lo - ref.min()) <= 1e-5 * abs(ref.min()) and abs(hi - ref.max()) <= 1e-5 * ref.max()
+    ctx.close()
+
+
+@pytest.mark.parametrize("n", [(12, 10, 66), (32, 16, 64), (70, 44, 104)])
+@pytest.mark.parametrize("rough", [False, True])
+def test_vjp_tiles_and_fallback(n, rough):
+    """The reverse pass with boxes in shared memory (smooth velocity) and with
+    boxes that do not fit (rough: every point moves on its own, so tiles take the
+    global-memory paths), against the oracle.  The image cotangent is a sum of
+    64 FP32 products per node (1e-5); the velocity cotangent of a rough map
+    has kinks at every cell face, so only the smooth one is compared (1e-4).
+    A cotangent scaled by a power of two scales the result exactly: the
+    fixed-point scale follows max |gbar|.  (Scaled down, the velocity
+    cotangent's FP32 products with small image gradients become subnormal and
+    lose bits, so only the image cotangent scales exactly there.)"""
+    rng = np.random.default_rng(5)
+    v = rng.uniform(-3, 3, (3,) + n) if rough else synth.mode_velocity(n, seed=4, vmax=1.0, kmax=2)
+    v = v.astype(np.float32)
+    m0 = synth.blob_template(n, seed=5, sigma=0.9).astype(np.float32)
+    gbar = rng.standard_normal(n).astype(np.float32)
+    gbar[rng.random(n) < 0.1] = 0.0
+    ctx = _ctx(n)
+    out = {}
+    for k in (0, 90, -90):
+        gm, gv = torch.empty(n, device="cuda"), torch.empty((3,) + n, device="cuda")
+        ctx.transport_vjp(_dev(v), _dev(m0), _dev(gbar * np.float32(2.0 ** k)), gm, gv)
+        out[k] = (gm, gv)
+    rm, rv = oracle.transport_vjp(m0.astype(np.float64), v.astype(np.float64), gbar.astype(np.float64),
+                                  oracle.Params(nt=4))
+    l2 = lambda a, b: float(np.linalg.norm(a.cpu().numpy().astype(np.float64) - b) / np.linalg.norm(b))
+    assert l2(out[0][0], rm) < 1e-5
+    if not rough:
+        assert l2(out[0][1], rv) < 1e-4
+    for k in (90, -90):
+        assert torch.equal(out[k][0], out[0][0] * 2.0 ** k)
+        if k > 0:
+            assert torch.equal(out[k][1], out[0][1] * 2.0 ** k)
+    ctx.close()
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_vjp_non_finite_cotangent_gives_nan(bad):
+    n = (16, 24, 8)
+    v = synth.mode_velocity(n, seed=4, vmax=0.5, kmax=2)
+    g = np.ones(n, dtype=np.float32)
+    g[3, 4, 5] = bad
+    ctx = _ctx(n)
+    gm = torch.empty(n, device="cuda")
+    ctx.transport_vjp(_dev(v), _dev(np.ones(n)), _dev(g), gm)
+    assert bool(torch.isnan(gm).all())
+    ctx.close()
