@@ -122,6 +122,9 @@ struct claire_ctx {
     // their tile-bounds tables, written by every backtrace into dS / dA (the
     // only writer of either field), read by the gathers at dS / dA
     int4 *tbS = nullptr, *tbA = nullptr;
+    // table of the characteristic that objective, transport, det-J and the
+    // reverse mode trace into z, where the same call's gathers read it
+    int4* tbZ = nullptr;
     char *divv = nullptr, *divXp = nullptr;
     char *m = nullptr, *gm = nullptr;     // (nt+1) N states m^j, (nt+1) 3N gradients (null when lowmem)
     char *l0 = nullptr, *l1 = nullptr;    // rolling scalar fields (FP32-sized: transport uses them as FP32)
@@ -345,8 +348,9 @@ struct Layout {
     }
 };
 
-size_t layout_floats(size_t N, size_t M, int nt, int red_blocks, size_t es, bool lowmem, Layout* L)
+size_t layout_floats(const int n[3], size_t N, size_t M, int nt, int red_blocks, size_t es, bool lowmem, Layout* L)
 {
+    const size_t tiles = tiled_grid_tiles(n[0], n[1], n[2]);
     Layout tmp;
     Layout& l = L ? *L : tmp;
     auto S = [&](size_t values) { return (values * es + 3) / 4; };  // storage-typed region, in floats
@@ -370,8 +374,9 @@ size_t layout_floats(size_t N, size_t M, int nt, int red_blocks, size_t es, bool
     l.add(6 * M);             // rh
     l.add(4 * red_blocks);    // partials (2 * red_blocks doubles)
     l.add(32);                // dres (16 doubles)
-    l.add(8 * ((N + 1023) / 1024));  // tbS (2 int4 per 1024-point tile)
-    l.add(8 * ((N + 1023) / 1024));  // tbA
+    l.add(8 * tiles);         // tbS (2 int4 per 4 x 8 x 32 tile)
+    l.add(8 * tiles);         // tbA
+    l.add(8 * tiles);         // tbZ
     return l.total;
 }
 
@@ -607,10 +612,12 @@ claire_status gather_src(claire_ctx* c, const void* f, int ncomp, const void** s
     return CLAIRE_OK;
 }
 
-// tile-bounds table of a displacement field of the context (null for others)
+// tile-bounds table of a displacement field of the context (null for others;
+// a kernels_only context has neither fields nor tables)
 int4* tile_table(claire_ctx* c, const float* d)
 {
-    return d == c->dS ? c->tbS : (d == c->dA ? c->tbA : nullptr);
+    if (!d || !c->tbS) return nullptr;
+    return d == c->dS ? c->tbS : (d == c->dA ? c->tbA : (d == c->z ? c->tbZ : nullptr));
 }
 
 claire_status backtrace(claire_ctx* c, const float* v, float* d, int sign)
@@ -1319,7 +1326,7 @@ claire_status claire_query_workspace(const int grid[3], int nt, const claire_opt
         *bytes = (2 * 152 * 8 + 16) * sizeof(double);  // reduction partials and device scalars
         return CLAIRE_OK;
     }
-    *bytes = layout_floats(N, M, nt, 152 * 8, storage_bytes(static_cast<Storage>(sto)), lowmem, nullptr) *
+    *bytes = layout_floats(grid, N, M, nt, 152 * 8, storage_bytes(static_cast<Storage>(sto)), lowmem, nullptr) *
              sizeof(float);
     return CLAIRE_OK;
 }
@@ -1408,7 +1415,7 @@ claire_status claire_create(claire_ctx** out, const int grid[3], double beta_v, 
     Layout L;
     c->sto = static_cast<Storage>(o.storage);
     c->es = storage_bytes(c->sto);
-    size_t floats = layout_floats(c->N, c->M, nt, c->red_blocks, c->es, o.lowmem != 0, &L);
+    size_t floats = layout_floats(grid, c->N, c->M, nt, c->red_blocks, c->es, o.lowmem != 0, &L);
     cudaError_t e = cudaMalloc(&c->arena, floats * sizeof(float));
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -1445,6 +1452,7 @@ claire_status claire_create(claire_ctx** out, const int grid[3], double beta_v, 
     c->dres = reinterpret_cast<double*>(base + L.off[k++]);
     c->tbS = reinterpret_cast<int4*>(base + L.off[k++]);
     c->tbA = reinterpret_cast<int4*>(base + L.off[k++]);
+    c->tbZ = reinterpret_cast<int4*>(base + L.off[k++]);
     if (cudaMemset(c->dres, 0, 16 * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
         return bail(CLAIRE_ECUDA);
@@ -1812,7 +1820,7 @@ claire_status claire_transport(claire_ctx* c, const float* v, const float* m_in,
             CL_TRY(gather_src(c, src, 1, &gs));
             KTimer t(c, KK_ADJ_STEP, 28.0 * N, 1.0 * N);
             launch_adj_step(c->grid, c->o.interp, gs, c->z, divv, divXp, static_cast<float>(c->dt), a,
-                            Storage::F32, c->stream);
+                            Storage::F32, c->stream, tile_table(c, c->z));
             CL_LAUNCHED(c);
             src = a;
             std::swap(a, b);

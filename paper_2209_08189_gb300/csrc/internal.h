@@ -77,11 +77,13 @@ __device__ __forceinline__ void block_minmax(double lo, double hi, double* pmin,
 #endif
 
 // ---- semi-Lagrangian and FD kernels (sl_kernels.cu) ----
+// CTAs of the tiled gathers on an n1 x n2 x n3 grid (entries of a tile-bounds table)
+size_t tiled_grid_tiles(int n1, int n2, int n3);
 // Pointers typed void* hold scalar fields in the storage type `sto` (FP32,
 // FP16 or BF16); float* ones are always FP32 (displacements, velocities,
 // vector work fields).
 // tb: the tile-bounds table of d written by launch_backtrace (or null: the
-// gathers reduce the bounds themselves); used on grids the tiles cover exactly
+// gathers reduce the bounds themselves)
 void launch_interp(const Grid& g, int order, const void* f, const float* d, void* out, Storage sto,
                    cudaStream_t st, const int4* tb = nullptr);
 // nf FP32 fields [nf][N] at one displacement into out [nf][N]
@@ -90,7 +92,7 @@ void launch_interp_fields(const Grid& g, int order, const float* f, int nf, cons
 // CTAs of the tiled gathers that took the global-memory path (device-wide counter)
 cudaError_t gather_fallback_tiles(unsigned long long* count, bool reset);
 // tb (may be null): also write the tile-bounds table of d (2 int4 per tile of
-// the tiled grid) on grids the tiles cover exactly
+// the tiled grid)
 void launch_backtrace(const Grid& g, int order, const float* v, const float* vc, float dt, int sign, float* d,
                       cudaStream_t st, int4* tb = nullptr);
 // One SL step of Eq. (4): lam = Heun(lam_next(X+), div v(X+), div v).

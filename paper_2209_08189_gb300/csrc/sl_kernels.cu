@@ -24,9 +24,9 @@ inline unsigned blocks_for(uint32_t n) { return (n + kThreads - 1) / kThreads; }
 // sign = -1 gives X+ = x + dt/2 [v(x) + v(x + dt v(x))]; d in grid units.
 // The three velocity gathers at the predictor point are served from a
 // shared-memory box per 4 x 8 x 32 tile (one box, staged once per component;
-// the predictor points of a tile share its bounds).  TBW (grids the tiles
-// cover exactly): also write the tile-bounds table of d (tile_index order),
-// from the same FP32 values that are stored, for the gathers at d.
+// the predictor points of a tile share its bounds).  TBW: also write the
+// tile-bounds table of d (tile_index order), from the same FP32 values that
+// are stored, for the gathers at d.
 template <int ORDER, bool FULL, bool TBW>
 __global__ void __launch_bounds__(kTileThreads, CLAIRE_TILE_MIN_BLOCKS)
     k_backtrace_tiled(Grid g, const float* __restrict__ v, const float* __restrict__ vc, float dt, float sign,
@@ -65,13 +65,12 @@ __global__ void __launch_bounds__(kTileThreads, CLAIRE_TILE_MIN_BLOCKS)
     const bool use_box = bp.E1 != 0;
     if (!use_box && threadIdx.x == 0) atomicAdd(&g_gather_global_tiles, 1ull);
     const float cc = -0.5f * sdt;
-    // bounds of the characteristic itself (TBW)
-    int lo[3] = {INT_MAX, INT_MAX, INT_MAX}, hi[3] = {INT_MIN, INT_MIN, INT_MIN};
-    bool dbad = false;
+    bool dbad = false;  // a component of the characteristic itself fails disp_ok (TBW)
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         const float* f = vc + c * N;
         const float ih = c == 0 ? g.ih1 : (c == 1 ? g.ih2 : g.ih3);
+        int lo = INT_MAX, hi = INT_MIN;  // bounds of the characteristic along axis c (TBW)
         // weights and offsets are formed anew per component: kept across the
         // three they do not fit the 64 registers
 #pragma unroll
@@ -92,18 +91,34 @@ __global__ void __launch_bounds__(kTileThreads, CLAIRE_TILE_MIN_BLOCKS)
             const float uc = c == 0 ? u1[q] : (c == 1 ? u2[q] : u3[q]);
             const float dc = cc * (uc + vsq * ih);
             d[c * N + p0 + q * g.n23] = dc;
-            if constexpr (TBW) bounds_add(c == 0 ? i : (c == 1 ? j : k), dc, lo[c], hi[c], dbad);
+            if constexpr (TBW) bounds_add(c == 0 ? i : (c == 1 ? j : k), dc, lo, hi, dbad);
+        }
+        if constexpr (TBW) {
+            // reduced per component, so that two bounds are live at a time (red is
+            // free again: tile_box read it before its last barrier)
+            lo = __reduce_min_sync(0xffffffffu, lo);
+            hi = __reduce_max_sync(0xffffffffu, hi);
+            if (lane == 0) {
+                red[c][warp] = lo;
+                red[3 + c][warp] = hi;
+            }
         }
         if (use_box) __syncthreads();  // every read of this component is done before the next staging
     }
     if constexpr (TBW) {
-        static_assert(FULL, "tile-bounds tables cover exactly tiled grids only");
-        int b[6];
-        const bool any_bad = tile_bounds(lo[0], lo[1], lo[2], hi[0], hi[1], hi[2], dbad, red, lane, warp, b);
-        if (threadIdx.x == 0) {
-            const unsigned t = tile_index();
-            tb[2 * t] = make_int4(b[0], b[1], b[2], any_bad ? 1 : 0);
-            tb[2 * t + 1] = make_int4(b[3], b[4], b[5], 0);
+        const bool any_bad = __syncthreads_or(dbad) != 0;
+        if (threadIdx.x < 6) {
+            // thread c: lower bound of axis c, thread 3 + c: upper bound
+            const int r = threadIdx.x;
+            int x = red[r][0];
+#pragma unroll
+            for (int w = 1; w < TILE2; ++w) x = r < 3 ? min(x, red[r][w]) : max(x, red[r][w]);
+            int* e = reinterpret_cast<int*>(tb + 2 * tile_index());
+            e[r < 3 ? r : r + 1] = x;
+            if (r == 0) {
+                e[3] = any_bad ? 1 : 0;
+                e[7] = 0;
+            }
         }
     }
 }
@@ -123,9 +138,12 @@ template <int ORDER>
 void launch_backtrace_tiled(const Grid& g, const float* v, const float* vc, float dt, float sign, float* d,
                             int4* tb, cudaStream_t st)
 {
-    if (tiles_cover_grid(g) && tb)
+    const bool full = tiles_cover_grid(g);
+    if (tb && full)
         launch_backtrace_tiled_as<ORDER, true, true>(g, v, vc, dt, sign, d, tb, st);
-    else if (tiles_cover_grid(g))
+    else if (tb)
+        launch_backtrace_tiled_as<ORDER, false, true>(g, v, vc, dt, sign, d, tb, st);
+    else if (full)
         launch_backtrace_tiled_as<ORDER, true, false>(g, v, vc, dt, sign, d, nullptr, st);
     else
         launch_backtrace_tiled_as<ORDER, false, false>(g, v, vc, dt, sign, d, nullptr, st);
@@ -679,6 +697,16 @@ void launch_interp_fields(const Grid& g, int order, const float* f, int nf, cons
         launch_fields_as<4, false>(g, f, nf, d, out, st);
     else
         launch_fields_as<1, false>(g, f, nf, d, out, st);
+}
+
+size_t tiled_grid_tiles(int n1, int n2, int n3)
+{
+    Grid g{};
+    g.n1 = n1;
+    g.n2 = n2;
+    g.n3 = n3;
+    const dim3 t = tiled_grid(g);
+    return static_cast<size_t>(t.x) * t.y * t.z;
 }
 
 cudaError_t gather_fallback_tiles(unsigned long long* count, bool reset)

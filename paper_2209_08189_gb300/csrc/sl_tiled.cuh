@@ -87,6 +87,26 @@ struct BoxPar {
     int S3;          // row stride, a multiple of 32
 };
 
+// The grid whose extents bound the box: an axis too short for a tile's usual
+// box (32 columns, 8 rows or 4 planes, the stencil and some spread) counts
+// double, since a field of period n also has period 2 n; the staging wraps
+// such indices twice.  Without this every tile of a grid with n3 < 40 or so
+// took the global-memory path (32^3 backtrace: 26 us against 13 us).
+__host__ __device__ __forceinline__ Grid box_grid(Grid g)
+{
+    g.n1 = g.n1 < 16 ? 2 * g.n1 : g.n1;
+    g.n2 = g.n2 < 24 ? 2 * g.n2 : g.n2;
+    g.n3 = g.n3 < 64 ? 2 * g.n3 : g.n3;
+    return g;
+}
+
+// Wrapped index of w + c for w in [0, n) and an offset c < 2 n inside a box.
+__device__ __forceinline__ int box_wrap(int x, int n)
+{
+    x = x >= n ? x - n : x;
+    return x >= n ? x - n : x;
+}
+
 // Box geometry from the bounds [a, z] (per axis) of the first-node cells
 // (before the -OFF shift) of a tile's stencils: par[0..2] the first node
 // (unwrapped grid coordinates), par[3..5] the extents and par[6] the row
@@ -95,44 +115,44 @@ struct BoxPar {
 // that a displacement of the tile failed disp_ok (non-finite or at least 2^20
 // cells).  Such a tile is gathered from global memory with the clamped split,
 // whose indices always wrap into range.
+// The x3 origin and extent are rounded to the widest chunk the row length
+// allows (16, 8 or 4 bytes), so that no chunk straddles the x3 wrap.
 // ES: bytes per stored value of the field (4, or 2 for FP16 / BF16 storage,
 // whose box is staged as raw 16-bit pairs before widening to FP32).
+// Unsigned 32-bit arithmetic (every thread of a tile with a tile-bounds table
+// runs this): spans are compared before anything is added to them.
 template <int ORDER, int ES = 4>
 __host__ __device__ __forceinline__ void box_geometry(const Grid& g, int a1, int a2, int a3, int z1, int z2, int z3,
                                                       bool bad, int par[7])
 {
-    constexpr int M = Scheme<ORDER>::M;
-    constexpr int OFF = Scheme<ORDER>::OFF;
+    constexpr unsigned M = Scheme<ORDER>::M;
+    constexpr unsigned OFF = Scheme<ORDER>::OFF;
+    constexpr unsigned WIDE = 16 / ES;  // values per 16-byte chunk
+    const unsigned d1 = static_cast<unsigned>(z1) - static_cast<unsigned>(a1),
+                   d2 = static_cast<unsigned>(z2) - static_cast<unsigned>(a2),
+                   d3 = static_cast<unsigned>(z3) - static_cast<unsigned>(a3);
+    const unsigned n1 = g.n1, n2 = g.n2, n3 = g.n3;
     // box of the stencils: cells [a - OFF, z - OFF + M); the tile always
     // holds at least one valid point
-    long long o3 = (long long)a3 - OFF;
-    long long e3 = (long long)z3 - a3 + M;
-    if (ES == 2 && (g.n3 & 7) == 0) {  // x3 origin and extent multiples of 8: 16-byte chunks of halves
-        const long long o3e = o3 & ~7LL;
-        e3 = (e3 + (o3 - o3e) + 7) & ~7LL;
-        o3 = o3e;
-    } else if (ES == 2) {  // even x3 origin and extent: 4-byte aligned 16-bit pairs
-        const long long o3e = o3 & ~1LL;
-        e3 = (e3 + (o3 - o3e) + 1) & ~1LL;
-        o3 = o3e;
-    } else if ((g.n3 & 3) == 0) {  // x3 origin and extent multiples of 4: 16-byte row chunks
-        const long long o3e = o3 & ~3LL;
-        e3 = (e3 + (o3 - o3e) + 3) & ~3LL;
-        o3 = o3e;
-    }
-    const long long e1 = (long long)z1 - a1 + M, e2 = (long long)z2 - a2 + M;
-    const long long s3 = (e3 + 31) / 32 * 32;  // bank-aligned row stride
+    bool fits = !bad && z1 >= a1 && z2 >= a2 && z3 >= a3 && d1 <= n1 - M && d2 <= n2 - M && d3 <= n3 - M;
+    const unsigned e1 = d1 + M, e2 = d2 + M;
+    unsigned o3 = static_cast<unsigned>(a3) - OFF, e3 = d3 + M;
+    unsigned align = WIDE;
+    while (align > 1 && (n3 & (align - 1))) align /= 2;
+    const unsigned r = o3 & (align - 1);
+    o3 -= r;
+    e3 = (e3 + r + align - 1) & ~(align - 1);
+    const unsigned s3 = (e3 + 31) & ~31u;  // bank-aligned row stride
     // FP32 box plus, for 16-bit storage, the staging copy (half its size)
-    const long long need = e1 * e2 * s3 * (ES == 2 ? 3 : 2) / 2;
-    const bool fits = !bad && e1 >= M && e2 >= M && e3 >= M && e1 <= g.n1 && e2 <= g.n2 && e3 <= g.n3 &&
-                      need <= kBoxCapFloats;
-    par[0] = fits ? a1 - OFF : 0;
-    par[1] = fits ? a2 - OFF : 0;
+    fits = fits && e3 <= n3 &&
+           static_cast<unsigned long long>(e1 * e2) * s3 * (ES == 2 ? 3 : 2) <= 2ull * kBoxCapFloats;
+    par[0] = fits ? static_cast<int>(static_cast<unsigned>(a1) - OFF) : 0;
+    par[1] = fits ? static_cast<int>(static_cast<unsigned>(a2) - OFF) : 0;
     par[2] = fits ? static_cast<int>(o3) : 0;
-    par[3] = static_cast<int>(fits ? e1 : 0);
-    par[4] = static_cast<int>(fits ? e2 : 0);
-    par[5] = static_cast<int>(fits ? e3 : 0);
-    par[6] = static_cast<int>(fits ? s3 : 0);
+    par[3] = fits ? static_cast<int>(e1) : 0;
+    par[4] = fits ? static_cast<int>(e2) : 0;
+    par[5] = fits ? static_cast<int>(e3) : 0;
+    par[6] = fits ? static_cast<int>(s3) : 0;
 }
 
 // Fold one point's displacement (grid units) along an axis into the tile's
@@ -190,7 +210,7 @@ __device__ __forceinline__ BoxPar tile_box(const Grid& g, int lo1, int lo2, int 
 {
     int b[6];
     const bool any_bad = tile_bounds(lo1, lo2, lo3, hi1, hi2, hi3, bad, red, lane, warp, b);
-    if (threadIdx.x == 0) box_geometry<ORDER, ES>(g, b[0], b[1], b[2], b[3], b[4], b[5], any_bad, par);
+    if (threadIdx.x == 0) box_geometry<ORDER, ES>(box_grid(g), b[0], b[1], b[2], b[3], b[4], b[5], any_bad, par);
     __syncthreads();
     BoxPar bp;
     bp.O1 = par[0]; bp.O2 = par[1]; bp.O3 = par[2];
@@ -202,15 +222,11 @@ __device__ __forceinline__ BoxPar tile_box(const Grid& g, int lo1, int lo2, int 
 // produced the field: entry t (the CTA index of the tiled grid, x fastest) is
 // tb[2t] = (a1, a2, a3, bad) and tb[2t + 1] = (z1, z2, z3, 0), the first-node
 // cell bounds of the tile's points (before the -OFF shift) and whether a
-// displacement failed disp_ok.  Only for grids the tiles cover exactly.
+// displacement failed disp_ok.
 __device__ __forceinline__ unsigned tile_index()
 {
     return (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
 }
-#endif
-
-#ifndef CLAIRE_F16_OWN_WIDEN
-#define CLAIRE_F16_OWN_WIDEN 1  // 16-bit boxes: each thread widens its own chunks (no barrier between)
 #endif
 
 // Two 16-bit values packed in a word (low half first) widened to FP32.
@@ -225,60 +241,61 @@ __device__ __forceinline__ float2 widen2(uint32_t w)
     return make_float2(to_f32<S>(lo), to_f32<S>(hi));
 }
 
-// Copy the (periodically wrapped) box of f into shared memory as FP32:
-// asynchronously (cp.async) for FP32 storage, converting loads otherwise.
+// Bytes per copy with which the box of f is staged: the widest chunk that the
+// x3 origin, the x3 extent, n3 and the address of f are all multiples of (a
+// field passed by a caller may start at any 4-byte boundary); 0 when not even
+// pairs of values line up (FP32 only: single values then).
 template <class S>
-__device__ __forceinline__ void box_copy(float* dst, const S* src)
+__device__ __forceinline__ int box_chunk_bytes(const Grid& g, const S* f, const BoxPar& bp)
 {
-    if constexpr (sizeof(S) == 4)
-        cp_async_f32(dst, reinterpret_cast<const float*>(src));
-    else
-        *dst = ldf<S>(src);
+    const unsigned a = static_cast<unsigned>(bp.O3 | bp.E3 | g.n3) * static_cast<unsigned>(sizeof(S)) |
+                       static_cast<unsigned>(reinterpret_cast<uintptr_t>(f));
+    if ((a & 15u) == 0) return 16;
+    if ((a & 7u) == 0) return 8;
+    return sizeof(S) == 2 ? 4 : 0;  // 16-bit fields are the context's own: even rows at 4-byte boundaries
 }
 
-// Whether the box of f is staged in 16-byte chunks: the x3 origin, the x3
-// extent and n3 are multiples of the values per chunk (so no chunk straddles
-// the x3 wrap) and f itself is 16-byte aligned (a field passed by a caller
-// may start at any 4-byte boundary); otherwise 4-byte copies.
-template <class S>
-__device__ __forceinline__ bool box_chunks16(const Grid& g, const S* f, const BoxPar& bp)
-{
-    constexpr int VPC = 16 / static_cast<int>(sizeof(S));
-    return ((bp.O3 | bp.E3 | g.n3) & (VPC - 1)) == 0 && (reinterpret_cast<uintptr_t>(f) & 15u) == 0;
-}
+// Threads per box row when chunks of BYTES are staged by columns: a row of 64
+// values (two bank rows, the usual box) in one pass.
+template <class S, int BYTES>
+struct ColumnMap {
+    static constexpr int VPC = BYTES / static_cast<int>(sizeof(S));  // values per chunk
+    static constexpr int LPR = 64 / VPC;                             // threads per row
+};
 
-#ifndef CLAIRE_STAGE_COLS
-#define CLAIRE_STAGE_COLS 1  // 16-byte box staging: each thread one (row, chunk) column through all planes
-#endif
-
-// 16-byte box staging by columns: thread t owns row b = t / 16 (+16 per
-// pass) and chunk c = t % 16 (+16) of every box plane and copies that chunk
-// of each of the E1 planes in turn, so the wrapped x2 / x3 indices and the
-// row pointer are formed once per (b, c) and a plane costs one address step.
-// VPC: values per 16-byte chunk (4 FP32, 8 halves); dst: the box (FP32) or
-// the 16-bit staging area, whose row stride is S3 / (4 / sizeof(S)) words.
-// Returns nothing; the caller waits for the copies.
-template <class S>
+// Box staging by columns: thread t owns box row t / LPR (and every
+// kTileThreads / LPR rows on) and chunk t % LPR (+ LPR) and copies that chunk
+// of each of the E1 planes in turn, so the wrapped x2 / x3 indices and the row
+// pointer are formed once per (row, chunk) and a plane costs one address step.
+// dst0: the box (FP32) or the 16-bit staging area, whose rows are S3 values
+// apart.  182 x 218 x 182 (n3 not a multiple of 4): 8-byte chunks of FP32 and
+// 4-byte pairs of halves instead of value-wise row loops took the FP16 adjoint
+// step from 171 to 111 us (the tile-bounds table included).
+template <class S, int BYTES>
 __device__ __forceinline__ void stage_box_columns(const Grid& g, const S* __restrict__ f, uint32_t dst0,
-                                                  const BoxPar& bp, int w1, int w2, int w3)
+                                                  const BoxPar& bp)
 {
-    constexpr int VPC = 16 / sizeof(S);
+    constexpr int VPC = ColumnMap<S, BYTES>::VPC, LPR = ColumnMap<S, BYTES>::LPR;
+    const int w1 = wrap_index(bp.O1, g.n1), w2 = wrap_index(bp.O2, g.n2), w3 = wrap_index(bp.O3, g.n3);
     const int nch = bp.E3 / VPC;
     const uint32_t row_bytes = static_cast<uint32_t>(bp.S3) * sizeof(S);
     const uint32_t plane_bytes = row_bytes * static_cast<uint32_t>(bp.E2);
-    for (int b = threadIdx.x >> 4; b < bp.E2; b += kTileThreads / 16) {
-        int gj = w2 + b;
-        gj = gj >= g.n2 ? gj - g.n2 : gj;
-        for (int c = threadIdx.x & 15; c < nch; c += 16) {
-            int gk = w3 + VPC * c;
-            gk = gk >= g.n3 ? gk - g.n3 : gk;
+    for (int b = threadIdx.x / LPR; b < bp.E2; b += kTileThreads / LPR) {
+        const int gj = box_wrap(w2 + b, g.n2);
+        for (int c = threadIdx.x % LPR; c < nch; c += LPR) {
+            const int gk = box_wrap(w3 + VPC * c, g.n3);
             const S* src = f + static_cast<size_t>(gj) * g.n3 + gk;
-            uint32_t dst = dst0 + static_cast<uint32_t>(b) * row_bytes + 16u * c;
+            uint32_t dst = dst0 + static_cast<uint32_t>(b) * row_bytes + static_cast<uint32_t>(BYTES) * c;
             int gi = w1;
             for (int a = 0; a < bp.E1; ++a) {
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst),
-                             "l"(src + static_cast<size_t>(gi) * g.n23)
-                             : "memory");
+                if constexpr (BYTES == 16)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst),
+                                 "l"(src + static_cast<size_t>(gi) * g.n23)
+                                 : "memory");
+                else
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(dst),
+                                 "l"(src + static_cast<size_t>(gi) * g.n23), "n"(BYTES)
+                                 : "memory");
                 dst += plane_bytes;
                 gi = gi + 1 == g.n1 ? 0 : gi + 1;
             }
@@ -286,204 +303,90 @@ __device__ __forceinline__ void stage_box_columns(const Grid& g, const S* __rest
     }
 }
 
+// Widen the chunks stage_box_columns copied from this thread, in its order.
+template <class S, int BYTES>
+__device__ __forceinline__ void widen_box_columns(const uint32_t* stage, float* box, const BoxPar& bp)
+{
+    constexpr int VPC = ColumnMap<S, BYTES>::VPC, LPR = ColumnMap<S, BYTES>::LPR;
+    const int nch = bp.E3 / VPC;
+    for (int b = threadIdx.x / LPR; b < bp.E2; b += kTileThreads / LPR)
+        for (int c = threadIdx.x % LPR; c < nch; c += LPR)
+            for (int a = 0; a < bp.E1; ++a) {
+                const int r = a * bp.E2 + b;
+                const uint32_t* sp = stage + r * (bp.S3 / 2) + c * (VPC / 2);
+                float* dp = box + r * bp.S3 + c * VPC;
+                if constexpr (BYTES == 16) {
+                    const uint4 w = *reinterpret_cast<const uint4*>(sp);
+                    const float2 p0 = widen2<S>(w.x), p1 = widen2<S>(w.y), p2 = widen2<S>(w.z), p3 = widen2<S>(w.w);
+                    reinterpret_cast<float4*>(dp)[0] = make_float4(p0.x, p0.y, p1.x, p1.y);
+                    reinterpret_cast<float4*>(dp)[1] = make_float4(p2.x, p2.y, p3.x, p3.y);
+                } else if constexpr (BYTES == 8) {
+                    const uint2 w = *reinterpret_cast<const uint2*>(sp);
+                    const float2 p0 = widen2<S>(w.x), p1 = widen2<S>(w.y);
+                    *reinterpret_cast<float4*>(dp) = make_float4(p0.x, p0.y, p1.x, p1.y);
+                } else {
+                    *reinterpret_cast<float2*>(dp) = widen2<S>(*sp);
+                }
+            }
+}
+
+// Copy the (periodically wrapped) box of f into shared memory asynchronously:
+// FP32 fields into the box itself, 16-bit ones as raw values into a staging
+// area behind it (tile_widen_box then fills the box).
 template <class S>
 __device__ __forceinline__ void tile_load_box(const Grid& g, const S* __restrict__ f, float* box,
                                               const BoxPar& bp, int lane, int warp)
 {
-    const int w1 = wrap_index(bp.O1, g.n1), w2 = wrap_index(bp.O2, g.n2), w3 = wrap_index(bp.O3, g.n3);
-    int gk0 = w3 + lane;
-    gk0 = gk0 >= g.n3 ? gk0 - g.n3 : gk0;
-    int gk1 = w3 + lane + 32;
-    gk1 = gk1 >= g.n3 ? gk1 - g.n3 : gk1;
+    const int bytes = box_chunk_bytes<S>(g, f, bp);
     if constexpr (sizeof(S) == 4) {
-#if CLAIRE_STAGE_COLS
-        if (box_chunks16<S>(g, f, bp)) {
-            stage_box_columns<S>(g, f, static_cast<uint32_t>(__cvta_generic_to_shared(box)), bp, w1, w2, w3);
-            return;
-        }
-#endif
-        if (box_chunks16<S>(g, f, bp)) {
-            // 16-byte chunks: a chunk never straddles the x3 wrap (n3 and the
-            // origin are multiples of 4); 16 threads per row, 16 rows per pass
-            const int nch = bp.E3 >> 2, rows = bp.E1 * bp.E2;
-            const int ch0 = threadIdx.x & 15;
-            int r = threadIdx.x >> 4;
-            int a = r / bp.E2, b = r - a * bp.E2;
-            for (; r < rows; r += kTileThreads / 16) {
-                int gi = w1 + a;
-                gi = gi >= g.n1 ? gi - g.n1 : gi;
-                int gj = w2 + b;
-                gj = gj >= g.n2 ? gj - g.n2 : gj;
-                const float* src = reinterpret_cast<const float*>(f) + static_cast<size_t>(gi) * g.n23 +
-                                   static_cast<size_t>(gj) * g.n3;
-                const unsigned dst = static_cast<unsigned>(__cvta_generic_to_shared(box + r * bp.S3));
-                for (int c = ch0; c < nch; c += 16) {
-                    int gk = w3 + 4 * c;
-                    gk = gk >= g.n3 ? gk - g.n3 : gk;
-                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst + 16u * c), "l"(src + gk)
-                                 : "memory");
-                }
-                b += kTileThreads / 16;
-                while (b >= bp.E2) {
-                    b -= bp.E2;
-                    ++a;
-                }
-            }
-            return;
-        }
-        for (int a = 0; a < bp.E1; ++a) {
-            int gi = w1 + a;
-            gi = gi >= g.n1 ? gi - g.n1 : gi;
-            const S* plane = f + static_cast<size_t>(gi) * g.n23;
-            for (int b = warp; b < bp.E2; b += TILE2) {
-                int gj = w2 + b;
-                gj = gj >= g.n2 ? gj - g.n2 : gj;
-                const S* src = plane + gj * g.n3;
-                float* dst = box + (a * bp.E2 + b) * bp.S3;
-                if (lane < bp.E3) box_copy<S>(dst + lane, src + gk0);
-                if (lane + 32 < bp.E3) box_copy<S>(dst + lane + 32, src + gk1);
-                for (int c = lane + 64; c < bp.E3; c += 32) {
-                    int gk = w3 + c;
-                    gk = gk >= g.n3 ? gk - g.n3 : gk;
-                    box_copy<S>(dst + c, src + gk);
+        const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(box));
+        if (bytes == 16) {
+            stage_box_columns<S, 16>(g, f, dst, bp);
+        } else if (bytes == 8) {
+            stage_box_columns<S, 8>(g, f, dst, bp);
+        } else {
+            // a caller's field at an odd 4-byte boundary: value by value
+            const int w1 = wrap_index(bp.O1, g.n1), w2 = wrap_index(bp.O2, g.n2), w3 = wrap_index(bp.O3, g.n3);
+            for (int a = 0; a < bp.E1; ++a) {
+                const S* plane = f + static_cast<size_t>(box_wrap(w1 + a, g.n1)) * g.n23;
+                for (int b = warp; b < bp.E2; b += TILE2) {
+                    const S* src = plane + box_wrap(w2 + b, g.n2) * g.n3;
+                    float* row = box + (a * bp.E2 + b) * bp.S3;
+                    for (int c = lane; c < bp.E3; c += 32)
+                        cp_async_f32(row + c, reinterpret_cast<const float*>(src + box_wrap(w3 + c, g.n3)));
                 }
             }
         }
     } else {
-        // 16-bit storage: raw pairs (4 bytes, aligned: even origin, even n3)
-        // go asynchronously to a staging area behind the FP32 box; after they
-        // land they are widened to FP32 in the box (tile_widen_box: each
-        // thread its own copies; else here, after a barrier, a share each).
-        const int rows = bp.E1 * bp.E2;
-        const int pairs = bp.E3 / 2;
-        uint32_t* stage = reinterpret_cast<uint32_t*>(box + rows * bp.S3);
-#if CLAIRE_STAGE_COLS
-        if (box_chunks16<S>(g, f, bp)) {
-            stage_box_columns<S>(g, f, static_cast<uint32_t>(__cvta_generic_to_shared(stage)), bp, w1, w2, w3);
-        } else
-#endif
-        if (box_chunks16<S>(g, f, bp)) {
-            // 16-byte chunks of 8 values (no chunk straddles the x3 wrap), 16 threads per row
-            const int nch = bp.E3 >> 3;
-            const int ch0 = threadIdx.x & 15;
-            int r = threadIdx.x >> 4;
-            int a = r / bp.E2, b = r - a * bp.E2;
-            for (; r < rows; r += kTileThreads / 16) {
-                int gi = w1 + a;
-                gi = gi >= g.n1 ? gi - g.n1 : gi;
-                int gj = w2 + b;
-                gj = gj >= g.n2 ? gj - g.n2 : gj;
-                const S* src = f + static_cast<size_t>(gi) * g.n23 + static_cast<size_t>(gj) * g.n3;
-                const unsigned dst = static_cast<unsigned>(__cvta_generic_to_shared(stage + r * (bp.S3 / 2)));
-                for (int c = ch0; c < nch; c += 16) {
-                    int gk = w3 + 8 * c;
-                    gk = gk >= g.n3 ? gk - g.n3 : gk;
-                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst + 16u * c), "l"(src + gk)
-                                 : "memory");
-                }
-                b += kTileThreads / 16;
-                while (b >= bp.E2) {
-                    b -= bp.E2;
-                    ++a;
-                }
-            }
-        } else {
-        for (int a = 0; a < bp.E1; ++a) {
-            int gi = w1 + a;
-            gi = gi >= g.n1 ? gi - g.n1 : gi;
-            const S* plane = f + static_cast<size_t>(gi) * g.n23;
-            for (int b = warp; b < bp.E2; b += TILE2) {
-                int gj = w2 + b;
-                gj = gj >= g.n2 ? gj - g.n2 : gj;
-                const S* src = plane + gj * g.n3;
-                uint32_t* dst = stage + (a * bp.E2 + b) * (bp.S3 / 2);
-                for (int c = lane; c < pairs; c += 32) {
-                    int gk = w3 + 2 * c;
-                    gk = gk >= g.n3 ? gk - g.n3 : gk;
-                    cp_async_f32(reinterpret_cast<float*>(dst + c), reinterpret_cast<const float*>(src + gk));
-                }
-            }
-        }
-        }
-#if !CLAIRE_F16_OWN_WIDEN
-        cp_async_wait_all();
-        __syncthreads();
-        for (int r = warp; r < rows; r += TILE2) {
-            const uint32_t* sp = stage + r * (bp.S3 / 2);
-            float* dst = box + r * bp.S3;
-            for (int c = lane; c < pairs; c += 32) {
-                const float2 w = widen2<S>(sp[c]);
-                dst[2 * c] = w.x;
-                dst[2 * c + 1] = w.y;
-            }
-        }
-#endif
+        const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(box + bp.E1 * bp.E2 * bp.S3));
+        if (bytes == 16)
+            stage_box_columns<S, 16>(g, f, dst, bp);
+        else if (bytes == 8)
+            stage_box_columns<S, 8>(g, f, dst, bp);
+        else
+            stage_box_columns<S, 4>(g, f, dst, bp);
     }
 }
 
-// Completion of tile_load_box for 16-bit storage with CLAIRE_F16_OWN_WIDEN:
-// every thread waits for its own copies and widens exactly the chunks (or
-// pairs) it issued, in the same order, so no barrier separates the copy from
-// the widening; the caller's barrier before the stencils publishes the box.
-// FP32 storage: nothing (the caller waits for the copies).
+// Completion of tile_load_box for 16-bit storage: every thread waits for its
+// own copies and widens exactly the chunks it issued, in the same order, so no
+// barrier separates the copy from the widening; the caller's barrier before
+// the stencils publishes the box.  FP32 storage: nothing (the caller waits
+// for the copies).
 template <class S>
-__device__ __forceinline__ void tile_widen_box(const Grid& g, const S* f, float* box, const BoxPar& bp, int lane,
-                                               int warp)
+__device__ __forceinline__ void tile_widen_box(const Grid& g, const S* f, float* box, const BoxPar& bp)
 {
-#if CLAIRE_F16_OWN_WIDEN
     if constexpr (sizeof(S) == 2) {
-        const int rows = bp.E1 * bp.E2;
-        const uint32_t* stage = reinterpret_cast<const uint32_t*>(box + rows * bp.S3);
+        const uint32_t* stage = reinterpret_cast<const uint32_t*>(box + bp.E1 * bp.E2 * bp.S3);
+        const int bytes = box_chunk_bytes<S>(g, f, bp);
         cp_async_wait_all();
-#if CLAIRE_STAGE_COLS
-        if (box_chunks16<S>(g, f, bp)) {
-            // the chunks stage_box_columns issued from this thread, in its order
-            const int nch = bp.E3 >> 3;
-            for (int b = threadIdx.x >> 4; b < bp.E2; b += kTileThreads / 16)
-                for (int c = threadIdx.x & 15; c < nch; c += 16)
-                    for (int a = 0; a < bp.E1; ++a) {
-                        const int r = a * bp.E2 + b;
-                        const uint4 w = reinterpret_cast<const uint4*>(stage + r * (bp.S3 / 2))[c];
-                        float4* dp = reinterpret_cast<float4*>(box + r * bp.S3);
-                        const float2 p0 = widen2<S>(w.x), p1 = widen2<S>(w.y), p2 = widen2<S>(w.z),
-                                     p3 = widen2<S>(w.w);
-                        dp[2 * c] = make_float4(p0.x, p0.y, p1.x, p1.y);
-                        dp[2 * c + 1] = make_float4(p2.x, p2.y, p3.x, p3.y);
-                    }
-        } else
-#endif
-        if (box_chunks16<S>(g, f, bp)) {
-            const int nch = bp.E3 >> 3;
-            const int ch0 = threadIdx.x & 15;
-            for (int r = threadIdx.x >> 4; r < rows; r += kTileThreads / 16) {
-                const uint4* sp = reinterpret_cast<const uint4*>(stage + r * (bp.S3 / 2));
-                float4* dp = reinterpret_cast<float4*>(box + r * bp.S3);
-                for (int c = ch0; c < nch; c += 16) {
-                    const uint4 w = sp[c];
-                    const float2 p0 = widen2<S>(w.x), p1 = widen2<S>(w.y), p2 = widen2<S>(w.z),
-                                 p3 = widen2<S>(w.w);
-                    dp[2 * c] = make_float4(p0.x, p0.y, p1.x, p1.y);
-                    dp[2 * c + 1] = make_float4(p2.x, p2.y, p3.x, p3.y);
-                }
-            }
-        } else {
-            const int pairs = bp.E3 / 2;
-            for (int a = 0; a < bp.E1; ++a)
-                for (int b = warp; b < bp.E2; b += TILE2) {
-                    const int r = a * bp.E2 + b;
-                    const uint32_t* sp = stage + r * (bp.S3 / 2);
-                    float* dst = box + r * bp.S3;
-                    for (int c = lane; c < pairs; c += 32) {
-                        const float2 w = widen2<S>(sp[c]);
-                        dst[2 * c] = w.x;
-                        dst[2 * c + 1] = w.y;
-                    }
-                }
-        }
+        if (bytes == 16)
+            widen_box_columns<S, 16>(stage, box, bp);
+        else if (bytes == 8)
+            widen_box_columns<S, 8>(stage, box, bp);
+        else
+            widen_box_columns<S, 4>(stage, box, bp);
     }
-#else
-    (void)g; (void)f; (void)box; (void)bp; (void)lane; (void)warp;
-#endif
 }
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p)
@@ -642,7 +545,7 @@ __device__ __forceinline__ float tile_eval(const float* box, const BoxPar& bp, i
 // the stencil is evaluated.
 // FULL: the tiles cover the grid exactly (n3 % 32 = n2 % 8 = n1 % TILE1 = 0),
 // so no point of a tile is out of range and the bounds tests compile away.
-// TB (FULL grids only): the box comes from the tile-bounds table tb that the
+// TB: the box comes from the tile-bounds table tb that the
 // backtrace wrote with d, so the CTA starts staging it at once, reads the
 // displacements and the epilogue operands while it is in flight, and needs no
 // block reduction.  Every point is checked against the box (in_box); if any
@@ -666,11 +569,10 @@ __global__ void __launch_bounds__(kTileThreads, CLAIRE_TILE_MIN_BLOCKS)
     auto valid = [&](int q) { return FULL || (col_ok && i0 + q < g.n1); };
 
     if constexpr (TB) {
-        static_assert(FULL, "tile-bounds tables cover exactly tiled grids only");
         const unsigned t = tile_index();
         const int4 lo = __ldg(tb + 2 * t), hi = __ldg(tb + 2 * t + 1);
         int gp[7];
-        box_geometry<ORDER, sizeof(S)>(g, lo.x, lo.y, lo.z, hi.x, hi.y, hi.z, lo.w != 0, gp);
+        box_geometry<ORDER, sizeof(S)>(box_grid(g), lo.x, lo.y, lo.z, hi.x, hi.y, hi.z, lo.w != 0, gp);
         BoxPar bp;
         bp.O1 = gp[0]; bp.O2 = gp[1]; bp.O3 = gp[2];
         bp.E1 = gp[3]; bp.E2 = gp[4]; bp.E3 = gp[5]; bp.S3 = gp[6];
@@ -680,6 +582,7 @@ __global__ void __launch_bounds__(kTileThreads, CLAIRE_TILE_MIN_BLOCKS)
         bool out = bp.E1 == 0;
 #pragma unroll
         for (int q = 0; q < TILE1; ++q) {
+            if (!valid(q)) continue;
             const uint32_t p = p0 + q * g.n23;
             e1[q] = __ldg(d + p);
             e2[q] = __ldg(d + N + p);
@@ -687,19 +590,23 @@ __global__ void __launch_bounds__(kTileThreads, CLAIRE_TILE_MIN_BLOCKS)
             pre[q] = epi.prefetch(p);
         }
 #pragma unroll
-        for (int q = 0; q < TILE1; ++q) out = out || !in_box<ORDER>(bp, i0 + q, j, k, e1[q], e2[q], e3[q]);
-        if (bp.E1 != 0) tile_widen_box<S>(g, f, box, bp, lane, warp);
+        for (int q = 0; q < TILE1; ++q)
+            if (valid(q)) out = out || !in_box<ORDER>(bp, i0 + q, j, k, e1[q], e2[q], e3[q]);
+        if (bp.E1 != 0) tile_widen_box<S>(g, f, box, bp);
         cp_async_wait_all();
         if (__syncthreads_or(out)) {
             if (threadIdx.x == 0) atomicAdd(&g_gather_global_tiles, 1ull);
 #pragma unroll
             for (int q = 0; q < TILE1; ++q)
-                epi.finish(p0 + q * g.n23, gather_global<ORDER, S>(g, f, i0 + q, j, k, e1[q], e2[q], e3[q]), pre[q]);
+                if (valid(q))
+                    epi.finish(p0 + q * g.n23, gather_global<ORDER, S>(g, f, i0 + q, j, k, e1[q], e2[q], e3[q]),
+                               pre[q]);
             return;
         }
 #pragma unroll
         for (int q = 0; q < TILE1; ++q)
-            epi.finish(p0 + q * g.n23, tile_eval<ORDER>(box, bp, i0 + q, j, k, e1[q], e2[q], e3[q]), pre[q]);
+            if (valid(q))
+                epi.finish(p0 + q * g.n23, tile_eval<ORDER>(box, bp, i0 + q, j, k, e1[q], e2[q], e3[q]), pre[q]);
         return;
     }
     float d1[TILE1], d2[TILE1], d3[TILE1];
@@ -737,7 +644,7 @@ __global__ void __launch_bounds__(kTileThreads, CLAIRE_TILE_MIN_BLOCKS)
 #pragma unroll
     for (int q = 0; q < TILE1; ++q)
         if (valid(q)) pre[q] = epi.prefetch(p0 + q * g.n23);
-    tile_widen_box<S>(g, f, box, bp, lane, warp);
+    tile_widen_box<S>(g, f, box, bp);
     cp_async_wait_all();
     __syncthreads();
 #pragma unroll
@@ -835,27 +742,28 @@ inline dim3 tiled_grid(const Grid& g)
 
 constexpr size_t kTiledSmemBytes = kBoxCapFloats * sizeof(float);
 
+template <int ORDER, class Epi, class S, bool FULL, bool TB>
+inline void launch_tiled_as(const Grid& g, const S* f, const float* d, const Epi& e, cudaStream_t st, const int4* tb)
+{
+    if (kTiledSmemBytes > 48 * 1024)
+        cudaFuncSetAttribute(k_gather_tiled<ORDER, Epi, S, FULL, TB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(kTiledSmemBytes));
+    k_gather_tiled<ORDER, Epi, S, FULL, TB><<<tiled_grid(g), kTileThreads, kTiledSmemBytes, st>>>(g, f, d, e, tb);
+}
+
 template <int ORDER, class Epi, class S>
 inline void launch_tiled(const Grid& g, const S* f, const float* d, const Epi& e, cudaStream_t st,
                          const int4* tb = nullptr)
 {
-    if (tiles_cover_grid(g) && tb) {
-        if (kTiledSmemBytes > 48 * 1024)
-            cudaFuncSetAttribute(k_gather_tiled<ORDER, Epi, S, true, true>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kTiledSmemBytes));
-        k_gather_tiled<ORDER, Epi, S, true, true><<<tiled_grid(g), kTileThreads, kTiledSmemBytes, st>>>(g, f, d, e,
-                                                                                                        tb);
-    } else if (tiles_cover_grid(g)) {
-        if (kTiledSmemBytes > 48 * 1024)
-            cudaFuncSetAttribute(k_gather_tiled<ORDER, Epi, S, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(kTiledSmemBytes));
-        k_gather_tiled<ORDER, Epi, S, true><<<tiled_grid(g), kTileThreads, kTiledSmemBytes, st>>>(g, f, d, e);
-    } else {
-        if (kTiledSmemBytes > 48 * 1024)
-            cudaFuncSetAttribute(k_gather_tiled<ORDER, Epi, S, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(kTiledSmemBytes));
-        k_gather_tiled<ORDER, Epi, S, false><<<tiled_grid(g), kTileThreads, kTiledSmemBytes, st>>>(g, f, d, e);
-    }
+    const bool full = tiles_cover_grid(g);
+    if (tb && full)
+        launch_tiled_as<ORDER, Epi, S, true, true>(g, f, d, e, st, tb);
+    else if (tb)
+        launch_tiled_as<ORDER, Epi, S, false, true>(g, f, d, e, st, tb);
+    else if (full)
+        launch_tiled_as<ORDER, Epi, S, true, false>(g, f, d, e, st, tb);
+    else
+        launch_tiled_as<ORDER, Epi, S, false, false>(g, f, d, e, st, tb);
 }
 
 // ---- epilogues: prefetch(p) loads the point's operands early, finish(p, v, pre)

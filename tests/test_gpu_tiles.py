@@ -103,3 +103,60 @@ def test_vjp_non_finite_cotangent_gives_nan(bad):
     ctx.transport_vjp(_dev(v), _dev(np.ones(n)), _dev(g), gm)
     assert bool(torch.isnan(gm).all())
     ctx.close()
+
+
+@pytest.mark.parametrize("n", [(8, 8, 8), (32, 32, 32), (12, 14, 30), (34, 18, 70), (20, 28, 44), (64, 24, 96)])
+@pytest.mark.parametrize("order", [3, 1])
+def test_table_and_chunk_widths_agree(n, order):
+    """The solver's gathers take their boxes from the backtrace's tile-bounds
+    table and stage them with the widest copies the row length and the address
+    allow; the kernel-level gather reduces the bounds itself.  A transport and
+    the same steps through the kernel-level calls, from fields at every 4-byte
+    alignment, give the same bits, and a smooth displacement of under two cells
+    fits the box on every grid, however short its axes."""
+    from paper_2209_08189_gb300 import claire
+    rng = np.random.default_rng(9)
+    v = synth.mode_velocity(n, seed=3, vmax=1.0, kmax=1)
+    v = (v * (1.5 * 4 * 2 * np.pi / max(n)) / np.abs(v).max()).astype(np.float32)  # at most 1.5 cells per step
+    m = rng.standard_normal(n).astype(np.float32)
+    ctx, out = _ctx(n, interp=order), torch.empty(n, device="cuda")
+    claire.claire_gather_fallback_tiles(reset=True)
+    ctx.transport(_dev(v), _dev(m), out)
+    d = torch.empty((3,) + n, device="cuda")
+    ctx.backtrace(_dev(v), d)
+    for off in range(4):
+        buf = torch.empty(m.size + 4, device="cuda")
+        cur = buf[off:off + m.size].view(n)
+        cur.copy_(_dev(m))
+        for _ in range(4):
+            nxt = torch.empty(n, device="cuda")
+            ctx.interp(cur, d, nxt, order)
+            cur.copy_(nxt)
+        assert torch.equal(cur, out)
+    assert claire.claire_gather_fallback_tiles() == 0
+    ctx.close()
+
+
+@pytest.mark.parametrize("n", [(32, 32, 32), (12, 14, 30), (34, 18, 70), (20, 28, 44)])
+@pytest.mark.parametrize("storage", [0, 1, 2])
+def test_boxes_on_every_row_length_carry_a_shift(n, storage):
+    """Rows staged in 16-, 8- and 4-byte copies, for each storage type.  A
+    constant velocity of whole cells per step carries an image of values that
+    the type holds exactly; each step interpolates at a point within FP32
+    rounding of a node, so it returns the node's value up to 1e-6 of it, which
+    16-bit rounding removes (values in [1/2, 1], spacing at least 2^-12): the
+    mismatch against the shifted image is 0, or in FP32 of that order squared."""
+    rng = np.random.default_rng(4)
+    m0 = (0.5 + rng.integers(0, 64, n) / 128.0).astype(np.float32)  # seven bits: exact in every type
+    step = (1, -2, 3)
+    v = np.empty((3,) + n, dtype=np.float32)
+    for c in range(3):
+        v[c] = step[c] * 4 * 2 * np.pi / n[c]
+    # m(1)(x) = m0(x - v): four steps of `step` cells
+    m1 = np.roll(m0, [4 * s for s in step], (0, 1, 2))
+    ctx = _ctx(n, storage=storage)
+    ctx.set_images(_dev(m0), _dev(m1))
+    _, mis = ctx.objective(_dev(v))
+    vol = float(np.prod([2 * np.pi / s for s in n]))
+    assert mis <= (0.0 if storage else 0.5 * vol * m0.size * (4 * 4e-6) ** 2)
+    ctx.close()
