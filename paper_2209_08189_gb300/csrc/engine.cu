@@ -137,7 +137,9 @@ struct claire_ctx {
     cufftComplex* rh = nullptr;           // PCG residual, Fourier space
     double* partials = nullptr;           // 2 * red_blocks
     double* dres = nullptr;               // device scalars
-    double* hres = nullptr;               // pinned host scalars
+    double* hres = nullptr;               // pinned host scalars, written by the reductions
+    double* hres_dev = nullptr;           // their device address
+    unsigned* ticket = nullptr;           // finished blocks of the running reduction (device, 0 at rest)
 
     // reverse-mode transport scratch, allocated by the first claire_transport_vjp
     // spectrum of the Gauss-Newton iterate inside claire_register (spectral_iterate = 1):
@@ -483,22 +485,43 @@ void collect_timing(claire_ctx* c)
 // building blocks on the context's stream
 // ---------------------------------------------------------------------------
 
-claire_status sync_scalars(claire_ctx* c, int count)
+// Wait for the scalars that the reductions write into hres.
+claire_status sync_scalars(claire_ctx* c)
 {
-    (void)count;
-    CL_CUDA(c, cudaMemcpyAsync(c->hres, c->dres, 16 * sizeof(double), cudaMemcpyDeviceToHost,
-                               c->stream));
     CL_CUDA(c, cudaStreamSynchronize(c->stream));
     return CLAIRE_OK;
 }
 
-// dres[slot] = scale * sum x*y  (device only; no sync)
+// Totals into dres[slot] (and slot + 1) and their host mirror, times scale.
+Reduction reduction(claire_ctx* c, int slot, double scale = 1.0)
+{
+    return Reduction{c->partials, c->red_blocks, scale, c->dres + slot, c->hres_dev + slot, c->ticket};
+}
+
+// Pinned scalars, their device address and the ticket (the last device scalar).
+bool make_scalars(claire_ctx* c)
+{
+    if (cudaMallocHost(&c->hres, 16 * sizeof(double)) != cudaSuccess) {
+        cudaGetLastError();
+        c->hres = nullptr;
+        return false;
+    }
+    void* dev = nullptr;
+    if (cudaHostGetDevicePointer(&dev, c->hres, 0) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    c->hres_dev = static_cast<double*>(dev);
+    c->ticket = reinterpret_cast<unsigned*>(c->dres + 15);
+    return true;
+}
+
+// dres[slot] = scale * sum x*y  (no sync)
 claire_status dot_async(claire_ctx* c, const float* x, const float* y, size_t n, double scale,
                         int slot)
 {
-    KTimer t(c, KK_REDUCE, 8.0 * n, 0, 2);
-    launch_dot_partial(x, y, n, c->partials, c->red_blocks, c->stream);
-    launch_final_sum(c->partials, c->red_blocks, scale, c->dres + slot, c->stream);
+    KTimer t(c, KK_REDUCE, 8.0 * n, 0);
+    launch_dot(x, y, n, reduction(c, slot, scale), c->stream);
     CL_LAUNCHED(c);
     return CLAIRE_OK;
 }
@@ -507,7 +530,7 @@ claire_status dot(claire_ctx* c, const float* x, const float* y, size_t n, doubl
 {
     PhaseScope ps(c, CLAIRE_PHASE_VECTOR);
     CL_TRY(dot_async(c, x, y, n, c->hvol, 0));
-    CL_TRY(sync_scalars(c, 1));
+    CL_TRY(sync_scalars(c));
     *out = c->hres[0];
     if (!std::isfinite(*out)) return fail(c, CLAIRE_ENONFINITE, "non-finite inner product");
     return CLAIRE_OK;
@@ -737,14 +760,13 @@ claire_status gradient_at_lin(claire_ctx* c, float* g)
     {
         PhaseScope ps(c, CLAIRE_PHASE_VECTOR);
         CL_TRY(dot_async(c, c->v, g, 3 * N, 0.5 * c->hvol, 0));
-        KTimer t(c, KK_REDUCE, 8.0 * N, 0, 2);
-        launch_sqdiff_partial(at(c, c->m, c->nt * N), c->m1, N, c->partials, c->red_blocks, c->sto, c->stream);
-        launch_final_sum(c->partials, c->red_blocks, 0.5 * c->hvol, c->dres + 1, c->stream);
+        KTimer t(c, KK_REDUCE, 8.0 * N, 0);
+        launch_sqdiff(at(c, c->m, c->nt * N), c->m1, N, c->sto, reduction(c, 1, 0.5 * c->hvol), c->stream);
         CL_LAUNCHED(c);
     }
     CL_TRY(adjoint_and_body(c, c->m1, at(c, c->m, c->nt * N), g));
     if (c->o.grad_form == 1) CL_TRY(spectral(c, g, g, SPEC_K));
-    CL_TRY(sync_scalars(c, 2));
+    CL_TRY(sync_scalars(c));
     c->reg_lin = c->hres[0];
     c->mis_lin = c->hres[1];
     c->J_lin = c->reg_lin + c->mis_lin;
@@ -858,12 +880,11 @@ claire_status objective_at(claire_ctx* c, const float* v, double* J, double* mis
     CL_TRY(spectral(c, v, c->r, SPEC_REG));
     CL_TRY(dot_async(c, v, c->r, 3 * N, 0.5 * c->hvol, 0));
     {
-        KTimer t(c, KK_REDUCE, 8.0 * N, 0, 2);
-        launch_sqdiff_partial(src, c->m1, N, c->partials, c->red_blocks, c->sto, c->stream);
-        launch_final_sum(c->partials, c->red_blocks, 0.5 * c->hvol, c->dres + 1, c->stream);
+        KTimer t(c, KK_REDUCE, 8.0 * N, 0);
+        launch_sqdiff(src, c->m1, N, c->sto, reduction(c, 1, 0.5 * c->hvol), c->stream);
         CL_LAUNCHED(c);
     }
-    CL_TRY(sync_scalars(c, 2));
+    CL_TRY(sync_scalars(c));
     if (mis) *mis = c->hres[1];
     if (J) *J = c->hres[0] + c->hres[1];
     if (!std::isfinite(c->hres[0] + c->hres[1]))
@@ -889,16 +910,11 @@ claire_status detj_of(claire_ctx* c, const float* v, double* lo, double* hi)
         std::swap(a, b);
     }
     {
-        KTimer t(c, KK_DETJ, 12.0 * N, 0, 2);
-        launch_detj_minmax(c->grid, a, c->partials + c->red_blocks, c->partials, c->red_blocks,
-                           c->stream);
-        launch_final_minmax(c->partials + c->red_blocks, c->partials, c->red_blocks, c->dres + 4,
-                            c->stream);
+        KTimer t(c, KK_DETJ, 12.0 * N, 0);
+        launch_detj_minmax(c->grid, a, reduction(c, 4), c->stream);
         CL_LAUNCHED(c);
     }
-    CL_CUDA(c, cudaMemcpyAsync(c->hres + 4, c->dres + 4, 2 * sizeof(double), cudaMemcpyDeviceToHost,
-                               c->stream));
-    CL_CUDA(c, cudaStreamSynchronize(c->stream));
+    CL_TRY(sync_scalars(c));
     *lo = c->hres[4];
     *hi = c->hres[5];
     return CLAIRE_OK;
@@ -907,14 +923,11 @@ claire_status detj_of(claire_ctx* c, const float* v, double* lo, double* hi)
 claire_status cfl_of(claire_ctx* c, const float* v, double* cfl)
 {
     {
-        KTimer t(c, KK_REDUCE, 12.0 * c->N, 0, 2);
-        launch_maxnorm3_partial(v, c->N, c->partials, c->red_blocks, c->stream);
-        launch_final_max(c->partials, c->red_blocks, c->dres + 6, c->stream);
+        KTimer t(c, KK_REDUCE, 12.0 * c->N, 0);
+        launch_maxnorm3(v, c->N, reduction(c, 7), c->stream);
         CL_LAUNCHED(c);
     }
-    CL_CUDA(c, cudaMemcpyAsync(c->hres + 6, c->dres + 6, 2 * sizeof(double), cudaMemcpyDeviceToHost,
-                               c->stream));
-    CL_CUDA(c, cudaStreamSynchronize(c->stream));
+    CL_TRY(sync_scalars(c));
     const double hmin = std::min(c->grid.h1, std::min(c->grid.h2, c->grid.h3));
     *cfl = std::sqrt(c->hres[7]) * c->dt / hmin;
     return CLAIRE_OK;
@@ -930,15 +943,18 @@ claire_status screen_velocity(claire_ctx* c, const float* v)
     return CLAIRE_OK;
 }
 
-// Final sums of the two partial-sum arrays of a Fourier-space PCG kernel
-// into dres[0], dres[1] (scaled to discrete inner products), then synchronise.
+// Totals of a Fourier-space PCG kernel into dres[slot], scaled to discrete
+// inner products (Parseval on scaled spectra).
+Reduction fs_reduction(claire_ctx* c, int slot)
+{
+    return reduction(c, slot, c->hvol * static_cast<double>(c->N));
+}
+
+// Wait for the first `count` of them (slot 0 on).
 claire_status fs_sums(claire_ctx* c, int count)
 {
-    const double scale = c->hvol * static_cast<double>(c->N);  // Parseval on scaled spectra
-    launch_final_sum(c->partials, c->red_blocks, scale, c->dres, c->stream);
-    if (count > 1) launch_final_sum(c->partials + c->red_blocks, c->red_blocks, scale, c->dres + 1, c->stream);
     CL_LAUNCHED(c);
-    CL_TRY(sync_scalars(c, count));
+    CL_TRY(sync_scalars(c));
     for (int i = 0; i < count; ++i)
         if (!std::isfinite(c->hres[i])) return fail(c, CLAIRE_ENONFINITE, "non-finite PCG inner product");
     return CLAIRE_OK;
@@ -1075,20 +1091,17 @@ claire_status tl_apply(claire_ctx* c, const cufftComplex* rf, cufftComplex* zf, 
 {
     TwoLevel* t = c->tl2;
     const SpectralOp op = c->o.grad_form == 1 ? SPEC_AINV : SPEC_INV;
-    const int rb = c->red_blocks;
     PhaseScope ps(c, CLAIRE_PHASE_SPECTRAL);
     *its = 0;
     {
-        KTimer kt(c, KK_SPECTRAL, 120.0 * t->M, 0, 2);
-        launch_tl_start(c->grid, rf, c->M, t->g, t->rh, t->xh, t->ph, t->cp, t->M, op, c->rp, c->partials,
-                        c->partials + rb, rb, c->stream);
+        KTimer kt(c, KK_SPECTRAL, 120.0 * t->M, 0);
+        launch_tl_start(c->grid, rf, c->M, t->g, t->rh, t->xh, t->ph, t->cp, t->M, op, c->rp, t->sc,
+                        fs_reduction(c, 0), c->stream);
     }
     CL_TRY(fs_sums(c, 2));
     const double r0 = std::sqrt(c->hres[0]);
     // rz stays on the device: alpha and beta are formed there (FP64, as the host
     // would), so an iteration reads back only |r|^2 and the breakdown flag
-    CL_CUDA(c, cudaMemcpyAsync(t->sc + kTlRz, c->dres + 1, sizeof(double), cudaMemcpyDeviceToDevice, c->stream));
-    const double scale = c->hvol * static_cast<double>(c->N);  // Parseval on scaled spectra, as fs_sums
     for (int it = 1; r0 > 0.0 && it <= c->o.pc_maxit; ++it) {
         {
             KTimer kt(c, KK_FFT, 0, 0);
@@ -1104,25 +1117,19 @@ claire_status tl_apply(claire_ctx* c, const cufftComplex* rf, cufftComplex* zf, 
             CL_FFT(c, cufftExecR2C(t->r2c, t->real, t->T));
         }
         {
-            KTimer kt(c, KK_SPECTRAL, 72.0 * t->M, 0, 3);
-            launch_tl_hp(t->g, t->T, t->ph, t->q, t->M, c->o.grad_form, c->rp, static_cast<float>(1.0 / t->N),
-                         c->partials, rb, c->stream);
-            launch_final_sum(c->partials, rb, scale, t->sc + kTlPq, c->stream);
-            launch_tl_scalars(t->sc, 0, c->stream);
+            KTimer kt(c, KK_SPECTRAL, 72.0 * t->M, 0);
+            launch_tl_hp(t->g, t->T, t->ph, t->q, t->M, c->o.grad_form, c->rp, static_cast<float>(1.0 / t->N), t->sc,
+                         fs_reduction(c, 8), c->stream);
             CL_LAUNCHED(c);
         }
         {
-            KTimer kt(c, KK_SPECTRAL, 144.0 * t->M, 0, 4);
-            launch_tl_update(t->g, t->ph, t->q, t->xh, t->rh, t->zh, t->M, t->sc + kTlAlpha, op, c->rp,
-                             c->partials, c->partials + rb, rb, c->stream);
-            launch_final_sum(c->partials, rb, scale, t->sc + kTlRr, c->stream);
-            launch_final_sum(c->partials + rb, rb, scale, t->sc + kTlRzNew, c->stream);
+            KTimer kt(c, KK_SPECTRAL, 144.0 * t->M, 0);
+            launch_tl_update(t->g, t->ph, t->q, t->xh, t->rh, t->zh, t->M, t->sc, op, c->rp, fs_reduction(c, 10),
+                             c->stream);
             CL_LAUNCHED(c);
         }
-        CL_CUDA(c, cudaMemcpyAsync(c->hres + 8, t->sc + kTlRr, 2 * sizeof(double), cudaMemcpyDeviceToHost,
-                                   c->stream));
-        CL_CUDA(c, cudaStreamSynchronize(c->stream));
-        const double rr = c->hres[8], flag = c->hres[9];
+        CL_TRY(sync_scalars(c));
+        const double rr = c->hres[10], flag = c->hres[9];
         *its = it;
         if (flag == 2.0) return fail(c, CLAIRE_ENONFINITE, "non-finite inner PCG curvature");
         if (flag != 0.0) break;  // pq <= 0: the update above ran with alpha = 0
@@ -1130,16 +1137,14 @@ claire_status tl_apply(claire_ctx* c, const cufftComplex* rf, cufftComplex* zf, 
         if (c->o.pc_tol > 0 && std::sqrt(rr) <= c->o.pc_tol * r0) break;
         if (it == c->o.pc_maxit) break;
         {
-            KTimer kt(c, KK_SPECTRAL, 72.0 * t->M, 0, 2);
-            launch_tl_scalars(t->sc, 1, c->stream);
+            KTimer kt(c, KK_SPECTRAL, 72.0 * t->M, 0);
             launch_dir_stored(t->g, t->zh, t->ph, t->cp, t->M, 0.0f, 0, c->stream, t->sc + kTlBeta);
             CL_LAUNCHED(c);
         }
     }
     {
-        KTimer kt(c, KK_SPECTRAL, (zold ? 72.0 : 48.0) * c->M, 0, 2);
-        launch_tl_finish(c->grid, rf, zf, zold, c->M, t->g, t->xh, t->M, op, c->rp, c->partials, c->partials + rb,
-                         rb, c->stream);
+        KTimer kt(c, KK_SPECTRAL, (zold ? 72.0 : 48.0) * c->M, 0);
+        launch_tl_finish(c->grid, rf, zf, zold, c->M, t->g, t->xh, t->M, op, c->rp, fs_reduction(c, 0), c->stream);
     }
     CL_TRY(fs_sums(c, 2));
     *rz = c->hres[0];
@@ -1169,9 +1174,8 @@ claire_status pcg(claire_ctx* c, double eta, int* its)
             KTimer t(c, KK_FFT, 0, 0);
             CL_FFT(c, cufftExecR2C(c->r2c, c->g, c->spec));
         }
-        KTimer t(c, KK_SPECTRAL, 72.0 * M, 0, 3);
-        launch_fs_start(c->grid, c->spec, c->rh, c->xh, c->M, op, c->rp, scale, c->partials,
-                        c->partials + c->red_blocks, c->red_blocks, c->stream);
+        KTimer t(c, KK_SPECTRAL, 72.0 * M, 0);
+        launch_fs_start(c->grid, c->spec, c->rh, c->xh, c->M, op, c->rp, scale, fs_reduction(c, 0), c->stream);
     }
     CL_TRY(fs_sums(c, 2));
     const double r0 = std::sqrt(c->hres[0]);
@@ -1212,9 +1216,9 @@ claire_status pcg(claire_ctx* c, double eta, int* its)
                 KTimer t(c, KK_FFT, 0, 0);
                 CL_FFT(c, cufftExecR2C(c->r2c, c->z, c->spec2));
             }
-            KTimer t(c, KK_SPECTRAL, 72.0 * M, 0, 2);
-            launch_fs_hp(c->grid, c->spec, c->spec2, c->phat, c->M, c->o.grad_form, c->rp, scale,
-                         c->partials, c->red_blocks, c->stream);
+            KTimer t(c, KK_SPECTRAL, 72.0 * M, 0);
+            launch_fs_hp(c->grid, c->spec, c->spec2, c->phat, c->M, c->o.grad_form, c->rp, scale, fs_reduction(c, 0),
+                         c->stream);
         }
         CL_TRY(fs_sums(c, 1));
         const double pq = c->hres[0];
@@ -1227,10 +1231,9 @@ claire_status pcg(claire_ctx* c, double eta, int* its)
         const double alpha = rz / pq;
         {
             PhaseScope ps(c, CLAIRE_PHASE_VECTOR);
-            KTimer t(c, KK_SPECTRAL, 144.0 * M, 0, 3);
+            KTimer t(c, KK_SPECTRAL, 144.0 * M, 0);
             launch_fs_update(c->grid, c->spec, c->phat, c->xh, c->rh, two_level ? c->tl2->zf : nullptr, c->M,
-                             static_cast<float>(alpha), op, c->rp, c->partials, c->partials + c->red_blocks,
-                             c->red_blocks, c->stream);
+                             static_cast<float>(alpha), op, c->rp, fs_reduction(c, 0), c->stream);
         }
         CL_TRY(fs_sums(c, 2));
         const double rr = c->hres[0];
@@ -1402,11 +1405,7 @@ claire_status claire_create(claire_ctx** out, const int grid[3], double beta_v, 
             cudaGetLastError();
             return bail(CLAIRE_ECUDA);
         }
-        if (cudaMallocHost(&c->hres, 16 * sizeof(double)) != cudaSuccess) {
-            cudaGetLastError();
-            c->hres = nullptr;
-            return bail(CLAIRE_ENOMEM);
-        }
+        if (!make_scalars(c)) return bail(CLAIRE_ENOMEM);
         st = claire_set_stream(c, nullptr);
         if (st != CLAIRE_OK) return bail(st);
         *out = c;
@@ -1457,11 +1456,7 @@ claire_status claire_create(claire_ctx** out, const int grid[3], double beta_v, 
         cudaGetLastError();
         return bail(CLAIRE_ECUDA);
     }
-    if (cudaMallocHost(&c->hres, 16 * sizeof(double)) != cudaSuccess) {
-        cudaGetLastError();
-        c->hres = nullptr;
-        return bail(CLAIRE_ENOMEM);
-    }
+    if (!make_scalars(c)) return bail(CLAIRE_ENOMEM);
     // both plans share one work area (they never run concurrently: one stream)
     int nn[3] = {grid[0], grid[1], grid[2]};
     size_t ws_r2c = 0, ws_c2r = 0;
@@ -1756,14 +1751,11 @@ claire_status claire_register(claire_ctx* c, float* v_inout, claire_report* rep)
     {
         double den;
         {
-            KTimer t(c, KK_REDUCE, 8.0 * N, 0, 2);
-            launch_sqdiff_partial(c->m0, c->m1, N, c->partials, c->red_blocks, c->sto, c->stream);
-            launch_final_sum(c->partials, c->red_blocks, 0.5 * c->hvol, c->dres + 2, c->stream);
+            KTimer t(c, KK_REDUCE, 8.0 * N, 0);
+            launch_sqdiff(c->m0, c->m1, N, c->sto, reduction(c, 2, 0.5 * c->hvol), c->stream);
             CL_LAUNCHED(c);
         }
-        CL_CUDA(c, cudaMemcpyAsync(c->hres + 2, c->dres + 2, sizeof(double), cudaMemcpyDeviceToHost,
-                                   c->stream));
-        CL_CUDA(c, cudaStreamSynchronize(c->stream));
+        CL_TRY(sync_scalars(c));
         den = c->hres[2];
         R.r = den > 0 ? c->mis_lin / den : 0.0;
     }
@@ -1826,7 +1818,7 @@ claire_status claire_transport(claire_ctx* c, const float* v, const float* m_in,
             std::swap(a, b);
         }
     }
-    CL_TRY(sync_scalars(c, 0));
+    CL_TRY(sync_scalars(c));
     CL_TRY(copy_out(c, m_out, src, N));
     collect_timing(c);
     return CLAIRE_OK;
@@ -1840,15 +1832,15 @@ claire_status scatter_transpose(claire_ctx* c, const float* yv, const float* d, 
 {
     // the fixed-point scale follows max |yv|, computed on the device (no host round trip)
     double* mx = c->dres + 8;
-    launch_maxabs(yv, c->N, c->partials, c->red_blocks, mx, c->stream);
+    launch_maxabs(yv, c->N, reduction(c, 8), c->stream);
     CL_LAUNCHED(c);
     {
         KTimer t(c, KK_VJP_SCATTER, (4.0 + 12.0) * c->N, 1.0 * c->N);
-        CL_CUDA(c, launch_scatter_fixed(c->grid, c->o.interp, yv, d, v, static_cast<float>(c->dt), mx + 1, c->vjp_acc,
+        CL_CUDA(c, launch_scatter_fixed(c->grid, c->o.interp, yv, d, v, static_cast<float>(c->dt), mx, c->vjp_acc,
                                         c->stream));
         CL_LAUNCHED(c);
     }
-    launch_fixed_to_float(c->vjp_acc, mx + 1, accumulate ? 1 : 0, mult, out, c->N, c->stream);
+    launch_fixed_to_float(c->vjp_acc, mx, accumulate ? 1 : 0, mult, out, c->N, c->stream);
     CL_LAUNCHED(c);
     return CLAIRE_OK;
 }
@@ -1986,7 +1978,7 @@ claire_status claire_interp(claire_ctx* c, const float* f, const float* d, float
         launch_interp(c->grid, order, f, d, out, Storage::F32, c->stream);
         CL_LAUNCHED(c);
     }
-    CL_TRY(sync_scalars(c, 0));
+    CL_TRY(sync_scalars(c));
     collect_timing(c);
     return CLAIRE_OK;
 }
@@ -2004,7 +1996,7 @@ claire_status claire_interp_fields(claire_ctx* c, const float* f, int nf, const 
         launch_interp_fields(c->grid, order, f, nf, d, out, c->stream);
         CL_LAUNCHED(c);
     }
-    CL_TRY(sync_scalars(c, 0));
+    CL_TRY(sync_scalars(c));
     collect_timing(c);
     return CLAIRE_OK;
 }
@@ -2016,16 +2008,12 @@ claire_status claire_dice(claire_ctx* c, const float* a, const float* b, size_t 
     CL_TRY(check_kernel_ptr(c, a));
     CL_TRY(check_kernel_ptr(c, b));
     {
-        KTimer t(c, KK_REDUCE, 8.0 * n, 0, 4);
-        launch_count_partial(a, b, n, 0.5f, 0, c->partials, c->partials + c->red_blocks, c->red_blocks, c->stream);
-        launch_final_sum(c->partials, c->red_blocks, 1.0, c->dres + 10, c->stream);
-        launch_final_sum(c->partials + c->red_blocks, c->red_blocks, 1.0, c->dres + 11, c->stream);
-        launch_count_partial(a, b, n, 0.5f, 1, c->partials, c->partials + c->red_blocks, c->red_blocks, c->stream);
-        launch_final_sum(c->partials, c->red_blocks, 1.0, c->dres + 12, c->stream);
+        KTimer t(c, KK_REDUCE, 8.0 * n, 0, 2);
+        launch_count(a, b, n, 0.5f, 0, reduction(c, 10), c->stream);
+        launch_count(a, b, n, 0.5f, 1, reduction(c, 12), c->stream);
         CL_LAUNCHED(c);
     }
-    CL_CUDA(c, cudaMemcpyAsync(c->hres + 10, c->dres + 10, 3 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    CL_CUDA(c, cudaStreamSynchronize(c->stream));
+    CL_TRY(sync_scalars(c));
     const double na = c->hres[10], nb = c->hres[11], nab = c->hres[12];
     *dice = (na + nb) > 0 ? 2.0 * nab / (na + nb) : 1.0;
     collect_timing(c);

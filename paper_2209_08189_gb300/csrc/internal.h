@@ -14,6 +14,22 @@
 namespace claire {
 
 // ---- block reductions (256-thread blocks, fixed order: deterministic) ----
+// A grid-wide FP64 reduction in one launch: every block writes its partial (one
+// or two arrays of nblocks doubles), and the block that finishes last adds
+// them up in a fixed order and stores the scaled totals at out (device) and
+// host (their mirror in mapped pinned memory, read after the stream has been
+// synchronised).  `ticket` counts finished blocks and is left at 0; launches
+// that share it must be ordered (one stream).  A separate one-block kernel and
+// a copy of the scalars, which this replaces, cost 4 and 3 us per reduction.
+struct Reduction {
+    double* partials;  // 2 nblocks doubles
+    int nblocks;
+    double scale;
+    double* out;
+    double* host;
+    unsigned* ticket;
+};
+
 #ifdef __CUDACC__
 __device__ __forceinline__ double warp_sum(double x)
 {
@@ -36,6 +52,89 @@ __device__ __forceinline__ void block_sum(double x, double* out)
         y = warp_sum(y);
         if (lane == 0) out[blockIdx.x] = y;
     }
+}
+
+// Whether this block is the last of the grid to get here; thread 0 has written
+// the block's partials.  Same answer in every thread.
+__device__ __forceinline__ bool last_block(unsigned* ticket)
+{
+    __shared__ bool last;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (last) __threadfence();
+    return last;
+}
+
+// Total of n partials in a fixed order (256 threads); valid in thread 0.
+__device__ __forceinline__ double total_of(const double* partials, int n)
+{
+    __shared__ double sh[8];
+    double x = 0.0;
+    for (int i = threadIdx.x; i < n; i += 256) x += __ldcg(partials + i);
+    x = warp_sum(x);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (lane == 0) sh[wid] = x;
+    __syncthreads();
+    double y = 0.0;
+    if (wid == 0) y = warp_sum(lane < 8 ? sh[lane] : 0.0);
+    __syncthreads();
+    return y;
+}
+
+__device__ __forceinline__ void put_result(const Reduction& r, int slot, double v)
+{
+    r.out[slot] = v;
+    if (r.host) r.host[slot] = v;
+}
+
+// Grid-wide sum of x (256-thread blocks).  True, with the scaled total stored
+// and returned in *total, in thread 0 of the block that finished last.
+__device__ __forceinline__ bool grid_sum(double x, const Reduction& r, double* total = nullptr)
+{
+    block_sum(x, r.partials);
+    if (!last_block(r.ticket)) return false;
+    const double t = total_of(r.partials, r.nblocks) * r.scale;
+    if (threadIdx.x != 0) return false;
+    put_result(r, 0, t);
+    if (total) *total = t;
+    return true;
+}
+
+// Block maximum of non-negative doubles given by their bit patterns (integers
+// order them the same way, NaN on top), then over the grid: result at out[0].
+__device__ __forceinline__ unsigned long long block_max_bits(unsigned long long hi)
+{
+    __shared__ unsigned long long sh[8];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long t = __shfl_xor_sync(0xffffffffu, hi, o);
+        hi = t > hi ? t : hi;
+    }
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = hi;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int w = 1; w < 8; ++w) hi = sh[w] > hi ? sh[w] : hi;
+    }
+    __syncthreads();
+    return hi;  // thread 0
+}
+
+__device__ __forceinline__ void grid_max_bits(unsigned long long hi, const Reduction& r)
+{
+    hi = block_max_bits(hi);
+    if (threadIdx.x == 0) r.partials[blockIdx.x] = __longlong_as_double(static_cast<long long>(hi));
+    if (!last_block(r.ticket)) return;
+    hi = 0;
+    for (int i = threadIdx.x; i < r.nblocks; i += 256) {
+        const unsigned long long t = static_cast<unsigned long long>(__double_as_longlong(__ldcg(r.partials + i)));
+        hi = t > hi ? t : hi;
+    }
+    hi = block_max_bits(hi);
+    if (threadIdx.x == 0) put_result(r, 0, __longlong_as_double(static_cast<long long>(hi)));
 }
 
 // min / max that keep a NaN operand (fmin / fmax return the other operand),
@@ -72,6 +171,39 @@ __device__ __forceinline__ void block_minmax(double lo, double hi, double* pmin,
             pmin[blockIdx.x] = a;
             pmax[blockIdx.x] = b;
         }
+    }
+}
+
+// Grid-wide minimum (out[0]) and maximum (out[1]); partial maxima first.
+__device__ __forceinline__ void grid_minmax(double lo, double hi, const Reduction& r)
+{
+    __shared__ double fin[16];
+    block_minmax(lo, hi, r.partials + r.nblocks, r.partials);
+    if (!last_block(r.ticket)) return;
+    lo = 1e300;
+    hi = -1e300;
+    for (int i = threadIdx.x; i < r.nblocks; i += 256) {
+        lo = min_nan(lo, __ldcg(r.partials + r.nblocks + i));
+        hi = max_nan(hi, __ldcg(r.partials + i));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        lo = min_nan(lo, __shfl_down_sync(0xffffffffu, lo, o));
+        hi = max_nan(hi, __shfl_down_sync(0xffffffffu, hi, o));
+    }
+    if ((threadIdx.x & 31) == 0) {
+        fin[threadIdx.x >> 5] = lo;
+        fin[8 + (threadIdx.x >> 5)] = hi;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int w = 1; w < 8; ++w) {
+            lo = min_nan(lo, fin[w]);
+            hi = max_nan(hi, fin[8 + w]);
+        }
+        put_result(r, 0, lo);
+        put_result(r, 1, hi);
     }
 }
 #endif
@@ -136,8 +268,8 @@ void launch_map_step(const Grid& g, int order, const float* u_prev, const float*
                      cudaStream_t st);
 void launch_fd8_grad(const Grid& g, const void* f, void* out, Storage sto, cudaStream_t st);
 void launch_fd8_div(const Grid& g, const float* v, void* out, Storage sto, cudaStream_t st);
-void launch_detj_minmax(const Grid& g, const float* u, double* pmin, double* pmax, int nblocks,
-                        cudaStream_t st);
+// totals: minimum at red.out[0], maximum at red.out[1] (scale unused)
+void launch_detj_minmax(const Grid& g, const float* u, const Reduction& red, cudaStream_t st);
 
 // ---- context accessors for host-side drivers in other units (engine.cu) ----
 cudaStream_t ctx_stream(const claire_ctx* c);
@@ -165,7 +297,8 @@ void launch_scale_add(float* y, float a, const float* x, size_t n, cudaStream_t 
 void launch_predictor_terms(const Grid& g, int order, const float* v, const float* vc, float dt, const float* dbar,
                             float* ubar, float* Ubar, cudaStream_t st);
 // out2[1] = max |x| (out2[0] scratch)
-void launch_maxabs(const float* x, size_t n, double* partials, int nblocks, double* out2, cudaStream_t st);
+// out[0] = max |x| (NaN: infinity)
+void launch_maxabs(const float* x, size_t n, const Reduction& r, cudaStream_t st);
 
 // ---- spectral scaling, vector ops and reductions (vec_kernels.cu) ----
 enum SpectralOp { SPEC_REG = 0, SPEC_INV = 1, SPEC_K = 2, SPEC_AINV = 3 };
@@ -181,31 +314,24 @@ struct RegParams {
 void launch_spectral(const Grid& g, cufftComplex* xh, size_t cstride, SpectralOp op,
                      RegParams rp, float scale, cudaStream_t st);
 
-// PCG preconditioner in Fourier space: xh <- scale * M(k) xh (SPEC_INV or
-// SPEC_AINV) with block partial sums of sum_x r z (Parseval) in partials.
-void launch_spectral_precond(const Grid& g, cufftComplex* xh, size_t cstride, SpectralOp op,
-                             RegParams rp, float scale, double* partials, int nblocks, cudaStream_t st);
 // PCG direction in Fourier space: ph = zh + beta ph (first: ph = zh), cp = ph, zh <- S ph.
 void launch_spectral_direction(const Grid& g, const cufftComplex* rh, cufftComplex* ph, cufftComplex* cp,
                                size_t cstride, float beta, int first, SpectralOp op, RegParams rp,
                                cudaStream_t st);
 
-// Fourier-space PCG (vectors are half spectra scaled by 1/N; partial sums are
+// Fourier-space PCG (vectors are half spectra scaled by 1/N; totals are
 // of sum_k wt Re(conj(a) b), wt the multiplicity of the mode):
-//   start:  r~ = -scale spec, x~ = 0, spec <- M r~;  partials |r~|^2 (prr), <r~, M r~> (prz)
-//   hp:     spec <- spec + scale spec2 (K applied if kform);  partials <p~, H p~>
-//   update: x~ += alpha p~, r~ -= alpha spec, spec <- M r~;  partials as in start
+//   start:  r~ = -scale spec, x~ = 0, spec <- M r~;  totals |r~|^2, <r~, M r~>
+//   hp:     spec <- spec + scale spec2 (K applied if kform);  total <p~, H p~>
+//   update: x~ += alpha p~, r~ -= alpha spec, spec <- M r~;  totals as in start
 void launch_fs_start(const Grid& g, cufftComplex* spec, cufftComplex* rh, cufftComplex* xh, size_t cs,
-                     SpectralOp op, RegParams rp, float scale, double* prr, double* prz, int nblocks,
-                     cudaStream_t st);
+                     SpectralOp op, RegParams rp, float scale, const Reduction& red, cudaStream_t st);
 void launch_fs_hp(const Grid& g, cufftComplex* spec, const cufftComplex* spec2, const cufftComplex* ph,
-                  size_t cs, int kform, RegParams rp, float scale, double* ppq, int nblocks, cudaStream_t st);
+                  size_t cs, int kform, RegParams rp, float scale, const Reduction& red, cudaStream_t st);
 void launch_fs_update(const Grid& g, cufftComplex* spec, const cufftComplex* ph, cufftComplex* xh,
                       cufftComplex* rh, const cufftComplex* zc, size_t cs, float alpha, SpectralOp op, RegParams rp,
-                      double* prr, double* prz, int nblocks, cudaStream_t st);
+                      const Reduction& red, cudaStream_t st);
 
-// Deterministic FP64 reductions: partial sums per block, then a one-block
-// final sum in fixed order.  `partials` holds at least nblocks doubles.
 // two-level zero-velocity preconditioner (coarse grid gc of the fine grid gf; cs* = component strides)
 void launch_mean_levels(const void* m, int nt, float w_end, float w_mid, size_t N, float* out, Storage sto,
                         cudaStream_t st);
@@ -216,45 +342,34 @@ void launch_tl_restrict(const Grid& gf, const cufftComplex* F, size_t csf, const
 void launch_tl_weight(float* gbar_c, const float* w, size_t n, cudaStream_t st);
 void launch_tl_start(const Grid& gf, const cufftComplex* rf, size_t csf, const Grid& gc, cufftComplex* rh,
                      cufftComplex* xh, cufftComplex* ph, cufftComplex* cp, size_t cs, SpectralOp op, RegParams rp,
-                     double* prr, double* prz, int nblocks, cudaStream_t st);
+                     double* sc, const Reduction& red, cudaStream_t st);
 void launch_tl_rank1(const float* gbar, float* p, size_t Nc, cudaStream_t st);
 void launch_tl_hp(const Grid& gc, const cufftComplex* T, const cufftComplex* ph, cufftComplex* q, size_t cs,
-                  int kform, RegParams rp, float scale, double* ppq, int nblocks, cudaStream_t st);
-// Device scalars of the inner PCG (slots of a small FP64 array)
-constexpr int kTlRz = 0, kTlPq = 1, kTlAlpha = 2, kTlRr = 3, kTlFlag = 4, kTlRzNew = 5, kTlBeta = 6, kTlSlots = 8;
-// stage 0: alpha = rz / pq (0 and the breakdown flag when pq <= 0); stage 1: beta = rz_new / rz, rz <- rz_new
-void launch_tl_scalars(double* s, int stage, cudaStream_t st);
+                  int kform, RegParams rp, float scale, double* sc, const Reduction& red, cudaStream_t st);
+// Device scalars sc of the inner PCG (slots of a small FP64 array).  The kernel
+// that ends a reduction also forms what follows from it: start stores
+// rz; hp forms alpha = rz / pq (0 and the breakdown flag when pq <= 0); update
+// forms beta = rz_new / rz and moves rz_new to rz.
+constexpr int kTlRz = 0, kTlAlpha = 1, kTlBeta = 2, kTlSlots = 4;
 void launch_tl_update(const Grid& gc, const cufftComplex* ph, const cufftComplex* q, cufftComplex* xh,
-                      cufftComplex* rh, cufftComplex* zh, size_t cs, const double* alpha_dev, SpectralOp op,
-                      RegParams rp, double* prr, double* prz, int nblocks, cudaStream_t st);
+                      cufftComplex* rh, cufftComplex* zh, size_t cs, double* sc, SpectralOp op, RegParams rp,
+                      const Reduction& red, cudaStream_t st);
 // beta from beta_dev when it is not null, else the host value
 void launch_dir_stored(const Grid& g, const cufftComplex* zh, cufftComplex* ph, cufftComplex* cp, size_t cs,
                        float beta, int first, cudaStream_t st, const double* beta_dev = nullptr);
 void launch_tl_finish(const Grid& gf, const cufftComplex* rf, cufftComplex* zf, const cufftComplex* zold, size_t csf,
-                      const Grid& gc, const cufftComplex* xc, size_t csc, SpectralOp op, RegParams rp, double* prz,
-                      double* pro, int nblocks, cudaStream_t st);
-void launch_dot_partial(const float* x, const float* y, size_t n, double* partials, int nblocks,
-                        cudaStream_t st);
-void launch_sqdiff_partial(const void* a, const void* b, size_t n, double* partials, int nblocks,
-                           Storage sto, cudaStream_t st);
-void launch_maxnorm3_partial(const float* v, size_t N, double* partials, int nblocks,
-                             cudaStream_t st);
+                      const Grid& gc, const cufftComplex* xc, size_t csc, SpectralOp op, RegParams rp,
+                      const Reduction& red, cudaStream_t st);
+// Deterministic FP64 reductions (struct Reduction): totals at red.out
+void launch_dot(const float* x, const float* y, size_t n, const Reduction& red, cudaStream_t st);
+void launch_sqdiff(const void* a, const void* b, size_t n, Storage sto, const Reduction& red, cudaStream_t st);
+void launch_maxnorm3(const float* v, size_t N, const Reduction& red, cudaStream_t st);
 // Dice counts: |a >= t| and |b >= t| (both = 0) or |(a >= t) and (b >= t)| (both = 1)
-void launch_count_partial(const float* a, const float* b, size_t n, float t, int both, double* pa, double* pb,
-                          int nblocks, cudaStream_t st);
-void launch_final_sum(const double* partials, int nblocks, double scale, double* out,
-                      cudaStream_t st);
-void launch_final_max(const double* partials, int nblocks, double* out, cudaStream_t st);
-void launch_final_minmax(const double* pmin, const double* pmax, int nblocks, double* out2,
-                         cudaStream_t st);
+void launch_count(const float* a, const float* b, size_t n, float t, int both, const Reduction& red, cudaStream_t st);
 
 // y = a x + y
 void launch_axpy(float a, const float* x, float* y, size_t n, cudaStream_t st);
 // z = x + a y
 void launch_xpay(const float* x, float a, const float* y, float* z, size_t n, cudaStream_t st);
-// x += alpha p; r -= alpha q; partial sums of r . r
-void launch_pcg_update(float alpha, const float* p, const float* q, float* x, float* r, size_t n,
-                       double* partials, int nblocks, cudaStream_t st);
-void launch_fill(float* x, float value, size_t n, cudaStream_t st);
 
 }  // namespace claire

@@ -534,7 +534,7 @@ __device__ __forceinline__ int ordered_int(float x)
 constexpr int kOrderedInf = 0x7f800000;  // +infinity; ~kOrderedInf is -infinity
 __device__ __forceinline__ float ordered_float(int i) { return __int_as_float(i ^ ((i >> 31) & 0x7fffffff)); }
 
-// det(I + grad u) in FP64 with block-wise min / max partials.
+// Extrema of det(I + grad u) in FP64.
 //
 // Bound: the nine FD8 differences per point.  The FP64 pipe of this part runs
 // 2 operations per clock and SM, so the 30 FP64 operations of every point's
@@ -548,7 +548,7 @@ __device__ __forceinline__ float ordered_float(int i) { return __int_as_float(i 
 // extrema are the FP64 ones, bit for bit.  Columns are walked by a fixed
 // number of CTAs (one partial each).  256^3: 328 us.
 __global__ void __launch_bounds__(kThreads) k_detj_minmax(Grid g, const float* __restrict__ u, int zlen, int ncol,
-                                                           double* __restrict__ pmin, double* __restrict__ pmax)
+                                                           Reduction red)
 {
     __shared__ float sh[2][3][kFdPlane];
     const int own = (static_cast<int>(threadIdx.x >> 5) + 4) * kFdCols + (threadIdx.x & 31) + 4;
@@ -640,7 +640,7 @@ __global__ void __launch_bounds__(kThreads) k_detj_minmax(Grid g, const float* _
             }
         }
     }
-    block_minmax(lo, hi, pmin, pmax);
+    grid_minmax(lo, hi, red);
 }
 
 }  // namespace
@@ -881,12 +881,11 @@ void launch_fd8_div(const Grid& g, const float* v, void* out, Storage sto, cudaS
     });
 }
 
-void launch_detj_minmax(const Grid& g, const float* u, double* pmin, double* pmax, int nblocks,
-                        cudaStream_t st)
+void launch_detj_minmax(const Grid& g, const float* u, const Reduction& red, cudaStream_t st)
 {
     const int z = fd_zlen(g);
     const dim3 cols = fd_grid(g, z);
-    k_detj_minmax<<<nblocks, kThreads, 0, st>>>(g, u, z, static_cast<int>(cols.x * cols.y * cols.z), pmin, pmax);
+    k_detj_minmax<<<red.nblocks, kThreads, 0, st>>>(g, u, z, static_cast<int>(cols.x * cols.y * cols.z), red);
 }
 
 }  // namespace claire

@@ -130,32 +130,6 @@ __global__ void __launch_bounds__(kThreads) k_spectral(Grid g, float2* __restric
     }
 }
 
-// Preconditioner in Fourier space: zh = scale * M(k) rh in place (M = S^{-1}
-// or (a I)^{-1}) and block partial sums of sum_k wt Re(conj(rh) zh), which is
-// sum_x r(x) z(x) by Parseval (zh already carries the 1/N of the inverse FFT).
-__global__ void __launch_bounds__(kThreads) k_spectral_precond(Grid g, float2* __restrict__ xh, size_t cs,
-                                                                int op, RegParams rp, float scale,
-                                                                double* __restrict__ partials)
-{
-    const int n3h = g.n3 / 2 + 1;
-    const size_t M = static_cast<size_t>(g.n1) * g.n2 * n3h;
-    double acc = 0.0;
-    for (size_t idx = blockIdx.x * static_cast<size_t>(kThreads) + threadIdx.x; idx < M;
-         idx += static_cast<size_t>(gridDim.x) * kThreads) {
-        const Mode m = mode_of(g, idx, n3h, rp);
-        const float2 x0 = xh[idx], x1 = xh[cs + idx], x2 = xh[2 * cs + idx];
-        float2 y0, y1, y2;
-        apply_inv(m, op, x0, x1, x2, y0, y1, y2);
-        y0 = cmul(scale, y0); y1 = cmul(scale, y1); y2 = cmul(scale, y2);
-        xh[idx] = y0;
-        xh[cs + idx] = y1;
-        xh[2 * cs + idx] = y2;
-        const float re = x0.x * y0.x + x0.y * y0.y + x1.x * y1.x + x1.y * y1.y + x2.x * y2.x + x2.y * y2.y;
-        acc += static_cast<double>(m.wt * re);
-    }
-    block_sum(acc, partials);
-}
-
 // PCG direction in Fourier space: z~ = M r~ (recomputed from r~, not
 // stored), p~ = z~ + beta p~ (p~ = z~ when first), copied to cp for the
 // inverse FFT that yields p (it overwrites its input).
@@ -219,6 +193,22 @@ __device__ __forceinline__ void block_sum2(double a, double b, double* pa, doubl
     }
 }
 
+// Grid-wide sums of a and b.  True, with the scaled totals stored and returned,
+// in thread 0 of the block that finished last.
+__device__ __forceinline__ bool grid_sum2(double a, double b, const Reduction& r, double tot[2])
+{
+    block_sum2(a, b, r.partials, r.partials + r.nblocks);
+    if (!last_block(r.ticket)) return false;
+    const double x = total_of(r.partials, r.nblocks) * r.scale;
+    const double y = total_of(r.partials + r.nblocks, r.nblocks) * r.scale;
+    if (threadIdx.x != 0) return false;
+    put_result(r, 0, x);
+    put_result(r, 1, y);
+    tot[0] = x;
+    tot[1] = y;
+    return true;
+}
+
 __device__ __forceinline__ float cdot3(float2 a0, float2 a1, float2 a2, float2 b0, float2 b1, float2 b2)
 {
     return a0.x * b0.x + a0.y * b0.y + a1.x * b1.x + a1.y * b1.y + a2.x * b2.x + a2.y * b2.y;
@@ -228,8 +218,7 @@ __device__ __forceinline__ float cdot3(float2 a0, float2 a1, float2 a2, float2 b
 // <r~, z~> with z~ = M r~ (recomputed by the direction kernel).
 __global__ void __launch_bounds__(kThreads) k_fs_start(Grid g, float2* __restrict__ spec,
                                                         float2* __restrict__ rh, float2* __restrict__ xh,
-                                                        size_t cs, int op, RegParams rp, float scale,
-                                                        double* __restrict__ prr, double* __restrict__ prz)
+                                                        size_t cs, int op, RegParams rp, float scale, Reduction red)
 {
     const int n3h = g.n3 / 2 + 1;
     const size_t M = static_cast<size_t>(g.n1) * g.n2 * n3h;
@@ -246,7 +235,8 @@ __global__ void __launch_bounds__(kThreads) k_fs_start(Grid g, float2* __restric
         arr += static_cast<double>(m.wt * cdot3(r0, r1, r2, r0, r1, r2));
         arz += static_cast<double>(m.wt * cdot3(r0, r1, r2, z0, z1, z2));
     }
-    block_sum2(arr, arz, prr, prz);
+    double tot[2];
+    grid_sum2(arr, arz, red, tot);
 }
 
 // H p~ = S p~ + scale F[body] (in spec2), or K of that for the paper's
@@ -254,7 +244,7 @@ __global__ void __launch_bounds__(kThreads) k_fs_start(Grid g, float2* __restric
 __global__ void __launch_bounds__(kThreads) k_fs_hp(Grid g, float2* __restrict__ spec,
                                                      const float2* __restrict__ spec2,
                                                      const float2* __restrict__ ph, size_t cs, int kform,
-                                                     RegParams rp, float scale, double* __restrict__ ppq)
+                                                     RegParams rp, float scale, Reduction red)
 {
     const int n3h = g.n3 / 2 + 1;
     const size_t M = static_cast<size_t>(g.n1) * g.n2 * n3h;
@@ -282,7 +272,7 @@ __global__ void __launch_bounds__(kThreads) k_fs_hp(Grid g, float2* __restrict__
         for (int c = 0; c < 3; ++c) spec[c * cs + idx] = h[c];
         acc += static_cast<double>(m.wt * cdot3(p0, p1, p2, h[0], h[1], h[2]));
     }
-    block_sum(acc, ppq);
+    grid_sum(acc, red);
 }
 
 // x~ += alpha p~, r~ -= alpha H p~ (H p~ in spec); partials of |r~|^2 and
@@ -292,8 +282,7 @@ __global__ void __launch_bounds__(kThreads) k_fs_update(Grid g, const float2* __
                                                          const float2* __restrict__ ph,
                                                          float2* __restrict__ xh, float2* __restrict__ rh,
                                                          const float2* __restrict__ zc, size_t cs, float alpha,
-                                                         int op, RegParams rp, double* __restrict__ prr,
-                                                         double* __restrict__ prz)
+                                                         int op, RegParams rp, Reduction red)
 {
     const int n3h = g.n3 / 2 + 1;
     const size_t M = static_cast<size_t>(g.n1) * g.n2 * n3h;
@@ -322,7 +311,8 @@ __global__ void __launch_bounds__(kThreads) k_fs_update(Grid g, const float2* __
             arz += static_cast<double>(m.wt * cdot3(r[0], r[1], r[2], z0, z1, z2));
         }
     }
-    block_sum2(arr, arz, prr, prz);
+    double tot[2];
+    grid_sum2(arr, arz, red, tot);
 }
 
 __device__ __forceinline__ bool aligned16(const void* p)
@@ -330,9 +320,8 @@ __device__ __forceinline__ bool aligned16(const void* p)
     return (reinterpret_cast<uintptr_t>(p) & 15u) == 0;
 }
 
-__global__ void __launch_bounds__(kThreads) k_dot_partial(const float* __restrict__ x,
-                                                           const float* __restrict__ y, size_t n,
-                                                           double* __restrict__ partials)
+__global__ void __launch_bounds__(kThreads) k_dot(const float* __restrict__ x, const float* __restrict__ y, size_t n,
+                                                   Reduction red)
 {
     double acc = 0.0;
     const size_t stride = static_cast<size_t>(gridDim.x) * kThreads;
@@ -349,12 +338,12 @@ __global__ void __launch_bounds__(kThreads) k_dot_partial(const float* __restric
         done = n4 * 4;
     }
     for (size_t i = done + t0; i < n; i += stride) acc += static_cast<double>(x[i] * y[i]);
-    block_sum(acc, partials);
+    grid_sum(acc, red);
 }
 
 template <class S>
-__global__ void __launch_bounds__(kThreads) k_sqdiff_partial(const S* __restrict__ a, const S* __restrict__ b,
-                                                              size_t n, double* __restrict__ partials)
+__global__ void __launch_bounds__(kThreads) k_sqdiff(const S* __restrict__ a, const S* __restrict__ b, size_t n,
+                                                      Reduction red)
 {
     double acc = 0.0;
     const size_t stride = static_cast<size_t>(gridDim.x) * kThreads;
@@ -377,11 +366,10 @@ __global__ void __launch_bounds__(kThreads) k_sqdiff_partial(const S* __restrict
         const float d = ldf<S>(a + i) - ldf<S>(b + i);
         acc += static_cast<double>(d * d);
     }
-    block_sum(acc, partials);
+    grid_sum(acc, red);
 }
 
-// max over points of |v|_2^2 in FP64; partials holds 2 * gridDim.x doubles (the
-// first half receives the block maxima, the second half is scratch).
+// max over points of |v|_2^2 in FP64.
 //
 // Bound: one pass over v (12 B per point, HBM).  The FP64 pipe of this part
 // runs 2 operations per clock and SM, so forming every |v|^2 in FP64 cost ten
@@ -444,11 +432,9 @@ __device__ __forceinline__ unsigned norm3_threshold(unsigned m, unsigned thr)
     return max(thr, __float_as_uint(f * (1.0f - 9.5367431640625e-07f)));
 }
 
-__global__ void __launch_bounds__(kThreads) k_maxnorm3_partial(const float* __restrict__ v, size_t N,
-                                                                double* __restrict__ partials)
+__global__ void __launch_bounds__(kThreads) k_maxnorm3(const float* __restrict__ v, size_t N, Reduction out)
 {
     __shared__ unsigned bthr;                       // the block's threshold (only ever rises)
-    __shared__ unsigned long long red[kThreads / 32];
     unsigned long long hi = 0;                      // bits of the FP64 maximum
     if (threadIdx.x == 0) bthr = 0;
     __syncthreads();
@@ -499,49 +485,14 @@ __global__ void __launch_bounds__(kThreads) k_maxnorm3_partial(const float* __re
             }
         }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long t = __shfl_xor_sync(0xffffffffu, hi, o);
-        hi = t > hi ? t : hi;
-    }
-    if (lane == 0) red[threadIdx.x >> 5] = hi;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int w = 1; w < kThreads / 32; ++w) hi = red[w] > hi ? red[w] : hi;
-        partials[blockIdx.x] = __longlong_as_double(static_cast<long long>(hi));
-    }
+    grid_max_bits(hi, out);
 }
 
-// Maximum of nb non-negative doubles (bit patterns; NaN on top) into out[0].
-__global__ void __launch_bounds__(kThreads) k_final_max(const double* __restrict__ p, int nb, double* __restrict__ out)
-{
-    __shared__ unsigned long long red[kThreads / 32];
-    unsigned long long hi = 0;
-    for (int i = threadIdx.x; i < nb; i += kThreads) {
-        const unsigned long long t = static_cast<unsigned long long>(__double_as_longlong(p[i])) & 0x7fffffffffffffffull;
-        hi = t > hi ? t : hi;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long t = __shfl_xor_sync(0xffffffffu, hi, o);
-        hi = t > hi ? t : hi;
-    }
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = hi;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int w = 1; w < kThreads / 32; ++w) hi = red[w] > hi ? red[w] : hi;
-        out[0] = __longlong_as_double(static_cast<long long>(hi));
-    }
-}
-
-// Dice counts (Sec. 4.1): both = 0 counts a >= t and b >= t into pa, pb;
-// both = 1 counts (a >= t) and (b >= t) into pa (pb gets zeros).  Per-block
+// Dice counts (Sec. 4.1): both = 0 counts a >= t and b >= t into totals 0 and
+// 1; both = 1 counts (a >= t) and (b >= t) into total 0 (1 is zero).
 // FP64 partial sums of integers: exact below 2^53.
-__global__ void __launch_bounds__(kThreads) k_count_partial(const float* __restrict__ a, const float* __restrict__ b,
-                                                             size_t n, float t, int both, double* __restrict__ pa,
-                                                             double* __restrict__ pb)
+__global__ void __launch_bounds__(kThreads) k_count(const float* __restrict__ a, const float* __restrict__ b, size_t n,
+                                                     float t, int both, Reduction red)
 {
     unsigned long long ca = 0, cb = 0;
     const size_t stride = static_cast<size_t>(gridDim.x) * kThreads;
@@ -554,30 +505,8 @@ __global__ void __launch_bounds__(kThreads) k_count_partial(const float* __restr
             cb += ib ? 1u : 0u;
         }
     }
-    block_sum2(static_cast<double>(ca), static_cast<double>(cb), pa, pb);
-}
-
-__global__ void __launch_bounds__(kThreads) k_final_sum(const double* __restrict__ partials, int nb,
-                                                         double scale, double* __restrict__ out)
-{
-    double acc = 0.0;
-    for (int i = threadIdx.x; i < nb; i += kThreads) acc += partials[i];
-    block_sum(acc, out);
-    if (threadIdx.x == 0) out[0] *= scale;
-}
-
-__global__ void __launch_bounds__(kThreads) k_final_minmax(const double* __restrict__ pmin,
-                                                            const double* __restrict__ pmax, int nb,
-                                                            double* __restrict__ out2)
-{
-    double lo = 1e300, hi = -1e300;
-    for (int i = threadIdx.x; i < nb; i += kThreads) {
-        const double a = pmin ? pmin[i] : lo;
-        const double b = pmax[i];
-        lo = min_nan(lo, a);
-        hi = max_nan(hi, b);
-    }
-    block_minmax(lo, hi, out2, out2 + 1);
+    double tot[2];
+    grid_sum2(static_cast<double>(ca), static_cast<double>(cb), red, tot);
 }
 
 // The vector updates take a float4 path when every pointer is 16-byte aligned
@@ -622,51 +551,6 @@ __global__ void __launch_bounds__(kThreads) k_xpay(const float* __restrict__ x, 
         done = n4 * 4;
     }
     for (size_t i = done + t0; i < n; i += stride) z[i] = fmaf(a, y[i], x[i]);
-}
-
-__global__ void __launch_bounds__(kThreads) k_pcg_update(float alpha, const float* __restrict__ p,
-                                                          const float* __restrict__ q,
-                                                          float* __restrict__ x,
-                                                          float* __restrict__ r, size_t n,
-                                                          double* __restrict__ partials)
-{
-    double acc = 0.0;
-    const size_t stride = static_cast<size_t>(gridDim.x) * kThreads;
-    const size_t t0 = blockIdx.x * static_cast<size_t>(kThreads) + threadIdx.x;
-    size_t done = 0;
-    if (aligned16(p) && aligned16(q) && aligned16(x) && aligned16(r)) {
-        const size_t n4 = n / 4;
-        const float4* p4 = reinterpret_cast<const float4*>(p);
-        const float4* q4 = reinterpret_cast<const float4*>(q);
-        float4* x4 = reinterpret_cast<float4*>(x);
-        float4* r4 = reinterpret_cast<float4*>(r);
-        for (size_t i = t0; i < n4; i += stride) {
-            const float4 pp = __ldg(p4 + i), qq = __ldg(q4 + i);
-            float4 xx = x4[i], rr = r4[i];
-            xx.x = fmaf(alpha, pp.x, xx.x); xx.y = fmaf(alpha, pp.y, xx.y);
-            xx.z = fmaf(alpha, pp.z, xx.z); xx.w = fmaf(alpha, pp.w, xx.w);
-            rr.x = fmaf(-alpha, qq.x, rr.x); rr.y = fmaf(-alpha, qq.y, rr.y);
-            rr.z = fmaf(-alpha, qq.z, rr.z); rr.w = fmaf(-alpha, qq.w, rr.w);
-            x4[i] = xx;
-            r4[i] = rr;
-            acc += static_cast<double>(rr.x * rr.x + rr.y * rr.y + rr.z * rr.z + rr.w * rr.w);
-        }
-        done = n4 * 4;
-    }
-    for (size_t i = done + t0; i < n; i += stride) {
-        x[i] = fmaf(alpha, p[i], x[i]);
-        const float ri = fmaf(-alpha, q[i], r[i]);
-        r[i] = ri;
-        acc += static_cast<double>(ri * ri);
-    }
-    block_sum(acc, partials);
-}
-
-__global__ void __launch_bounds__(kThreads) k_fill(float* __restrict__ x, float value, size_t n)
-{
-    const size_t stride = static_cast<size_t>(gridDim.x) * kThreads;
-    for (size_t i = blockIdx.x * static_cast<size_t>(kThreads) + threadIdx.x; i < n; i += stride)
-        x[i] = value;
 }
 
 unsigned stream_blocks(size_t n)
@@ -775,8 +659,7 @@ __global__ void __launch_bounds__(kThreads) k_tl_restrict(Grid gf, const float2*
 __global__ void __launch_bounds__(kThreads) k_tl_start(Grid gf, const float2* __restrict__ rf, size_t csf,
                                                         Grid gc, float2* __restrict__ rh, float2* __restrict__ xh,
                                                         float2* __restrict__ ph, float2* __restrict__ cp, size_t cs,
-                                                        int op, RegParams rp, double* __restrict__ prr,
-                                                        double* __restrict__ prz)
+                                                        int op, RegParams rp, double* __restrict__ sc, Reduction red)
 {
     const int n3h = gc.n3 / 2 + 1;
     const size_t Mc = static_cast<size_t>(gc.n1) * gc.n2 * n3h;
@@ -804,7 +687,8 @@ __global__ void __launch_bounds__(kThreads) k_tl_start(Grid gf, const float2* __
         arr += static_cast<double>(m.wt * cdot3(r[0], r[1], r[2], r[0], r[1], r[2]));
         arz += static_cast<double>(m.wt * cdot3(r[0], r[1], r[2], z[0], z[1], z[2]));
     }
-    block_sum2(arr, arz, prr, prz);
+    double tot[2];
+    if (grid_sum2(arr, arz, red, tot)) sc[kTlRz] = tot[1];
 }
 
 // In place on the coarse real fields: p <- gbar (gbar . p).
@@ -826,7 +710,7 @@ __global__ void __launch_bounds__(kThreads) k_tl_rank1(const float* __restrict__
 __global__ void __launch_bounds__(kThreads) k_tl_hp(Grid gc, const float2* __restrict__ T,
                                                      const float2* __restrict__ ph, float2* __restrict__ q,
                                                      size_t cs, int kform, RegParams rp, float scale,
-                                                     double* __restrict__ ppq)
+                                                     double* __restrict__ sc, Reduction red)
 {
     const int n3h = gc.n3 / 2 + 1;
     const size_t Mc = static_cast<size_t>(gc.n1) * gc.n2 * n3h;
@@ -858,33 +742,23 @@ __global__ void __launch_bounds__(kThreads) k_tl_hp(Grid gc, const float2* __res
         for (int c = 0; c < 3; ++c) q[c * cs + idx] = h[c];
         acc += static_cast<double>(m.wt * cdot3(p0, p1, p2, h[0], h[1], h[2]));
     }
-    block_sum(acc, ppq);
-}
-
-// x += alpha p, r -= alpha q, z = M r (stored); partials of |r|^2 and <r, z>.
-// Scalars of the inner PCG kept on the device (slots of TlScalar): after the
-// curvature pq (stage 0) alpha = rz / pq, or 0 with the breakdown flag set
-// when pq <= 0 (1) or NaN (2); before the direction update (stage 1) beta = rz_new / rz and
-// rz <- rz_new.  FP64 divisions, as the host would do them.
-__global__ void k_tl_scalars(double* __restrict__ s, int stage)
-{
-    if (stage == 0) {
-        const double pq = s[kTlPq];
-        s[kTlAlpha] = pq > 0.0 ? s[kTlRz] / pq : 0.0;
-        s[kTlFlag] = pq > 0.0 ? 0.0 : (pq == pq ? 1.0 : 2.0);  // 2: pq is NaN
-    } else {
-        s[kTlBeta] = s[kTlRzNew] / s[kTlRz];
-        s[kTlRz] = s[kTlRzNew];
+    double pq;
+    if (grid_sum(acc, red, &pq)) {
+        // alpha = rz / pq, or 0 with the breakdown flag set when pq <= 0 (1) or
+        // NaN (2); FP64 divisions, as the host would do them
+        sc[kTlAlpha] = pq > 0.0 ? sc[kTlRz] / pq : 0.0;
+        put_result(red, 1, pq > 0.0 ? 0.0 : (pq == pq ? 1.0 : 2.0));
     }
 }
 
+// x += alpha p, r -= alpha q, z = M r (stored); totals |r|^2 and <r, z>, then
+// beta = rz_new / rz and rz <- rz_new for the next direction.
 __global__ void __launch_bounds__(kThreads) k_tl_update(Grid gc, const float2* __restrict__ ph,
                                                          const float2* __restrict__ q, float2* __restrict__ xh,
                                                          float2* __restrict__ rh, float2* __restrict__ zh, size_t cs,
-                                                         const double* __restrict__ alpha_dev, int op, RegParams rp,
-                                                         double* __restrict__ prr, double* __restrict__ prz)
+                                                         double* __restrict__ sc, int op, RegParams rp, Reduction red)
 {
-    const float alpha = static_cast<float>(*alpha_dev);
+    const float alpha = static_cast<float>(sc[kTlAlpha]);
     const int n3h = gc.n3 / 2 + 1;
     const size_t Mc = static_cast<size_t>(gc.n1) * gc.n2 * n3h;
     double arr = 0.0, arz = 0.0;
@@ -908,7 +782,11 @@ __global__ void __launch_bounds__(kThreads) k_tl_update(Grid gc, const float2* _
         arr += static_cast<double>(m.wt * cdot3(r[0], r[1], r[2], r[0], r[1], r[2]));
         arz += static_cast<double>(m.wt * cdot3(r[0], r[1], r[2], z0, z1, z2));
     }
-    block_sum2(arr, arz, prr, prz);
+    double tot[2];
+    if (grid_sum2(arr, arz, red, tot)) {
+        sc[kTlBeta] = tot[1] / sc[kTlRz];
+        sc[kTlRz] = tot[1];
+    }
 }
 
 // p = z + beta p (p = z when first) and its copy cp for the inverse transform;
@@ -941,8 +819,7 @@ __global__ void __launch_bounds__(kThreads) k_dir_stored(Grid g, const float2* _
 __global__ void __launch_bounds__(kThreads) k_tl_finish(Grid gf, const float2* __restrict__ rf,
                                                          float2* __restrict__ zf, const float2* __restrict__ zold,
                                                          size_t csf, Grid gc, const float2* __restrict__ xc,
-                                                         size_t csc, int op, RegParams rp, double* __restrict__ prz,
-                                                         double* __restrict__ pro)
+                                                         size_t csc, int op, RegParams rp, Reduction red)
 {
     const int n3h = gf.n3 / 2 + 1;
     const size_t M = static_cast<size_t>(gf.n1) * gf.n2 * n3h;
@@ -968,7 +845,8 @@ __global__ void __launch_bounds__(kThreads) k_tl_finish(Grid gf, const float2* _
         if (zold)
             ao += static_cast<double>(m.wt * cdot3(r0, r1, r2, zold[idx], zold[csf + idx], zold[2 * csf + idx]));
     }
-    block_sum2(az, ao, prz, pro);
+    double tot[2];
+    grid_sum2(az, ao, red, tot);
 }
 
 }  // namespace
@@ -979,13 +857,6 @@ void launch_spectral(const Grid& g, cufftComplex* xh, size_t cstride, SpectralOp
     const size_t M = static_cast<size_t>(g.n1) * g.n2 * (g.n3 / 2 + 1);
     k_spectral<<<stream_blocks(M), kThreads, 0, st>>>(g, reinterpret_cast<float2*>(xh), cstride,
                                                      static_cast<int>(op), rp, scale);
-}
-
-void launch_spectral_precond(const Grid& g, cufftComplex* xh, size_t cstride, SpectralOp op,
-                             RegParams rp, float scale, double* partials, int nblocks, cudaStream_t st)
-{
-    k_spectral_precond<<<nblocks, kThreads, 0, st>>>(g, reinterpret_cast<float2*>(xh), cstride,
-                                                    static_cast<int>(op), rp, scale, partials);
 }
 
 void launch_spectral_direction(const Grid& g, const cufftComplex* rh, cufftComplex* ph, cufftComplex* cp,
@@ -999,31 +870,30 @@ void launch_spectral_direction(const Grid& g, const cufftComplex* rh, cufftCompl
 }
 
 void launch_fs_start(const Grid& g, cufftComplex* spec, cufftComplex* rh, cufftComplex* xh, size_t cs,
-                     SpectralOp op, RegParams rp, float scale, double* prr, double* prz, int nblocks,
-                     cudaStream_t st)
+                     SpectralOp op, RegParams rp, float scale, const Reduction& red, cudaStream_t st)
 {
-    k_fs_start<<<nblocks, kThreads, 0, st>>>(g, reinterpret_cast<float2*>(spec), reinterpret_cast<float2*>(rh),
+    k_fs_start<<<red.nblocks, kThreads, 0, st>>>(g, reinterpret_cast<float2*>(spec), reinterpret_cast<float2*>(rh),
                                              reinterpret_cast<float2*>(xh), cs, static_cast<int>(op), rp,
-                                             scale, prr, prz);
+                                             scale, red);
 }
 
 void launch_fs_hp(const Grid& g, cufftComplex* spec, const cufftComplex* spec2, const cufftComplex* ph,
-                  size_t cs, int kform, RegParams rp, float scale, double* ppq, int nblocks, cudaStream_t st)
+                  size_t cs, int kform, RegParams rp, float scale, const Reduction& red, cudaStream_t st)
 {
-    k_fs_hp<<<nblocks, kThreads, 0, st>>>(g, reinterpret_cast<float2*>(spec),
+    k_fs_hp<<<red.nblocks, kThreads, 0, st>>>(g, reinterpret_cast<float2*>(spec),
                                           reinterpret_cast<const float2*>(spec2),
-                                          reinterpret_cast<const float2*>(ph), cs, kform, rp, scale, ppq);
+                                          reinterpret_cast<const float2*>(ph), cs, kform, rp, scale, red);
 }
 
 void launch_fs_update(const Grid& g, cufftComplex* spec, const cufftComplex* ph, cufftComplex* xh,
                       cufftComplex* rh, const cufftComplex* zc, size_t cs, float alpha, SpectralOp op, RegParams rp,
-                      double* prr, double* prz, int nblocks, cudaStream_t st)
+                      const Reduction& red, cudaStream_t st)
 {
-    k_fs_update<<<nblocks, kThreads, 0, st>>>(g, reinterpret_cast<const float2*>(spec),
+    k_fs_update<<<red.nblocks, kThreads, 0, st>>>(g, reinterpret_cast<const float2*>(spec),
                                               reinterpret_cast<const float2*>(ph),
                                               reinterpret_cast<float2*>(xh), reinterpret_cast<float2*>(rh),
                                               reinterpret_cast<const float2*>(zc), cs, alpha, static_cast<int>(op),
-                                              rp, prr, prz);
+                                              rp, red);
 }
 
 void launch_mean_levels(const void* m, int nt, float w_end, float w_mid, size_t N, float* out, Storage sto,
@@ -1069,12 +939,12 @@ void launch_tl_restrict(const Grid& gf, const cufftComplex* F, size_t csf, const
 
 void launch_tl_start(const Grid& gf, const cufftComplex* rf, size_t csf, const Grid& gc, cufftComplex* rh,
                      cufftComplex* xh, cufftComplex* ph, cufftComplex* cp, size_t cs, SpectralOp op, RegParams rp,
-                     double* prr, double* prz, int nblocks, cudaStream_t st)
+                     double* sc, const Reduction& red, cudaStream_t st)
 {
-    k_tl_start<<<nblocks, kThreads, 0, st>>>(gf, reinterpret_cast<const float2*>(rf), csf, gc,
+    k_tl_start<<<red.nblocks, kThreads, 0, st>>>(gf, reinterpret_cast<const float2*>(rf), csf, gc,
                                              reinterpret_cast<float2*>(rh), reinterpret_cast<float2*>(xh),
                                              reinterpret_cast<float2*>(ph), reinterpret_cast<float2*>(cp), cs,
-                                             static_cast<int>(op), rp, prr, prz);
+                                             static_cast<int>(op), rp, sc, red);
 }
 
 void launch_tl_rank1(const float* gbar, float* p, size_t Nc, cudaStream_t st)
@@ -1083,25 +953,20 @@ void launch_tl_rank1(const float* gbar, float* p, size_t Nc, cudaStream_t st)
 }
 
 void launch_tl_hp(const Grid& gc, const cufftComplex* T, const cufftComplex* ph, cufftComplex* q, size_t cs,
-                  int kform, RegParams rp, float scale, double* ppq, int nblocks, cudaStream_t st)
+                  int kform, RegParams rp, float scale, double* sc, const Reduction& red, cudaStream_t st)
 {
-    k_tl_hp<<<nblocks, kThreads, 0, st>>>(gc, reinterpret_cast<const float2*>(T), reinterpret_cast<const float2*>(ph),
-                                          reinterpret_cast<float2*>(q), cs, kform, rp, scale, ppq);
+    k_tl_hp<<<red.nblocks, kThreads, 0, st>>>(gc, reinterpret_cast<const float2*>(T), reinterpret_cast<const float2*>(ph),
+                                          reinterpret_cast<float2*>(q), cs, kform, rp, scale, sc, red);
 }
 
 void launch_tl_update(const Grid& gc, const cufftComplex* ph, const cufftComplex* q, cufftComplex* xh,
-                      cufftComplex* rh, cufftComplex* zh, size_t cs, const double* alpha_dev, SpectralOp op,
-                      RegParams rp, double* prr, double* prz, int nblocks, cudaStream_t st)
+                      cufftComplex* rh, cufftComplex* zh, size_t cs, double* sc, SpectralOp op, RegParams rp,
+                      const Reduction& red, cudaStream_t st)
 {
-    k_tl_update<<<nblocks, kThreads, 0, st>>>(gc, reinterpret_cast<const float2*>(ph),
+    k_tl_update<<<red.nblocks, kThreads, 0, st>>>(gc, reinterpret_cast<const float2*>(ph),
                                               reinterpret_cast<const float2*>(q), reinterpret_cast<float2*>(xh),
                                               reinterpret_cast<float2*>(rh), reinterpret_cast<float2*>(zh), cs,
-                                              alpha_dev, static_cast<int>(op), rp, prr, prz);
-}
-
-void launch_tl_scalars(double* s, int stage, cudaStream_t st)
-{
-    k_tl_scalars<<<1, 1, 0, st>>>(s, stage);
+                                              sc, static_cast<int>(op), rp, red);
 }
 
 void launch_dir_stored(const Grid& g, const cufftComplex* zh, cufftComplex* ph, cufftComplex* cp, size_t cs,
@@ -1114,58 +979,36 @@ void launch_dir_stored(const Grid& g, const cufftComplex* zh, cufftComplex* ph, 
 }
 
 void launch_tl_finish(const Grid& gf, const cufftComplex* rf, cufftComplex* zf, const cufftComplex* zold, size_t csf,
-                      const Grid& gc, const cufftComplex* xc, size_t csc, SpectralOp op, RegParams rp, double* prz,
-                      double* pro, int nblocks, cudaStream_t st)
+                      const Grid& gc, const cufftComplex* xc, size_t csc, SpectralOp op, RegParams rp,
+                      const Reduction& red, cudaStream_t st)
 {
-    k_tl_finish<<<nblocks, kThreads, 0, st>>>(gf, reinterpret_cast<const float2*>(rf), reinterpret_cast<float2*>(zf),
+    k_tl_finish<<<red.nblocks, kThreads, 0, st>>>(gf, reinterpret_cast<const float2*>(rf), reinterpret_cast<float2*>(zf),
                                               reinterpret_cast<const float2*>(zold), csf, gc,
-                                              reinterpret_cast<const float2*>(xc), csc, static_cast<int>(op), rp, prz,
-                                              pro);
+                                              reinterpret_cast<const float2*>(xc), csc, static_cast<int>(op), rp,
+                                              red);
 }
 
-void launch_dot_partial(const float* x, const float* y, size_t n, double* partials, int nblocks,
-                        cudaStream_t st)
+void launch_dot(const float* x, const float* y, size_t n, const Reduction& red, cudaStream_t st)
 {
-    k_dot_partial<<<nblocks, kThreads, 0, st>>>(x, y, n, partials);
+    k_dot<<<red.nblocks, kThreads, 0, st>>>(x, y, n, red);
 }
 
-void launch_sqdiff_partial(const void* a, const void* b, size_t n, double* partials, int nblocks,
-                           Storage sto, cudaStream_t st)
+void launch_sqdiff(const void* a, const void* b, size_t n, Storage sto, const Reduction& red, cudaStream_t st)
 {
     CLAIRE_STORAGE_DISPATCH(sto, {
-        k_sqdiff_partial<SType><<<nblocks, kThreads, 0, st>>>(static_cast<const SType*>(a),
-                                                             static_cast<const SType*>(b), n, partials);
+        k_sqdiff<SType><<<red.nblocks, kThreads, 0, st>>>(static_cast<const SType*>(a), static_cast<const SType*>(b), n,
+                                                          red);
     });
 }
 
-void launch_maxnorm3_partial(const float* v, size_t N, double* partials, int nblocks,
-                             cudaStream_t st)
+void launch_maxnorm3(const float* v, size_t N, const Reduction& red, cudaStream_t st)
 {
-    k_maxnorm3_partial<<<nblocks, kThreads, 0, st>>>(v, N, partials);
+    k_maxnorm3<<<red.nblocks, kThreads, 0, st>>>(v, N, red);
 }
 
-void launch_count_partial(const float* a, const float* b, size_t n, float t, int both, double* pa, double* pb,
-                          int nblocks, cudaStream_t st)
+void launch_count(const float* a, const float* b, size_t n, float t, int both, const Reduction& red, cudaStream_t st)
 {
-    k_count_partial<<<nblocks, kThreads, 0, st>>>(a, b, n, t, both, pa, pb);
-}
-
-void launch_final_sum(const double* partials, int nblocks, double scale, double* out,
-                      cudaStream_t st)
-{
-    k_final_sum<<<1, kThreads, 0, st>>>(partials, nblocks, scale, out);
-}
-
-void launch_final_max(const double* partials, int nblocks, double* out, cudaStream_t st)
-{
-    // out[0] is left alone, out[1] receives the maximum
-    k_final_max<<<1, kThreads, 0, st>>>(partials, nblocks, out + 1);
-}
-
-void launch_final_minmax(const double* pmin, const double* pmax, int nblocks, double* out2,
-                         cudaStream_t st)
-{
-    k_final_minmax<<<1, kThreads, 0, st>>>(pmin, pmax, nblocks, out2);
+    k_count<<<red.nblocks, kThreads, 0, st>>>(a, b, n, t, both, red);
 }
 
 void launch_axpy(float a, const float* x, float* y, size_t n, cudaStream_t st)
@@ -1176,17 +1019,6 @@ void launch_axpy(float a, const float* x, float* y, size_t n, cudaStream_t st)
 void launch_xpay(const float* x, float a, const float* y, float* z, size_t n, cudaStream_t st)
 {
     k_xpay<<<stream_blocks(n), kThreads, 0, st>>>(x, a, y, z, n);
-}
-
-void launch_pcg_update(float alpha, const float* p, const float* q, float* x, float* r, size_t n,
-                       double* partials, int nblocks, cudaStream_t st)
-{
-    k_pcg_update<<<nblocks, kThreads, 0, st>>>(alpha, p, q, x, r, n, partials);
-}
-
-void launch_fill(float* x, float value, size_t n, cudaStream_t st)
-{
-    k_fill<<<stream_blocks(n), kThreads, 0, st>>>(x, value, n);
 }
 
 }  // namespace claire

@@ -654,13 +654,11 @@ __global__ void __launch_bounds__(kThreads) k_scale_add(float* __restrict__ y, f
     if (p < n) y[p] = a * (y[p] + x[p]);
 }
 
-// max |x| over n values (as doubles) into the first gridDim.x partials.  The
+// max |x| over n values (as a double).  The
 // maximum is taken on the FP32 bit patterns, which order like the magnitudes;
 // NaN becomes infinity, which the reductions keep.
-__global__ void __launch_bounds__(kThreads) k_maxabs_partial(const float* __restrict__ x, size_t n,
-                                                              double* __restrict__ partials)
+__global__ void __launch_bounds__(kThreads) k_maxabs(const float* __restrict__ x, size_t n, Reduction red)
 {
-    __shared__ unsigned red[kThreads / 32];
     unsigned hi = 0;
     const size_t stride = static_cast<size_t>(gridDim.x) * kThreads;
     const size_t t0 = blockIdx.x * static_cast<size_t>(kThreads) + threadIdx.x;
@@ -675,14 +673,8 @@ __global__ void __launch_bounds__(kThreads) k_maxabs_partial(const float* __rest
         done = 4 * n4;
     }
     for (size_t i = done + t0; i < n; i += stride) hi = max(hi, __float_as_uint(x[i]) & 0x7fffffffu);
-    hi = __reduce_max_sync(0xffffffffu, hi);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = hi;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int w = 1; w < kThreads / 32; ++w) hi = max(hi, red[w]);
-        partials[blockIdx.x] = __uint_as_float(min(hi, 0x7f800000u));
-    }
+    const double m = __uint_as_float(min(hi, 0x7f800000u));
+    grid_max_bits(static_cast<unsigned long long>(__double_as_longlong(m)), red);
 }
 
 }  // namespace
@@ -770,10 +762,9 @@ void launch_scale_add(float* y, float a, const float* x, size_t n, cudaStream_t 
     k_scale_add<<<blocks_for(n), kThreads, 0, st>>>(y, a, x, n);
 }
 
-void launch_maxabs(const float* x, size_t n, double* partials, int nblocks, double* out2, cudaStream_t st)
+void launch_maxabs(const float* x, size_t n, const Reduction& red, cudaStream_t st)
 {
-    k_maxabs_partial<<<nblocks, kThreads, 0, st>>>(x, n, partials);
-    launch_final_max(partials, nblocks, out2, st);
+    k_maxabs<<<red.nblocks, kThreads, 0, st>>>(x, n, red);
 }
 
 }  // namespace claire
