@@ -266,6 +266,21 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t saddr, uint32_t lbo, uint
            (static_cast<uint64_t>((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46);
 }
 
+// One MMA (M = 128 or 64 by the instruction descriptor, BF16, FP32 accumulator at
+// dt) issued by this thread.  A descriptor is given by its two words: stepping
+// an operand's start address (16-byte units, below 2^14) changes only the low
+// one, one 32-bit addition.  A single thread issues all MMAs of a CTA, so the
+// instructions around each of them are on the critical path: with 64-bit
+// descriptors rebuilt per MMA in rolled loops an issue took 100 cycles
+// (forward) to 300 (weight gradient), several times the MMA itself.
+__device__ __forceinline__ void umma(uint32_t dt, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
+                                     uint32_t idesc, uint32_t accum)
+{
+    asm volatile("{\n .reg .pred p;\n .reg .b64 a, b;\n mov.b64 a, {%1, %2};\n mov.b64 b, {%3, %4};\n"
+                 " setp.ne.b32 p, %6, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n}\n" ::"r"(dt),
+                 "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accum));
+}
+
 __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity)
 {
     const uint32_t limit = g_tc_spin_limit;
@@ -331,7 +346,8 @@ __device__ __forceinline__ void cp_async_wait_group()
 
 struct TcShape {
     int bdc;        // D planes per brick
-    int ccols;      // TMEM columns per plane (Cout rounded up to 32)
+    int stack;      // 1: the kd taps are stacked along N (3 Cout <= 256)
+    int ccols;      // TMEM columns per plane (Cout; unstacked: rounded up to 32)
     int nstage;     // 1 or 2 staging buffers
     int plane;      // bytes of one 8-channel half plane of the halo
     int stage;      // bytes of one stage (halo + weights)
@@ -357,8 +373,55 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3d_tc(const __nv_bfloat16*
     const int h0 = (r % nbh) * kTcBH; r /= nbh;
     const int d0 = (r % nbd) * bdc;
     const int b = r / nbd;
-    const int slots = (bdc + 2) * kTcPlaneSlots;
     const uint32_t smem_s = smem_addr(tc_smem), mbar_s = smem_addr(&mbar);
+    const int nchunks = Cin / 16;
+    // staging: 16-byte pieces of the halo plane e = tid + 128 u < 360, piece e =
+    // half e & 1 (8 channels) of slot e >> 1 = (sh * 10 + sw); the wrapped (h, w)
+    // offsets are formed once, a plane costs one pointer step
+    uint32_t goff[3], soff[3];
+#pragma unroll
+    for (int u = 0; u < 3; ++u) {
+        const int e = min(tid + u * kConvThreads, 2 * kTcPlaneSlots - 1);
+        const int sl = e >> 1, hlf = e & 1, shh = sl / kTcHaloW, sw = sl - shh * kTcHaloW;
+        goff[u] = (static_cast<uint32_t>(wrapi(h0 + shh - 1, v.H)) * v.W + wrapi(w0 + sw - 1, v.W)) * Cxs + 8 * hlf;
+        soff[u] = hlf * sh.plane + sl * 16;
+    }
+    const bool third = tid + 2 * kConvThreads < 2 * kTcPlaneSlots;
+    const size_t plane_elems = static_cast<size_t>(v.H) * v.W * Cxs;
+    auto issue = [&](int c, int stg) {
+        const int c0 = 16 * c;
+        uint32_t dst = smem_s + stg * sh.stage;
+        const uint32_t wb = dst + 2 * sh.plane;
+        const __nv_bfloat16* xb = X + static_cast<size_t>(b) * v.D * plane_elems + c0;
+        int d = wrapi(d0 - 1, v.D);
+        for (int sd = 0; sd < bdc + 2; ++sd) {
+            const __nv_bfloat16* xp = xb + d * plane_elems;
+            cp_async16(dst + soff[0], xp + goff[0]);
+            cp_async16(dst + soff[1], xp + goff[1]);
+            if (third) cp_async16(dst + soff[2], xp + goff[2]);
+            dst += kTcPlaneSlots * 16;
+            d = d + 1 == v.D ? 0 : d + 1;
+        }
+        // weights: 16 output channels x 8 (tap, half) pieces at a time.  Stacked: row
+        // block 2 - kd of the (kh, kw) tap; else the tap's own rows.
+        const int co16 = tid & 15, q0 = tid >> 4;
+        for (int co = co16; co < Cout; co += 16) {
+            const __nv_bfloat16* src = Wt + static_cast<size_t>(co) * 27 * Cin + c0;
+            for (int q = q0; q < 54; q += 8) {
+                const int tap = q >> 1, hlf = q & 1;
+                int row;  // 16-byte rows from wb
+                if (sh.stack) {
+                    const int kd = tap / 9;
+                    row = ((tap - 9 * kd) * 2 + hlf) * 3 * Cout + (2 - kd) * Cout + co;
+                } else {
+                    row = q * Cout + co;
+                }
+                cp_async16(wb + row * 16, src + tap * Cin + 8 * hlf);
+            }
+        }
+        cp_async_commit();
+    };
+    issue(0, 0);  // in flight while tensor memory is allocated
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&tmem_slot)),
                      "r"(sh.cols));
@@ -379,30 +442,10 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3d_tc(const __nv_bfloat16*
     bool ok = true;
     if (stall) ok = __syncthreads_and(mbar_wait(mbar_s, 0)) != 0;
     const bool stalled = !ok;  // gave up before any MMA was issued
-    // instruction descriptor: D F32, A and B BF16, both K-major, N = Cout, M = 128
-    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((static_cast<uint32_t>(Cout) >> 3) << 17) |
-                           ((128u >> 4) << 24);
-    const int nchunks = Cin / 16;
-    // stage a slice: halo slot s = (sd * 18 + sh) * 10 + sw in half plane h; weight piece (tap, half, co)
-    auto issue = [&](int c, int stg) {
-        const int c0 = 16 * c;
-        const uint32_t base = smem_s + stg * sh.stage;
-        for (int e = tid; e < 2 * slots; e += kConvThreads) {
-            const int hlf = e / slots, sl = e - hlf * slots;
-            const int sw = sl % kTcHaloW, shh = (sl / kTcHaloW) % kTcHaloH, sd = sl / kTcPlaneSlots;
-            const int d = wrapi(d0 + sd - 1, v.D), h = wrapi(h0 + shh - 1, v.H), w = wrapi(w0 + sw - 1, v.W);
-            const size_t vox = ((static_cast<size_t>(b) * v.D + d) * v.H + h) * v.W + w;
-            cp_async16(base + hlf * sh.plane + sl * 16, X + vox * Cxs + c0 + 8 * hlf);
-        }
-        const uint32_t wb = base + 2 * sh.plane;
-        const int npieces = 27 * 2 * Cout;
-        for (int e = tid; e < npieces; e += kConvThreads) {
-            const int co = e % Cout, hlf = (e / Cout) & 1, tap = e / (2 * Cout);
-            cp_async16(wb + e * 16, Wt + (static_cast<size_t>(co) * 27 + tap) * Cin + c0 + 8 * hlf);
-        }
-        cp_async_commit();
+    // instruction descriptor: D F32, A and B BF16, both K-major, M = 128, N = n
+    auto idesc = [](int n) {
+        return (1u << 4) | (1u << 7) | (1u << 10) | ((static_cast<uint32_t>(n) >> 3) << 17) | ((128u >> 4) << 24);
     };
-    if (ok) issue(0, 0);
     for (int c = 0; c < nchunks && ok; ++c) {
         const int stg = sh.nstage == 2 ? (c & 1) : 0;
         // every completion phase is waited for exactly once and in order, so
@@ -427,21 +470,46 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3d_tc(const __nv_bfloat16*
         asm volatile("tcgen05.fence::after_thread_sync;");
         if (tid == 0) {
             const uint32_t base = smem_s + stg * sh.stage;
-            const uint32_t wb = base + 2 * sh.plane;
-#pragma unroll 1
-            for (int z = 0; z < bdc; ++z)
-#pragma unroll 1
-                for (int tap = 0; tap < 27; ++tap) {
-                    const int kd = tap / 9, kh = (tap / 3) % 3, kw = tap % 3;
-                    const uint32_t a_addr = base + (((z + kd) * kTcHaloH + kh) * kTcHaloW + kw) * 16;
-                    const uint64_t ad = umma_desc(a_addr, sh.plane, kTcHaloW * 16);
-                    const uint64_t bd = umma_desc(wb + tap * 2 * Cout * 16, Cout * 16, 128);
-                    const uint32_t accum = (c > 0 || tap > 0) ? 1u : 0u;
-                    const uint32_t dt = tmem + static_cast<uint32_t>(z * sh.ccols);
-                    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                                 " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dt),
-                                 "l"(ad), "l"(bd), "r"(idesc), "r"(accum));
+            const uint64_t ad = umma_desc(base, sh.plane, kTcHaloW * 16);
+            const uint64_t bd = umma_desc(base + 2 * sh.plane, (sh.stack ? 3 : 1) * Cout * 16, 128);
+            const uint32_t a_lo = static_cast<uint32_t>(ad), a_hi = static_cast<uint32_t>(ad >> 32);
+            const uint32_t b_lo = static_cast<uint32_t>(bd), b_hi = static_cast<uint32_t>(bd >> 32);
+            if (sh.stack) {
+                // input plane sd feeds the output planes z = sd - kd: blocks j = 2 - kd
+                // of N, at the columns of z = sd - 2 + j, clipped to the brick
+                const uint32_t bstep = 6u * Cout;
+                for (int sd = 0; sd < bdc + 2; ++sd) {
+                    const int j0 = sd < 2 ? 2 - sd : 0, j1 = sd < bdc ? 3 : bdc + 2 - sd;
+                    const uint32_t ap = a_lo + static_cast<uint32_t>(sd * kTcPlaneSlots);
+                    const uint32_t bp = b_lo + static_cast<uint32_t>(j0 * Cout);
+                    const uint32_t dt = tmem + static_cast<uint32_t>((sd - 2 + j0) * Cout);
+                    const uint32_t id = idesc((j1 - j0) * Cout);
+                    // plane z = sd sees its first product here (kd = 0): written, not added
+                    if (c == 0 && j1 == 3) {
+                        if (j0 < 2) umma(dt, ap, a_hi, bp, b_hi, idesc((2 - j0) * Cout), 1u);
+                        umma(tmem + static_cast<uint32_t>(sd * Cout), ap, a_hi, b_lo + 2u * Cout, b_hi, idesc(Cout), 0u);
+                    } else {
+                        umma(dt, ap, a_hi, bp, b_hi, id, 1u);
+                    }
+#pragma unroll
+                    for (int t = 1; t < 9; ++t)
+                        umma(dt, ap + (t / 3) * kTcHaloW + t % 3, a_hi, bp + t * bstep, b_hi, id, 1u);
                 }
+            } else {
+                const uint32_t id = idesc(Cout), bstep = 2u * Cout;
+                for (int z = 0; z < bdc; ++z) {
+                    const uint32_t dt = tmem + static_cast<uint32_t>(z * sh.ccols);
+                    uint32_t ap = a_lo + static_cast<uint32_t>(z * kTcPlaneSlots), bp = b_lo;
+                    for (int kd = 0; kd < 3; ++kd) {
+                        umma(dt, ap, a_hi, bp, b_hi, id, c > 0 || kd > 0 ? 1u : 0u);
+#pragma unroll
+                        for (int t = 1; t < 9; ++t)
+                            umma(dt, ap + (t / 3) * kTcHaloW + t % 3, a_hi, bp + t * bstep, b_hi, id, 1u);
+                        ap += kTcPlaneSlots;
+                        bp += 9 * bstep;
+                    }
+                }
+            }
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar_s)
                          : "memory");
         }
@@ -618,14 +686,19 @@ __global__ void __launch_bounds__(kWgThreads) k_wgrad_tc(const __nv_bfloat16* __
         const int nl = kWgLoaders / S;
         const int grp = (tid - 64) / nl, lt = (tid - 64) - grp * nl;
         // a row's pieces are spread over the group's threads (several rows
-        // per pass when a row has fewer pieces than the group has threads)
+        // per pass when a row has fewer pieces than the group has threads, as
+        // it does unless the layer is wide: then a thread keeps its voxel slot
+        // and channel block, and a row costs two address steps)
         const int tja = 8 * cbn;  // dY: pieces per brick row
-        const int rppa = tja <= nl ? nl / tja : 1, stepa = tja <= nl ? tja : nl;
+        const int rppa = tja <= nl ? nl / tja : 1;
         const int ja_r = tja <= nl ? lt / tja : 0, ja0 = tja <= nl ? lt - ja_r * tja : lt;
+        const int a_vox = ja0 / cbn, a_cb = ja0 - a_vox * cbn;
         const int tjx = kTcHaloW * nq;  // X: pieces per halo row
         const int rppx = tjx <= nl ? nl / tjx : 1, stepx = tjx <= nl ? tjx : nl;
         const int jx_r = tjx <= nl ? lt / tjx : 0, jx0 = tjx <= nl ? lt - jx_r * tjx : lt;
-        const size_t row_y = static_cast<size_t>(v.W) * Cys, row_x = static_cast<size_t>(v.W) * Cxs;
+        const uint32_t row_y = static_cast<uint32_t>(v.W) * Cys, row_x = static_cast<uint32_t>(v.W) * Cxs;
+        const size_t plane_y = static_cast<size_t>(v.H) * row_y, plane_x = static_cast<size_t>(v.H) * row_x;
+        const uint32_t xrow_s = static_cast<uint32_t>(nq) * (wg.nkw == 1 ? 160 : 3 * 128);  // bytes of a staged halo row
         const int nbw = v.W / kTcBW, nbh = v.H / kTcBH;
         const uint32_t a_s = s0 + grp * stage_bytes, h_s = a_s + wg.abytes;
         for (int j = grp; j < nbr; j += S) {
@@ -647,41 +720,56 @@ __global__ void __launch_bounds__(kWgThreads) k_wgrad_tc(const __nv_bfloat16* __
             const int w0 = (r % nbw) * kTcBW; r /= nbw;
             const int h0 = (r % nbh) * kTcBH;
             const int b = r / nbh;
-            // dY rows (s, hr): 8 voxels x cbn pieces -> hr * albo + (s * cbn + cb) * 128 + voxel * 16
+            // dY rows (sb, hr): 8 voxels x cbn pieces -> hr * albo + (sb * cbn + cb) * 128 + voxel * 16
             if (ja_r < rppa) {
-                for (int rr = ja_r; rr < 16 * wg.nsa; rr += rppa) {
-                    const int sb = rr >> 4, hr = rr & 15;
+                for (int sb = 0; sb < wg.nsa; ++sb) {
                     const int d = wg.nsa == 3 ? wrapi(d0 + sb - 1, v.D) : d0;
-                    const __nv_bfloat16* rowp = dY + ((static_cast<size_t>(b) * v.D + d) * v.H + h0 + hr) * row_y +
-                                                static_cast<size_t>(w0) * Cys + co0;
-                    for (int jj = ja0; jj < tja; jj += stepa) {
-                        const int vox = jj / cbn, cb = jj - vox * cbn;
-                        cp_async16(a_s + hr * albo + (sb * cbn + cb) * 128 + vox * 16,
-                                   rowp + static_cast<size_t>(vox) * Cys + 8 * cb);
+                    const __nv_bfloat16* rowp = dY + (static_cast<size_t>(b) * v.D + d) * plane_y +
+                                                static_cast<uint32_t>(h0 + ja_r) * row_y +
+                                                static_cast<uint32_t>(w0) * Cys + co0;
+                    uint32_t dst = a_s + ja_r * albo + sb * cbn * 128;
+                    if (tja <= nl) {
+                        rowp += static_cast<uint32_t>(a_vox) * Cys + 8 * a_cb;
+                        dst += a_cb * 128 + a_vox * 16;
+                        for (int hr = ja_r; hr < kTcBH; hr += rppa) {
+                            cp_async16(dst, rowp);
+                            rowp += rppa * row_y;
+                            dst += rppa * albo;
+                        }
+                    } else {
+                        for (int hr = 0; hr < kTcBH; ++hr) {
+                            for (int jj = ja0; jj < tja; jj += nl) {
+                                const int vox = jj / cbn, cb = jj - vox * cbn;
+                                cp_async16(dst + cb * 128 + vox * 16, rowp + static_cast<size_t>(vox) * Cys + 8 * cb);
+                            }
+                            rowp += row_y;
+                            dst += albo;
+                        }
                     }
                 }
             }
             // X halo rows (sd, sh): 10 voxel slots x nq pieces
             if (jx_r < rppx) {
-                for (int rr = jx_r; rr < kTcHaloH * wg.npl; rr += rppx) {
-                    const int sd = rr / kTcHaloH, sh = rr - sd * kTcHaloH;
-                    const int d = wg.npl == 3 ? wrapi(d0 + sd - 1, v.D) : d0;
-                    const int h = wrapi(h0 + sh - 1, v.H);
-                    const __nv_bfloat16* rowp =
-                        X + ((static_cast<size_t>(b) * v.D + d) * v.H + h) * row_x + ci0;
-                    for (int jj = jx0; jj < tjx; jj += stepx) {
-                        const int x_sw = jj / nq, x_q = jj - x_sw * nq;
-                        const __nv_bfloat16* src =
-                            rowp + static_cast<size_t>(wrapi(w0 + x_sw - 1, v.W)) * Cxs + 8 * x_q;
-                        if (wg.nkw == 1) {
-                            cp_async16(h_s + (rr * nq + x_q) * 160 + x_sw * 16, src);
-                        } else {
+                for (int jj = jx0; jj < tjx; jj += stepx) {
+                    const int x_sw = jj / nq, x_q = jj - x_sw * nq;
+                    const uint32_t woff = static_cast<uint32_t>(wrapi(w0 + x_sw - 1, v.W)) * Cxs + 8 * x_q + ci0;
+                    for (int sd = 0; sd < wg.npl; ++sd) {
+                        const int d = wg.npl == 3 ? wrapi(d0 + sd - 1, v.D) : d0;
+                        const __nv_bfloat16* plane = X + (static_cast<size_t>(b) * v.D + d) * plane_x + woff;
+                        uint32_t dst = h_s + (sd * kTcHaloH + jx_r) * xrow_s + (wg.nkw == 1 ? x_q * 160 : x_q * 128) +
+                                       x_sw * 16;
+                        for (int sh = jx_r; sh < kTcHaloH; sh += rppx) {
+                            const __nv_bfloat16* src = plane + static_cast<uint32_t>(wrapi(h0 + sh - 1, v.H)) * row_x;
+                            if (wg.nkw == 1) {
+                                cp_async16(dst, src);
+                            } else {
+                                // the kw-shifted copies: voxel slot x_sw - kw of the brick's eight
 #pragma unroll
-                            for (int kw = 0; kw < 3; ++kw) {
-                                const int ww = x_sw - kw;
-                                if (ww >= 0 && ww < 8)
-                                    cp_async16_ca(h_s + ((rr * 3 + kw) * nq + x_q) * 128 + ww * 16, src);
+                                for (int kw = 0; kw < 3; ++kw)
+                                    if (x_sw - kw >= 0 && x_sw - kw < 8)
+                                        cp_async16_ca(dst + kw * (nq * 128 - 16), src);
                             }
+                            dst += rppx * xrow_s;
                         }
                     }
                 }
@@ -707,24 +795,21 @@ __global__ void __launch_bounds__(kWgThreads) k_wgrad_tc(const __nv_bfloat16* __
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;");
                 const uint32_t a_s = s0 + sidx * stage_bytes, h_s = a_s + wg.abytes;
-#pragma unroll 1
-                for (int ks = 0; ks < 8; ++ks) {
-                    const uint64_t ad = umma_desc(a_s + 2 * ks * albo, albo, 128);
-                    const uint32_t accum = (j > 0 || ks > 0) ? 1u : 0u;
-#pragma unroll 1
-                    for (int jj = 0; jj < nun; ++jj) {
-                        const int u = u0 + jj, kd = u / nkwu, kw = u - kd * nkwu;
-                        const int sd = wg.npl == 3 ? kd : 0;
-                        uint64_t bd;
-                        if (wg.nkw == 1)
-                            bd = umma_desc(h_s + (sd * kTcHaloH + 2 * ks) * nq * 160 + kw * 16, nq * 160, 160);
-                        else
-                            bd = umma_desc(h_s + (sd * kTcHaloH + 2 * ks) * 3 * nq * 128, 3 * nq * 128, 128);
-                        asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                                     " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
-                                         tmem + static_cast<uint32_t>(N * jj)),
-                                     "l"(ad), "l"(bd), "r"(idesc), "r"(accum));
-                    }
+                const uint64_t ad = umma_desc(a_s, albo, 128);
+                const uint32_t a_lo = static_cast<uint32_t>(ad), a_hi = static_cast<uint32_t>(ad >> 32);
+                const uint32_t astep = 2u * albo / 16u;
+                for (int jj = 0; jj < nun; ++jj) {
+                    const int u = u0 + jj, kd = u / nkwu, kw = u - kd * nkwu;
+                    const int sd = wg.npl == 3 ? kd : 0;
+                    const uint64_t bd = wg.nkw == 1
+                                            ? umma_desc(h_s + sd * kTcHaloH * nq * 160 + kw * 16, nq * 160, 160)
+                                            : umma_desc(h_s + sd * kTcHaloH * 3 * nq * 128, 3 * nq * 128, 128);
+                    const uint32_t b_lo = static_cast<uint32_t>(bd), b_hi = static_cast<uint32_t>(bd >> 32);
+                    const uint32_t bstep = 2u * nq * (wg.nkw == 1 ? 10u : 24u);
+                    const uint32_t dt = tmem + static_cast<uint32_t>(N * jj);
+                    umma(dt, a_lo, a_hi, b_lo, b_hi, idesc, j > 0 ? 1u : 0u);
+#pragma unroll
+                    for (int ks = 1; ks < 8; ++ks) umma(dt, a_lo + ks * astep, a_hi, b_lo + ks * bstep, b_hi, idesc, 1u);
                 }
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                                  smem_addr(&empty[sidx]))
@@ -1369,16 +1454,26 @@ cudaError_t conv3d(const void* X, int Cxs, int Cin, const void* Wt, const float*
         // tcgen05 path: bricks of bdc x 16 x 8 voxels; the deepest brick whose
         // TMEM columns (bdc planes x Cout rounded to 32) and shared memory fit
         TcShape sh{};
-        sh.ccols = (Cout + 31) / 32 * 32;
+        // stacked up to 64 output channels: an MMA reads 128 x 32 B of halo and N x 32 B
+        // of weights from shared memory whatever its N, so three kd taps per read
+        // of the halo save more than the clipped edge planes of a brick cost
+        sh.stack = 3 * Cout <= 256 ? 1 : 0;
+        sh.ccols = sh.stack ? Cout : (Cout + 31) / 32 * 32;
         const int wbytes = 27 * 2 * Cout * 16;
         int nsm = 0, dev = 0;
         cudaGetDevice(&dev);
         if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1) nsm = 152;
-        // choose the brick depth and staging: the deepest brick (halo shared
-        // by more planes, weights staged once for more voxels) that still
-        // leaves two waves of CTAs at the occupancy that its shared memory and
-        // TMEM allow; one stage unless a forced setting asks for two
-        for (int bdc = 4; bdc >= 1; bdc >>= 1) {
+        // choose the brick depth by a model of the SM with the most CTAs (n of
+        // them, r resident): per 16-channel slice an SM spends the larger of its
+        // MMAs' time and a CTA's whole turn over r.  Cycles: an MMA reads 128
+        // halo rows at half rate (the 10-voxel rows straddle bank lines) and N
+        // weight rows, (8192 + 32 N) / 128; a staged 16-byte piece costs 1/2; the
+        // latencies of a turn 2000.  The deepest brick with two waves of CTAs,
+        // the rule before, left small volumes one plane deep: 32^3 x 4, 192 ->
+        // 64 channels 274 us against 125 at four planes.  One stage unless a
+        // forced setting asks for two.
+        double best = 0.0;
+        for (int bdc = sh.stack ? 8 : 4; bdc >= 1; bdc >>= 1) {
             if (D % bdc || bdc * sh.ccols > 512) continue;
             if (g_tc_force_bdc && bdc != g_tc_force_bdc) continue;
             const int plane = (bdc + 2) * kTcPlaneSlots * 16;
@@ -1389,12 +1484,20 @@ cudaError_t conv3d(const void* X, int Cxs, int Cin, const void* Wt, const float*
             while (cols < static_cast<uint32_t>(bdc * sh.ccols)) cols <<= 1;
             const int per_sm = std::max(1, std::min(kTcMaxSmem / (nstage * stage), static_cast<int>(512 / cols)));
             const long long grid = static_cast<long long>(B) * (D / bdc) * (H / kTcBH) * (W / kTcBW);
-            if (!g_tc_force_bdc && bdc > 1 && grid < 2LL * nsm * per_sm) continue;
+            const double n = static_cast<double>((grid + nsm - 1) / nsm);
+            double mma = 0.0;
+            for (int sd = 0; sd < bdc + 2; ++sd) {
+                const int blocks = std::min(3, bdc + 2 - sd) - std::max(0, 2 - sd);
+                mma += sh.stack ? 9 * (64.0 + 0.25 * blocks * Cout) : 9 * blocks * (64.0 + 0.25 * Cout);
+            }
+            const double turn = mma + 0.5 * ((bdc + 2) * 360 + 54 * Cout) + 2000.0;
+            const double t = n * std::max(mma, turn / std::min(static_cast<double>(per_sm), n));
+            if (sh.bdc != 0 && t >= best) continue;
+            best = t;
             sh.bdc = bdc;
             sh.plane = plane;
             sh.stage = stage;
             sh.nstage = nstage;
-            break;
         }
         if (sh.bdc == 0) return cudaErrorInvalidValue;
         sh.cols = 32;
