@@ -73,10 +73,11 @@ struct TwoLevel {
     void* block = nullptr;
     float* gbar = nullptr;  // 3 Nc
     float* real = nullptr;  // 3 Nc scratch
-    cufftComplex *xh = nullptr, *rh = nullptr, *zh = nullptr, *ph = nullptr, *cp = nullptr, *q = nullptr,
-                 *T = nullptr;  // 3 Mc each
+    // 3 Mc each; cp holds the copy of p for the inverse transform, then the
+    // transform of gbar (gbar . p)
+    cufftComplex *xh = nullptr, *rh = nullptr, *ph = nullptr, *cp = nullptr;
     cufftComplex* zf = nullptr;  // 3 M (fine): the stored preconditioned residual
-    double* sc = nullptr;        // kTlSlots FP64 scalars of the inner PCG (device)
+    double* sc = nullptr;        // kPcgSlots FP64 scalars of the inner PCG (device)
     ~TwoLevel()
     {
         if (plans) {
@@ -140,6 +141,7 @@ struct claire_ctx {
     double* hres = nullptr;               // pinned host scalars, written by the reductions
     double* hres_dev = nullptr;           // their device address
     unsigned* ticket = nullptr;           // finished blocks of the running reduction (device, 0 at rest)
+    double* psc = nullptr;                // kPcgSlots scalars of the outer PCG (device)
 
     // reverse-mode transport scratch, allocated by the first claire_transport_vjp
     // spectrum of the Gauss-Newton iterate inside claire_register (spectral_iterate = 1):
@@ -336,6 +338,10 @@ Grid grid_of(int n1, int n2, int n3)
     return g;
 }
 
+// FP64 device scalars of a context: 15 results with a host mirror, the ticket of
+// the reductions, then the outer PCG's.
+constexpr int kDres = 16 + kPcgSlots;
+
 // Layout of the workspace arena in floats (each region 256-byte aligned).
 struct Layout {
     size_t off[32];
@@ -375,7 +381,7 @@ size_t layout_floats(const int n[3], size_t N, size_t M, int nt, int red_blocks,
     l.add(6 * M);             // xh
     l.add(6 * M);             // rh
     l.add(4 * red_blocks);    // partials (2 * red_blocks doubles)
-    l.add(32);                // dres (16 doubles)
+    l.add(2 * kDres);         // dres
     l.add(8 * tiles);         // tbS (2 int4 per 4 x 8 x 32 tile)
     l.add(8 * tiles);         // tbA
     l.add(8 * tiles);         // tbZ
@@ -498,7 +504,7 @@ Reduction reduction(claire_ctx* c, int slot, double scale = 1.0)
     return Reduction{c->partials, c->red_blocks, scale, c->dres + slot, c->hres_dev + slot, c->ticket};
 }
 
-// Pinned scalars, their device address and the ticket (the last device scalar).
+// Pinned scalars, their device address the ticket and the PCG's scalars.
 bool make_scalars(claire_ctx* c)
 {
     if (cudaMallocHost(&c->hres, 16 * sizeof(double)) != cudaSuccess) {
@@ -513,6 +519,7 @@ bool make_scalars(claire_ctx* c)
     }
     c->hres_dev = static_cast<double*>(dev);
     c->ticket = reinterpret_cast<unsigned*>(c->dres + 15);
+    c->psc = c->dres + 16;
     return true;
 }
 
@@ -536,8 +543,9 @@ claire_status dot(claire_ctx* c, const float* x, const float* y, size_t n, doubl
     return CLAIRE_OK;
 }
 
-// out = F^{-1}[M(k) F[in]] for a 3N vector field
-claire_status spectral(claire_ctx* c, const float* in, float* out, SpectralOp op)
+// out = F^{-1}[M(k) F[in]] for a 3N vector field.  energy >= 0: also 1/2 <in, M in>
+// into that result slot.
+claire_status spectral(claire_ctx* c, const float* in, float* out, SpectralOp op, int energy = -1)
 {
     PhaseScope ps(c, CLAIRE_PHASE_SPECTRAL);
     {
@@ -546,7 +554,10 @@ claire_status spectral(claire_ctx* c, const float* in, float* out, SpectralOp op
     }
     {
         KTimer t(c, KK_SPECTRAL, 48.0 * c->M, 0);
-        launch_spectral(c->grid, c->spec, c->M, op, c->rp, static_cast<float>(1.0 / c->N), c->stream);
+        // Parseval: sum_x = (1/N) sum_k over the unnormalised transform
+        const Reduction red = reduction(c, std::max(energy, 0), 0.5 * c->hvol / static_cast<double>(c->N));
+        launch_spectral(c->grid, c->spec, c->spec, c->M, op, c->rp, static_cast<float>(1.0 / c->N),
+                        energy >= 0 ? &red : nullptr, c->stream);
         CL_LAUNCHED(c);
     }
     {
@@ -557,22 +568,44 @@ claire_status spectral(claire_ctx* c, const float* in, float* out, SpectralOp op
 }
 
 // out = F^{-1}[M(k) vh] for the iterate's spectrum vh (scaled by 1/N like the
-// PCG spectra); vh is copied to the transform buffer first (C2R overwrites its
+// PCG spectra), through the transform buffer (C2R overwrites its
 // input).  No forward transform: its FP32 roundoff, which the symbol M(k)
-// would amplify at high |k|, never enters.
-claire_status spectral_hat(claire_ctx* c, const cufftComplex* vh, float* out, SpectralOp op)
+// would amplify at high |k|, never enters.  1/2 <v, M v> into slot `energy`.
+claire_status spectral_hat(claire_ctx* c, const cufftComplex* vh, float* out, SpectralOp op, int energy)
 {
     PhaseScope ps(c, CLAIRE_PHASE_SPECTRAL);
-    CL_CUDA(c, cudaMemcpyAsync(c->spec, vh, 3 * c->M * sizeof(cufftComplex), cudaMemcpyDeviceToDevice, c->stream));
     {
         KTimer t(c, KK_SPECTRAL, 48.0 * c->M, 0);
-        launch_spectral(c->grid, c->spec, c->M, op, c->rp, 1.0f, c->stream);
+        const Reduction red = reduction(c, energy, 0.5 * c->hvol * static_cast<double>(c->N));
+        launch_spectral(c->grid, vh, c->spec, c->M, op, c->rp, 1.0f, &red, c->stream);
         CL_LAUNCHED(c);
     }
     {
         KTimer t(c, KK_FFT, 0, 0);
         CL_FFT(c, cufftExecC2R(c->c2r, c->spec, out));
     }
+    return CLAIRE_OK;
+}
+
+// The regularisation energy 1/2 <v, S v> into slot `slot`: from a transform of v,
+// or, when alpha is given, of the trial v = iterate + alpha x of the line
+// search from the spectra that the solver carries.
+claire_status reg_energy(claire_ctx* c, const float* v, const double* alpha, int slot)
+{
+    PhaseScope ps(c, CLAIRE_PHASE_SPECTRAL);
+    if (!alpha) {
+        KTimer t(c, KK_FFT, 0, 0);
+        CL_FFT(c, cufftExecR2C(c->r2c, const_cast<float*>(v), c->spec));
+    }
+    KTimer t(c, KK_SPECTRAL, (alpha ? 48.0 : 24.0) * c->M, 0);
+    const double N = static_cast<double>(c->N);
+    if (alpha)
+        launch_reg_energy(c->grid, c->vh, c->xh, c->M, static_cast<float>(*alpha), c->rp,
+                          reduction(c, slot, 0.5 * c->hvol * N), c->stream);
+    else
+        launch_reg_energy(c->grid, c->spec, nullptr, c->M, 0.0f, c->rp, reduction(c, slot, 0.5 * c->hvol / N),
+                          c->stream);
+    CL_LAUNCHED(c);
     return CLAIRE_OK;
 }
 
@@ -643,13 +676,15 @@ int4* tile_table(claire_ctx* c, const float* d)
     return d == c->dS ? c->tbS : (d == c->dA ? c->tbA : (d == c->z ? c->tbZ : nullptr));
 }
 
-claire_status backtrace(claire_ctx* c, const float* v, float* d, int sign)
+// table = false: no later gather reads d's tile-bounds table (writing it costs 20 us
+// at 256^3, reading it saves a gather 5 to 15).
+claire_status backtrace(claire_ctx* c, const float* v, float* d, int sign, bool table = true)
 {
     const void* vc;
     CL_TRY(gather_src(c, v, 3, &vc));
     KTimer t(c, KK_BACKTRACE, 24.0 * c->N, 3.0 * c->N);
     launch_backtrace(c->grid, c->o.interp, v, static_cast<const float*>(vc), static_cast<float>(c->dt), sign, d,
-                     c->stream, tile_table(c, d));
+                     c->stream, table ? tile_table(c, d) : nullptr);
     CL_LAUNCHED(c);
     return CLAIRE_OK;
 }
@@ -754,12 +789,11 @@ claire_status gradient_at_lin(claire_ctx* c, float* g)
 {
     const size_t N = c->N;
     if (c->vh_on)
-        CL_TRY(spectral_hat(c, c->vh, g, SPEC_REG));
+        CL_TRY(spectral_hat(c, c->vh, g, SPEC_REG, 0));
     else
-        CL_TRY(spectral(c, c->v, g, SPEC_REG));
+        CL_TRY(spectral(c, c->v, g, SPEC_REG, 0));
     {
         PhaseScope ps(c, CLAIRE_PHASE_VECTOR);
-        CL_TRY(dot_async(c, c->v, g, 3 * N, 0.5 * c->hvol, 0));
         KTimer t(c, KK_REDUCE, 8.0 * N, 0);
         launch_sqdiff(at(c, c->m, c->nt * N), c->m1, N, c->sto, reduction(c, 1, 0.5 * c->hvol), c->stream);
         CL_LAUNCHED(c);
@@ -855,12 +889,13 @@ claire_status precond(claire_ctx* c, const float* r, float* z)
     return spectral(c, r, z, c->o.grad_form == 1 ? SPEC_AINV : SPEC_INV);
 }
 
-// J(v) for a trial v (device, 3N); uses z (displacement), l0/l1, r (S v).
+// J(v) for a trial v (device, 3N); uses z (displacement), l0/l1.  alpha (the line
+// search): v is the iterate plus alpha times the PCG solution.
 // With into_state the characteristic and the states m^1..m^nt are written to
 // c->dS and c->m (the line search, once the linearisation point is spent),
 // so that an accepted trial seeds the next linearisation.
 claire_status objective_at(claire_ctx* c, const float* v, double* J, double* mis,
-                           bool into_state = false)
+                           bool into_state = false, const double* alpha = nullptr)
 {
     if (!c->have_images) return fail(c, CLAIRE_ESTATE, "images not set (claire_set_images)");
     const size_t N = c->N;
@@ -877,8 +912,7 @@ claire_status objective_at(claire_ctx* c, const float* v, double* J, double* mis
         src = dst;
         std::swap(a, b);
     }
-    CL_TRY(spectral(c, v, c->r, SPEC_REG));
-    CL_TRY(dot_async(c, v, c->r, 3 * N, 0.5 * c->hvol, 0));
+    CL_TRY(reg_energy(c, v, c->vh_on ? alpha : nullptr, 0));
     {
         KTimer t(c, KK_REDUCE, 8.0 * N, 0);
         launch_sqdiff(src, c->m1, N, c->sto, reduction(c, 1, 0.5 * c->hvol), c->stream);
@@ -897,7 +931,7 @@ claire_status objective_at(claire_ctx* c, const float* v, double* J, double* mis
 claire_status detj_of(claire_ctx* c, const float* v, double* lo, double* hi)
 {
     const size_t N = c->N;
-    CL_TRY(backtrace(c, v, c->z, +1));
+    CL_TRY(backtrace(c, v, c->z, +1, false));  // the map steps reduce their own bounds
     float* a = c->r;
     float* b = c->p;
     CL_CUDA(c, cudaMemsetAsync(a, 0, 3 * N * sizeof(float), c->stream));
@@ -981,7 +1015,7 @@ claire_status tl_ensure(claire_ctx* c)
     auto up = [](size_t b) { return (b + 255) / 256 * 256; };
     const size_t realb = up(3 * t->N * sizeof(float)), specb = up(3 * t->M * sizeof(cufftComplex)),
                  fineb = up(3 * c->M * sizeof(cufftComplex));
-    const size_t total = 2 * realb + 7 * specb + fineb + up(kTlSlots * sizeof(double));
+    const size_t total = 2 * realb + 4 * specb + fineb + up(kPcgSlots * sizeof(double));
     if (cudaMalloc(&t->block, total) != cudaSuccess) {
         cudaGetLastError();
         t->block = nullptr;
@@ -991,7 +1025,7 @@ claire_status tl_ensure(claire_ctx* c)
     char* b = static_cast<char*>(t->block);
     t->gbar = reinterpret_cast<float*>(b); b += realb;
     t->real = reinterpret_cast<float*>(b); b += realb;
-    cufftComplex** sp[7] = {&t->xh, &t->rh, &t->zh, &t->ph, &t->cp, &t->q, &t->T};
+    cufftComplex** sp[4] = {&t->xh, &t->rh, &t->ph, &t->cp};
     for (auto q : sp) {
         *q = reinterpret_cast<cufftComplex*>(b);
         b += specb;
@@ -1084,10 +1118,10 @@ claire_status tl_prepare(claire_ctx* c)
     return CLAIRE_OK;
 }
 
-// zf = P^{-1} rf on scaled fine half spectra; *rz = <rf, zf>, *ro = <rf, zold>
+// zf = P^{-1} (rscale rf) on fine half spectra, rscale rf the scaled residual; *rz = <rf, zf>, *ro = <rf, zold>
 // (0 when zold is null); *its = inner PCG iterations.
-claire_status tl_apply(claire_ctx* c, const cufftComplex* rf, cufftComplex* zf, const cufftComplex* zold,
-                       double* rz, double* ro, int* its)
+claire_status tl_apply(claire_ctx* c, const cufftComplex* rf, float rscale, cufftComplex* zf,
+                       const cufftComplex* zold, double* rz, double* ro, int* its)
 {
     TwoLevel* t = c->tl2;
     const SpectralOp op = c->o.grad_form == 1 ? SPEC_AINV : SPEC_INV;
@@ -1095,13 +1129,14 @@ claire_status tl_apply(claire_ctx* c, const cufftComplex* rf, cufftComplex* zf, 
     *its = 0;
     {
         KTimer kt(c, KK_SPECTRAL, 120.0 * t->M, 0);
-        launch_tl_start(c->grid, rf, c->M, t->g, t->rh, t->xh, t->ph, t->cp, t->M, op, c->rp, t->sc,
-                        fs_reduction(c, 0), c->stream);
+        launch_tl_start(c->grid, rf, c->M, t->g, t->rh, t->xh, t->ph, t->cp, t->M, op, c->rp, rscale,
+                        t->sc, fs_reduction(c, 0), c->stream);
     }
     CL_TRY(fs_sums(c, 2));
     const double r0 = std::sqrt(c->hres[0]);
     // rz stays on the device: alpha and beta are formed there (FP64, as the host
     // would), so an iteration reads back only |r|^2 and the breakdown flag
+    const float tscale = static_cast<float>(1.0 / t->N);
     for (int it = 1; r0 > 0.0 && it <= c->o.pc_maxit; ++it) {
         {
             KTimer kt(c, KK_FFT, 0, 0);
@@ -1114,18 +1149,17 @@ claire_status tl_apply(claire_ctx* c, const cufftComplex* rf, cufftComplex* zf, 
         }
         {
             KTimer kt(c, KK_FFT, 0, 0);
-            CL_FFT(c, cufftExecR2C(t->r2c, t->real, t->T));
+            CL_FFT(c, cufftExecR2C(t->r2c, t->real, t->cp));
         }
         {
-            KTimer kt(c, KK_SPECTRAL, 72.0 * t->M, 0);
-            launch_tl_hp(t->g, t->T, t->ph, t->q, t->M, c->o.grad_form, c->rp, static_cast<float>(1.0 / t->N), t->sc,
-                         fs_reduction(c, 8), c->stream);
+            KTimer kt(c, KK_SPECTRAL, 48.0 * t->M, 0);
+            launch_tl_hp(t->g, t->cp, t->ph, t->M, c->o.grad_form, c->rp, tscale, t->sc, fs_reduction(c, 8), c->stream);
             CL_LAUNCHED(c);
         }
         {
             KTimer kt(c, KK_SPECTRAL, 144.0 * t->M, 0);
-            launch_tl_update(t->g, t->ph, t->q, t->xh, t->rh, t->zh, t->M, t->sc, op, c->rp, fs_reduction(c, 10),
-                             c->stream);
+            launch_tl_update(t->g, t->cp, t->ph, t->xh, t->rh, t->M, c->o.grad_form, op, c->rp, tscale, t->sc,
+                             fs_reduction(c, 10), c->stream);
             CL_LAUNCHED(c);
         }
         CL_TRY(sync_scalars(c));
@@ -1137,14 +1171,15 @@ claire_status tl_apply(claire_ctx* c, const cufftComplex* rf, cufftComplex* zf, 
         if (c->o.pc_tol > 0 && std::sqrt(rr) <= c->o.pc_tol * r0) break;
         if (it == c->o.pc_maxit) break;
         {
-            KTimer kt(c, KK_SPECTRAL, 72.0 * t->M, 0);
-            launch_dir_stored(t->g, t->zh, t->ph, t->cp, t->M, 0.0f, 0, c->stream, t->sc + kTlBeta);
+            KTimer kt(c, KK_SPECTRAL, 96.0 * t->M, 0);
+            launch_spectral_direction(t->g, t->rh, t->ph, t->cp, t->M, t->sc, 0, op, c->rp, c->stream);
             CL_LAUNCHED(c);
         }
     }
     {
         KTimer kt(c, KK_SPECTRAL, (zold ? 72.0 : 48.0) * c->M, 0);
-        launch_tl_finish(c->grid, rf, zf, zold, c->M, t->g, t->xh, t->M, op, c->rp, fs_reduction(c, 0), c->stream);
+        launch_tl_finish(c->grid, rf, zf, zold, c->M, t->g, t->xh, t->M, op, c->rp, rscale,
+                         c->psc, fs_reduction(c, 0), c->stream);
     }
     CL_TRY(fs_sums(c, 2));
     *rz = c->hres[0];
@@ -1175,7 +1210,7 @@ claire_status pcg(claire_ctx* c, double eta, int* its)
             CL_FFT(c, cufftExecR2C(c->r2c, c->g, c->spec));
         }
         KTimer t(c, KK_SPECTRAL, 72.0 * M, 0);
-        launch_fs_start(c->grid, c->spec, c->rh, c->xh, c->M, op, c->rp, scale, fs_reduction(c, 0), c->stream);
+        launch_fs_start(c->grid, c->spec, c->rh, c->xh, c->M, op, c->rp, scale, c->psc, fs_reduction(c, 0), c->stream);
     }
     CL_TRY(fs_sums(c, 2));
     const double r0 = std::sqrt(c->hres[0]);
@@ -1189,7 +1224,7 @@ claire_status pcg(claire_ctx* c, double eta, int* its)
     int inner_its = 0;
     if (two_level) {
         double ro;
-        CL_TRY(tl_apply(c, c->rh, c->tl2->zf, nullptr, &rz, &ro, &inner_its));
+        CL_TRY(tl_apply(c, c->rh, 1.0f, c->tl2->zf, nullptr, &rz, &ro, &inner_its));
     }
     double beta = 0.0;
     for (int it = 1; it <= c->o.max_pcg; ++it) {
@@ -1202,8 +1237,8 @@ claire_status pcg(claire_ctx* c, double eta, int* its)
                     launch_dir_stored(c->grid, c->tl2->zf, c->phat, c->spec2, c->M, static_cast<float>(beta),
                                       it == 1 ? 1 : 0, c->stream);
                 else
-                    launch_spectral_direction(c->grid, c->rh, c->phat, c->spec2, c->M, static_cast<float>(beta),
-                                              it == 1 ? 1 : 0, op, c->rp, c->stream);
+                    launch_spectral_direction(c->grid, c->rh, c->phat, c->spec2, c->M, c->psc, it == 1 ? 1 : 0, op,
+                                              c->rp, c->stream);
                 CL_LAUNCHED(c);
             }
             KTimer t(c, KK_FFT, 0, 0);
@@ -1216,39 +1251,41 @@ claire_status pcg(claire_ctx* c, double eta, int* its)
                 KTimer t(c, KK_FFT, 0, 0);
                 CL_FFT(c, cufftExecR2C(c->r2c, c->z, c->spec2));
             }
-            KTimer t(c, KK_SPECTRAL, 72.0 * M, 0);
-            launch_fs_hp(c->grid, c->spec, c->spec2, c->phat, c->M, c->o.grad_form, c->rp, scale, fs_reduction(c, 0),
-                         c->stream);
+            {
+                KTimer t(c, KK_SPECTRAL, 48.0 * M, 0);
+                launch_fs_hp(c->grid, c->spec2, c->phat, c->M, c->o.grad_form, c->rp, scale, c->psc, fs_reduction(c, 8),
+                             c->stream);
+                CL_LAUNCHED(c);
+            }
+            // with the step length formed on the device, the update follows at once
+            // (it moves nothing when the curvature is not positive)
+            KTimer t(c, KK_SPECTRAL, 144.0 * M, 0);
+            launch_fs_update(c->grid, c->spec2, c->phat, c->xh, c->rh, two_level ? c->tl2->zf : nullptr, c->M,
+                             c->o.grad_form, op, c->rp, scale, c->psc, fs_reduction(c, 0), c->stream);
         }
-        CL_TRY(fs_sums(c, 1));
-        const double pq = c->hres[0];
+        CL_TRY(fs_sums(c, 0));
+        const double pq = c->hres[8], alpha = c->hres[9];
+        if (!std::isfinite(pq)) return fail(c, CLAIRE_ENONFINITE, "non-finite PCG inner product");
         if (pq <= 0.0) {
             if (it == 1)
                 CL_CUDA(c, cudaMemcpyAsync(c->xh, c->phat, 3 * c->M * sizeof(cufftComplex),
                                            cudaMemcpyDeviceToDevice, c->stream));
             break;
         }
-        const double alpha = rz / pq;
-        {
-            PhaseScope ps(c, CLAIRE_PHASE_VECTOR);
-            KTimer t(c, KK_SPECTRAL, 144.0 * M, 0);
-            launch_fs_update(c->grid, c->spec, c->phat, c->xh, c->rh, two_level ? c->tl2->zf : nullptr, c->M,
-                             static_cast<float>(alpha), op, c->rp, fs_reduction(c, 0), c->stream);
-        }
-        CL_TRY(fs_sums(c, 2));
         const double rr = c->hres[0];
+        if (!std::isfinite(rr) || !std::isfinite(c->hres[1]))
+            return fail(c, CLAIRE_ENONFINITE, "non-finite PCG inner product");
         if (!c->o.pcg_fixed && std::sqrt(rr) <= eta * r0) break;
         if (it == c->o.max_pcg) break;
         if (two_level) {
             // <r_new, z_old> = <r_old, z_old> - alpha <H p, z_old>; z_new overwrites z_old
             const double ro = rz - alpha * c->hres[1];
             double rz_new, unused;
-            CL_TRY(tl_apply(c, c->rh, c->tl2->zf, nullptr, &rz_new, &unused, &inner_its));
+            CL_TRY(tl_apply(c, c->rh, 1.0f, c->tl2->zf, nullptr, &rz_new, &unused, &inner_its));
             beta = (rz_new - ro) / rz;
             rz = rz_new;
         } else {
-            beta = c->hres[1] / rz;
-            rz = c->hres[1];
+            rz = c->hres[1];  // beta: on the device
         }
     }
     {
@@ -1326,7 +1363,7 @@ claire_status claire_query_workspace(const int grid[3], int nt, const claire_opt
     if (sto < 0 || sto > 2) return CLAIRE_EINVAL;
     const bool lowmem = opts ? opts->lowmem != 0 : false;
     if (opts && opts->kernels_only) {
-        *bytes = (2 * 152 * 8 + 16) * sizeof(double);  // reduction partials and device scalars
+        *bytes = (2 * 152 * 8 + kDres) * sizeof(double);  // reduction partials and device scalars
         return CLAIRE_OK;
     }
     *bytes = layout_floats(grid, N, M, nt, 152 * 8, storage_bytes(static_cast<Storage>(sto)), lowmem, nullptr) *
@@ -1392,7 +1429,7 @@ claire_status claire_create(claire_ctx** out, const int grid[3], double beta_v, 
     c->red_blocks = std::max(1, c->nsm) * 4;
     if (o.kernels_only) {
         // reduction partials and the device scalars only: no fields, no plans
-        const size_t bytes = (2 * static_cast<size_t>(c->red_blocks) + 16) * sizeof(double);
+        const size_t bytes = (2 * static_cast<size_t>(c->red_blocks) + kDres) * sizeof(double);
         if (cudaMalloc(&c->arena, bytes) != cudaSuccess) {
             cudaGetLastError();
             c->arena = nullptr;
@@ -1401,7 +1438,7 @@ claire_status claire_create(claire_ctx** out, const int grid[3], double beta_v, 
         c->arena_bytes = bytes;
         c->partials = static_cast<double*>(c->arena);
         c->dres = c->partials + 2 * c->red_blocks;
-        if (cudaMemset(c->dres, 0, 16 * sizeof(double)) != cudaSuccess) {
+        if (cudaMemset(c->dres, 0, kDres * sizeof(double)) != cudaSuccess) {
             cudaGetLastError();
             return bail(CLAIRE_ECUDA);
         }
@@ -1452,7 +1489,7 @@ claire_status claire_create(claire_ctx** out, const int grid[3], double beta_v, 
     c->tbS = reinterpret_cast<int4*>(base + L.off[k++]);
     c->tbA = reinterpret_cast<int4*>(base + L.off[k++]);
     c->tbZ = reinterpret_cast<int4*>(base + L.off[k++]);
-    if (cudaMemset(c->dres, 0, 16 * sizeof(double)) != cudaSuccess) {
+    if (cudaMemset(c->dres, 0, kDres * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
         return bail(CLAIRE_ECUDA);
     }
@@ -1596,11 +1633,9 @@ claire_status claire_precond(claire_ctx* c, const float* r, float* z)
     if (c->o.precond == CLAIRE_PRECOND_TWO_LEVEL) {
         CL_TRY(tl_prepare(c));
         CL_FFT(c, cufftExecR2C(c->r2c, const_cast<float*>(dr), c->rh));
-        launch_cscale(c->rh, 3 * c->M, static_cast<float>(1.0 / c->N), c->stream);
-        CL_LAUNCHED(c);
         double rz, ro;
         int its;
-        CL_TRY(tl_apply(c, c->rh, c->tl2->zf, nullptr, &rz, &ro, &its));
+        CL_TRY(tl_apply(c, c->rh, static_cast<float>(1.0 / c->N), c->tl2->zf, nullptr, &rz, &ro, &its));
         CL_FFT(c, cufftExecC2R(c->c2r, c->tl2->zf, c->r));
     } else {
         CL_TRY(precond(c, dr, c->r));
@@ -1710,7 +1745,7 @@ claire_status claire_register(claire_ctx* c, float* v_inout, claire_report* rep)
                     CL_LAUNCHED(c);
                 }
                 double Jt;
-                CL_TRY(objective_at(c, c->p, &Jt, nullptr, true));
+                CL_TRY(objective_at(c, c->p, &Jt, nullptr, true, &alpha));
                 if (Jt <= c->J_lin + c->o.armijo_c1 * alpha * gtx) {
                     ok = true;
                     break;

@@ -308,29 +308,40 @@ struct RegParams {
     int reg;  // 1 = H1 seminorm, 2 = H2 seminorm
 };
 
-// In-place scaling of the three half-spectra xh[c], c = 0..2 (each
+// Scaling of the three half-spectra xh[c] into yh[c] (may be xh), c = 0..2 (each
 // n1 * n2 * (n3/2+1) complex values, stride cstride) by the 3x3 symbol of op,
-// times scale (the 1/N of the unnormalised inverse transform).
-void launch_spectral(const Grid& g, cufftComplex* xh, size_t cstride, SpectralOp op,
-                     RegParams rp, float scale, cudaStream_t st);
+// times scale (the 1/N of the unnormalised inverse transform); energy (may be
+// null): also the total of the quadratic form of the operator.
+void launch_spectral(const Grid& g, const cufftComplex* xh, cufftComplex* yh, size_t cstride, SpectralOp op,
+                     RegParams rp, float scale, const Reduction* energy, cudaStream_t st);
+// total of sum_k wt Re(conj(w) S w), w = vh + alpha xh (xh may be null)
+void launch_reg_energy(const Grid& g, const cufftComplex* vh, const cufftComplex* xh, size_t cs, float alpha,
+                       RegParams rp, const Reduction& red, cudaStream_t st);
 
-// PCG direction in Fourier space: ph = zh + beta ph (first: ph = zh), cp = ph, zh <- S ph.
+// Device scalars sc of a PCG iteration (FP64).  The kernel that ends a reduction
+// also forms what follows from it: start (and the two-level finish) store rz;
+// hp forms alpha = rz / pq (0 when pq <= 0 or NaN); update forms beta = rz_new /
+// rz and moves rz_new to rz.
+constexpr int kPcgRz = 0, kPcgAlpha = 1, kPcgBeta = 2, kPcgSlots = 4;
+
+// PCG direction in Fourier space: ph = z~ + beta ph (first: ph = z~), z~ = M rh, cp = ph.
 void launch_spectral_direction(const Grid& g, const cufftComplex* rh, cufftComplex* ph, cufftComplex* cp,
-                               size_t cstride, float beta, int first, SpectralOp op, RegParams rp,
+                               size_t cstride, const double* sc, int first, SpectralOp op, RegParams rp,
                                cudaStream_t st);
 
 // Fourier-space PCG (vectors are half spectra scaled by 1/N; totals are
-// of sum_k wt Re(conj(a) b), wt the multiplicity of the mode):
-//   start:  r~ = -scale spec, x~ = 0, spec <- M r~;  totals |r~|^2, <r~, M r~>
-//   hp:     spec <- spec + scale spec2 (K applied if kform);  total <p~, H p~>
-//   update: x~ += alpha p~, r~ -= alpha spec, spec <- M r~;  totals as in start
+// of sum_k wt Re(conj(a) b), wt the multiplicity of the mode; H p~ = S p~ + scale T, K
+// of it if kform, is formed where it is used):
+//   start:  r~ = -scale spec, x~ = 0;  totals |r~|^2, <r~, M r~>
+//   hp:     totals <p~, H p~> and (second result) alpha
+//   update: x~ += alpha p~, r~ -= alpha H p~;  totals as in start, or with zc |r~|^2, <H p~, zc>
 void launch_fs_start(const Grid& g, cufftComplex* spec, cufftComplex* rh, cufftComplex* xh, size_t cs,
-                     SpectralOp op, RegParams rp, float scale, const Reduction& red, cudaStream_t st);
-void launch_fs_hp(const Grid& g, cufftComplex* spec, const cufftComplex* spec2, const cufftComplex* ph,
-                  size_t cs, int kform, RegParams rp, float scale, const Reduction& red, cudaStream_t st);
-void launch_fs_update(const Grid& g, cufftComplex* spec, const cufftComplex* ph, cufftComplex* xh,
-                      cufftComplex* rh, const cufftComplex* zc, size_t cs, float alpha, SpectralOp op, RegParams rp,
-                      const Reduction& red, cudaStream_t st);
+                     SpectralOp op, RegParams rp, float scale, double* sc, const Reduction& red, cudaStream_t st);
+void launch_fs_hp(const Grid& g, const cufftComplex* T, const cufftComplex* ph, size_t cs, int kform, RegParams rp,
+                  float scale, double* sc, const Reduction& red, cudaStream_t st);
+void launch_fs_update(const Grid& g, const cufftComplex* T, const cufftComplex* ph, cufftComplex* xh,
+                      cufftComplex* rh, const cufftComplex* zc, size_t cs, int kform, SpectralOp op, RegParams rp,
+                      float scale, double* sc, const Reduction& red, cudaStream_t st);
 
 // two-level zero-velocity preconditioner (coarse grid gc of the fine grid gf; cs* = component strides)
 void launch_mean_levels(const void* m, int nt, float w_end, float w_mid, size_t N, float* out, Storage sto,
@@ -342,24 +353,19 @@ void launch_tl_restrict(const Grid& gf, const cufftComplex* F, size_t csf, const
 void launch_tl_weight(float* gbar_c, const float* w, size_t n, cudaStream_t st);
 void launch_tl_start(const Grid& gf, const cufftComplex* rf, size_t csf, const Grid& gc, cufftComplex* rh,
                      cufftComplex* xh, cufftComplex* ph, cufftComplex* cp, size_t cs, SpectralOp op, RegParams rp,
-                     double* sc, const Reduction& red, cudaStream_t st);
+                     float rscale, double* sc, const Reduction& red, cudaStream_t st);
 void launch_tl_rank1(const float* gbar, float* p, size_t Nc, cudaStream_t st);
-void launch_tl_hp(const Grid& gc, const cufftComplex* T, const cufftComplex* ph, cufftComplex* q, size_t cs,
-                  int kform, RegParams rp, float scale, double* sc, const Reduction& red, cudaStream_t st);
-// Device scalars sc of the inner PCG (slots of a small FP64 array).  The kernel
-// that ends a reduction also forms what follows from it: start stores
-// rz; hp forms alpha = rz / pq (0 and the breakdown flag when pq <= 0); update
-// forms beta = rz_new / rz and moves rz_new to rz.
-constexpr int kTlRz = 0, kTlAlpha = 1, kTlBeta = 2, kTlSlots = 4;
-void launch_tl_update(const Grid& gc, const cufftComplex* ph, const cufftComplex* q, cufftComplex* xh,
-                      cufftComplex* rh, cufftComplex* zh, size_t cs, double* sc, SpectralOp op, RegParams rp,
+// second result: the breakdown flag (0; 1: pq <= 0; 2: pq is NaN)
+void launch_tl_hp(const Grid& gc, const cufftComplex* T, const cufftComplex* ph, size_t cs, int kform, RegParams rp,
+                  float scale, double* sc, const Reduction& red, cudaStream_t st);
+void launch_tl_update(const Grid& gc, const cufftComplex* T, const cufftComplex* ph, cufftComplex* xh,
+                      cufftComplex* rh, size_t cs, int kform, SpectralOp op, RegParams rp, float scale, double* sc,
                       const Reduction& red, cudaStream_t st);
-// beta from beta_dev when it is not null, else the host value
 void launch_dir_stored(const Grid& g, const cufftComplex* zh, cufftComplex* ph, cufftComplex* cp, size_t cs,
-                       float beta, int first, cudaStream_t st, const double* beta_dev = nullptr);
+                       float beta, int first, cudaStream_t st);
 void launch_tl_finish(const Grid& gf, const cufftComplex* rf, cufftComplex* zf, const cufftComplex* zold, size_t csf,
-                      const Grid& gc, const cufftComplex* xc, size_t csc, SpectralOp op, RegParams rp,
-                      const Reduction& red, cudaStream_t st);
+                      const Grid& gc, const cufftComplex* xc, size_t csc, SpectralOp op, RegParams rp, float rscale,
+                      double* sc, const Reduction& red, cudaStream_t st);
 // Deterministic FP64 reductions (struct Reduction): totals at red.out
 void launch_dot(const float* x, const float* y, size_t n, const Reduction& red, cudaStream_t st);
 void launch_sqdiff(const void* a, const void* b, size_t n, Storage sto, const Reduction& red, cudaStream_t st);

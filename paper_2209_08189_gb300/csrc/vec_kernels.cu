@@ -21,13 +21,14 @@ struct Mode {
     float u1, u2, u3, a, c, kk, wt;
 };
 
-__device__ __forceinline__ Mode mode_of(const Grid& g, size_t idx, int n3h, const RegParams& rp)
+// idx: index of the mode on the half spectrum (below 2^31: 32-bit divisions).
+__device__ __forceinline__ Mode mode_of(const Grid& g, uint32_t idx, int n3h, const RegParams& rp)
 {
     Mode m;
-    const int k3i = static_cast<int>(idx % n3h);
-    const size_t r = idx / n3h;
-    const int j = static_cast<int>(r % g.n2);
-    const int i = static_cast<int>(r / g.n2);
+    const uint32_t r = idx / static_cast<uint32_t>(n3h);
+    const int k3i = static_cast<int>(idx - r * static_cast<uint32_t>(n3h));
+    const int i = static_cast<int>(r / static_cast<uint32_t>(g.n2));
+    const int j = static_cast<int>(r) - i * g.n2;
     const float k1 = static_cast<float>(i <= g.n1 / 2 ? i : i - g.n1);
     const float k2 = static_cast<float>(j <= g.n2 / 2 ? j : j - g.n2);
     const float k3 = static_cast<float>(k3i);
@@ -73,60 +74,24 @@ __device__ __forceinline__ void apply_inv(const Mode& m, int op, float2 x0, floa
     y2 = cmul(ia, make_float2(x2.x - f * m.u3 * ud.x, x2.y - f * m.u3 * ud.y));
 }
 
-// In place: xh <- scale * M(k) xh for the three half-spectra.
-__global__ void __launch_bounds__(kThreads) k_spectral(Grid g, float2* __restrict__ xh, size_t cs,
-                                                        int op, RegParams rp, float scale)
+// y = M x for one mode and any of the operators.
+__device__ __forceinline__ void apply_op(const Mode& m, int op, float2 x0, float2 x1, float2 x2, float2& y0,
+                                         float2& y1, float2& y2)
 {
-    const int n3h = g.n3 / 2 + 1;
-    const size_t M = static_cast<size_t>(g.n1) * g.n2 * n3h;
-    for (size_t idx = blockIdx.x * static_cast<size_t>(kThreads) + threadIdx.x; idx < M;
-         idx += static_cast<size_t>(gridDim.x) * kThreads) {
-        const int k3i = static_cast<int>(idx % n3h);
-        const size_t r = idx / n3h;
-        const int j = static_cast<int>(r % g.n2);
-        const int i = static_cast<int>(r / g.n2);
-        const float k1 = static_cast<float>(i <= g.n1 / 2 ? i : i - g.n1);
-        const float k2 = static_cast<float>(j <= g.n2 / 2 ? j : j - g.n2);
-        const float k3 = static_cast<float>(k3i);
-        const float kk = k1 * k1 + k2 * k2 + k3 * k3;
-        const float u1 = (2 * i == g.n1) ? 0.0f : k1;
-        const float u2 = (2 * j == g.n2) ? 0.0f : k2;
-        const float u3 = (2 * k3i == g.n3) ? 0.0f : k3;
-        const float a = rp.beta_v * (rp.reg == 2 ? kk * kk : kk);
-        const float c = rp.beta_w * (1.0f + kk);
-        float2 x0 = xh[idx], x1 = xh[cs + idx], x2 = xh[2 * cs + idx];
-        const float2 ud = make_float2(u1 * x0.x + u2 * x1.x + u3 * x2.x,
-                                      u1 * x0.y + u2 * x1.y + u3 * x2.y);
-        float2 y0, y1, y2;
-        if (op == SPEC_REG) {
-            y0 = make_float2(a * x0.x + c * u1 * ud.x, a * x0.y + c * u1 * ud.y);
-            y1 = make_float2(a * x1.x + c * u2 * ud.x, a * x1.y + c * u2 * ud.y);
-            y2 = make_float2(a * x2.x + c * u3 * ud.x, a * x2.y + c * u3 * ud.y);
-        } else if (kk == 0.0f) {
-            y0 = x0;
-            y1 = x1;
-            y2 = x2;
-        } else if (op == SPEC_AINV) {
-            const float ia = 1.0f / a;
-            y0 = cmul(ia, x0);
-            y1 = cmul(ia, x1);
-            y2 = cmul(ia, x2);
-        } else {
-            // K = I - c u u^T / (a + c |u|^2);  S^{-1} = K / a  (Sherman-Morrison)
-            const float f = c / (a + c * (u1 * u1 + u2 * u2 + u3 * u3));
-            y0 = make_float2(x0.x - f * u1 * ud.x, x0.y - f * u1 * ud.y);
-            y1 = make_float2(x1.x - f * u2 * ud.x, x1.y - f * u2 * ud.y);
-            y2 = make_float2(x2.x - f * u3 * ud.x, x2.y - f * u3 * ud.y);
-            if (op == SPEC_INV) {
-                const float ia = 1.0f / a;
-                y0 = cmul(ia, y0);
-                y1 = cmul(ia, y1);
-                y2 = cmul(ia, y2);
-            }
-        }
-        xh[idx] = cmul(scale, y0);
-        xh[cs + idx] = cmul(scale, y1);
-        xh[2 * cs + idx] = cmul(scale, y2);
+    if (op == SPEC_REG) {
+        apply_S(m, x0, x1, x2, y0, y1, y2);
+    } else if (op != SPEC_K) {
+        apply_inv(m, op, x0, x1, x2, y0, y1, y2);
+    } else if (m.kk == 0.0f) {
+        y0 = x0; y1 = x1; y2 = x2;
+    } else {
+        // K = I - c u u^T / (a + c |u|^2);  S^{-1} = K / a  (Sherman-Morrison)
+        const float2 ud = make_float2(m.u1 * x0.x + m.u2 * x1.x + m.u3 * x2.x,
+                                      m.u1 * x0.y + m.u2 * x1.y + m.u3 * x2.y);
+        const float f = m.c / (m.a + m.c * (m.u1 * m.u1 + m.u2 * m.u2 + m.u3 * m.u3));
+        y0 = make_float2(x0.x - f * m.u1 * ud.x, x0.y - f * m.u1 * ud.y);
+        y1 = make_float2(x1.x - f * m.u2 * ud.x, x1.y - f * m.u2 * ud.y);
+        y2 = make_float2(x2.x - f * m.u3 * ud.x, x2.y - f * m.u3 * ud.y);
     }
 }
 
@@ -136,12 +101,13 @@ __global__ void __launch_bounds__(kThreads) k_spectral(Grid g, float2* __restric
 __global__ void __launch_bounds__(kThreads) k_spectral_direction(Grid g, const float2* __restrict__ rh,
                                                                   float2* __restrict__ ph,
                                                                   float2* __restrict__ cp, size_t cs,
-                                                                  float beta, int first, int op, RegParams rp)
+                                                                  const double* __restrict__ sc, int first, int op,
+                                                                  RegParams rp)
 {
+    const float beta = first ? 0.0f : static_cast<float>(sc[kPcgBeta]);
     const int n3h = g.n3 / 2 + 1;
-    const size_t M = static_cast<size_t>(g.n1) * g.n2 * n3h;
-    for (size_t idx = blockIdx.x * static_cast<size_t>(kThreads) + threadIdx.x; idx < M;
-         idx += static_cast<size_t>(gridDim.x) * kThreads) {
+    const uint32_t M = static_cast<uint32_t>(g.n1) * g.n2 * n3h;
+    for (uint32_t idx = blockIdx.x * kThreads + threadIdx.x; idx < M; idx += gridDim.x * kThreads) {
         const Mode m = mode_of(g, idx, n3h, rp);
         float2 z[3];
         apply_inv(m, op, rh[idx], rh[cs + idx], rh[2 * cs + idx], z[0], z[1], z[2]);
@@ -214,17 +180,68 @@ __device__ __forceinline__ float cdot3(float2 a0, float2 a1, float2 a2, float2 b
     return a0.x * b0.x + a0.y * b0.y + a1.x * b1.x + a1.y * b1.y + a2.x * b2.x + a2.y * b2.y;
 }
 
+// yh = scale * M(k) xh for the three half-spectra (in place when yh = xh); with
+// ENERGY also the total of sum_k wt Re(conj(xh) M xh), the quadratic form of
+// the operator (Parseval), so that no pass over the physical fields forms it.
+template <bool ENERGY>
+__global__ void __launch_bounds__(kThreads) k_spectral(Grid g, const float2* xh, float2* yh, size_t cs, int op,
+                                                        RegParams rp, float scale, Reduction red)
+{
+    const int n3h = g.n3 / 2 + 1;
+    const uint32_t M = static_cast<uint32_t>(g.n1) * g.n2 * n3h;
+    double acc = 0.0;
+    for (uint32_t idx = blockIdx.x * kThreads + threadIdx.x; idx < M; idx += gridDim.x * kThreads) {
+        const Mode m = mode_of(g, idx, n3h, rp);
+        const float2 x0 = xh[idx], x1 = xh[cs + idx], x2 = xh[2 * cs + idx];
+        float2 y0, y1, y2;
+        apply_op(m, op, x0, x1, x2, y0, y1, y2);
+        yh[idx] = cmul(scale, y0);
+        yh[cs + idx] = cmul(scale, y1);
+        yh[2 * cs + idx] = cmul(scale, y2);
+        if constexpr (ENERGY) acc += static_cast<double>(m.wt * cdot3(x0, x1, x2, y0, y1, y2));
+    }
+    if constexpr (ENERGY) grid_sum(acc, red);
+}
+
+// Total of sum_k wt Re(conj(w) S w) for w = vh + alpha xh (xh may be null): the
+// regularisation energy of a trial velocity from the spectra the solver
+// carries, without transforming it.
+__global__ void __launch_bounds__(kThreads) k_reg_energy(Grid g, const float2* __restrict__ vh,
+                                                          const float2* __restrict__ xh, size_t cs, float alpha,
+                                                          RegParams rp, Reduction red)
+{
+    const int n3h = g.n3 / 2 + 1;
+    const uint32_t M = static_cast<uint32_t>(g.n1) * g.n2 * n3h;
+    double acc = 0.0;
+    for (uint32_t idx = blockIdx.x * kThreads + threadIdx.x; idx < M; idx += gridDim.x * kThreads) {
+        float2 w[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            w[c] = vh[c * cs + idx];
+            if (xh) {
+                const float2 x = xh[c * cs + idx];
+                w[c] = make_float2(fmaf(alpha, x.x, w[c].x), fmaf(alpha, x.y, w[c].y));
+            }
+        }
+        const Mode m = mode_of(g, idx, n3h, rp);
+        float2 y0, y1, y2;
+        apply_S(m, w[0], w[1], w[2], y0, y1, y2);
+        acc += static_cast<double>(m.wt * cdot3(w[0], w[1], w[2], y0, y1, y2));
+    }
+    grid_sum(acc, red);
+}
+
 // Start: r~ = -scale g^ (spec holds F[g]), x~ = 0; partials of |r~|^2 and
 // <r~, z~> with z~ = M r~ (recomputed by the direction kernel).
 __global__ void __launch_bounds__(kThreads) k_fs_start(Grid g, float2* __restrict__ spec,
                                                         float2* __restrict__ rh, float2* __restrict__ xh,
-                                                        size_t cs, int op, RegParams rp, float scale, Reduction red)
+                                                        size_t cs, int op, RegParams rp, float scale,
+                                                        double* __restrict__ sc, Reduction red)
 {
     const int n3h = g.n3 / 2 + 1;
-    const size_t M = static_cast<size_t>(g.n1) * g.n2 * n3h;
+    const uint32_t M = static_cast<uint32_t>(g.n1) * g.n2 * n3h;
     double arr = 0.0, arz = 0.0;
-    for (size_t idx = blockIdx.x * static_cast<size_t>(kThreads) + threadIdx.x; idx < M;
-         idx += static_cast<size_t>(gridDim.x) * kThreads) {
+    for (uint32_t idx = blockIdx.x * kThreads + threadIdx.x; idx < M; idx += gridDim.x * kThreads) {
         const Mode m = mode_of(g, idx, n3h, rp);
         const float2 r0 = cmul(-scale, spec[idx]), r1 = cmul(-scale, spec[cs + idx]),
                      r2 = cmul(-scale, spec[2 * cs + idx]);
@@ -236,75 +253,90 @@ __global__ void __launch_bounds__(kThreads) k_fs_start(Grid g, float2* __restric
         arz += static_cast<double>(m.wt * cdot3(r0, r1, r2, z0, z1, z2));
     }
     double tot[2];
-    grid_sum2(arr, arz, red, tot);
+    if (grid_sum2(arr, arz, red, tot)) sc[kPcgRz] = tot[1];
 }
 
-// H p~ = S p~ + scale F[body] (in spec2), or K of that for the paper's
-// gradient form; written into spec; partials of <p~, H p~>.
-__global__ void __launch_bounds__(kThreads) k_fs_hp(Grid g, float2* __restrict__ spec,
-                                                     const float2* __restrict__ spec2,
+// h = S p~ + scale F[body] (T holds F[body]), or K of that for the paper's
+// gradient form: one mode of H p~.
+__device__ __forceinline__ void hp_mode(const Mode& m, const float2 p[3], const float2* __restrict__ T, size_t cs,
+                                        uint32_t idx, int kform, float scale, float2 h[3])
+{
+    apply_S(m, p[0], p[1], p[2], h[0], h[1], h[2]);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const float2 b = T[c * cs + idx];
+        h[c] = make_float2(fmaf(scale, b.x, h[c].x), fmaf(scale, b.y, h[c].y));
+    }
+    if (kform && m.kk != 0.0f) {
+        const float2 ud = make_float2(m.u1 * h[0].x + m.u2 * h[1].x + m.u3 * h[2].x,
+                                      m.u1 * h[0].y + m.u2 * h[1].y + m.u3 * h[2].y);
+        const float f = m.c / (m.a + m.c * (m.u1 * m.u1 + m.u2 * m.u2 + m.u3 * m.u3));
+        h[0] = make_float2(h[0].x - f * m.u1 * ud.x, h[0].y - f * m.u1 * ud.y);
+        h[1] = make_float2(h[1].x - f * m.u2 * ud.x, h[1].y - f * m.u2 * ud.y);
+        h[2] = make_float2(h[2].x - f * m.u3 * ud.x, h[2].y - f * m.u3 * ud.y);
+    }
+}
+
+// Step length of a CG iteration from its curvature pq: alpha = rz / pq, or 0
+// when pq <= 0 or NaN (the caller sees pq).  FP64, as the host would do it.
+__device__ __forceinline__ double cg_alpha(double rz, double pq) { return pq > 0.0 ? rz / pq : 0.0; }
+
+// Total of <p~, H p~>, then alpha.  H p~ is not stored: the update forms it again
+// from p~ and T, the same reads as of a stored H p~ (256^3: 30 us less per
+// iteration than writing it).
+__global__ void __launch_bounds__(kThreads) k_fs_hp(Grid g, const float2* __restrict__ T,
                                                      const float2* __restrict__ ph, size_t cs, int kform,
-                                                     RegParams rp, float scale, Reduction red)
+                                                     RegParams rp, float scale, double* __restrict__ sc, Reduction red)
 {
     const int n3h = g.n3 / 2 + 1;
-    const size_t M = static_cast<size_t>(g.n1) * g.n2 * n3h;
+    const uint32_t M = static_cast<uint32_t>(g.n1) * g.n2 * n3h;
     double acc = 0.0;
-    for (size_t idx = blockIdx.x * static_cast<size_t>(kThreads) + threadIdx.x; idx < M;
-         idx += static_cast<size_t>(gridDim.x) * kThreads) {
+    for (uint32_t idx = blockIdx.x * kThreads + threadIdx.x; idx < M; idx += gridDim.x * kThreads) {
         const Mode m = mode_of(g, idx, n3h, rp);
-        const float2 p0 = ph[idx], p1 = ph[cs + idx], p2 = ph[2 * cs + idx];
+        const float2 p[3] = {ph[idx], ph[cs + idx], ph[2 * cs + idx]};
         float2 h[3];
-        apply_S(m, p0, p1, p2, h[0], h[1], h[2]);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const float2 b = spec2[c * cs + idx];
-            h[c] = make_float2(fmaf(scale, b.x, h[c].x), fmaf(scale, b.y, h[c].y));
-        }
-        if (kform && m.kk != 0.0f) {
-            const float2 ud = make_float2(m.u1 * h[0].x + m.u2 * h[1].x + m.u3 * h[2].x,
-                                          m.u1 * h[0].y + m.u2 * h[1].y + m.u3 * h[2].y);
-            const float f = m.c / (m.a + m.c * (m.u1 * m.u1 + m.u2 * m.u2 + m.u3 * m.u3));
-            h[0] = make_float2(h[0].x - f * m.u1 * ud.x, h[0].y - f * m.u1 * ud.y);
-            h[1] = make_float2(h[1].x - f * m.u2 * ud.x, h[1].y - f * m.u2 * ud.y);
-            h[2] = make_float2(h[2].x - f * m.u3 * ud.x, h[2].y - f * m.u3 * ud.y);
-        }
-#pragma unroll
-        for (int c = 0; c < 3; ++c) spec[c * cs + idx] = h[c];
-        acc += static_cast<double>(m.wt * cdot3(p0, p1, p2, h[0], h[1], h[2]));
+        hp_mode(m, p, T, cs, idx, kform, scale, h);
+        acc += static_cast<double>(m.wt * cdot3(p[0], p[1], p[2], h[0], h[1], h[2]));
     }
-    grid_sum(acc, red);
+    double pq;
+    if (grid_sum(acc, red, &pq)) {
+        sc[kPcgAlpha] = cg_alpha(sc[kPcgRz], pq);
+        put_result(red, 1, sc[kPcgAlpha]);
+    }
 }
 
-// x~ += alpha p~, r~ -= alpha H p~ (H p~ in spec); partials of |r~|^2 and
-// <r~, z~> with z~ = M r~ (recomputed by the next direction kernel), or, when
-// a stored preconditioned residual zc is given, of <H p~, zc> instead.
-__global__ void __launch_bounds__(kThreads) k_fs_update(Grid g, const float2* __restrict__ spec,
+// x~ += alpha p~, r~ -= alpha H p~; totals |r~|^2 and <r~, z~> with z~ = M r~
+// (recomputed by the next direction kernel), or, when a stored preconditioned
+// residual zc is given, <H p~, zc> instead.  Without zc also beta and the new
+// rz for the next direction.
+__global__ void __launch_bounds__(kThreads) k_fs_update(Grid g, const float2* __restrict__ T,
                                                          const float2* __restrict__ ph,
                                                          float2* __restrict__ xh, float2* __restrict__ rh,
-                                                         const float2* __restrict__ zc, size_t cs, float alpha,
-                                                         int op, RegParams rp, Reduction red)
+                                                         const float2* __restrict__ zc, size_t cs, int kform, int op,
+                                                         RegParams rp, float scale, double* __restrict__ sc,
+                                                         Reduction red)
 {
+    const float alpha = static_cast<float>(sc[kPcgAlpha]);
     const int n3h = g.n3 / 2 + 1;
-    const size_t M = static_cast<size_t>(g.n1) * g.n2 * n3h;
+    const uint32_t M = static_cast<uint32_t>(g.n1) * g.n2 * n3h;
     double arr = 0.0, arz = 0.0;
-    for (size_t idx = blockIdx.x * static_cast<size_t>(kThreads) + threadIdx.x; idx < M;
-         idx += static_cast<size_t>(gridDim.x) * kThreads) {
-        float2 r[3];
+    for (uint32_t idx = blockIdx.x * kThreads + threadIdx.x; idx < M; idx += gridDim.x * kThreads) {
+        const Mode m = mode_of(g, idx, n3h, rp);
+        const float2 p[3] = {ph[idx], ph[cs + idx], ph[2 * cs + idx]};
+        float2 h[3], r[3];
+        hp_mode(m, p, T, cs, idx, kform, scale, h);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            const float2 p = ph[c * cs + idx], hp = spec[c * cs + idx];
             float2 x = xh[c * cs + idx], rr = rh[c * cs + idx];
-            x = make_float2(fmaf(alpha, p.x, x.x), fmaf(alpha, p.y, x.y));
-            rr = make_float2(fmaf(-alpha, hp.x, rr.x), fmaf(-alpha, hp.y, rr.y));
+            x = make_float2(fmaf(alpha, p[c].x, x.x), fmaf(alpha, p[c].y, x.y));
+            rr = make_float2(fmaf(-alpha, h[c].x, rr.x), fmaf(-alpha, h[c].y, rr.y));
             xh[c * cs + idx] = x;
             rh[c * cs + idx] = rr;
             r[c] = rr;
         }
-        const Mode m = mode_of(g, idx, n3h, rp);
         arr += static_cast<double>(m.wt * cdot3(r[0], r[1], r[2], r[0], r[1], r[2]));
         if (zc) {
-            arz += static_cast<double>(m.wt * cdot3(spec[idx], spec[cs + idx], spec[2 * cs + idx], zc[idx],
-                                                     zc[cs + idx], zc[2 * cs + idx]));
+            arz += static_cast<double>(m.wt * cdot3(h[0], h[1], h[2], zc[idx], zc[cs + idx], zc[2 * cs + idx]));
         } else {
             float2 z0, z1, z2;
             apply_inv(m, op, r[0], r[1], r[2], z0, z1, z2);
@@ -312,7 +344,10 @@ __global__ void __launch_bounds__(kThreads) k_fs_update(Grid g, const float2* __
         }
     }
     double tot[2];
-    grid_sum2(arr, arz, red, tot);
+    if (grid_sum2(arr, arz, red, tot) && !zc) {
+        sc[kPcgBeta] = tot[1] / sc[kPcgRz];
+        sc[kPcgRz] = tot[1];
+    }
 }
 
 __device__ __forceinline__ bool aligned16(const void* p)
@@ -581,16 +616,39 @@ __global__ void k_bspline_scale(Grid g, cufftComplex* __restrict__ spec, size_t 
     spec[e].x *= f;
     spec[e].y *= f;
 }
-// out = w_end (m^0 + m^nt) + w_mid (m^1 + ... + m^{nt-1}) (trapezoid over the stored levels)
+// out = w_end (m^0 + m^nt) + w_mid (m^1 + ... + m^{nt-1}) (trapezoid over the
+// stored levels; N is a multiple of 8 and the levels are the context's own, so
+// four points go together).
+template <class S>
+__device__ __forceinline__ float4 load4(const S* p)
+{
+    if constexpr (sizeof(S) == 4) {
+        return __ldg(reinterpret_cast<const float4*>(p));
+    } else {
+        const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
+        S v[4];
+        memcpy(v, &u, 8);
+        return make_float4(to_f32<S>(v[0]), to_f32<S>(v[1]), to_f32<S>(v[2]), to_f32<S>(v[3]));
+    }
+}
+
 template <class S>
 __global__ void __launch_bounds__(kThreads) k_mean_levels(const S* __restrict__ m, int nt, float w_end,
                                                            float w_mid, size_t N, float* __restrict__ out)
 {
-    for (size_t i = blockIdx.x * static_cast<size_t>(kThreads) + threadIdx.x; i < N;
-         i += static_cast<size_t>(gridDim.x) * kThreads) {
-        float acc = w_end * (ldf<S>(m + i) + ldf<S>(m + static_cast<size_t>(nt) * N + i));
-        for (int j = 1; j < nt; ++j) acc = fmaf(w_mid, ldf<S>(m + static_cast<size_t>(j) * N + i), acc);
-        out[i] = acc;
+    for (size_t i = 4 * (blockIdx.x * static_cast<size_t>(kThreads) + threadIdx.x); i < N;
+         i += static_cast<size_t>(gridDim.x) * (4 * kThreads)) {
+        const float4 a = load4(m + i), b = load4(m + static_cast<size_t>(nt) * N + i);
+        float4 acc = make_float4(w_end * (a.x + b.x), w_end * (a.y + b.y), w_end * (a.z + b.z), w_end * (a.w + b.w));
+#pragma unroll 4
+        for (int j = 1; j < nt; ++j) {
+            const float4 v = load4(m + static_cast<size_t>(j) * N + i);
+            acc.x = fmaf(w_mid, v.x, acc.x);
+            acc.y = fmaf(w_mid, v.y, acc.y);
+            acc.z = fmaf(w_mid, v.z, acc.z);
+            acc.w = fmaf(w_mid, v.w, acc.w);
+        }
+        *reinterpret_cast<float4*>(out + i) = acc;
     }
 }
 
@@ -609,13 +667,13 @@ __global__ void __launch_bounds__(kThreads) k_cscale(float2* __restrict__ x, siz
 // restriction and prolongation copy them).
 
 // Wavenumbers of half-spectrum mode idx of grid g.
-__device__ __forceinline__ void wavenumbers(const Grid& g, size_t idx, int& k1, int& k2, int& k3)
+__device__ __forceinline__ void wavenumbers(const Grid& g, uint32_t idx, int& k1, int& k2, int& k3)
 {
-    const int n3h = g.n3 / 2 + 1;
-    k3 = static_cast<int>(idx % n3h);
-    const size_t r = idx / n3h;
-    const int j = static_cast<int>(r % g.n2);
-    const int i = static_cast<int>(r / g.n2);
+    const uint32_t n3h = g.n3 / 2 + 1;
+    const uint32_t r = idx / n3h;
+    k3 = static_cast<int>(idx - r * n3h);
+    const int i = static_cast<int>(r / static_cast<uint32_t>(g.n2));
+    const int j = static_cast<int>(r) - i * g.n2;
     k1 = i <= g.n1 / 2 ? i : i - g.n1;
     k2 = j <= g.n2 / 2 ? j : j - g.n2;
 }
@@ -642,8 +700,7 @@ __global__ void __launch_bounds__(kThreads) k_tl_restrict(Grid gf, const float2*
                                                            float invN)
 {
     const size_t Mc = static_cast<size_t>(gc.n1) * gc.n2 * (gc.n3 / 2 + 1);
-    for (size_t idx = blockIdx.x * static_cast<size_t>(kThreads) + threadIdx.x; idx < Mc;
-         idx += static_cast<size_t>(gridDim.x) * kThreads) {
+    for (uint32_t idx = blockIdx.x * kThreads + threadIdx.x; idx < Mc; idx += gridDim.x * kThreads) {
         int k1, k2, k3;
         wavenumbers(gc, idx, k1, k2, k3);
         const bool keep = below_nyquist(gc, k1, k2, k3);
@@ -653,19 +710,19 @@ __global__ void __launch_bounds__(kThreads) k_tl_restrict(Grid gf, const float2*
     }
 }
 
-// Start of the inner PCG: r = Q R rf (kept modes of the fine residual), x = 0,
-// z = M r, p = z (and its copy cp for the inverse transform); partials of
+// Start of the inner PCG: r = Q R (rscale rf) (kept modes of the fine residual),
+// x = 0, z = M r, p = z (and its copy cp for the inverse transform); totals
 // |r|^2 and <r, z>.
 __global__ void __launch_bounds__(kThreads) k_tl_start(Grid gf, const float2* __restrict__ rf, size_t csf,
                                                         Grid gc, float2* __restrict__ rh, float2* __restrict__ xh,
                                                         float2* __restrict__ ph, float2* __restrict__ cp, size_t cs,
-                                                        int op, RegParams rp, double* __restrict__ sc, Reduction red)
+                                                        int op, RegParams rp, float rscale, double* __restrict__ sc,
+                                                        Reduction red)
 {
     const int n3h = gc.n3 / 2 + 1;
-    const size_t Mc = static_cast<size_t>(gc.n1) * gc.n2 * n3h;
+    const uint32_t Mc = static_cast<uint32_t>(gc.n1) * gc.n2 * n3h;
     double arr = 0.0, arz = 0.0;
-    for (size_t idx = blockIdx.x * static_cast<size_t>(kThreads) + threadIdx.x; idx < Mc;
-         idx += static_cast<size_t>(gridDim.x) * kThreads) {
+    for (uint32_t idx = blockIdx.x * kThreads + threadIdx.x; idx < Mc; idx += gridDim.x * kThreads) {
         int k1, k2, k3;
         wavenumbers(gc, idx, k1, k2, k3);
         const bool keep = below_nyquist(gc, k1, k2, k3) && (k1 | k2 | k3) != 0;
@@ -673,7 +730,7 @@ __global__ void __launch_bounds__(kThreads) k_tl_start(Grid gf, const float2* __
         const float2 zero = make_float2(0.f, 0.f);
         float2 r[3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) r[c] = keep ? rf[c * csf + f] : zero;
+        for (int c = 0; c < 3; ++c) r[c] = keep ? cmul(rscale, rf[c * csf + f]) : zero;
         const Mode m = mode_of(gc, idx, n3h, rp);
         float2 z[3];
         apply_inv(m, op, r[0], r[1], r[2], z[0], z[1], z[2]);
@@ -688,7 +745,7 @@ __global__ void __launch_bounds__(kThreads) k_tl_start(Grid gf, const float2* __
         arz += static_cast<double>(m.wt * cdot3(r[0], r[1], r[2], z[0], z[1], z[2]));
     }
     double tot[2];
-    if (grid_sum2(arr, arz, red, tot)) sc[kTlRz] = tot[1];
+    if (grid_sum2(arr, arz, red, tot)) sc[kPcgRz] = tot[1];
 }
 
 // In place on the coarse real fields: p <- gbar (gbar . p).
@@ -705,101 +762,89 @@ __global__ void __launch_bounds__(kThreads) k_tl_rank1(const float* __restrict__
     }
 }
 
-// q = Q (S p + scale T) (K of the sum for the paper's gradient form), T the
-// unnormalised transform of gbar (gbar . p); partials of <p, q>.
+// One mode of q = Q (S p + scale T) (K of the sum for the paper's gradient
+// form), T the unnormalised transform of gbar (gbar . p).
+__device__ __forceinline__ void tl_q(const Grid& gc, uint32_t idx, const Mode& m, const float2 p[3],
+                                     const float2* __restrict__ T, size_t cs, int kform, float scale, float2 h[3])
+{
+    hp_mode(m, p, T, cs, idx, kform, scale, h);
+    int k1, k2, k3;
+    wavenumbers(gc, idx, k1, k2, k3);
+    if (!(below_nyquist(gc, k1, k2, k3) && (k1 | k2 | k3) != 0)) h[0] = h[1] = h[2] = make_float2(0.f, 0.f);
+}
+
+// Total of <p, q>, then alpha.  Neither q nor the preconditioned residual is
+// stored in the inner PCG: the update and the direction form them again from
+// what they read anyway, and T lives where the copy of p was, so that an
+// iteration's five coarse arrays (26 MB each at 128^3) stay near the L2 size
+// instead of eight.
 __global__ void __launch_bounds__(kThreads) k_tl_hp(Grid gc, const float2* __restrict__ T,
-                                                     const float2* __restrict__ ph, float2* __restrict__ q,
-                                                     size_t cs, int kform, RegParams rp, float scale,
-                                                     double* __restrict__ sc, Reduction red)
+                                                     const float2* __restrict__ ph, size_t cs, int kform,
+                                                     RegParams rp, float scale, double* __restrict__ sc, Reduction red)
 {
     const int n3h = gc.n3 / 2 + 1;
-    const size_t Mc = static_cast<size_t>(gc.n1) * gc.n2 * n3h;
+    const uint32_t Mc = static_cast<uint32_t>(gc.n1) * gc.n2 * n3h;
     double acc = 0.0;
-    for (size_t idx = blockIdx.x * static_cast<size_t>(kThreads) + threadIdx.x; idx < Mc;
-         idx += static_cast<size_t>(gridDim.x) * kThreads) {
-        int k1, k2, k3;
-        wavenumbers(gc, idx, k1, k2, k3);
-        const bool keep = below_nyquist(gc, k1, k2, k3) && (k1 | k2 | k3) != 0;
+    for (uint32_t idx = blockIdx.x * kThreads + threadIdx.x; idx < Mc; idx += gridDim.x * kThreads) {
         const Mode m = mode_of(gc, idx, n3h, rp);
-        const float2 p0 = ph[idx], p1 = ph[cs + idx], p2 = ph[2 * cs + idx];
+        const float2 p[3] = {ph[idx], ph[cs + idx], ph[2 * cs + idx]};
         float2 h[3];
-        apply_S(m, p0, p1, p2, h[0], h[1], h[2]);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const float2 b = T[c * cs + idx];
-            h[c] = make_float2(fmaf(scale, b.x, h[c].x), fmaf(scale, b.y, h[c].y));
-        }
-        if (kform && m.kk != 0.0f) {
-            const float2 ud = make_float2(m.u1 * h[0].x + m.u2 * h[1].x + m.u3 * h[2].x,
-                                          m.u1 * h[0].y + m.u2 * h[1].y + m.u3 * h[2].y);
-            const float f = m.c / (m.a + m.c * (m.u1 * m.u1 + m.u2 * m.u2 + m.u3 * m.u3));
-            h[0] = make_float2(h[0].x - f * m.u1 * ud.x, h[0].y - f * m.u1 * ud.y);
-            h[1] = make_float2(h[1].x - f * m.u2 * ud.x, h[1].y - f * m.u2 * ud.y);
-            h[2] = make_float2(h[2].x - f * m.u3 * ud.x, h[2].y - f * m.u3 * ud.y);
-        }
-        if (!keep) h[0] = h[1] = h[2] = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) q[c * cs + idx] = h[c];
-        acc += static_cast<double>(m.wt * cdot3(p0, p1, p2, h[0], h[1], h[2]));
+        tl_q(gc, idx, m, p, T, cs, kform, scale, h);
+        acc += static_cast<double>(m.wt * cdot3(p[0], p[1], p[2], h[0], h[1], h[2]));
     }
     double pq;
     if (grid_sum(acc, red, &pq)) {
-        // alpha = rz / pq, or 0 with the breakdown flag set when pq <= 0 (1) or
-        // NaN (2); FP64 divisions, as the host would do them
-        sc[kTlAlpha] = pq > 0.0 ? sc[kTlRz] / pq : 0.0;
-        put_result(red, 1, pq > 0.0 ? 0.0 : (pq == pq ? 1.0 : 2.0));
+        sc[kPcgAlpha] = cg_alpha(sc[kPcgRz], pq);
+        put_result(red, 1, pq > 0.0 ? 0.0 : (pq == pq ? 1.0 : 2.0));  // breakdown flag; 2: pq is NaN
     }
 }
 
-// x += alpha p, r -= alpha q, z = M r (stored); totals |r|^2 and <r, z>, then
-// beta = rz_new / rz and rz <- rz_new for the next direction.
-__global__ void __launch_bounds__(kThreads) k_tl_update(Grid gc, const float2* __restrict__ ph,
-                                                         const float2* __restrict__ q, float2* __restrict__ xh,
-                                                         float2* __restrict__ rh, float2* __restrict__ zh, size_t cs,
-                                                         double* __restrict__ sc, int op, RegParams rp, Reduction red)
+// x += alpha p, r -= alpha q; totals |r|^2 and <r, z> with z = M r, then beta =
+// rz_new / rz and rz <- rz_new for the next direction.
+__global__ void __launch_bounds__(kThreads) k_tl_update(Grid gc, const float2* __restrict__ T,
+                                                         const float2* __restrict__ ph, float2* __restrict__ xh,
+                                                         float2* __restrict__ rh, size_t cs, int kform, int op,
+                                                         RegParams rp, float scale, double* __restrict__ sc,
+                                                         Reduction red)
 {
-    const float alpha = static_cast<float>(sc[kTlAlpha]);
+    const float alpha = static_cast<float>(sc[kPcgAlpha]);
     const int n3h = gc.n3 / 2 + 1;
-    const size_t Mc = static_cast<size_t>(gc.n1) * gc.n2 * n3h;
+    const uint32_t Mc = static_cast<uint32_t>(gc.n1) * gc.n2 * n3h;
     double arr = 0.0, arz = 0.0;
-    for (size_t idx = blockIdx.x * static_cast<size_t>(kThreads) + threadIdx.x; idx < Mc;
-         idx += static_cast<size_t>(gridDim.x) * kThreads) {
-        float2 r[3];
+    for (uint32_t idx = blockIdx.x * kThreads + threadIdx.x; idx < Mc; idx += gridDim.x * kThreads) {
+        const Mode m = mode_of(gc, idx, n3h, rp);
+        const float2 p[3] = {ph[idx], ph[cs + idx], ph[2 * cs + idx]};
+        float2 h[3], r[3];
+        tl_q(gc, idx, m, p, T, cs, kform, scale, h);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            const float2 p = ph[c * cs + idx], hq = q[c * cs + idx];
             float2 x = xh[c * cs + idx], rr = rh[c * cs + idx];
-            x = make_float2(fmaf(alpha, p.x, x.x), fmaf(alpha, p.y, x.y));
-            rr = make_float2(fmaf(-alpha, hq.x, rr.x), fmaf(-alpha, hq.y, rr.y));
+            x = make_float2(fmaf(alpha, p[c].x, x.x), fmaf(alpha, p[c].y, x.y));
+            rr = make_float2(fmaf(-alpha, h[c].x, rr.x), fmaf(-alpha, h[c].y, rr.y));
             xh[c * cs + idx] = x;
             rh[c * cs + idx] = rr;
             r[c] = rr;
         }
-        const Mode m = mode_of(gc, idx, n3h, rp);
         float2 z0, z1, z2;
         apply_inv(m, op, r[0], r[1], r[2], z0, z1, z2);
-        zh[idx] = z0; zh[cs + idx] = z1; zh[2 * cs + idx] = z2;
         arr += static_cast<double>(m.wt * cdot3(r[0], r[1], r[2], r[0], r[1], r[2]));
         arz += static_cast<double>(m.wt * cdot3(r[0], r[1], r[2], z0, z1, z2));
     }
     double tot[2];
     if (grid_sum2(arr, arz, red, tot)) {
-        sc[kTlBeta] = tot[1] / sc[kTlRz];
-        sc[kTlRz] = tot[1];
+        sc[kPcgBeta] = tot[1] / sc[kPcgRz];
+        sc[kPcgRz] = tot[1];
     }
 }
 
-// p = z + beta p (p = z when first) and its copy cp for the inverse transform;
-// on any grid (the inner PCG, and the outer PCG when z is stored).
+// p = z + beta p (p = z when first) and its copy cp for the inverse transform:
+// the outer PCG when z is stored.
 __global__ void __launch_bounds__(kThreads) k_dir_stored(Grid g, const float2* __restrict__ zh,
                                                           float2* __restrict__ ph, float2* __restrict__ cp, size_t cs,
-                                                          float beta_host, const double* __restrict__ beta_dev,
-                                                          int first)
+                                                          float beta, int first)
 {
-    const float beta = beta_dev ? static_cast<float>(*beta_dev) : beta_host;
-    const size_t M = static_cast<size_t>(g.n1) * g.n2 * (g.n3 / 2 + 1);
-    for (size_t idx = blockIdx.x * static_cast<size_t>(kThreads) + threadIdx.x; idx < M;
-         idx += static_cast<size_t>(gridDim.x) * kThreads) {
+    const uint32_t M = static_cast<uint32_t>(g.n1) * g.n2 * (g.n3 / 2 + 1);
+    for (uint32_t idx = blockIdx.x * kThreads + threadIdx.x; idx < M; idx += gridDim.x * kThreads) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             const float2 z = zh[c * cs + idx];
@@ -814,23 +859,24 @@ __global__ void __launch_bounds__(kThreads) k_dir_stored(Grid g, const float2* _
     }
 }
 
-// Outer preconditioned residual: z = E x (kept coarse modes), r on the mean,
-// M r on every other mode; partials of <r, z> and <r, zold> (zold may be null).
+// Outer preconditioned residual of r = rscale rf: z = E x (kept coarse modes), r
+// on the mean, M r on every other mode; totals <r, z> (also the outer PCG's
+// rz) and <r, zold> (zold may be null).
 __global__ void __launch_bounds__(kThreads) k_tl_finish(Grid gf, const float2* __restrict__ rf,
                                                          float2* __restrict__ zf, const float2* __restrict__ zold,
                                                          size_t csf, Grid gc, const float2* __restrict__ xc,
-                                                         size_t csc, int op, RegParams rp, Reduction red)
+                                                         size_t csc, int op, RegParams rp, float rscale,
+                                                         double* __restrict__ sc, Reduction red)
 {
     const int n3h = gf.n3 / 2 + 1;
-    const size_t M = static_cast<size_t>(gf.n1) * gf.n2 * n3h;
+    const uint32_t M = static_cast<uint32_t>(gf.n1) * gf.n2 * n3h;
     double az = 0.0, ao = 0.0;
-    for (size_t idx = blockIdx.x * static_cast<size_t>(kThreads) + threadIdx.x; idx < M;
-         idx += static_cast<size_t>(gridDim.x) * kThreads) {
+    for (uint32_t idx = blockIdx.x * kThreads + threadIdx.x; idx < M; idx += gridDim.x * kThreads) {
         int k1, k2, k3;
         wavenumbers(gf, idx, k1, k2, k3);
         const bool low = below_nyquist(gc, k1, k2, k3) && (k1 | k2 | k3) != 0;
         const Mode m = mode_of(gf, idx, n3h, rp);
-        const float2 r0 = rf[idx], r1 = rf[csf + idx], r2 = rf[2 * csf + idx];
+        const float2 r0 = cmul(rscale, rf[idx]), r1 = cmul(rscale, rf[csf + idx]), r2 = cmul(rscale, rf[2 * csf + idx]);
         float2 z[3];
         if (low) {
             const size_t ci = mode_index(gc, k1, k2, k3);
@@ -846,61 +892,71 @@ __global__ void __launch_bounds__(kThreads) k_tl_finish(Grid gf, const float2* _
             ao += static_cast<double>(m.wt * cdot3(r0, r1, r2, zold[idx], zold[csf + idx], zold[2 * csf + idx]));
     }
     double tot[2];
-    grid_sum2(az, ao, red, tot);
+    if (grid_sum2(az, ao, red, tot)) sc[kPcgRz] = tot[0];
 }
 
 }  // namespace
 
-void launch_spectral(const Grid& g, cufftComplex* xh, size_t cstride, SpectralOp op, RegParams rp,
-                     float scale, cudaStream_t st)
+void launch_spectral(const Grid& g, const cufftComplex* xh, cufftComplex* yh, size_t cstride, SpectralOp op,
+                     RegParams rp, float scale, const Reduction* energy, cudaStream_t st)
 {
     const size_t M = static_cast<size_t>(g.n1) * g.n2 * (g.n3 / 2 + 1);
-    k_spectral<<<stream_blocks(M), kThreads, 0, st>>>(g, reinterpret_cast<float2*>(xh), cstride,
-                                                     static_cast<int>(op), rp, scale);
+    auto x = reinterpret_cast<const float2*>(xh);
+    auto y = reinterpret_cast<float2*>(yh);
+    if (energy)
+        k_spectral<true><<<energy->nblocks, kThreads, 0, st>>>(g, x, y, cstride, static_cast<int>(op), rp, scale, *energy);
+    else
+        k_spectral<false><<<stream_blocks(M), kThreads, 0, st>>>(g, x, y, cstride, static_cast<int>(op), rp, scale,
+                                                                Reduction{});
+}
+
+void launch_reg_energy(const Grid& g, const cufftComplex* vh, const cufftComplex* xh, size_t cs, float alpha,
+                       RegParams rp, const Reduction& red, cudaStream_t st)
+{
+    k_reg_energy<<<red.nblocks, kThreads, 0, st>>>(g, reinterpret_cast<const float2*>(vh),
+                                                   reinterpret_cast<const float2*>(xh), cs, alpha, rp, red);
 }
 
 void launch_spectral_direction(const Grid& g, const cufftComplex* rh, cufftComplex* ph, cufftComplex* cp,
-                               size_t cstride, float beta, int first, SpectralOp op, RegParams rp,
+                               size_t cstride, const double* sc, int first, SpectralOp op, RegParams rp,
                                cudaStream_t st)
 {
     const size_t M = static_cast<size_t>(g.n1) * g.n2 * (g.n3 / 2 + 1);
     k_spectral_direction<<<stream_blocks(M), kThreads, 0, st>>>(
         g, reinterpret_cast<const float2*>(rh), reinterpret_cast<float2*>(ph), reinterpret_cast<float2*>(cp),
-        cstride, beta, first, static_cast<int>(op), rp);
+        cstride, sc, first, static_cast<int>(op), rp);
 }
 
 void launch_fs_start(const Grid& g, cufftComplex* spec, cufftComplex* rh, cufftComplex* xh, size_t cs,
-                     SpectralOp op, RegParams rp, float scale, const Reduction& red, cudaStream_t st)
+                     SpectralOp op, RegParams rp, float scale, double* sc, const Reduction& red, cudaStream_t st)
 {
     k_fs_start<<<red.nblocks, kThreads, 0, st>>>(g, reinterpret_cast<float2*>(spec), reinterpret_cast<float2*>(rh),
-                                             reinterpret_cast<float2*>(xh), cs, static_cast<int>(op), rp,
-                                             scale, red);
+                                                 reinterpret_cast<float2*>(xh), cs, static_cast<int>(op), rp, scale,
+                                                 sc, red);
 }
 
-void launch_fs_hp(const Grid& g, cufftComplex* spec, const cufftComplex* spec2, const cufftComplex* ph,
-                  size_t cs, int kform, RegParams rp, float scale, const Reduction& red, cudaStream_t st)
+void launch_fs_hp(const Grid& g, const cufftComplex* T, const cufftComplex* ph, size_t cs, int kform, RegParams rp,
+                  float scale, double* sc, const Reduction& red, cudaStream_t st)
 {
-    k_fs_hp<<<red.nblocks, kThreads, 0, st>>>(g, reinterpret_cast<float2*>(spec),
-                                          reinterpret_cast<const float2*>(spec2),
-                                          reinterpret_cast<const float2*>(ph), cs, kform, rp, scale, red);
+    k_fs_hp<<<red.nblocks, kThreads, 0, st>>>(g, reinterpret_cast<const float2*>(T),
+                                              reinterpret_cast<const float2*>(ph), cs, kform, rp, scale, sc, red);
 }
 
-void launch_fs_update(const Grid& g, cufftComplex* spec, const cufftComplex* ph, cufftComplex* xh,
-                      cufftComplex* rh, const cufftComplex* zc, size_t cs, float alpha, SpectralOp op, RegParams rp,
-                      const Reduction& red, cudaStream_t st)
+void launch_fs_update(const Grid& g, const cufftComplex* T, const cufftComplex* ph, cufftComplex* xh,
+                      cufftComplex* rh, const cufftComplex* zc, size_t cs, int kform, SpectralOp op, RegParams rp,
+                      float scale, double* sc, const Reduction& red, cudaStream_t st)
 {
-    k_fs_update<<<red.nblocks, kThreads, 0, st>>>(g, reinterpret_cast<const float2*>(spec),
-                                              reinterpret_cast<const float2*>(ph),
-                                              reinterpret_cast<float2*>(xh), reinterpret_cast<float2*>(rh),
-                                              reinterpret_cast<const float2*>(zc), cs, alpha, static_cast<int>(op),
-                                              rp, red);
+    k_fs_update<<<red.nblocks, kThreads, 0, st>>>(g, reinterpret_cast<const float2*>(T),
+                                                  reinterpret_cast<const float2*>(ph), reinterpret_cast<float2*>(xh),
+                                                  reinterpret_cast<float2*>(rh), reinterpret_cast<const float2*>(zc),
+                                                  cs, kform, static_cast<int>(op), rp, scale, sc, red);
 }
 
 void launch_mean_levels(const void* m, int nt, float w_end, float w_mid, size_t N, float* out, Storage sto,
                         cudaStream_t st)
 {
     CLAIRE_STORAGE_DISPATCH(sto, {
-        k_mean_levels<SType><<<stream_blocks(N), kThreads, 0, st>>>(static_cast<const SType*>(m), nt, w_end, w_mid,
+        k_mean_levels<SType><<<stream_blocks(N / 4), kThreads, 0, st>>>(static_cast<const SType*>(m), nt, w_end, w_mid,
                                                                     N, out);
     });
 }
@@ -939,12 +995,12 @@ void launch_tl_restrict(const Grid& gf, const cufftComplex* F, size_t csf, const
 
 void launch_tl_start(const Grid& gf, const cufftComplex* rf, size_t csf, const Grid& gc, cufftComplex* rh,
                      cufftComplex* xh, cufftComplex* ph, cufftComplex* cp, size_t cs, SpectralOp op, RegParams rp,
-                     double* sc, const Reduction& red, cudaStream_t st)
+                     float rscale, double* sc, const Reduction& red, cudaStream_t st)
 {
     k_tl_start<<<red.nblocks, kThreads, 0, st>>>(gf, reinterpret_cast<const float2*>(rf), csf, gc,
-                                             reinterpret_cast<float2*>(rh), reinterpret_cast<float2*>(xh),
-                                             reinterpret_cast<float2*>(ph), reinterpret_cast<float2*>(cp), cs,
-                                             static_cast<int>(op), rp, sc, red);
+                                                 reinterpret_cast<float2*>(rh), reinterpret_cast<float2*>(xh),
+                                                 reinterpret_cast<float2*>(ph), reinterpret_cast<float2*>(cp), cs,
+                                                 static_cast<int>(op), rp, rscale, sc, red);
 }
 
 void launch_tl_rank1(const float* gbar, float* p, size_t Nc, cudaStream_t st)
@@ -952,40 +1008,40 @@ void launch_tl_rank1(const float* gbar, float* p, size_t Nc, cudaStream_t st)
     k_tl_rank1<<<stream_blocks(Nc), kThreads, 0, st>>>(gbar, p, Nc);
 }
 
-void launch_tl_hp(const Grid& gc, const cufftComplex* T, const cufftComplex* ph, cufftComplex* q, size_t cs,
-                  int kform, RegParams rp, float scale, double* sc, const Reduction& red, cudaStream_t st)
+void launch_tl_hp(const Grid& gc, const cufftComplex* T, const cufftComplex* ph, size_t cs, int kform, RegParams rp,
+                  float scale, double* sc, const Reduction& red, cudaStream_t st)
 {
-    k_tl_hp<<<red.nblocks, kThreads, 0, st>>>(gc, reinterpret_cast<const float2*>(T), reinterpret_cast<const float2*>(ph),
-                                          reinterpret_cast<float2*>(q), cs, kform, rp, scale, sc, red);
+    k_tl_hp<<<red.nblocks, kThreads, 0, st>>>(gc, reinterpret_cast<const float2*>(T),
+                                              reinterpret_cast<const float2*>(ph), cs, kform, rp, scale, sc, red);
 }
 
-void launch_tl_update(const Grid& gc, const cufftComplex* ph, const cufftComplex* q, cufftComplex* xh,
-                      cufftComplex* rh, cufftComplex* zh, size_t cs, double* sc, SpectralOp op, RegParams rp,
+void launch_tl_update(const Grid& gc, const cufftComplex* T, const cufftComplex* ph, cufftComplex* xh,
+                      cufftComplex* rh, size_t cs, int kform, SpectralOp op, RegParams rp, float scale, double* sc,
                       const Reduction& red, cudaStream_t st)
 {
-    k_tl_update<<<red.nblocks, kThreads, 0, st>>>(gc, reinterpret_cast<const float2*>(ph),
-                                              reinterpret_cast<const float2*>(q), reinterpret_cast<float2*>(xh),
-                                              reinterpret_cast<float2*>(rh), reinterpret_cast<float2*>(zh), cs,
-                                              sc, static_cast<int>(op), rp, red);
+    k_tl_update<<<red.nblocks, kThreads, 0, st>>>(gc, reinterpret_cast<const float2*>(T),
+                                                  reinterpret_cast<const float2*>(ph), reinterpret_cast<float2*>(xh),
+                                                  reinterpret_cast<float2*>(rh), cs, kform, static_cast<int>(op), rp,
+                                                  scale, sc, red);
 }
 
 void launch_dir_stored(const Grid& g, const cufftComplex* zh, cufftComplex* ph, cufftComplex* cp, size_t cs,
-                       float beta, int first, cudaStream_t st, const double* beta_dev)
+                       float beta, int first, cudaStream_t st)
 {
     const size_t M = static_cast<size_t>(g.n1) * g.n2 * (g.n3 / 2 + 1);
     k_dir_stored<<<stream_blocks(M), kThreads, 0, st>>>(g, reinterpret_cast<const float2*>(zh),
                                                         reinterpret_cast<float2*>(ph), reinterpret_cast<float2*>(cp),
-                                                        cs, beta, beta_dev, first);
+                                                        cs, beta, first);
 }
 
 void launch_tl_finish(const Grid& gf, const cufftComplex* rf, cufftComplex* zf, const cufftComplex* zold, size_t csf,
-                      const Grid& gc, const cufftComplex* xc, size_t csc, SpectralOp op, RegParams rp,
-                      const Reduction& red, cudaStream_t st)
+                      const Grid& gc, const cufftComplex* xc, size_t csc, SpectralOp op, RegParams rp, float rscale,
+                      double* sc, const Reduction& red, cudaStream_t st)
 {
-    k_tl_finish<<<red.nblocks, kThreads, 0, st>>>(gf, reinterpret_cast<const float2*>(rf), reinterpret_cast<float2*>(zf),
-                                              reinterpret_cast<const float2*>(zold), csf, gc,
-                                              reinterpret_cast<const float2*>(xc), csc, static_cast<int>(op), rp,
-                                              red);
+    k_tl_finish<<<red.nblocks, kThreads, 0, st>>>(gf, reinterpret_cast<const float2*>(rf),
+                                                  reinterpret_cast<float2*>(zf), reinterpret_cast<const float2*>(zold),
+                                                  csf, gc, reinterpret_cast<const float2*>(xc), csc,
+                                                  static_cast<int>(op), rp, rscale, sc, red);
 }
 
 void launch_dot(const float* x, const float* y, size_t n, const Reduction& red, cudaStream_t st)
