@@ -720,17 +720,14 @@ claire_status characteristics(claire_ctx* c, const float* v, float* dS, float* d
 
 
 // Set the linearisation point: characteristics, states m^j and grad m^j, S v,
-// objective pieces.  v (device) is copied into c->v unless it already is c->v.
+// objective pieces.  v: device.
 // With have_state the state characteristic X (c->dS) and the states
 // m^1..m^nt of this v are already in place (an accepted line-search trial).
 claire_status linearise(claire_ctx* c, const float* v, bool have_state = false)
 {
     if (!c->have_images) return fail(c, CLAIRE_ESTATE, "images not set (claire_set_images)");
     c->have_lin = false;
-    if (v != c->v)
-        CL_CUDA(c, cudaMemcpyAsync(c->v, v, 3 * c->N * sizeof(float), cudaMemcpyDeviceToDevice,
-                                   c->stream));
-    CL_TRY(characteristics(c, c->v, have_state ? nullptr : c->dS, c->dA, c->divv, c->divXp, c->sto));
+    CL_TRY(characteristics(c, v, have_state ? nullptr : c->dS, c->dA, c->divv, c->divXp, c->sto));
     {
         PhaseScope ps(c, CLAIRE_PHASE_STATE);
         const size_t N = c->N;
@@ -783,15 +780,16 @@ claire_status adjoint_and_body(claire_ctx* c, const void* a, const void* s, floa
     return CLAIRE_OK;
 }
 
-// g = S v + b (grad_form 0) or K(S v + b) at the current linearisation point;
+// g = S v + b (grad_form 0) or K(S v + b) at the current linearisation point, whose
+// velocity is v (device, 16-byte aligned: a transform reads it);
 // also returns J, mismatch, reg energy.
-claire_status gradient_at_lin(claire_ctx* c, float* g)
+claire_status gradient_at_lin(claire_ctx* c, const float* v, float* g)
 {
     const size_t N = c->N;
     if (c->vh_on)
         CL_TRY(spectral_hat(c, c->vh, g, SPEC_REG, 0));
     else
-        CL_TRY(spectral(c, c->v, g, SPEC_REG, 0));
+        CL_TRY(spectral(c, v, g, SPEC_REG, 0));
     {
         PhaseScope ps(c, CLAIRE_PHASE_VECTOR);
         KTimer t(c, KK_REDUCE, 8.0 * N, 0);
@@ -1317,10 +1315,25 @@ claire_status device_input(claire_ctx* c, const float* src, size_t n, float* scr
 claire_status copy_out(claire_ctx* c, float* dst, const float* src, size_t n)
 {
     if (!dst) return fail(c, CLAIRE_EINVAL, "null output argument");
-    if (dst == src) return CLAIRE_OK;
+    if (dst == src) {  // formed in place
+        CL_CUDA(c, cudaStreamSynchronize(c->stream));
+        return CLAIRE_OK;
+    }
     CL_CUDA(c, cudaMemcpyAsync(dst, src, n * sizeof(float), cudaMemcpyDefault, c->stream));
     CL_CUDA(c, cudaStreamSynchronize(c->stream));
     return CLAIRE_OK;
+}
+
+// Where a result of n floats is formed: the caller's array itself when it is
+// device memory at a 16-byte boundary (what the transforms and the vector loads
+// need) and shares no byte with the input of m floats; else the context's
+// scratch, from which copy_out then copies it.  A copy moves 8 bytes per value:
+// 60 us for a velocity at 256^3.
+float* result_array(float* dst, size_t n, const float* in, size_t m, float* scratch)
+{
+    const uintptr_t d = reinterpret_cast<uintptr_t>(dst), i = reinterpret_cast<uintptr_t>(in);
+    if ((d & 15u) || (d < i + m * sizeof(float) && i < d + n * sizeof(float)) || !is_device_ptr(dst)) return scratch;
+    return dst;
 }
 
 claire_status check_kernel_ptr(claire_ctx* c, const void* p)
@@ -1602,10 +1615,15 @@ claire_status claire_gradient(claire_ctx* c, const float* v, float* g, double* J
     const float* dv = nullptr;
     CL_TRY(device_input(c, v, 3 * c->N, c->v, &dv));
     CL_TRY(screen_velocity(c, dv));
+    if (reinterpret_cast<uintptr_t>(dv) & 15u) {
+        CL_CUDA(c, cudaMemcpyAsync(c->v, dv, 3 * c->N * sizeof(float), cudaMemcpyDeviceToDevice, c->stream));
+        dv = c->v;
+    }
+    float* out = result_array(g, 3 * c->N, dv, 3 * c->N, c->g);
     CL_TRY(linearise(c, dv));
-    CL_TRY(gradient_at_lin(c, c->g));
+    CL_TRY(gradient_at_lin(c, dv, out));
     if (J) *J = c->J_lin;
-    CL_TRY(copy_out(c, g, c->g, 3 * c->N));
+    CL_TRY(copy_out(c, g, out, 3 * c->N));
     collect_timing(c);
     return CLAIRE_OK;
 }
@@ -1617,8 +1635,9 @@ claire_status claire_hessian_matvec(claire_ctx* c, const float* vt, float* Hvt)
     if (!vt || !Hvt) return fail(c, CLAIRE_EINVAL, "null argument");
     const float* dvt = nullptr;
     CL_TRY(device_input(c, vt, 3 * c->N, c->p, &dvt));
-    CL_TRY(matvec(c, dvt, c->r));
-    CL_TRY(copy_out(c, Hvt, c->r, 3 * c->N));
+    float* out = result_array(Hvt, 3 * c->N, dvt, 3 * c->N, c->r);
+    CL_TRY(matvec(c, dvt, out));
+    CL_TRY(copy_out(c, Hvt, out, 3 * c->N));
     collect_timing(c);
     return CLAIRE_OK;
 }
@@ -1630,17 +1649,18 @@ claire_status claire_precond(claire_ctx* c, const float* r, float* z)
     if (!r || !z) return fail(c, CLAIRE_EINVAL, "null argument");
     const float* dr = nullptr;
     CL_TRY(device_input(c, r, 3 * c->N, c->p, &dr));
+    float* out = result_array(z, 3 * c->N, dr, 3 * c->N, c->r);
     if (c->o.precond == CLAIRE_PRECOND_TWO_LEVEL) {
         CL_TRY(tl_prepare(c));
         CL_FFT(c, cufftExecR2C(c->r2c, const_cast<float*>(dr), c->rh));
         double rz, ro;
         int its;
         CL_TRY(tl_apply(c, c->rh, static_cast<float>(1.0 / c->N), c->tl2->zf, nullptr, &rz, &ro, &its));
-        CL_FFT(c, cufftExecC2R(c->c2r, c->tl2->zf, c->r));
+        CL_FFT(c, cufftExecC2R(c->c2r, c->tl2->zf, out));
     } else {
-        CL_TRY(precond(c, dr, c->r));
+        CL_TRY(precond(c, dr, out));
     }
-    CL_TRY(copy_out(c, z, c->r, 3 * c->N));
+    CL_TRY(copy_out(c, z, out, 3 * c->N));
     collect_timing(c);
     return CLAIRE_OK;
 }
@@ -1694,7 +1714,7 @@ claire_status claire_register(claire_ctx* c, float* v_inout, claire_report* rep)
         return std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
     };
     CL_TRY(linearise(c, c->v));
-    CL_TRY(gradient_at_lin(c, c->g));
+    CL_TRY(gradient_at_lin(c, c->v, c->g));
     double gn;
     CL_TRY(dot(c, c->g, c->g, n3, &gn));
     // the tolerance and the PCG forcing are relative to g0_ref when given
@@ -1725,7 +1745,7 @@ claire_status claire_register(claire_ctx* c, float* v_inout, claire_report* rep)
                 ++R.pc_fallbacks;
                 // the trials overwrote the state characteristic and states: linearise again at v
                 CL_TRY(linearise(c, c->v));
-                CL_TRY(gradient_at_lin(c, c->g));
+                CL_TRY(gradient_at_lin(c, c->v, c->g));
                 c->o.precond = CLAIRE_PRECOND_SPECTRAL;
             }
             int its = 0;
@@ -1774,7 +1794,7 @@ claire_status claire_register(claire_ctx* c, float* v_inout, claire_report* rep)
         }
         R.gn_iters = k + 1;
         CL_TRY(linearise(c, c->v, true));  // c->v equals the accepted trial c->p bit for bit
-        CL_TRY(gradient_at_lin(c, c->g));
+        CL_TRY(gradient_at_lin(c, c->v, c->g));
         CL_TRY(dot(c, c->g, c->g, n3, &gn));
         rel = std::sqrt(gn) / g0;
         if (rel <= c->o.gtol) st = CLAIRE_OK;
@@ -1831,11 +1851,14 @@ claire_status claire_transport(claire_ctx* c, const float* v, const float* m_in,
     CL_TRY(device_input(c, m_in, N, reinterpret_cast<float*>(c->l0), &src));
     float* a = reinterpret_cast<float*>(c->l1);
     float* b = reinterpret_cast<float*>(c->l0);
+    // the last step writes the caller's array (the only one to read m_in when nt = 1)
+    float* last = c->nt > 1 ? result_array(m_out, N, nullptr, 0, nullptr) : result_array(m_out, N, m_in, N, nullptr);
     if (flags == CLAIRE_TRANSPORT_FWD) {
         CL_TRY(backtrace(c, dv, c->z, +1));
         for (int j = 0; j < c->nt; ++j) {
-            CL_TRY(interp(c, src, c->z, a, Storage::F32));
-            src = a;
+            float* dst = j + 1 == c->nt && last ? last : a;
+            CL_TRY(interp(c, src, c->z, dst, Storage::F32));
+            src = dst;
             std::swap(a, b);
         }
     } else {
@@ -1846,14 +1869,14 @@ claire_status claire_transport(claire_ctx* c, const float* v, const float* m_in,
             const void* gs;
             CL_TRY(gather_src(c, src, 1, &gs));
             KTimer t(c, KK_ADJ_STEP, 28.0 * N, 1.0 * N);
-            launch_adj_step(c->grid, c->o.interp, gs, c->z, divv, divXp, static_cast<float>(c->dt), a,
+            float* dst = j + 1 == c->nt && last ? last : a;
+            launch_adj_step(c->grid, c->o.interp, gs, c->z, divv, divXp, static_cast<float>(c->dt), dst,
                             Storage::F32, c->stream, tile_table(c, c->z));
             CL_LAUNCHED(c);
-            src = a;
+            src = dst;
             std::swap(a, b);
         }
     }
-    CL_TRY(sync_scalars(c));
     CL_TRY(copy_out(c, m_out, src, N));
     collect_timing(c);
     return CLAIRE_OK;
@@ -1940,6 +1963,7 @@ extern "C" claire_status claire_transport_vjp(claire_ctx* c, const float* v, con
             launch_grad_accum(c->grid, c->o.interp, mjc, d, mb, dbar, j == nt - 1, c->stream);
             CL_LAUNCHED(c);
         }
+        if (j == 0 && gm0 && c->o.interp != 4) mb2 = result_array(gm0, N, dv, 3 * N, mb2);
         CL_TRY(scatter_transpose(c, mb, d, nullptr, mb2, false, 1.0f));
         if (c->o.interp == 4) {
             // the transpose of "prefilter, then interpolate": scatter, then the
@@ -1952,7 +1976,7 @@ extern "C" claire_status claire_transport_vjp(claire_ctx* c, const float* v, con
     }
     if (gm0) CL_TRY(copy_out(c, gm0, mb, N));
     if (gv) {
-        float* ub = c->p;
+        float* ub = result_array(gv, 3 * N, dv, 3 * N, c->p);
         float* Ub = reinterpret_cast<float*>(c->spec);  // 6 M >= 3 N floats, unused here
         const void* vsrc;
         CL_TRY(gather_src(c, dv, 3, &vsrc));  // v, or its B-spline coefficients

@@ -288,22 +288,31 @@ __device__ __forceinline__ void scatter_disp(const Grid& g, const float* __restr
 constexpr float kFixMagic = 12582912.0f;             // 1.5 2^23, bits 0x4b400000
 constexpr float kFixDown = 7.450580596923828125e-9f;  // 2^-27
 
-// The term, its h biased by the magic's bits: term + kFixBias 2^32 mod 2^64
-// (the bias 0x4b400000 2^27 has only a high word).
+// The term as two words, its h biased by the magic's bits: term + kFixBias 2^32
+// mod 2^64 (the bias 0x4b400000 2^27 has only a high word).
 constexpr unsigned kFixBias = 0x4b400000u >> 5;
 
-__device__ __forceinline__ unsigned long long fixed_term_biased(float wab, float wab_down, float wc)
+struct FixedTerm {
+    unsigned lo, hi;
+};
+
+__device__ __forceinline__ FixedTerm fixed_term_biased(float wab, float wab_down, float wc)
 {
     const float p = wab * wc;
     const float x = fmaf(wab_down, wc, kFixMagic);
-    const float r = fmaf(__fsub_rn(x, kFixMagic), -134217728.0f, p);
-    return static_cast<unsigned long long>(static_cast<long long>(__float_as_int(x)) * 134217728ll +
-                                           __float2int_rn(r));
+    const int r = __float2int_rn(fmaf(__fsub_rn(x, kFixMagic), -134217728.0f, p));
+    FixedTerm t;
+    asm("{\n .reg .u32 a, b, s;\n shl.b32 a, %2, 27;\n add.cc.u32 %0, a, %3;\n shr.u32 b, %2, 5;\n"
+        " shr.s32 s, %3, 31;\n addc.u32 %1, b, s;\n}\n"
+        : "=r"(t.lo), "=r"(t.hi)
+        : "r"(__float_as_int(x)), "r"(r));
+    return t;
 }
 
 __device__ __forceinline__ unsigned long long fixed_term(float wab, float wc)
 {
-    return fixed_term_biased(wab, wab * kFixDown, wc) - (static_cast<unsigned long long>(kFixBias) << 32);
+    const FixedTerm t = fixed_term_biased(wab, wab * kFixDown, wc);
+    return (static_cast<unsigned long long>(t.hi - kFixBias) << 32) | t.lo;
 }
 
 // 64-bit addition of a biased term into shared memory as two 32-bit additions:
@@ -312,21 +321,17 @@ __device__ __forceinline__ unsigned long long fixed_term(float wab, float wc)
 // compare-and-swap loop on this part.)  The sum of all additions is exact
 // whatever their order.
 template <int BYTE_OFF>
-__device__ __forceinline__ unsigned add_low(uint32_t lo, unsigned long long v)
+__device__ __forceinline__ unsigned add_low(uint32_t lo, const FixedTerm& t)
 {
     unsigned old;
-    asm volatile("atom.shared.add.u32 %0, [%1+%2], %3;" : "=r"(old) : "r"(lo), "n"(BYTE_OFF),
-                 "r"(static_cast<unsigned>(v)) : "memory");
+    asm volatile("atom.shared.add.u32 %0, [%1+%2], %3;" : "=r"(old) : "r"(lo), "n"(BYTE_OFF), "r"(t.lo) : "memory");
     return old;
 }
 template <int BYTE_OFF>
-__device__ __forceinline__ void add_high(uint32_t hi, unsigned long long v, unsigned old)
+__device__ __forceinline__ void add_high(uint32_t hi, const FixedTerm& t, unsigned old)
 {
-    unsigned lo, h;
-    asm("add.cc.u32 %0, %2, %3;\n\taddc.u32 %1, %4, %5;"
-        : "=r"(lo), "=r"(h)
-        : "r"(old), "r"(static_cast<unsigned>(v)), "r"(static_cast<unsigned>(v >> 32)), "n"(0u - kFixBias));
-    asm volatile("red.shared.add.u32 [%0+%1], %2;" ::"r"(hi), "n"(BYTE_OFF), "r"(h) : "memory");
+    asm volatile("{\n .reg .u32 a, b;\n add.cc.u32 a, %2, %3;\n addc.u32 b, %4, %5;\n red.shared.add.u32 [%0+%1], b;\n}\n"
+                 ::"r"(hi), "n"(BYTE_OFF), "r"(old), "r"(t.lo), "r"(t.hi), "n"(0u - kFixBias) : "memory");
 }
 
 // Scatter-transpose tiles: a CTA owns a 4 x 8 x 32 tile of source points
@@ -461,7 +466,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_scatter_tiled(Grid g, const flo
                 const float wab = ys * (w1[a] * w2[b]), wd = wab * kFixDown;
                 const uint32_t lo = lo_s + 4u * static_cast<uint32_t>(first + (a * e2 + b) * e3);
                 const uint32_t hi = lo + hi_off;
-                unsigned long long t[M];
+                FixedTerm t[M];
                 unsigned old[M];
 #pragma unroll
                 for (int c = 0; c < M; ++c) t[c] = fixed_term_biased(wab, wd, w3[c]);

@@ -160,3 +160,52 @@ def test_boxes_on_every_row_length_carry_a_shift(n, storage):
     vol = float(np.prod([2 * np.pi / s for s in n]))
     assert mis <= (0.0 if storage else 0.5 * vol * m0.size * (4 * 4e-6) ** 2)
     ctx.close()
+
+
+@pytest.mark.parametrize("nt", [1, 4])
+def test_results_formed_in_the_callers_array(nt):
+    """Results are formed in the caller's array when it is aligned and shares no
+    byte with the input, else in scratch and copied: outputs into separate,
+    unaligned and partly or fully shared arrays hold the same bits, and an input
+    that is not shared is left alone."""
+    from paper_2209_08189_gb300 import claire
+    n = (16, 24, 40)
+    N = n[0] * n[1] * n[2]
+    ctx = claire.Context(n, 1e-2, nt, stream=torch.cuda.current_stream().cuda_stream)
+    v = _dev(synth.mode_velocity(n, seed=3, vmax=0.4, kmax=2))
+    vt = _dev(synth.mode_velocity(n, seed=4, vmax=0.4, kmax=2))
+    m0, m1 = _dev(synth.blob_template(n, seed=1, sigma=0.9)), _dev(synth.blob_template(n, seed=2, sigma=0.9))
+    ctx.set_images(m0, m1)
+    new = lambda k: torch.empty(k * N, device="cuda")
+
+    def layouts(x, k):
+        """(input, output) views of k N floats; the input holds x."""
+        size = x.numel()
+        for out_off, shared in ((0, None), (1, None), (0, 0), (0, 4), (0, 3)):
+            if shared is None:  # separate arrays, output at out_off
+                inp, out = x.clone().reshape(-1), new(k + 1)[out_off:out_off + k * N]
+            else:               # one array, output `shared` floats behind the input
+                buf = new(max(k, size // N) + 1)
+                inp, out = buf[:size], buf[shared:shared + k * N]
+                inp.copy_(x.reshape(-1))
+            yield inp, out, shared is None
+
+    calls = {
+        "gradient": (v, 3, lambda i, o: ctx.gradient(i, o)),
+        "matvec": (vt, 3, lambda i, o: (ctx.gradient(v, new(3)), ctx.hessian_matvec(i, o))),
+        "precond": (vt, 3, lambda i, o: ctx.precond(i, o)),
+        "forward": (m0, 1, lambda i, o: ctx.transport(v, i, o)),
+        "adjoint": (m0, 1, lambda i, o: ctx.transport(v, i, o, claire.TRANSPORT_ADJ)),
+        "vjp": (v, 3, lambda i, o: ctx.transport_vjp(i, m0, m1, new(1), o)),
+        "vjp_image": (m1, 1, lambda i, o: ctx.transport_vjp(v, m0, i, o)),
+    }
+    for name, (x, k, call) in calls.items():
+        want = None
+        for inp, out, separate in layouts(x, k):
+            call(inp, out)
+            got = out.clone()
+            want = got if want is None else want
+            assert torch.equal(got, want), name
+            if separate:
+                assert torch.equal(inp, x.reshape(-1)), name
+    ctx.close()
