@@ -28,7 +28,7 @@ inline unsigned blocks_for(uint32_t n) { return (n + kThreads - 1) / kThreads; }
 // tile-bounds table of d (tile_index order), from the same FP32 values that
 // are stored, for the gathers at d.
 template <int ORDER, bool FULL, bool TBW>
-__global__ void __launch_bounds__(kTileThreads, CLAIRE_TILE_MIN_BLOCKS)
+__global__ void __launch_bounds__(kTileThreads, tile_min_blocks<ORDER>())
     k_backtrace_tiled(Grid g, const float* __restrict__ v, const float* __restrict__ vc, float dt, float sign,
                       float* __restrict__ d, int4* __restrict__ tb)
 {
@@ -127,10 +127,10 @@ template <int ORDER, bool FULL, bool TBW>
 void launch_backtrace_tiled_as(const Grid& g, const float* v, const float* vc, float dt, float sign, float* d,
                                int4* tb, cudaStream_t st)
 {
-    if (kTiledSmemBytes > 48 * 1024)
+    if (tiled_smem_bytes<ORDER>() > 48 * 1024)
         cudaFuncSetAttribute(k_backtrace_tiled<ORDER, FULL, TBW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(kTiledSmemBytes));
-    k_backtrace_tiled<ORDER, FULL, TBW><<<tiled_grid(g), kTileThreads, kTiledSmemBytes, st>>>(g, v, vc, dt, sign,
+                             static_cast<int>(tiled_smem_bytes<ORDER>()));
+    k_backtrace_tiled<ORDER, FULL, TBW><<<tiled_grid(g), kTileThreads, tiled_smem_bytes<ORDER>(), st>>>(g, v, vc, dt, sign,
                                                                                               d, tb);
 }
 
@@ -673,10 +673,10 @@ void launch_interp(const Grid& g, int order, const void* f, const float* d, void
 template <int ORDER, bool FULL, bool MAP>
 void launch_fields_tiles(const Grid& g, const float* f, int nf, const float* d, float* out, cudaStream_t st)
 {
-    if (kTiledSmemBytes > 48 * 1024)
+    if (tiled_smem_bytes<ORDER>() > 48 * 1024)
         cudaFuncSetAttribute(k_gather_tiled_fields<ORDER, FULL, MAP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(kTiledSmemBytes));
-    k_gather_tiled_fields<ORDER, FULL, MAP><<<tiled_grid(g), kTileThreads, kTiledSmemBytes, st>>>(g, f, nf, d, out);
+                             static_cast<int>(tiled_smem_bytes<ORDER>()));
+    k_gather_tiled_fields<ORDER, FULL, MAP><<<tiled_grid(g), kTileThreads, tiled_smem_bytes<ORDER>(), st>>>(g, f, nf, d, out);
 }
 
 template <int ORDER, bool MAP>

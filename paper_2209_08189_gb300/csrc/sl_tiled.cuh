@@ -49,6 +49,24 @@ static __device__ unsigned long long g_gather_global_tiles = 0;
 constexpr int kTileThreads = TILE2 * 32;
 constexpr int kBoxCapFloats = CLAIRE_BOX_CAP;
 
+// Trilinear FP32 tiles: a point reads 8 values, so a tile is mostly the latency of
+// its staging, and six CTAs per SM with boxes of 36 KB (a stencil two nodes wide
+// needs half the box) hide it better than four of 46 KB: 256 x 300 x 256
+// transport of eight steps 1277 -> 1130 us (five: 1205, seven: 1122 but 5 %
+// slower adjoint steps).  16-bit fields, whose boxes also hold the staging copy,
+// lose 2 % with six and keep four.
+constexpr int kBoxCapLinear = 9216;
+template <int ORDER, int ES = 4>
+__host__ __device__ constexpr int box_cap()
+{
+    return ORDER == 1 && ES == 4 && kBoxCapLinear < kBoxCapFloats ? kBoxCapLinear : kBoxCapFloats;
+}
+template <int ORDER, int ES = 4>
+constexpr int tile_min_blocks()
+{
+    return ORDER == 1 && ES == 4 ? 6 : CLAIRE_TILE_MIN_BLOCKS;
+}
+
 __device__ __forceinline__ void cp_async_f32(float* smem_dst, const float* gmem_src)
 {
     const unsigned s = static_cast<unsigned>(__cvta_generic_to_shared(smem_dst));
@@ -145,7 +163,7 @@ __host__ __device__ __forceinline__ void box_geometry(const Grid& g, int a1, int
     const unsigned s3 = (e3 + 31) & ~31u;  // bank-aligned row stride
     // FP32 box plus, for 16-bit storage, the staging copy (half its size)
     fits = fits && e3 <= n3 &&
-           static_cast<unsigned long long>(e1 * e2) * s3 * (ES == 2 ? 3 : 2) <= 2ull * kBoxCapFloats;
+           static_cast<unsigned long long>(e1 * e2) * s3 * (ES == 2 ? 3 : 2) <= 2ull * box_cap<ORDER, ES>();
     par[0] = fits ? static_cast<int>(static_cast<unsigned>(a1) - OFF) : 0;
     par[1] = fits ? static_cast<int>(static_cast<unsigned>(a2) - OFF) : 0;
     par[2] = fits ? static_cast<int>(o3) : 0;
@@ -552,7 +570,7 @@ __device__ __forceinline__ float tile_eval(const float* box, const BoxPar& bp, i
 // fails, which a table written with this d never causes, the tile takes the
 // global-memory path.
 template <int ORDER, class Epi, class S, bool FULL, bool TB = false>
-__global__ void __launch_bounds__(kTileThreads, CLAIRE_TILE_MIN_BLOCKS)
+__global__ void __launch_bounds__(kTileThreads, tile_min_blocks<ORDER, sizeof(S)>())
     k_gather_tiled(Grid g, const S* __restrict__ f, const float* __restrict__ d, Epi epi,
                    const int4* __restrict__ tb = nullptr)
 {
@@ -664,7 +682,7 @@ __global__ void __launch_bounds__(kTileThreads, CLAIRE_TILE_MIN_BLOCKS)
 // box as the gathers do; the per-point kernel it replaced fetched them through
 // L1 (256^3, CFL 3.4: 0.80 ms per step; from the box 0.56 ms).
 template <int ORDER, bool FULL, bool MAP = false>
-__global__ void __launch_bounds__(kTileThreads, CLAIRE_TILE_MIN_BLOCKS)
+__global__ void __launch_bounds__(kTileThreads, tile_min_blocks<ORDER>())
     k_gather_tiled_fields(Grid g, const float* __restrict__ f, int nf, const float* __restrict__ d,
                           float* __restrict__ out)
 {
@@ -740,15 +758,19 @@ inline dim3 tiled_grid(const Grid& g)
     return dim3((g.n3 + TILE3 - 1) / TILE3, (g.n2 + TILE2 - 1) / TILE2, (g.n1 + TILE1 - 1) / TILE1);
 }
 
-constexpr size_t kTiledSmemBytes = kBoxCapFloats * sizeof(float);
+template <int ORDER, int ES = 4>
+constexpr size_t tiled_smem_bytes()
+{
+    return box_cap<ORDER, ES>() * sizeof(float);
+}
 
 template <int ORDER, class Epi, class S, bool FULL, bool TB>
 inline void launch_tiled_as(const Grid& g, const S* f, const float* d, const Epi& e, cudaStream_t st, const int4* tb)
 {
-    if (kTiledSmemBytes > 48 * 1024)
+    if (tiled_smem_bytes<ORDER, sizeof(S)>() > 48 * 1024)
         cudaFuncSetAttribute(k_gather_tiled<ORDER, Epi, S, FULL, TB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(kTiledSmemBytes));
-    k_gather_tiled<ORDER, Epi, S, FULL, TB><<<tiled_grid(g), kTileThreads, kTiledSmemBytes, st>>>(g, f, d, e, tb);
+                             static_cast<int>(tiled_smem_bytes<ORDER, sizeof(S)>()));
+    k_gather_tiled<ORDER, Epi, S, FULL, TB><<<tiled_grid(g), kTileThreads, tiled_smem_bytes<ORDER, sizeof(S)>(), st>>>(g, f, d, e, tb);
 }
 
 template <int ORDER, class Epi, class S>

@@ -209,3 +209,4 @@ def test_results_formed_in_the_callers_array(nt):
             if separate:
                 assert torch.equal(inp, x.reshape(-1)), name
     ctx.close()
+
