@@ -498,10 +498,15 @@ claire_status sync_scalars(claire_ctx* c)
     return CLAIRE_OK;
 }
 
-// Totals into dres[slot] (and slot + 1) and their host mirror, times scale.
-Reduction reduction(claire_ctx* c, int slot, double scale = 1.0)
+// Totals into dres[slot] (and slot + 1) and their host mirror, times scale, over
+// `work` items a thread each at a time: no more blocks than they fill (a block
+// without work still pays its block sums and its turn at the ticket: 3 us for
+// the 608 blocks of a 32^3 screen).
+Reduction reduction(claire_ctx* c, int slot, size_t work, double scale = 1.0)
 {
-    return Reduction{c->partials, c->red_blocks, scale, c->dres + slot, c->hres_dev + slot, c->ticket};
+    const size_t blocks = std::min<size_t>(c->red_blocks, (work + 255) / 256);
+    return Reduction{c->partials, static_cast<int>(std::max<size_t>(blocks, 1)), scale, c->dres + slot,
+                     c->hres_dev + slot, c->ticket};
 }
 
 // Pinned scalars, their device address the ticket and the PCG's scalars.
@@ -528,7 +533,7 @@ claire_status dot_async(claire_ctx* c, const float* x, const float* y, size_t n,
                         int slot)
 {
     KTimer t(c, KK_REDUCE, 8.0 * n, 0);
-    launch_dot(x, y, n, reduction(c, slot, scale), c->stream);
+    launch_dot(x, y, n, reduction(c, slot, n / 4, scale), c->stream);
     CL_LAUNCHED(c);
     return CLAIRE_OK;
 }
@@ -555,7 +560,7 @@ claire_status spectral(claire_ctx* c, const float* in, float* out, SpectralOp op
     {
         KTimer t(c, KK_SPECTRAL, 48.0 * c->M, 0);
         // Parseval: sum_x = (1/N) sum_k over the unnormalised transform
-        const Reduction red = reduction(c, std::max(energy, 0), 0.5 * c->hvol / static_cast<double>(c->N));
+        const Reduction red = reduction(c, std::max(energy, 0), c->M, 0.5 * c->hvol / static_cast<double>(c->N));
         launch_spectral(c->grid, c->spec, c->spec, c->M, op, c->rp, static_cast<float>(1.0 / c->N),
                         energy >= 0 ? &red : nullptr, c->stream);
         CL_LAUNCHED(c);
@@ -576,7 +581,7 @@ claire_status spectral_hat(claire_ctx* c, const cufftComplex* vh, float* out, Sp
     PhaseScope ps(c, CLAIRE_PHASE_SPECTRAL);
     {
         KTimer t(c, KK_SPECTRAL, 48.0 * c->M, 0);
-        const Reduction red = reduction(c, energy, 0.5 * c->hvol * static_cast<double>(c->N));
+        const Reduction red = reduction(c, energy, c->M, 0.5 * c->hvol * static_cast<double>(c->N));
         launch_spectral(c->grid, vh, c->spec, c->M, op, c->rp, 1.0f, &red, c->stream);
         CL_LAUNCHED(c);
     }
@@ -601,9 +606,9 @@ claire_status reg_energy(claire_ctx* c, const float* v, const double* alpha, int
     const double N = static_cast<double>(c->N);
     if (alpha)
         launch_reg_energy(c->grid, c->vh, c->xh, c->M, static_cast<float>(*alpha), c->rp,
-                          reduction(c, slot, 0.5 * c->hvol * N), c->stream);
+                          reduction(c, slot, c->M, 0.5 * c->hvol * N), c->stream);
     else
-        launch_reg_energy(c->grid, c->spec, nullptr, c->M, 0.0f, c->rp, reduction(c, slot, 0.5 * c->hvol / N),
+        launch_reg_energy(c->grid, c->spec, nullptr, c->M, 0.0f, c->rp, reduction(c, slot, c->M, 0.5 * c->hvol / N),
                           c->stream);
     CL_LAUNCHED(c);
     return CLAIRE_OK;
@@ -793,7 +798,7 @@ claire_status gradient_at_lin(claire_ctx* c, const float* v, float* g)
     {
         PhaseScope ps(c, CLAIRE_PHASE_VECTOR);
         KTimer t(c, KK_REDUCE, 8.0 * N, 0);
-        launch_sqdiff(at(c, c->m, c->nt * N), c->m1, N, c->sto, reduction(c, 1, 0.5 * c->hvol), c->stream);
+        launch_sqdiff(at(c, c->m, c->nt * N), c->m1, N, c->sto, reduction(c, 1, N / 4, 0.5 * c->hvol), c->stream);
         CL_LAUNCHED(c);
     }
     CL_TRY(adjoint_and_body(c, c->m1, at(c, c->m, c->nt * N), g));
@@ -913,7 +918,7 @@ claire_status objective_at(claire_ctx* c, const float* v, double* J, double* mis
     CL_TRY(reg_energy(c, v, c->vh_on ? alpha : nullptr, 0));
     {
         KTimer t(c, KK_REDUCE, 8.0 * N, 0);
-        launch_sqdiff(src, c->m1, N, c->sto, reduction(c, 1, 0.5 * c->hvol), c->stream);
+        launch_sqdiff(src, c->m1, N, c->sto, reduction(c, 1, N / 4, 0.5 * c->hvol), c->stream);
         CL_LAUNCHED(c);
     }
     CL_TRY(sync_scalars(c));
@@ -943,7 +948,7 @@ claire_status detj_of(claire_ctx* c, const float* v, double* lo, double* hi)
     }
     {
         KTimer t(c, KK_DETJ, 12.0 * N, 0);
-        launch_detj_minmax(c->grid, a, reduction(c, 4), c->stream);
+        launch_detj_minmax(c->grid, a, reduction(c, 4, N), c->stream);
         CL_LAUNCHED(c);
     }
     CL_TRY(sync_scalars(c));
@@ -956,7 +961,7 @@ claire_status cfl_of(claire_ctx* c, const float* v, double* cfl)
 {
     {
         KTimer t(c, KK_REDUCE, 12.0 * c->N, 0);
-        launch_maxnorm3(v, c->N, reduction(c, 7), c->stream);
+        launch_maxnorm3(v, c->N, reduction(c, 7, c->N / 8), c->stream);
         CL_LAUNCHED(c);
     }
     CL_TRY(sync_scalars(c));
@@ -977,9 +982,9 @@ claire_status screen_velocity(claire_ctx* c, const float* v)
 
 // Totals of a Fourier-space PCG kernel into dres[slot], scaled to discrete
 // inner products (Parseval on scaled spectra).
-Reduction fs_reduction(claire_ctx* c, int slot)
+Reduction fs_reduction(claire_ctx* c, int slot, size_t modes)
 {
-    return reduction(c, slot, c->hvol * static_cast<double>(c->N));
+    return reduction(c, slot, modes, c->hvol * static_cast<double>(c->N));
 }
 
 // Wait for the first `count` of them (slot 0 on).
@@ -1128,7 +1133,7 @@ claire_status tl_apply(claire_ctx* c, const cufftComplex* rf, float rscale, cuff
     {
         KTimer kt(c, KK_SPECTRAL, 120.0 * t->M, 0);
         launch_tl_start(c->grid, rf, c->M, t->g, t->rh, t->xh, t->ph, t->cp, t->M, op, c->rp, rscale,
-                        t->sc, fs_reduction(c, 0), c->stream);
+                        t->sc, fs_reduction(c, 0, t->M), c->stream);
     }
     CL_TRY(fs_sums(c, 2));
     const double r0 = std::sqrt(c->hres[0]);
@@ -1151,13 +1156,14 @@ claire_status tl_apply(claire_ctx* c, const cufftComplex* rf, float rscale, cuff
         }
         {
             KTimer kt(c, KK_SPECTRAL, 48.0 * t->M, 0);
-            launch_tl_hp(t->g, t->cp, t->ph, t->M, c->o.grad_form, c->rp, tscale, t->sc, fs_reduction(c, 8), c->stream);
+            launch_tl_hp(t->g, t->cp, t->ph, t->M, c->o.grad_form, c->rp, tscale, t->sc,
+                         fs_reduction(c, 8, t->M), c->stream);
             CL_LAUNCHED(c);
         }
         {
             KTimer kt(c, KK_SPECTRAL, 144.0 * t->M, 0);
             launch_tl_update(t->g, t->cp, t->ph, t->xh, t->rh, t->M, c->o.grad_form, op, c->rp, tscale, t->sc,
-                             fs_reduction(c, 10), c->stream);
+                             fs_reduction(c, 10, t->M), c->stream);
             CL_LAUNCHED(c);
         }
         CL_TRY(sync_scalars(c));
@@ -1177,7 +1183,7 @@ claire_status tl_apply(claire_ctx* c, const cufftComplex* rf, float rscale, cuff
     {
         KTimer kt(c, KK_SPECTRAL, (zold ? 72.0 : 48.0) * c->M, 0);
         launch_tl_finish(c->grid, rf, zf, zold, c->M, t->g, t->xh, t->M, op, c->rp, rscale,
-                         c->psc, fs_reduction(c, 0), c->stream);
+                         c->psc, fs_reduction(c, 0, c->M), c->stream);
     }
     CL_TRY(fs_sums(c, 2));
     *rz = c->hres[0];
@@ -1208,7 +1214,7 @@ claire_status pcg(claire_ctx* c, double eta, int* its)
             CL_FFT(c, cufftExecR2C(c->r2c, c->g, c->spec));
         }
         KTimer t(c, KK_SPECTRAL, 72.0 * M, 0);
-        launch_fs_start(c->grid, c->spec, c->rh, c->xh, c->M, op, c->rp, scale, c->psc, fs_reduction(c, 0), c->stream);
+        launch_fs_start(c->grid, c->spec, c->rh, c->xh, c->M, op, c->rp, scale, c->psc, fs_reduction(c, 0, c->M), c->stream);
     }
     CL_TRY(fs_sums(c, 2));
     const double r0 = std::sqrt(c->hres[0]);
@@ -1251,7 +1257,7 @@ claire_status pcg(claire_ctx* c, double eta, int* its)
             }
             {
                 KTimer t(c, KK_SPECTRAL, 48.0 * M, 0);
-                launch_fs_hp(c->grid, c->spec2, c->phat, c->M, c->o.grad_form, c->rp, scale, c->psc, fs_reduction(c, 8),
+                launch_fs_hp(c->grid, c->spec2, c->phat, c->M, c->o.grad_form, c->rp, scale, c->psc, fs_reduction(c, 8, c->M),
                              c->stream);
                 CL_LAUNCHED(c);
             }
@@ -1259,7 +1265,7 @@ claire_status pcg(claire_ctx* c, double eta, int* its)
             // (it moves nothing when the curvature is not positive)
             KTimer t(c, KK_SPECTRAL, 144.0 * M, 0);
             launch_fs_update(c->grid, c->spec2, c->phat, c->xh, c->rh, two_level ? c->tl2->zf : nullptr, c->M,
-                             c->o.grad_form, op, c->rp, scale, c->psc, fs_reduction(c, 0), c->stream);
+                             c->o.grad_form, op, c->rp, scale, c->psc, fs_reduction(c, 0, c->M), c->stream);
         }
         CL_TRY(fs_sums(c, 0));
         const double pq = c->hres[8], alpha = c->hres[9];
@@ -1807,7 +1813,7 @@ claire_status claire_register(claire_ctx* c, float* v_inout, claire_report* rep)
         double den;
         {
             KTimer t(c, KK_REDUCE, 8.0 * N, 0);
-            launch_sqdiff(c->m0, c->m1, N, c->sto, reduction(c, 2, 0.5 * c->hvol), c->stream);
+            launch_sqdiff(c->m0, c->m1, N, c->sto, reduction(c, 2, N / 4, 0.5 * c->hvol), c->stream);
             CL_LAUNCHED(c);
         }
         CL_TRY(sync_scalars(c));
@@ -1890,7 +1896,7 @@ claire_status scatter_transpose(claire_ctx* c, const float* yv, const float* d, 
 {
     // the fixed-point scale follows max |yv|, computed on the device (no host round trip)
     double* mx = c->dres + 8;
-    launch_maxabs(yv, c->N, reduction(c, 8), c->stream);
+    launch_maxabs(yv, c->N, reduction(c, 8, c->N / 4), c->stream);
     CL_LAUNCHED(c);
     {
         KTimer t(c, KK_VJP_SCATTER, (4.0 + 12.0) * c->N, 1.0 * c->N);
@@ -2068,8 +2074,8 @@ claire_status claire_dice(claire_ctx* c, const float* a, const float* b, size_t 
     CL_TRY(check_kernel_ptr(c, b));
     {
         KTimer t(c, KK_REDUCE, 8.0 * n, 0, 2);
-        launch_count(a, b, n, 0.5f, 0, reduction(c, 10), c->stream);
-        launch_count(a, b, n, 0.5f, 1, reduction(c, 12), c->stream);
+        launch_count(a, b, n, 0.5f, 0, reduction(c, 10, n), c->stream);
+        launch_count(a, b, n, 0.5f, 1, reduction(c, 12, n), c->stream);
         CL_LAUNCHED(c);
     }
     CL_TRY(sync_scalars(c));

@@ -129,50 +129,11 @@ __global__ void __launch_bounds__(kThreads) k_spectral_direction(Grid g, const f
 // inverse FFT returns u and sum_x u(x) w(x) = N sum_k wt Re(conj(u~) w~)
 // (Parseval on the half spectrum; wt = multiplicity of the mode).
 
-__device__ __forceinline__ void block_sum2(double a, double b, double* pa, double* pb)
+// Grid-wide sums of a and b (grid_sums).
+__device__ __forceinline__ bool grid_sum2(double a, double b, const Reduction& r, double (&tot)[2])
 {
-    __shared__ double sa[32], sb[32];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_down_sync(0xffffffffu, a, o);
-        b += __shfl_down_sync(0xffffffffu, b, o);
-    }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) {
-        sa[wid] = a;
-        sb[wid] = b;
-    }
-    __syncthreads();
-    if (wid == 0) {
-        const int nw = (blockDim.x + 31) >> 5;
-        double x = lane < nw ? sa[lane] : 0.0;
-        double y = lane < nw ? sb[lane] : 0.0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            x += __shfl_down_sync(0xffffffffu, x, o);
-            y += __shfl_down_sync(0xffffffffu, y, o);
-        }
-        if (lane == 0) {
-            pa[blockIdx.x] = x;
-            pb[blockIdx.x] = y;
-        }
-    }
-}
-
-// Grid-wide sums of a and b.  True, with the scaled totals stored and returned,
-// in thread 0 of the block that finished last.
-__device__ __forceinline__ bool grid_sum2(double a, double b, const Reduction& r, double tot[2])
-{
-    block_sum2(a, b, r.partials, r.partials + r.nblocks);
-    if (!last_block(r.ticket)) return false;
-    const double x = total_of(r.partials, r.nblocks) * r.scale;
-    const double y = total_of(r.partials + r.nblocks, r.nblocks) * r.scale;
-    if (threadIdx.x != 0) return false;
-    put_result(r, 0, x);
-    put_result(r, 1, y);
-    tot[0] = x;
-    tot[1] = y;
-    return true;
+    const double v[2] = {a, b};
+    return grid_sums<2>(v, r, tot);
 }
 
 __device__ __forceinline__ float cdot3(float2 a0, float2 a1, float2 a2, float2 b0, float2 b1, float2 b2)
