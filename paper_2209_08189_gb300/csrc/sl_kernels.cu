@@ -520,7 +520,11 @@ __global__ void __launch_bounds__(kThreads) k_fd8_div_tiled(Grid g, const float*
         __syncthreads();
         const float d1 = fd_queue_diff(q), d2 = fd_sh_diff<32>(&sh2[b][(warp + 4) * 32 + lane]),
                     d3 = fd_sh_diff<1>(&sh3[b][warp * kFdCols + lane + 4]);
-        if (ok) stf<S>(out + static_cast<size_t>(i) * g.n23 + col, d1 * g.ih1 + d2 * g.ih2 + d3 * g.ih3);
+        // one order of rounding for all storage types and grids: a 16-bit div v
+        // turns another order's last FP32 bit into 2^-11 of the value
+        if (ok)
+            stf<S>(out + static_cast<size_t>(i) * g.n23 + col,
+                   fmaf(d3, g.ih3, fmaf(d1, g.ih1, __fmul_rn(d2, g.ih2))));
         fd_queue_push(q, qn);
     }
 }
