@@ -155,8 +155,8 @@ claire_status claire_net_pcw_weight(const float* o, float* w, size_t n, void* st
 /* Tiling of the tcgen05 convolution for this process: bricks of bdc x 16 x 8
  * voxels (bdc 1, 2 or 4: D planes sharing one staged halo) and nstage 1 or 2
  * shared-memory stages (2: the next channel slice is staged while the tensor
- * cores work).  0 restores the automatic choice (the deepest brick that
- * leaves two waves of CTAs, one stage).  A forced setting that does not fit a
+ * cores work).  0 restores the automatic choice (1 to 8 planes by a
+ * model of the fullest SM, one stage).  A forced setting that does not fit a
  * shape (D % bdc, TMEM or shared memory) makes that call fail with
  * CLAIRE_ECUDA.  Meant for tuning and tests; not thread-safe. */
 claire_status claire_net_set_conv_tiling(int bdc, int nstage);

@@ -233,8 +233,9 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3d(const __nv_bfloat16* __
 // with cp.async, the brick's halo ((BDc+2) x 18 x 10 voxels) and the slice of
 // all 27 taps' weights into shared memory in the no-swizzle K-major
 // core-matrix layout (8 rows x 16 bytes per core matrix, two 8-channel half
-// planes), then one elected thread issues 27 x BDc tcgen05.mma.kind::f16
-// (M128 x N x K16): the A operand of a (plane, tap) pair is the halo at a
+// planes), then one elected thread issues tcgen05.mma.kind::f16 (M128 x N x
+// K16), 27 x BDc of them or, with the kd taps stacked along N (TcShape::stack),
+// 9 x (BDc + 2): the A operand of a (plane, tap) pair is the halo at a
 // shifted start address, because every core matrix is 8 consecutive voxels
 // along W and the next one is the next H row (a constant stride).  The halo
 // is shared by the BDc planes; with two stages the next slice is staged while
@@ -1481,7 +1482,7 @@ cudaError_t conv3d(const void* X, int Cxs, int Cin, const void* Wt, const float*
         // tcgen05 path: bricks of bdc x 16 x 8 voxels; the deepest brick whose
         // TMEM columns (bdc planes x Cout rounded to 32) and shared memory fit
         TcShape sh{};
-        // stacked up to 64 output channels: an MMA reads 128 x 32 B of halo and N x 32 B
+        // stacked up to 80 output channels (N <= 256): an MMA reads 128 x 32 B of halo and N x 32 B
         // of weights from shared memory whatever its N, so three kd taps per read
         // of the halo save more than the clipped edge planes of a brick cost
         sh.stack = 3 * Cout <= 256 ? 1 : 0;
