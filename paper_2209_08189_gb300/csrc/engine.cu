@@ -1330,16 +1330,18 @@ claire_status copy_out(claire_ctx* c, float* dst, const float* src, size_t n)
     return CLAIRE_OK;
 }
 
-// Where a result of n floats is formed: the caller's array itself when it is
-// device memory at a 16-byte boundary (what the transforms and the vector loads
-// need) and shares no byte with the input of m floats; else the context's
+// Where a result of n floats is formed: the caller's array itself when
+// forms_in_place allows it (m floats of input at in), else the context's
 // scratch, from which copy_out then copies it.  A copy moves 8 bytes per value:
 // 60 us for a velocity at 256^3.
-float* result_array(float* dst, size_t n, const float* in, size_t m, float* scratch)
+float* result_array(const claire_ctx* c, float* dst, size_t n, const float* in, size_t m, float* scratch)
 {
-    const uintptr_t d = reinterpret_cast<uintptr_t>(dst), i = reinterpret_cast<uintptr_t>(in);
-    if ((d & 15u) || (d < i + m * sizeof(float) && i < d + n * sizeof(float)) || !is_device_ptr(dst)) return scratch;
-    return dst;
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, dst) != cudaSuccess) {
+        cudaGetLastError();
+        return scratch;
+    }
+    return forms_in_place(a, c->device, dst, n, in, m) ? dst : scratch;
 }
 
 claire_status check_kernel_ptr(claire_ctx* c, const void* p)
@@ -1625,7 +1627,7 @@ claire_status claire_gradient(claire_ctx* c, const float* v, float* g, double* J
         CL_CUDA(c, cudaMemcpyAsync(c->v, dv, 3 * c->N * sizeof(float), cudaMemcpyDeviceToDevice, c->stream));
         dv = c->v;
     }
-    float* out = result_array(g, 3 * c->N, dv, 3 * c->N, c->g);
+    float* out = result_array(c, g, 3 * c->N, dv, 3 * c->N, c->g);
     CL_TRY(linearise(c, dv));
     CL_TRY(gradient_at_lin(c, dv, out));
     if (J) *J = c->J_lin;
@@ -1641,7 +1643,7 @@ claire_status claire_hessian_matvec(claire_ctx* c, const float* vt, float* Hvt)
     if (!vt || !Hvt) return fail(c, CLAIRE_EINVAL, "null argument");
     const float* dvt = nullptr;
     CL_TRY(device_input(c, vt, 3 * c->N, c->p, &dvt));
-    float* out = result_array(Hvt, 3 * c->N, dvt, 3 * c->N, c->r);
+    float* out = result_array(c, Hvt, 3 * c->N, dvt, 3 * c->N, c->r);
     CL_TRY(matvec(c, dvt, out));
     CL_TRY(copy_out(c, Hvt, out, 3 * c->N));
     collect_timing(c);
@@ -1655,7 +1657,7 @@ claire_status claire_precond(claire_ctx* c, const float* r, float* z)
     if (!r || !z) return fail(c, CLAIRE_EINVAL, "null argument");
     const float* dr = nullptr;
     CL_TRY(device_input(c, r, 3 * c->N, c->p, &dr));
-    float* out = result_array(z, 3 * c->N, dr, 3 * c->N, c->r);
+    float* out = result_array(c, z, 3 * c->N, dr, 3 * c->N, c->r);
     if (c->o.precond == CLAIRE_PRECOND_TWO_LEVEL) {
         CL_TRY(tl_prepare(c));
         CL_FFT(c, cufftExecR2C(c->r2c, const_cast<float*>(dr), c->rh));
@@ -1858,7 +1860,7 @@ claire_status claire_transport(claire_ctx* c, const float* v, const float* m_in,
     float* a = reinterpret_cast<float*>(c->l1);
     float* b = reinterpret_cast<float*>(c->l0);
     // the last step writes the caller's array (the only one to read m_in when nt = 1)
-    float* last = c->nt > 1 ? result_array(m_out, N, nullptr, 0, nullptr) : result_array(m_out, N, m_in, N, nullptr);
+    float* last = c->nt > 1 ? result_array(c, m_out, N, nullptr, 0, nullptr) : result_array(c, m_out, N, m_in, N, nullptr);
     if (flags == CLAIRE_TRANSPORT_FWD) {
         CL_TRY(backtrace(c, dv, c->z, +1));
         for (int j = 0; j < c->nt; ++j) {
@@ -1969,7 +1971,7 @@ extern "C" claire_status claire_transport_vjp(claire_ctx* c, const float* v, con
             launch_grad_accum(c->grid, c->o.interp, mjc, d, mb, dbar, j == nt - 1, c->stream);
             CL_LAUNCHED(c);
         }
-        if (j == 0 && gm0 && c->o.interp != 4) mb2 = result_array(gm0, N, dv, 3 * N, mb2);
+        if (j == 0 && gm0 && c->o.interp != 4) mb2 = result_array(c, gm0, N, dv, 3 * N, mb2);
         CL_TRY(scatter_transpose(c, mb, d, nullptr, mb2, false, 1.0f));
         if (c->o.interp == 4) {
             // the transpose of "prefilter, then interpolate": scatter, then the
@@ -1982,7 +1984,7 @@ extern "C" claire_status claire_transport_vjp(claire_ctx* c, const float* v, con
     }
     if (gm0) CL_TRY(copy_out(c, gm0, mb, N));
     if (gv) {
-        float* ub = result_array(gv, 3 * N, dv, 3 * N, c->p);
+        float* ub = result_array(c, gv, 3 * N, dv, 3 * N, c->p);
         float* Ub = reinterpret_cast<float*>(c->spec);  // 6 M >= 3 N floats, unused here
         const void* vsrc;
         CL_TRY(gather_src(c, dv, 3, &vsrc));  // v, or its B-spline coefficients

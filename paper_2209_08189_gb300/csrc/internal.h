@@ -297,6 +297,19 @@ void launch_fd8_div(const Grid& g, const float* v, void* out, Storage sto, cudaS
 // totals: minimum at red.out[0], maximum at red.out[1] (scale unused)
 void launch_detj_minmax(const Grid& g, const float* u, const Reduction& red, cudaStream_t st);
 
+// Whether a context of GPU `device` may form a result of n floats at dst itself
+// (a: dst's pointer attributes): managed memory or memory of that GPU (kernels of
+// this GPU cannot store to another's unless peer access happens to be enabled, a
+// copy can), at a 16-byte boundary (what the transforms and the vector loads
+// need), sharing no byte with the input of m floats.
+inline bool forms_in_place(const cudaPointerAttributes& a, int device, const void* dst, size_t n, const void* in,
+                           size_t m)
+{
+    const uintptr_t d = reinterpret_cast<uintptr_t>(dst), i = reinterpret_cast<uintptr_t>(in);
+    if ((d & 15u) || (d < i + m * sizeof(float) && i < d + n * sizeof(float))) return false;
+    return a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == device);
+}
+
 // ---- context accessors for host-side drivers in other units (engine.cu) ----
 cudaStream_t ctx_stream(const claire_ctx* c);
 size_t ctx_points(const claire_ctx* c);
