@@ -323,6 +323,21 @@ void launch_bspline_scale(const Grid& g, cufftComplex* spec, size_t M, int ncomp
 // first: dbar is written instead of added to
 void launch_grad_accum(const Grid& g, int order, const float* m, const float* d, const float* mbar, float* dbar,
                        bool first, cudaStream_t st);
+// Whether the scatter-transpose of a tile fits its shared-memory box: first nodes
+// of the points' stencils in [a, z] per axis, stencils of m nodes, cap nodes in
+// the box.  Displacements are clamped to 2^20 cells only, so an extent may reach
+// 2^21: each is compared before they are multiplied (the product of three would
+// not fit 63 bits).
+__host__ __device__ inline bool scatter_box_fits(const int a[3], const int z[3], int m, int cap, int e[3])
+{
+    bool fits = true;
+    for (int c = 0; c < 3; ++c) {
+        e[c] = z[c] - a[c] + m;  // |a|, |z| below 2^30
+        fits = fits && e[c] >= m && e[c] <= cap;
+    }
+    return fits && static_cast<long long>(e[0]) * e[1] * e[2] <= cap;
+}
+
 // acc += fixed-point(W(x + disp)^T yv), scale from *maxabs = max |yv| (device);
 // disp = d, or -sdt v / h when d is null
 cudaError_t launch_scatter_fixed(const Grid& g, int order, const float* yv, const float* d, const float* v, float sdt,

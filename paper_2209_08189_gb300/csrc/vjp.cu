@@ -396,19 +396,18 @@ __global__ void __launch_bounds__(kThreads, 4) k_scatter_tiled(Grid g, const flo
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        int a1 = INT_MAX, a2 = INT_MAX, a3 = INT_MAX, z1 = INT_MIN, z2 = INT_MIN, z3 = INT_MIN;
-        for (int w = 0; w < kST2; ++w) {
-            a1 = min(a1, red[0][w]); a2 = min(a2, red[1][w]); a3 = min(a3, red[2][w]);
-            z1 = max(z1, red[3][w]); z2 = max(z2, red[4][w]); z3 = max(z3, red[5][w]);
-        }
-        par[0] = a1; par[1] = a2; par[2] = a3;
-        if (a1 > z1) {
+        int a[3] = {INT_MAX, INT_MAX, INT_MAX}, z[3] = {INT_MIN, INT_MIN, INT_MIN}, e[3];
+        for (int w = 0; w < kST2; ++w)
+            for (int c = 0; c < 3; ++c) {
+                a[c] = min(a[c], red[c][w]);
+                z[c] = max(z[c], red[3 + c][w]);
+            }
+        par[0] = a[0]; par[1] = a[1]; par[2] = a[2];
+        if (a[0] > z[0]) {
             par[6] = 0;  // no non-zero point in the tile
         } else {
-            const long long e1 = (long long)z1 - a1 + M, e2 = (long long)z2 - a2 + M, e3 = (long long)z3 - a3 + M;
-            const bool fits = e1 * e2 * e3 <= kScatterCap;
-            par[3] = (int)e1; par[4] = (int)e2; par[5] = (int)e3;
-            par[6] = fits ? 1 : 2;
+            par[6] = scatter_box_fits(a, z, M, kScatterCap, e) ? 1 : 2;
+            par[3] = e[0]; par[4] = e[1]; par[5] = e[2];
         }
     }
     __syncthreads();

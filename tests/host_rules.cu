@@ -43,6 +43,33 @@ void result_arrays()
     check(forms_in_place(own, 1, dst, 1000, nullptr, 0), "no input: in place");
 }
 
+// The box of a scatter tile holds every node that its points add to, whatever the
+// displacements (clamped to 2^20 cells, either sign, so extents reach 2^21).
+void scatter_boxes()
+{
+    constexpr int cap = 6976, m = 4;
+    const int lim = 1 << 20;
+    int e[3];
+    auto fits = [&](int s1, int s2, int s3) {
+        const int a[3] = {0, -5, 7}, z[3] = {s1, s2 - 5, s3 + 7};
+        return scatter_box_fits(a, z, m, cap, e);
+    };
+    check(fits(3, 7, 31) && e[0] == 7 && e[1] == 11 && e[2] == 35, "tile at rest");
+    check(fits(12, 12, 23) && e[0] * e[1] * e[2] == 6912, "box just below the cap");
+    check(!fits(12, 12, 24), "box just above the cap");
+    check(fits(0, 0, 432) && !fits(0, 0, 433), "long rows up to the cap");
+    // spans whose product wraps past 63 bits, to a negative, a small or a zero value
+    check(!fits(2 * lim, 2 * lim, 2 * lim), "2^21 on every axis");
+    check(!fits(2 * lim - 4, 2 * lim - 4, 2 * lim - 4), "extents 2^21: product 2^63");
+    check(!fits((1 << 22) - 4, (1 << 21) - 4, (1 << 21) - 4), "product 2^64");
+    for (int s1 : {0, 40, lim, 2 * lim})
+        for (int s2 : {0, 40, lim, 2 * lim})
+            for (int s3 : {0, 40, lim, 2 * lim}) {
+                const bool want = (s1 + 4.0) * (s2 + 4.0) * (s3 + 4.0) <= cap;
+                check(fits(s1, s2, s3) == want, "span grid");
+            }
+}
+
 }  // namespace
 
 int main(int argc, char** argv)
@@ -50,6 +77,8 @@ int main(int argc, char** argv)
     const char* group = argc > 1 ? argv[1] : "";
     if (!std::strcmp(group, "result_arrays"))
         result_arrays();
+    else if (!std::strcmp(group, "scatter_boxes"))
+        scatter_boxes();
     else
         check(false, "unknown group");
     if (!g_failures) std::printf("OK\n");

@@ -31,7 +31,7 @@ def host_rules(tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("group", ["result_arrays"])
+@pytest.mark.parametrize("group", ["result_arrays", "scatter_boxes"])
 def test_host_rules(host_rules, group):
     run = subprocess.run([host_rules, group], capture_output=True, text=True, timeout=120)
     assert run.returncode == 0 and run.stdout.strip() == "OK", run.stdout + run.stderr
