@@ -18,6 +18,7 @@
 // = input channels, reduction over voxels) with per-chunk FP32 partials
 // reduced in a fixed order, so results are deterministic.
 #include "claire_net.h"
+#include "conv_schedule.cuh"
 
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -235,7 +236,8 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3d(const __nv_bfloat16* __
 // core-matrix layout (8 rows x 16 bytes per core matrix, two 8-channel half
 // planes), then one elected thread issues tcgen05.mma.kind::f16 (M128 x N x
 // K16), 27 x BDc of them or, with the kd taps stacked along N (TcShape::stack),
-// 9 x (BDc + 2): the A operand of a (plane, tap) pair is the halo at a
+// 9 x (BDc + 2) in three groups (conv_schedule.cuh; 128^3 x 4, 16 -> 16 channels
+// 266 us, 257 without the two waits that keep overlapping MMAs apart): the A operand of a (plane, tap) pair is the halo at a
 // shifted start address, because every core matrix is 8 consecutive voxels
 // along W and the next one is the next H row (a constant stride).  The halo
 // is shared by the BDc planes; with two stages the next slice is staged while
@@ -362,7 +364,7 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3d_tc(const __nv_bfloat16*
                                                             TcShape sh, Vol v, int* __restrict__ err)
 {
     extern __shared__ __align__(128) unsigned char tc_smem[];
-    __shared__ __align__(8) uint64_t mbar, drain;
+    __shared__ __align__(8) uint64_t mbar, group, drain;
     __shared__ uint32_t tmem_slot;
     __shared__ int stall;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -374,7 +376,7 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3d_tc(const __nv_bfloat16*
     const int h0 = (r % nbh) * kTcBH; r /= nbh;
     const int d0 = (r % nbd) * bdc;
     const int b = r / nbd;
-    const uint32_t smem_s = smem_addr(tc_smem), mbar_s = smem_addr(&mbar);
+    const uint32_t smem_s = smem_addr(tc_smem), mbar_s = smem_addr(&mbar), group_s = smem_addr(&group);
     const int nchunks = Cin / 16;
     // staging: 16-byte pieces of the halo plane e = tid + 128 u < 360, piece e =
     // half e & 1 (8 channels) of slot e >> 1 = (sh * 10 + sw); the wrapped (h, w)
@@ -431,6 +433,7 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3d_tc(const __nv_bfloat16*
     const uint32_t drain_s = smem_addr(&drain);
     if (tid == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(mbar_s), "r"(1));
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(group_s), "r"(1));
         asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(drain_s), "r"(1));
         stall = g_tc_test_stall;
     }
@@ -475,26 +478,29 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3d_tc(const __nv_bfloat16*
             const uint64_t bd = umma_desc(base + 2 * sh.plane, (sh.stack ? 3 : 1) * Cout * 16, 128);
             const uint32_t a_lo = static_cast<uint32_t>(ad), a_hi = static_cast<uint32_t>(ad >> 32);
             const uint32_t b_lo = static_cast<uint32_t>(bd), b_hi = static_cast<uint32_t>(bd >> 32);
+            bool issued = true;
             if (sh.stack) {
-                // input plane sd feeds the output planes z = sd - kd: blocks j = 2 - kd
-                // of N, at the columns of z = sd - 2 + j, clipped to the brick
                 const uint32_t bstep = 6u * Cout;
-                for (int sd = 0; sd < bdc + 2; ++sd) {
-                    const int j0 = sd < 2 ? 2 - sd : 0, j1 = sd < bdc ? 3 : bdc + 2 - sd;
-                    const uint32_t ap = a_lo + static_cast<uint32_t>(sd * kTcPlaneSlots);
-                    const uint32_t bp = b_lo + static_cast<uint32_t>(j0 * Cout);
-                    const uint32_t dt = tmem + static_cast<uint32_t>((sd - 2 + j0) * Cout);
-                    const uint32_t id = idesc((j1 - j0) * Cout);
-                    // plane z = sd sees its first product here (kd = 0): written, not added
-                    if (c == 0 && j1 == 3) {
-                        if (j0 < 2) umma(dt, ap, a_hi, bp, b_hi, idesc((2 - j0) * Cout), 1u);
-                        umma(tmem + static_cast<uint32_t>(sd * Cout), ap, a_hi, b_lo + 2u * Cout, b_hi, idesc(Cout), 0u);
-                    } else {
-                        umma(dt, ap, a_hi, bp, b_hi, id, 1u);
+                for (int grp = 0; grp < kStackGroups && issued; ++grp) {
+                    if (stacked_wait(bdc, grp)) {
+                        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::
+                                         "r"(group_s)
+                                     : "memory");
+                        // two phases per slice, waited for by this thread alone
+                        issued = mbar_wait(group_s, (grp - 1) & 1);
+                        asm volatile("tcgen05.fence::after_thread_sync;");
                     }
+                    for (int sd = grp; sd < bdc + 2 && issued; sd += kStackGroups) {
+                        const StackedPlane sp = stacked_plane(bdc, sd);
+                        const uint32_t ap = a_lo + static_cast<uint32_t>(sd * kTcPlaneSlots);
+                        const uint32_t bp = b_lo + static_cast<uint32_t>((2 - (sd - sp.z0)) * Cout);
+                        const uint32_t dt = tmem + static_cast<uint32_t>(sp.z0 * Cout);
+                        const uint32_t id = idesc(sp.nz * Cout);
+                        umma(dt, ap, a_hi, bp, b_hi, id, c > 0 || grp > 0 ? 1u : 0u);
 #pragma unroll
-                    for (int t = 1; t < 9; ++t)
-                        umma(dt, ap + (t / 3) * kTcHaloW + t % 3, a_hi, bp + t * bstep, b_hi, id, 1u);
+                        for (int t = 1; t < 9; ++t)
+                            umma(dt, ap + (t / 3) * kTcHaloW + t % 3, a_hi, bp + t * bstep, b_hi, id, 1u);
+                    }
                 }
             } else {
                 const uint32_t id = idesc(Cout), bstep = 2u * Cout;
@@ -511,8 +517,10 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3d_tc(const __nv_bfloat16*
                     }
                 }
             }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar_s)
-                         : "memory");
+            // a group that gave up leaves the phase open: every wait for it runs out
+            if (issued)
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar_s)
+                             : "memory");
         }
     }
     if (ok) ok = __syncthreads_and(mbar_wait(mbar_s, (nchunks - 1) & 1)) != 0;

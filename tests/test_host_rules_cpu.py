@@ -1,6 +1,7 @@
-"""Rules that decide where a kernel may store, compiled for the host from the
-kernels' own headers (host_rules.cu): faults in them would be stores out of
-range or to memory of another GPU, so they are tested without a GPU."""
+"""Rules that decide where a kernel may store and in which order, compiled for
+the host from the kernels' own headers (host_rules.cu): faults in them would be
+stores out of range, to memory of another GPU, or in an undefined order, so they
+are tested without a GPU."""
 import os
 import shutil
 import subprocess
@@ -31,7 +32,7 @@ def host_rules(tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("group", ["result_arrays", "scatter_boxes"])
+@pytest.mark.parametrize("group", ["result_arrays", "scatter_boxes", "conv_schedule"])
 def test_host_rules(host_rules, group):
     run = subprocess.run([host_rules, group], capture_output=True, text=True, timeout=120)
     assert run.returncode == 0 and run.stdout.strip() == "OK", run.stdout + run.stderr
