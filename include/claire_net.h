@@ -153,7 +153,7 @@ claire_status claire_net_pcw_loss(const float* o, const float* num, const float*
 claire_status claire_net_pcw_weight(const float* o, float* w, size_t n, void* stream);
 
 /* Tiling of the tcgen05 convolution for this process: bricks of bdc x 16 x 8
- * voxels (bdc 1, 2 or 4: D planes sharing one staged halo) and nstage 1 or 2
+ * voxels (bdc 1, 2, 4 or, up to 64 output channels, 8: D planes sharing one staged halo) and nstage 1 or 2
  * shared-memory stages (2: the next channel slice is staged while the tensor
  * cores work).  0 restores the automatic choice (1 to 8 planes by a
  * model of the fullest SM, one stage).  A forced setting that does not fit a

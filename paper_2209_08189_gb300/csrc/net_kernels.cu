@@ -2180,8 +2180,8 @@ extern "C" claire_status claire_net_set_wgrad_tiling(int nc)
 
 extern "C" claire_status claire_net_set_conv_tiling(int bdc, int nstage)
 {
-    if ((bdc != 0 && bdc != 1 && bdc != 2 && bdc != 4) || nstage < 0 || nstage > 2)
-        return net_fail("set_conv_tiling: bdc in {0, 1, 2, 4}, nstage in {0, 1, 2}");
+    if ((bdc != 0 && bdc != 1 && bdc != 2 && bdc != 4 && bdc != 8) || nstage < 0 || nstage > 2)
+        return net_fail("set_conv_tiling: bdc in {0, 1, 2, 4, 8}, nstage in {0, 1, 2}");
     g_tc_force_bdc = bdc;
     g_tc_force_nstage = nstage;
     return CLAIRE_OK;

@@ -127,6 +127,41 @@ def test_conv3d_tcgen05_tilings(env, tiling):
     assert net.device_errors() == 0
 
 
+@pytest.mark.parametrize("co", [16, 32, 48, 64, 96])
+def test_conv3d_tcgen05_every_depth(env, co):
+    """Brick depths 1 to 8 with one and two stages: stacked depth taps up to 64 output
+    channels (three blocks of 64 are the widest), plain ones at 96; three channel
+    slices.  A depth that does not fit (TMEM columns, shared memory, more than four
+    planes unstacked) is refused.  Tolerance: the parity test's."""
+    torch, net = env
+    B, D, H, W, ci = 2, 16, 16, 8, 48
+    r = np.random.default_rng(co)
+    xbuf = bf16(torch, r.standard_normal((B, D, H, W, ci)))
+    w = bf16(torch, r.standard_normal((co, 27, ci)) / np.sqrt(27 * ci))
+    bias = torch.from_numpy(r.standard_normal(co).astype(np.float32)).cuda()
+    ref = onet.conv3d(f64(xbuf), f64(w), f64(bias), act=True, slope=0.1)
+    depths = 0
+    try:
+        for bdc in (1, 2, 4, 8):
+            for nstage in (1, 2):
+                fits = (nstage * (2 * (bdc + 2) * 2880 + 27 * 32 * co) <= 231424 and
+                        bdc * co <= 512 and (bdc <= 4 or co <= 64))
+                net.set_conv_tiling(bdc, nstage)
+                y = torch.zeros((B, D, H, W, co), dtype=torch.bfloat16, device="cuda")
+                if not fits:
+                    with pytest.raises(Exception):
+                        net.conv3d(net.Act(xbuf, 0, ci), w, bias, net.Act(y, 0, co), 0.1, 1, stream(torch))
+                    continue
+                net.conv3d(net.Act(xbuf, 0, ci), w, bias, net.Act(y, 0, co), 0.1, 1, stream(torch))
+                torch.cuda.synchronize()
+                assert close_bf16(f64(y), ref) <= 0, (bdc, nstage)
+                depths = max(depths, bdc)
+    finally:
+        net.set_conv_tiling(0, 0)
+    assert depths == (8 if co <= 64 else 4)
+    assert net.device_errors() == 0
+
+
 @pytest.mark.parametrize("case", CONV_CASES)
 def test_conv3d_weight_gradient(env, case):
     torch, net = env
