@@ -3,6 +3,7 @@
 // solves, 8th-order finite differences, deformation-map transport and the
 // Jacobian determinant.  Method: "CLAIRE at scale" (arXiv 2209.08189),
 // Sec. 2.2 (SL with RK2, FD8) and Sec. 3 (IP and FD kernels).
+#include "detj.cuh"
 #include "internal.h"
 #include "sl_tiled.cuh"
 
@@ -544,13 +545,10 @@ __device__ __forceinline__ float ordered_float(int i) { return __int_as_float(i 
 // 2 operations per clock and SM, so the 30 FP64 operations of every point's
 // determinant were most of the kernel (256^3: 933 us).  Each determinant is
 // first formed in FP32 with an error bound E; only points that may be below
-// the block's smallest or above its largest value so far are formed in FP64.
-// E = 4e-6 m^3, m the largest |entry|: each of the six triple products (at
-// most m^3) carries three entry roundings, two products and up to three sums
-// of relative error 2^-24, together below 6 * 8 * 2^-24 m^3 = 2.9e-6 m^3.
-// A NaN or an overflow fails both comparisons and is formed in FP64.  The
-// extrema are the FP64 ones, bit for bit.  Columns are walked by a fixed
-// number of CTAs (one partial each).  256^3: 328 us.
+// the block's smallest or above its largest value so far are formed in FP64
+// (det_bounds).  A NaN or an overflow fails both comparisons and is formed in
+// FP64.  The extrema are the FP64 ones of the same FP32 differences, bit for bit.
+// Columns are walked by a fixed number of CTAs (one partial each).  256^3: 328 us.
 __global__ void __launch_bounds__(kThreads) k_detj_minmax(Grid g, const float* __restrict__ u, int zlen, int ncol,
                                                            Reduction red)
 {
@@ -600,24 +598,16 @@ __global__ void __launch_bounds__(kThreads) k_detj_minmax(Grid g, const float* _
             // any value a lane reads here bounds the block's extrema; the warp takes lane 0's
             float flo = ordered_float(__shfl_sync(0xffffffffu, *static_cast<volatile int*>(&blo), 0)),
                   fhi = ordered_float(__shfl_sync(0xffffffffu, *static_cast<volatile int*>(&bhi), 0));
-            float e[3][3], f[3][3], m = 0.0f;
+            float e[3][3];
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                e[c][0] = fd_queue_diff(q[c]) * g.ih1;
-                e[c][1] = fd_sh_diff<kFdCols>(sh[par][c] + own) * g.ih2;
-                e[c][2] = fd_sh_diff<1>(sh[par][c] + own) * g.ih3;
+                e[c][0] = __fmul_rn(fd_queue_diff(q[c]), g.ih1);
+                e[c][1] = __fmul_rn(fd_sh_diff<kFdCols>(sh[par][c] + own), g.ih2);
+                e[c][2] = __fmul_rn(fd_sh_diff<1>(sh[par][c] + own), g.ih3);
                 fd_queue_push(q[c], qn[c]);
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    f[c][a] = a == c ? 1.0f + e[c][a] : e[c][a];
-                    m = fmaxf(m, fabsf(f[c][a]));
-                }
             }
-            const float det = f[0][0] * (f[1][1] * f[2][2] - f[1][2] * f[2][1]) -
-                              f[0][1] * (f[1][0] * f[2][2] - f[1][2] * f[2][0]) +
-                              f[0][2] * (f[1][0] * f[2][1] - f[1][1] * f[2][0]);
-            const float E = 4e-6f * m * m * m;
-            const float dlo = det - E, dhi = det + E;
+            float dlo, dhi;
+            det_bounds(e, dlo, dhi);
             // dhi bounds lo from above, dlo bounds hi from below (finite ones only);
             // the bounds are raised by the plane's own points before it is tested
             const bool fin = t.ok && fabsf(dlo) < 3e38f && fabsf(dhi) < 3e38f;
@@ -629,16 +619,7 @@ __global__ void __launch_bounds__(kThreads) k_detj_minmax(Grid g, const float* _
                 atomicMax(&bhi, ordered_int(fhi));
             }
             if (t.ok && !(dlo > flo && dhi < fhi)) {
-                double F[3][3];
-#pragma unroll
-                for (int c = 0; c < 3; ++c)
-#pragma unroll
-                    for (int a = 0; a < 3; ++a) F[c][a] = e[c][a];
-#pragma unroll
-                for (int c = 0; c < 3; ++c) F[c][c] += 1.0;
-                const double d = F[0][0] * (F[1][1] * F[2][2] - F[1][2] * F[2][1]) -
-                                 F[0][1] * (F[1][0] * F[2][2] - F[1][2] * F[2][0]) +
-                                 F[0][2] * (F[1][0] * F[2][1] - F[1][1] * F[2][0]);
+                const double d = det_exact(e);
                 lo = min_nan(lo, d);  // a NaN propagates to both extrema
                 hi = max_nan(hi, d);
             }

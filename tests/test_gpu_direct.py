@@ -1,0 +1,112 @@
+"""GPU tests of single kernels on inputs that the entry points cannot give them
+directly (direct_calls.cu, linked against libclaire.so)."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+import __graft_entry__ as entry
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+@pytest.fixture(scope="module")
+def direct(tmp_path_factory):
+    entry.build()
+    from paper_2209_08189_gb300 import build
+    so = str(tmp_path_factory.mktemp("direct") / "direct_calls.so")
+    cmd = [os.path.join(build._cuda_home(), "bin", "nvcc"), *build.ARCH, "-O1", "-std=c++17", "-Xcompiler", "-fPIC",
+           "-shared", "-cudart", "shared", "--expt-relaxed-constexpr", "-I" + build.INCLUDE, "-I" + build.CSRC,
+           os.path.join(ROOT, "tests", "direct_calls.cu"), build.LIB, "-Xlinker", "-rpath=" + build.PKG, "-o", so]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    assert res.returncode == 0, res.stdout + res.stderr
+    return ctypes.CDLL(so)
+
+
+def _ptr(t):
+    return ctypes.c_void_p(t.data_ptr())
+
+
+def _differences(n, u):
+    """The nine FP32 differences of u, as the FD8 gradient forms them."""
+    from paper_2209_08189_gb300 import claire
+    ctx = claire.Context(n, 1e-2, 4, stream=torch.cuda.current_stream().cuda_stream, kernels_only=1)
+    out = np.empty((3, 3) + n)
+    for c in range(3):
+        g = torch.empty((3,) + n, device="cuda")
+        ctx.fd8_grad(u[c], g)
+        out[c] = g.cpu().numpy()
+    ctx.close()
+    return out
+
+
+def _det(e):
+    F = e + np.eye(3).reshape(3, 3, 1, 1, 1)
+    return (F[0, 0] * (F[1, 1] * F[2, 2] - F[1, 2] * F[2, 1]) - F[0, 1] * (F[1, 0] * F[2, 2] - F[1, 2] * F[2, 0]) +
+            F[0, 2] * (F[1, 0] * F[2, 1] - F[1, 1] * F[2, 0]))
+
+
+def _plateau(n, slope):
+    """Periodic function with the slope `slope` on a third of the period."""
+    x = np.arange(n) * 2 * np.pi / n
+    ramp = np.clip((np.abs(x - np.pi) - np.pi / 3) / (2 * np.pi / 3), 0, 1)
+    bump = ramp ** 3 * (10 - 15 * ramp + 6 * ramp ** 2)     # 0 on the plateau
+    d = slope * (1 - bump / bump.mean())
+    u = np.cumsum(d + np.roll(d, 1)) * np.pi / n
+    return u - u[n // 2]
+
+
+@pytest.mark.parametrize("size", [10.0, 1.0, 1e-1, 1e-2, 1e-3, 3e-6, 1e-12])
+def test_det_bounds_hold(direct, size):
+    """det(I + e) in FP64 lies between its FP32 bounds for entries of I + e up to
+    `size`, down to maps that compress a thousandfold and to products that
+    underflow, and the bounds are no wider than stated (8e-6 m^3 and its rounding)."""
+    n, rng = 1 << 18, np.random.default_rng(7)
+    ih = np.array([64, 90, 52], dtype=np.float32) / np.float32(2 * np.pi)
+    F = rng.uniform(-size, size, (3, 3, n)) * 10.0 ** rng.uniform(-1, 0, (3, 3, n))
+    diff = ((F - np.eye(3)[:, :, None]) / ih[None, :, None]).astype(np.float32)
+    d, i = torch.from_numpy(diff).cuda(), torch.from_numpy(ih).cuda()
+    lo, hi = torch.empty(n, device="cuda"), torch.empty(n, device="cuda")
+    det = torch.empty(n, device="cuda", dtype=torch.float64)
+    assert direct.direct_det_bounds(_ptr(d), _ptr(i), n, _ptr(lo), _ptr(det), _ptr(hi)) == 0
+    assert bool((lo.double() <= det).all()) and bool((det <= hi.double()).all())
+    assert float((hi - lo).max()) <= 1.1e-5 * max(size, 2e-7) ** 3 + 3e-36
+    e = (diff * ih[None, :, None]).astype(np.float64)
+    assert np.abs(det.cpu().numpy() - _det(e.reshape(3, 3, 1, 1, n)).ravel()).max() <= 1e-14 * max(size, 2e-7) ** 3 + 1e-300
+
+
+@pytest.mark.parametrize("compression", [1e-1, 1e-2])
+def test_detj_extrema_of_a_compressing_map(direct, compression):
+    """The FP32 filter of the determinant never loses an extremum: where the map
+    compresses by 1 / compression on every axis the entries of I + grad u are
+    small and thousands of points nearly tie.  The extrema are those of the
+    determinants in FP64 of the same FP32 differences, up to the rounding of the
+    FP64 formula (1e-14 of six products of the largest entries)."""
+    n = (48, 40, 64)
+    for seed in range(4):
+        rng = np.random.default_rng(seed)
+        ax = [_plateau(s, compression - 1.0) for s in n]
+        u = np.stack([np.broadcast_to(ax[c].reshape([-1 if a == c else 1 for a in range(3)]), n) for c in range(3)])
+        u = u + rng.uniform(-1, 1, u.shape) * 2e-8
+        d = torch.from_numpy(u.astype(np.float32)).cuda()
+        det = _det(_differences(n, d))
+        assert (det < 2 * det.min()).sum() > 1000  # near ties
+        out = (ctypes.c_double * 2)()
+        assert direct.direct_detj(*n, _ptr(d), 608, out) == 0
+        assert abs(out[0] - det.min()) <= 1e-14 * 6 * (2 * compression) ** 3
+        assert abs(out[1] - det.max()) <= 1e-14 * 6 * 3.0 ** 3
+
+
+@pytest.mark.parametrize("where", [(0, 0, 0), (47, 39, 63), (20, 17, 31)])
+def test_detj_keeps_a_nan(direct, where):
+    n = (48, 40, 64)
+    u = torch.zeros((3,) + n, device="cuda")
+    u[1][where] = float("nan")
+    out = (ctypes.c_double * 2)()
+    assert direct.direct_detj(*n, _ptr(u), 608, out) == 0
+    assert np.isnan(out[0]) and np.isnan(out[1])
