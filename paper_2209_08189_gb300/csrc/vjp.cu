@@ -537,6 +537,7 @@ __device__ __forceinline__ float fixed_value(long long a, const FixedScale& s, i
     f2 = s.down1 * (s.down0 * (f2 * pe));
     if (!accumulate) return mult * (f1 + f2);
     const float t = __fadd_rn(old, f1);
+    if (!(fabsf(t) < INFINITY)) return mult * t;  // the error terms below would make a NaN of an infinity
     const float bb = __fsub_rn(t, old);
     const float err = __fadd_rn(__fsub_rn(old, __fsub_rn(t, bb)), __fsub_rn(f1, bb));
     return mult * __fadd_rn(t, __fadd_rn(err, f2));

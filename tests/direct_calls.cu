@@ -57,3 +57,12 @@ extern "C" int direct_detj(int n1, int n2, int n3, const float* u, int blocks, d
     cudaFree(dev);
     return e;
 }
+
+// out = mult ((accumulate ? out : 0) + acc / scale(maxabs)); all arrays on the device.
+extern "C" int direct_fixed_to_float(unsigned long long* acc, const double* maxabs, int accumulate, float mult, float* out,
+                                     long long n)
+{
+    launch_fixed_to_float(acc, maxabs, accumulate, mult, out, static_cast<size_t>(n), nullptr);
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? cudaDeviceSynchronize() : e;
+}

@@ -110,3 +110,25 @@ def test_detj_keeps_a_nan(direct, where):
     out = (ctypes.c_double * 2)()
     assert direct.direct_detj(*n, _ptr(u), 608, out) == 0
     assert np.isnan(out[0]) and np.isnan(out[1])
+
+
+def _fixed_to_float(direct, acc, maxabs, out, mult=1.0, accumulate=True):
+    a = torch.from_numpy(np.asarray(acc, dtype=np.int64)).cuda()
+    m = torch.tensor([maxabs], dtype=torch.float64, device="cuda")
+    o = torch.from_numpy(np.asarray(out, dtype=np.float32)).cuda()
+    assert direct.direct_fixed_to_float(_ptr(a), _ptr(m), int(accumulate), ctypes.c_float(mult), _ptr(o),
+                                        ctypes.c_longlong(o.numel())) == 0
+    assert int(a.abs().max()) == 0  # cleared for the next scatter
+    return o.cpu().numpy()
+
+
+def test_fixed_point_sum_onto_infinities(direct):
+    """Added to an infinity the sum is that infinity, as it is in FP64; a NaN stays a
+    NaN, and a finite sum beyond the FP32 range becomes an infinity.  Seven values:
+    the vector path and the tail."""
+    big = np.float32(3e38)
+    old = [np.inf, -np.inf, np.nan, big, 1.0, np.inf, -big]
+    acc = [1 << 40, 1 << 40, 5, 1 << 47, 1 << 20, 0, -(1 << 47)]
+    got = _fixed_to_float(direct, acc, 2.5e38, old, mult=2.0)  # 2^47 stands for 2^127
+    assert got[0] == np.inf and got[1] == -np.inf and np.isnan(got[2]) and got[3] == np.inf
+    assert got[5] == np.inf and got[6] == -np.inf
