@@ -497,50 +497,63 @@ __global__ void __launch_bounds__(kThreads, 4) k_scatter_tiled(Grid g, const flo
     }
 }
 
-// The 64-bit integer a as (f1 + f2) 2^e up to 2^-48 of it: f1 its leading 24 bits, f2
-// the next 32 rounded to FP32.  (The 64-bit conversion instructions run on the
+// The 64-bit integer a as (f1 + f2 + f3) 2^e, exactly: f1 its leading 24 bits, f2 the
+// next 24, f3 the last 16.  (The 64-bit conversion instructions run on the
 // FP64 pipe, at some 300 cycles per warp and SM: at 128^3 they alone were 60 us
 // of the 69 us of this kernel.)
-__device__ __forceinline__ void ll_split(long long a, float& f1, float& f2, int& e)
+__device__ __forceinline__ void ll_split(long long a, float& f1, float& f2, float& f3, int& e)
 {
     const unsigned long long m = static_cast<unsigned long long>(a < 0 ? -a : a);
     if (m == 0) {
-        f1 = f2 = 0.0f;
+        f1 = f2 = f3 = 0.0f;
         e = 0;
         return;
     }
     const int z = __clzll(static_cast<long long>(m));
     const unsigned long long n = m << z;  // top bit set
-    f1 = static_cast<float>(static_cast<unsigned>(n >> 40));                                    // exact
-    f2 = static_cast<float>(static_cast<unsigned>(n >> 8)) * 2.3283064365386963e-10f;  // 2^-32
+    f1 = static_cast<float>(static_cast<unsigned>(n >> 40));
+    f2 = static_cast<float>(static_cast<unsigned>(n >> 16) & 0xffffffu) * 5.9604644775390625e-8f;  // 2^-24
+    f3 = static_cast<float>(static_cast<unsigned>(n) & 0xffffu) * 9.094947017729282379e-13f;       // 2^-40
     if (a < 0) {
         f1 = -f1;
         f2 = -f2;
+        f3 = -f3;
     }
     e = 40 - z;
 }
 
+// a + b as s + r, exactly.
+__device__ __forceinline__ void two_sum(float a, float b, float& s, float& r)
+{
+    s = __fadd_rn(a, b);
+    const float bb = __fsub_rn(s, a);
+    r = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+}
+
 // out = mult ((accumulate ? out : 0) + acc / scale); acc is cleared for reuse.
 // Bound: HBM (20 B per point, 24 when accumulating).  The scaling is by powers of
-// two; the sum with out is formed with its rounding error (two-sum), so that
-// the result is rounded to FP32 once, up to 2^-48 of the terms.  Four points
-// per thread when the arrays are 16-byte aligned.  128^3: 10 us; 81 us with
-// 64-bit conversions and FP64 sums.
+// two, and the sum with out carries its rounding errors (two-sums), so the 64
+// bits enter it whole; it is rounded to FP32, then the product with mult.  Four
+// points per thread when the arrays are 16-byte aligned.  128^3: 10 us; 81 us
+// with 64-bit conversions and FP64 sums.
 __device__ __forceinline__ float fixed_value(long long a, const FixedScale& s, int accumulate, float mult, float old)
 {
     if (s.kind == 2) return __int_as_float(0x7fffffff);  // non-finite cotangent: propagate NaN
-    float f1, f2;
+    float f1, f2, f3;
     int e;
-    ll_split(a, f1, f2, e);
+    ll_split(a, f1, f2, f3, e);
     const float pe = pow2f(e);  // -23 <= e <= 40
     f1 = s.down1 * (s.down0 * (f1 * pe));
     f2 = s.down1 * (s.down0 * (f2 * pe));
-    if (!accumulate) return mult * (f1 + f2);
-    const float t = __fadd_rn(old, f1);
-    if (!(fabsf(t) < INFINITY)) return mult * t;  // the error terms below would make a NaN of an infinity
-    const float bb = __fsub_rn(t, old);
-    const float err = __fadd_rn(__fsub_rn(old, __fsub_rn(t, bb)), __fsub_rn(f1, bb));
-    return mult * __fadd_rn(t, __fadd_rn(err, f2));
+    f3 = s.down1 * (s.down0 * (f3 * pe));
+    if (!accumulate) return mult * (f1 + (f2 + f3));
+    float t, u, v, w, hi, lo;
+    two_sum(old, f1, t, u);
+    if (!(fabsf(t) < INFINITY)) return mult * t;  // the error terms would make a NaN of an infinity
+    two_sum(u, f2, v, w);
+    two_sum(t, v, hi, lo);
+    if (!(fabsf(hi) < INFINITY)) return mult * hi;
+    return mult * __fadd_rn(hi, __fadd_rn(lo, __fadd_rn(w, f3)));
 }
 
 __global__ void __launch_bounds__(kThreads) k_fixed_to_float(unsigned long long* __restrict__ acc,

@@ -132,3 +132,23 @@ def test_fixed_point_sum_onto_infinities(direct):
     got = _fixed_to_float(direct, acc, 2.5e38, old, mult=2.0)  # 2^47 stands for 2^127
     assert got[0] == np.inf and got[1] == -np.inf and np.isnan(got[2]) and got[3] == np.inf
     assert got[5] == np.inf and got[6] == -np.inf
+
+
+@pytest.mark.parametrize("n", [1, 6, 4096])
+def test_fixed_point_sum_uses_all_bits(direct, n):
+    """acc / scale enters the sum with all 64 bits.  Added to minus its FP32 rounding
+    the rest remains, held to 2^-22 of it (three FP32 roundings), however many
+    bits of the sum cancel; plain, it is the FP32 rounding (2^-23, for ties that
+    an intermediate rounding makes)."""
+    rng = np.random.default_rng(3)
+    acc = [int(rng.integers(1, 1 << 62)) >> int(rng.integers(0, 62)) for _ in range(n)]
+    acc = [((a >> 40) << 40 | (a & ((1 << int(rng.integers(1, 33))) - 1))) or 1 for a in acc]  # low words after zeros
+    acc = [a if rng.random() < 0.5 else -a for a in acc]
+    maxabs = 1.0  # 2^47 stands for 1
+    val = [a / 2 ** 47 for a in acc]  # a Python division is correctly rounded
+    plain = _fixed_to_float(direct, acc, maxabs, np.zeros(n), accumulate=False)
+    assert np.all(np.abs(plain - np.array(val)) <= 2.0 ** -23 * np.abs(val))
+    got = _fixed_to_float(direct, acc, maxabs, -plain)
+    for a, p, g in zip(acc, plain, got):
+        rest = a - int(float(p) * 2 ** 47)  # exact: p is an FP32 value of at least 2^-47
+        assert abs(float(g) * 2 ** 47 - rest) <= 2.0 ** -22 * abs(rest), (a, p, g)
