@@ -17,7 +17,13 @@ struct Grid {
     uint32_t N;           // n1 * n2 * n3 (< 2^31)
     float h1, h2, h3;     // 2 pi / n_c
     float ih1, ih2, ih3;  // n_c / (2 pi)
+    // trilinear FP32 tiles take the wide box (sl_tiled.cuh): displacements so large
+    // that many tiles would not fit the narrow one; no value depends on it
+    int wide = 0;
 };
+
+// Largest displacement per step, in cells, with the narrow box (figures at box_cap).
+constexpr double kWideCfl = 14.0;
 
 __host__ __device__ __forceinline__ int wrap_index(int x, int n)
 {

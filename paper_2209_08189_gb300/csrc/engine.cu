@@ -892,6 +892,21 @@ claire_status precond(claire_ctx* c, const float* r, float* z)
     return spectral(c, r, z, c->o.grad_form == 1 ? SPEC_AINV : SPEC_INV);
 }
 
+// max |v(x)|^2 into result slot 7 (no sync), and the CFL number that it gives.
+claire_status maxnorm_async(claire_ctx* c, const float* v)
+{
+    KTimer t(c, KK_REDUCE, 12.0 * c->N, 0);
+    launch_maxnorm3(v, c->N, reduction(c, 7, c->N / 8), c->stream);
+    CL_LAUNCHED(c);
+    return CLAIRE_OK;
+}
+
+double cfl_of_maxnorm(const claire_ctx* c)
+{
+    const double hmin = std::min(c->grid.h1, std::min(c->grid.h2, c->grid.h3));
+    return std::sqrt(c->hres[7]) * c->dt / hmin;
+}
+
 // J(v) for a trial v (device, 3N); uses z (displacement), l0/l1.  alpha (the line
 // search): v is the iterate plus alpha times the PCG solution.
 // With into_state the characteristic and the states m^1..m^nt are written to
@@ -916,12 +931,17 @@ claire_status objective_at(claire_ctx* c, const float* v, double* J, double* mis
         std::swap(a, b);
     }
     CL_TRY(reg_energy(c, v, c->vh_on ? alpha : nullptr, 0));
+    // the trilinear boxes follow the iterate of a registration, which was screened
+    // at its start only
+    const bool track = into_state && c->o.interp == CLAIRE_INTERP_LINEAR;
+    if (track) CL_TRY(maxnorm_async(c, v));
     {
         KTimer t(c, KK_REDUCE, 8.0 * N, 0);
         launch_sqdiff(src, c->m1, N, c->sto, reduction(c, 1, N / 4, 0.5 * c->hvol), c->stream);
         CL_LAUNCHED(c);
     }
     CL_TRY(sync_scalars(c));
+    if (track) c->grid.wide = cfl_of_maxnorm(c) > kWideCfl;  // false for a NaN, which J reports
     if (mis) *mis = c->hres[1];
     if (J) *J = c->hres[0] + c->hres[1];
     if (!std::isfinite(c->hres[0] + c->hres[1]))
@@ -959,14 +979,9 @@ claire_status detj_of(claire_ctx* c, const float* v, double* lo, double* hi)
 
 claire_status cfl_of(claire_ctx* c, const float* v, double* cfl)
 {
-    {
-        KTimer t(c, KK_REDUCE, 12.0 * c->N, 0);
-        launch_maxnorm3(v, c->N, reduction(c, 7, c->N / 8), c->stream);
-        CL_LAUNCHED(c);
-    }
+    CL_TRY(maxnorm_async(c, v));
     CL_TRY(sync_scalars(c));
-    const double hmin = std::min(c->grid.h1, std::min(c->grid.h2, c->grid.h3));
-    *cfl = std::sqrt(c->hres[7]) * c->dt / hmin;
+    *cfl = cfl_of_maxnorm(c);
     return CLAIRE_OK;
 }
 
@@ -977,6 +992,7 @@ claire_status screen_velocity(claire_ctx* c, const float* v)
     double cfl;
     CL_TRY(cfl_of(c, v, &cfl));
     if (!std::isfinite(cfl)) return fail(c, CLAIRE_ENONFINITE, "non-finite velocity");
+    c->grid.wide = cfl > kWideCfl;
     return CLAIRE_OK;
 }
 

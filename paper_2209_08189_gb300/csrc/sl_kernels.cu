@@ -128,10 +128,10 @@ template <int ORDER, bool FULL, bool TBW>
 void launch_backtrace_tiled_as(const Grid& g, const float* v, const float* vc, float dt, float sign, float* d,
                                int4* tb, cudaStream_t st)
 {
-    if (tiled_smem_bytes<ORDER>() > 48 * 1024)
+    if (tiled_smem_bytes<ORDER>(g) > 48 * 1024)
         cudaFuncSetAttribute(k_backtrace_tiled<ORDER, FULL, TBW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(tiled_smem_bytes<ORDER>()));
-    k_backtrace_tiled<ORDER, FULL, TBW><<<tiled_grid(g), kTileThreads, tiled_smem_bytes<ORDER>(), st>>>(g, v, vc, dt, sign,
+                             static_cast<int>(tiled_smem_bytes<ORDER>(g)));
+    k_backtrace_tiled<ORDER, FULL, TBW><<<tiled_grid(g), kTileThreads, tiled_smem_bytes<ORDER>(g), st>>>(g, v, vc, dt, sign,
                                                                                               d, tb);
 }
 
@@ -658,10 +658,10 @@ void launch_interp(const Grid& g, int order, const void* f, const float* d, void
 template <int ORDER, bool FULL, bool MAP>
 void launch_fields_tiles(const Grid& g, const float* f, int nf, const float* d, float* out, cudaStream_t st)
 {
-    if (tiled_smem_bytes<ORDER>() > 48 * 1024)
+    if (tiled_smem_bytes<ORDER>(g) > 48 * 1024)
         cudaFuncSetAttribute(k_gather_tiled_fields<ORDER, FULL, MAP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(tiled_smem_bytes<ORDER>()));
-    k_gather_tiled_fields<ORDER, FULL, MAP><<<tiled_grid(g), kTileThreads, tiled_smem_bytes<ORDER>(), st>>>(g, f, nf, d, out);
+                             static_cast<int>(tiled_smem_bytes<ORDER>(g)));
+    k_gather_tiled_fields<ORDER, FULL, MAP><<<tiled_grid(g), kTileThreads, tiled_smem_bytes<ORDER>(g), st>>>(g, f, nf, d, out);
 }
 
 template <int ORDER, bool MAP>

@@ -55,11 +55,21 @@ constexpr int kBoxCapFloats = CLAIRE_BOX_CAP;
 // transport of eight steps 1277 -> 1130 us (five: 1205, seven: 1122 but 5 %
 // slower adjoint steps).  16-bit fields, whose boxes also hold the staging copy,
 // lose 2 % with six and keep four.
+// The narrow box holds tiles whose cells spread over 5 nodes, the wide one 6, and a
+// tile that fits neither costs most where six CTAs leave the L1 28 KB.  So large
+// displacements (Grid::wide, set by the context where |v| dt is more than kWideCfl
+// cells somewhere) take the wide box.  Four steps at 512^3, modes up to 24, share
+// of tiles that overflow and time, narrow / wide: CFL 12: 13 % 5.3 ms / 1.4 % 5.6;
+// CFL 16: 42 % 7.6 / 14 % 6.4; CFL 24: 74 % 15.2 / 54 % 8.5; CFL 41: 91 % 29.4 /
+// 83 % 11.6.  Modes up to 6, CFL 12: 0.3 % 4.6 / 0 5.3; CFL 24: 19 % 5.7 / 7 % 5.9.
+// 320^3, up to 24, CFL 10: 16 % 1.44 / 1 % 1.45; CFL 15: 69 % 3.3 / 32 % 1.9.
+// Half boxes of 16 columns for the tiles that overflow: 1.3 to 1.9 times the
+// wide box's time.
 constexpr int kBoxCapLinear = 9216;
 template <int ORDER, int ES = 4>
-__host__ __device__ constexpr int box_cap()
+__host__ __device__ __forceinline__ int box_cap(const Grid& g)
 {
-    return ORDER == 1 && ES == 4 && kBoxCapLinear < kBoxCapFloats ? kBoxCapLinear : kBoxCapFloats;
+    return ORDER == 1 && ES == 4 && !g.wide ? kBoxCapLinear : kBoxCapFloats;
 }
 template <int ORDER, int ES = 4>
 constexpr int tile_min_blocks()
@@ -87,13 +97,31 @@ __device__ __forceinline__ void axis_weights(float t, float w[4])
 // Direct global-memory gather for tiles whose departure box does not fit
 // (kept out of line so that it does not add to the register budget of the
 // shared-memory path).
+// Trilinear: the operations of tile_eval in its order, so that a value does not
+// depend on whether the tile's box fits (Grid::wide chooses the box by speed alone).
 template <int ORDER, class S>
 __device__ __noinline__ float gather_global(const Grid g, const S* __restrict__ f, int i, int j,
                                             int k, float d1, float d2, float d3)
 {
     Stencil<ORDER> s;
     s.build(g, i, j, k, d1, d2, d3);
-    return s.template eval<S>(f);
+    if constexpr (ORDER == 1) {
+        float val = 0.0f;
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+            float acc[2];
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                const S* row = f + s.a1.idx[a] + s.a2.idx[b];
+                acc[b] = __fmul_rn(__fmul_rn(s.a2.w[b], s.a3.w[0]), ldf<S>(row + s.a3.idx[0]));
+                acc[b] = __fmaf_rn(__fmul_rn(s.a2.w[b], s.a3.w[1]), ldf<S>(row + s.a3.idx[1]), acc[b]);
+            }
+            val = fmaf(s.a1.w[a], __fadd_rn(acc[0], acc[1]), val);
+        }
+        return val;
+    } else {
+        return s.template eval<S>(f);
+    }
 }
 
 // ---- building blocks of the tiled gathers ----
@@ -163,7 +191,7 @@ __host__ __device__ __forceinline__ void box_geometry(const Grid& g, int a1, int
     const unsigned s3 = (e3 + 31) & ~31u;  // bank-aligned row stride
     // FP32 box plus, for 16-bit storage, the staging copy (half its size)
     fits = fits && e3 <= n3 &&
-           static_cast<unsigned long long>(e1 * e2) * s3 * (ES == 2 ? 3 : 2) <= 2ull * box_cap<ORDER, ES>();
+           static_cast<unsigned long long>(e1 * e2) * s3 * (ES == 2 ? 3 : 2) <= 2ull * box_cap<ORDER, ES>(g);
     par[0] = fits ? static_cast<int>(static_cast<unsigned>(a1) - OFF) : 0;
     par[1] = fits ? static_cast<int>(static_cast<unsigned>(a2) - OFF) : 0;
     par[2] = fits ? static_cast<int>(o3) : 0;
@@ -759,18 +787,18 @@ inline dim3 tiled_grid(const Grid& g)
 }
 
 template <int ORDER, int ES = 4>
-constexpr size_t tiled_smem_bytes()
+size_t tiled_smem_bytes(const Grid& g)
 {
-    return box_cap<ORDER, ES>() * sizeof(float);
+    return box_cap<ORDER, ES>(g) * sizeof(float);
 }
 
 template <int ORDER, class Epi, class S, bool FULL, bool TB>
 inline void launch_tiled_as(const Grid& g, const S* f, const float* d, const Epi& e, cudaStream_t st, const int4* tb)
 {
-    if (tiled_smem_bytes<ORDER, sizeof(S)>() > 48 * 1024)
+    if (tiled_smem_bytes<ORDER, sizeof(S)>(g) > 48 * 1024)
         cudaFuncSetAttribute(k_gather_tiled<ORDER, Epi, S, FULL, TB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(tiled_smem_bytes<ORDER, sizeof(S)>()));
-    k_gather_tiled<ORDER, Epi, S, FULL, TB><<<tiled_grid(g), kTileThreads, tiled_smem_bytes<ORDER, sizeof(S)>(), st>>>(g, f, d, e, tb);
+                             static_cast<int>(tiled_smem_bytes<ORDER, sizeof(S)>(g)));
+    k_gather_tiled<ORDER, Epi, S, FULL, TB><<<tiled_grid(g), kTileThreads, tiled_smem_bytes<ORDER, sizeof(S)>(g), st>>>(g, f, d, e, tb);
 }
 
 template <int ORDER, class Epi, class S>

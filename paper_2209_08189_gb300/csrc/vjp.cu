@@ -702,12 +702,12 @@ void launch_grad_accum_as(const Grid& g, const float* m, const float* d, const f
                           cudaStream_t st)
 {
     if (first)
-        k_grad_accum<ORDER, FULL, true><<<tiled_grid(g), kTileThreads, tiled_smem_bytes<ORDER>(), st>>>(g, m, d, mbar, dbar);
+        k_grad_accum<ORDER, FULL, true><<<tiled_grid(g), kTileThreads, tiled_smem_bytes<ORDER>(g), st>>>(g, m, d, mbar, dbar);
     else
-        k_grad_accum<ORDER, FULL, false><<<tiled_grid(g), kTileThreads, tiled_smem_bytes<ORDER>(), st>>>(g, m, d, mbar, dbar);
+        k_grad_accum<ORDER, FULL, false><<<tiled_grid(g), kTileThreads, tiled_smem_bytes<ORDER>(g), st>>>(g, m, d, mbar, dbar);
 }
 
-static_assert(tiled_smem_bytes<3>() <= 48 * 1024, "the kernels of this file launch with the default shared-memory limit");
+static_assert(kBoxCapFloats * sizeof(float) <= 48 * 1024, "the kernels of this file launch with the default shared-memory limit");
 
 void launch_grad_accum(const Grid& g, int order, const float* m, const float* d, const float* mbar, float* dbar,
                        bool first, cudaStream_t st)
@@ -757,10 +757,10 @@ void launch_predictor_as(const Grid& g, const float* v, const float* vc, float d
                          float* Ubar, cudaStream_t st)
 {
     if (tiles_cover_grid(g))
-        k_predictor_terms<ORDER, true><<<tiled_grid(g), kTileThreads, tiled_smem_bytes<ORDER>(), st>>>(g, v, vc, dt, dbar, ubar,
+        k_predictor_terms<ORDER, true><<<tiled_grid(g), kTileThreads, tiled_smem_bytes<ORDER>(g), st>>>(g, v, vc, dt, dbar, ubar,
                                                                                              Ubar);
     else
-        k_predictor_terms<ORDER, false><<<tiled_grid(g), kTileThreads, tiled_smem_bytes<ORDER>(), st>>>(g, v, vc, dt, dbar, ubar,
+        k_predictor_terms<ORDER, false><<<tiled_grid(g), kTileThreads, tiled_smem_bytes<ORDER>(g), st>>>(g, v, vc, dt, dbar, ubar,
                                                                                               Ubar);
 }
 

@@ -210,3 +210,34 @@ def test_results_formed_in_the_callers_array(nt):
                 assert torch.equal(inp, x.reshape(-1)), name
     ctx.close()
 
+
+
+@pytest.mark.parametrize("n", [(64, 64, 64), (70, 44, 104)])
+def test_trilinear_values_do_not_depend_on_the_box(n):
+    """Trilinear tiles take a wider box where the displacement is large, and go to
+    global memory where no box holds them.  The value at a point is the same bits on
+    every path: a displacement below the line, one above it whose tiles fit, and
+    tiles made to overflow by one far point each, whose other points are compared."""
+    from paper_2209_08189_gb300 import claire
+    rng = np.random.default_rng(2)
+    f = _dev(rng.standard_normal(n))
+    far = np.zeros((3,) + n, dtype=np.float32)
+    far[:, ::4, ::8, ::32] = 40.0  # the first point of every tile
+    near = rng.uniform(-1.5, 1.5, (3,) + n).astype(np.float32)
+    out = {}
+    for vmax in (0.5, 20.0):  # below and above 14 cells per step on these grids
+        v = synth.mode_velocity(n, seed=3, vmax=vmax, kmax=1).astype(np.float32)
+        ctx = _ctx(n, interp=claire.INTERP_LINEAR)
+        d = torch.empty((3,) + n, device="cuda")
+        ctx.backtrace(_dev(v), d)
+        for name, disp in (("near", near), ("far", near + far)):
+            claire.claire_gather_fallback_tiles(reset=True)
+            o = torch.empty(n, device="cuda")
+            ctx.interp(f, _dev(disp), o, claire.INTERP_LINEAR)
+            tiles = -(-n[0] // 4) * -(-n[1] // 8) * -(-n[2] // 32)
+            assert claire.claire_gather_fallback_tiles() == (tiles if name == "far" else 0)
+            out[name, vmax] = o.cpu().numpy()
+        ctx.close()
+    same = far[0] == 0
+    for key in out:
+        assert np.array_equal(out[key][same], out["near", 0.5][same]), key
