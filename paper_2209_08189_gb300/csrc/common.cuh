@@ -23,7 +23,7 @@ struct Grid {
 };
 
 // Largest displacement per step, in cells, with the narrow box (figures at box_cap).
-constexpr double kWideCfl = 14.0;
+constexpr double kWideCfl = 12.0;
 
 __host__ __device__ __forceinline__ int wrap_index(int x, int n)
 {

@@ -655,22 +655,29 @@ void launch_interp(const Grid& g, int order, const void* f, const float* d, void
     });
 }
 
-template <int ORDER, bool FULL, bool MAP>
+template <int ORDER, bool FULL, bool MAP, bool WIDE>
 void launch_fields_tiles(const Grid& g, const float* f, int nf, const float* d, float* out, cudaStream_t st)
 {
-    if (tiled_smem_bytes<ORDER>(g) > 48 * 1024)
-        cudaFuncSetAttribute(k_gather_tiled_fields<ORDER, FULL, MAP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(tiled_smem_bytes<ORDER>(g)));
-    k_gather_tiled_fields<ORDER, FULL, MAP><<<tiled_grid(g), kTileThreads, tiled_smem_bytes<ORDER>(g), st>>>(g, f, nf, d, out);
+    const size_t smem = tiled_smem_bytes<ORDER>(g);
+    if (smem > 48 * 1024)
+        cudaFuncSetAttribute(k_gather_tiled_fields<ORDER, FULL, MAP, WIDE>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    k_gather_tiled_fields<ORDER, FULL, MAP, WIDE><<<tiled_grid(g), kTileThreads, smem, st>>>(g, f, nf, d, out);
 }
 
 template <int ORDER, bool MAP>
 void launch_fields_as(const Grid& g, const float* f, int nf, const float* d, float* out, cudaStream_t st)
 {
-    if (tiles_cover_grid(g))
-        launch_fields_tiles<ORDER, true, MAP>(g, f, nf, d, out, st);
-    else
-        launch_fields_tiles<ORDER, false, MAP>(g, f, nf, d, out, st);
+    const bool full = tiles_cover_grid(g);
+    if constexpr (ORDER == 1) {
+        if (g.wide) {
+            full ? launch_fields_tiles<ORDER, true, MAP, true>(g, f, nf, d, out, st)
+                 : launch_fields_tiles<ORDER, false, MAP, true>(g, f, nf, d, out, st);
+            return;
+        }
+    }
+    full ? launch_fields_tiles<ORDER, true, MAP, false>(g, f, nf, d, out, st)
+         : launch_fields_tiles<ORDER, false, MAP, false>(g, f, nf, d, out, st);
 }
 
 void launch_interp_fields(const Grid& g, int order, const float* f, int nf, const float* d, float* out,

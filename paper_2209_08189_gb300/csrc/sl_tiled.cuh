@@ -709,8 +709,12 @@ __global__ void __launch_bounds__(kTileThreads, tile_min_blocks<ORDER, sizeof(S)
 // (X - x) in physical units, nf = 3.  It reads its 192 stencil values from the
 // box as the gathers do; the per-point kernel it replaced fetched them through
 // L1 (256^3, CFL 3.4: 0.80 ms per step; from the box 0.56 ms).
-template <int ORDER, bool FULL, bool MAP = false>
-__global__ void __launch_bounds__(kTileThreads, tile_min_blocks<ORDER>())
+// WIDE: the registers of four CTAs per SM, for the wide box (trilinear; the narrow
+// box has the registers of six).  With the narrow kernel's registers tiles that
+// overflow took 1.25 times as long (256^3, three fields, 30 cells per step: 659 us
+// against 540); small displacements: 214 us narrow, 239 wide.
+template <int ORDER, bool FULL, bool MAP, bool WIDE>
+__global__ void __launch_bounds__(kTileThreads, WIDE ? CLAIRE_TILE_MIN_BLOCKS : tile_min_blocks<ORDER>())
     k_gather_tiled_fields(Grid g, const float* __restrict__ f, int nf, const float* __restrict__ d,
                           float* __restrict__ out)
 {

@@ -225,7 +225,7 @@ def test_trilinear_values_do_not_depend_on_the_box(n):
     far[:, ::4, ::8, ::32] = 40.0  # the first point of every tile
     near = rng.uniform(-1.5, 1.5, (3,) + n).astype(np.float32)
     out = {}
-    for vmax in (0.5, 20.0):  # below and above 14 cells per step on these grids
+    for vmax in (0.5, 20.0):  # below and above 12 cells per step on these grids
         v = synth.mode_velocity(n, seed=3, vmax=vmax, kmax=1).astype(np.float32)
         ctx = _ctx(n, interp=claire.INTERP_LINEAR)
         d = torch.empty((3,) + n, device="cuda")
