@@ -289,7 +289,10 @@ constexpr float kFixMagic = 12582912.0f;             // 1.5 2^23, bits 0x4b40000
 constexpr float kFixDown = 7.450580596923828125e-9f;  // 2^-27
 
 // The term as two words, its h biased by the magic's bits: term + kFixBias 2^32
-// mod 2^64 (the bias 0x4b400000 2^27 has only a high word).
+// mod 2^64 (the bias 0x4b400000 2^27 has only a high word).  The carries are in PTX
+// here and in add_high: written in C++ (64-bit sum, old + lo < old) the bits are the
+// same and the reverse pass takes longer (128^3 2.23 ms against 2.16, 182 x 218 x 182
+// 6.8 against 6.45).
 constexpr unsigned kFixBias = 0x4b400000u >> 5;
 
 struct FixedTerm {
