@@ -1137,10 +1137,9 @@ claire_status tl_prepare(claire_ctx* c)
     return CLAIRE_OK;
 }
 
-// zf = P^{-1} (rscale rf) on fine half spectra, rscale rf the scaled residual; *rz = <rf, zf>, *ro = <rf, zold>
-// (0 when zold is null); *its = inner PCG iterations.
-claire_status tl_apply(claire_ctx* c, const cufftComplex* rf, float rscale, cufftComplex* zf,
-                       const cufftComplex* zold, double* rz, double* ro, int* its)
+// zf = P^{-1} (rscale rf) on fine half spectra, rscale rf the scaled residual; *rz = <rf, zf>; *its = inner PCG
+// iterations.
+claire_status tl_apply(claire_ctx* c, const cufftComplex* rf, float rscale, cufftComplex* zf, double* rz, int* its)
 {
     TwoLevel* t = c->tl2;
     const SpectralOp op = c->o.grad_form == 1 ? SPEC_AINV : SPEC_INV;
@@ -1197,13 +1196,12 @@ claire_status tl_apply(claire_ctx* c, const cufftComplex* rf, float rscale, cuff
         }
     }
     {
-        KTimer kt(c, KK_SPECTRAL, (zold ? 72.0 : 48.0) * c->M, 0);
-        launch_tl_finish(c->grid, rf, zf, zold, c->M, t->g, t->xh, t->M, op, c->rp, rscale,
+        KTimer kt(c, KK_SPECTRAL, 48.0 * c->M, 0);
+        launch_tl_finish(c->grid, rf, zf, c->M, t->g, t->xh, t->M, op, c->rp, rscale,
                          c->psc, fs_reduction(c, 0, c->M), c->stream);
     }
-    CL_TRY(fs_sums(c, 2));
+    CL_TRY(fs_sums(c, 1));
     *rz = c->hres[0];
-    *ro = zold ? c->hres[1] : 0.0;
     c->pc_inner_total += *its;
     return CLAIRE_OK;
 }
@@ -1243,8 +1241,7 @@ claire_status pcg(claire_ctx* c, double eta, int* its)
     // the flexible one, beta = <r_new, z_new - z_old> / <r_old, z_old>
     int inner_its = 0;
     if (two_level) {
-        double ro;
-        CL_TRY(tl_apply(c, c->rh, 1.0f, c->tl2->zf, nullptr, &rz, &ro, &inner_its));
+        CL_TRY(tl_apply(c, c->rh, 1.0f, c->tl2->zf, &rz, &inner_its));
     }
     double beta = 0.0;
     for (int it = 1; it <= c->o.max_pcg; ++it) {
@@ -1300,8 +1297,8 @@ claire_status pcg(claire_ctx* c, double eta, int* its)
         if (two_level) {
             // <r_new, z_old> = <r_old, z_old> - alpha <H p, z_old>; z_new overwrites z_old
             const double ro = rz - alpha * c->hres[1];
-            double rz_new, unused;
-            CL_TRY(tl_apply(c, c->rh, 1.0f, c->tl2->zf, nullptr, &rz_new, &unused, &inner_its));
+            double rz_new;
+            CL_TRY(tl_apply(c, c->rh, 1.0f, c->tl2->zf, &rz_new, &inner_its));
             beta = (rz_new - ro) / rz;
             rz = rz_new;
         } else {
@@ -1677,9 +1674,9 @@ claire_status claire_precond(claire_ctx* c, const float* r, float* z)
     if (c->o.precond == CLAIRE_PRECOND_TWO_LEVEL) {
         CL_TRY(tl_prepare(c));
         CL_FFT(c, cufftExecR2C(c->r2c, const_cast<float*>(dr), c->rh));
-        double rz, ro;
+        double rz;
         int its;
-        CL_TRY(tl_apply(c, c->rh, static_cast<float>(1.0 / c->N), c->tl2->zf, nullptr, &rz, &ro, &its));
+        CL_TRY(tl_apply(c, c->rh, static_cast<float>(1.0 / c->N), c->tl2->zf, &rz, &its));
         CL_FFT(c, cufftExecC2R(c->c2r, c->tl2->zf, out));
     } else {
         CL_TRY(precond(c, dr, out));

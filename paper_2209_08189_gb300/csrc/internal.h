@@ -350,7 +350,6 @@ void launch_fixed_to_float(unsigned long long* acc, const double* maxabs, int ac
 void launch_scale_add(float* y, float a, const float* x, size_t n, cudaStream_t st);
 void launch_predictor_terms(const Grid& g, int order, const float* v, const float* vc, float dt, const float* dbar,
                             float* ubar, float* Ubar, cudaStream_t st);
-// out2[1] = max |x| (out2[0] scratch)
 // out[0] = max |x| (NaN: infinity)
 void launch_maxabs(const float* x, size_t n, const Reduction& r, cudaStream_t st);
 
@@ -417,9 +416,9 @@ void launch_tl_update(const Grid& gc, const cufftComplex* T, const cufftComplex*
                       const Reduction& red, cudaStream_t st);
 void launch_dir_stored(const Grid& g, const cufftComplex* zh, cufftComplex* ph, cufftComplex* cp, size_t cs,
                        float beta, int first, cudaStream_t st);
-void launch_tl_finish(const Grid& gf, const cufftComplex* rf, cufftComplex* zf, const cufftComplex* zold, size_t csf,
-                      const Grid& gc, const cufftComplex* xc, size_t csc, SpectralOp op, RegParams rp, float rscale,
-                      double* sc, const Reduction& red, cudaStream_t st);
+void launch_tl_finish(const Grid& gf, const cufftComplex* rf, cufftComplex* zf, size_t csf, const Grid& gc,
+                      const cufftComplex* xc, size_t csc, SpectralOp op, RegParams rp, float rscale, double* sc,
+                      const Reduction& red, cudaStream_t st);
 // Deterministic FP64 reductions (struct Reduction): totals at red.out
 void launch_dot(const float* x, const float* y, size_t n, const Reduction& red, cudaStream_t st);
 void launch_sqdiff(const void* a, const void* b, size_t n, Storage sto, const Reduction& red, cudaStream_t st);

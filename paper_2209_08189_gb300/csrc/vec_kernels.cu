@@ -857,17 +857,16 @@ __global__ void __launch_bounds__(kThreads) k_dir_stored(Grid g, const float2* _
 }
 
 // Outer preconditioned residual of r = rscale rf: z = E x (kept coarse modes), r
-// on the mean, M r on every other mode; totals <r, z> (also the outer PCG's
-// rz) and <r, zold> (zold may be null).
+// on the mean, M r on every other mode; total <r, z> (also the outer PCG's rz).
 __global__ void __launch_bounds__(kThreads) k_tl_finish(Grid gf, const float2* __restrict__ rf,
-                                                         float2* __restrict__ zf, const float2* __restrict__ zold,
-                                                         size_t csf, Grid gc, const float2* __restrict__ xc,
-                                                         size_t csc, int op, RegParams rp, float rscale,
-                                                         double* __restrict__ sc, Reduction red)
+                                                         float2* __restrict__ zf, size_t csf, Grid gc,
+                                                         const float2* __restrict__ xc, size_t csc, int op,
+                                                         RegParams rp, float rscale, double* __restrict__ sc,
+                                                         Reduction red)
 {
     const int n3h = gf.n3 / 2 + 1;
     const uint32_t M = static_cast<uint32_t>(gf.n1) * gf.n2 * n3h;
-    double az = 0.0, ao = 0.0;
+    double az = 0.0;
     for (uint32_t idx = blockIdx.x * kThreads + threadIdx.x; idx < M; idx += gridDim.x * kThreads) {
         int k1, k2, k3;
         wavenumbers(gf, idx, k1, k2, k3);
@@ -885,11 +884,9 @@ __global__ void __launch_bounds__(kThreads) k_tl_finish(Grid gf, const float2* _
 #pragma unroll
         for (int c = 0; c < 3; ++c) zf[c * csf + idx] = z[c];
         az += static_cast<double>(m.wt * cdot3(r0, r1, r2, z[0], z[1], z[2]));
-        if (zold)
-            ao += static_cast<double>(m.wt * cdot3(r0, r1, r2, zold[idx], zold[csf + idx], zold[2 * csf + idx]));
     }
-    double tot[2];
-    if (grid_sum2(az, ao, red, tot)) sc[kPcgRz] = tot[0];
+    double rz;
+    if (grid_sum(az, red, &rz)) sc[kPcgRz] = rz;
 }
 
 }  // namespace
@@ -1031,14 +1028,14 @@ void launch_dir_stored(const Grid& g, const cufftComplex* zh, cufftComplex* ph, 
                                                         cs, beta, first);
 }
 
-void launch_tl_finish(const Grid& gf, const cufftComplex* rf, cufftComplex* zf, const cufftComplex* zold, size_t csf,
-                      const Grid& gc, const cufftComplex* xc, size_t csc, SpectralOp op, RegParams rp, float rscale,
-                      double* sc, const Reduction& red, cudaStream_t st)
+void launch_tl_finish(const Grid& gf, const cufftComplex* rf, cufftComplex* zf, size_t csf, const Grid& gc,
+                      const cufftComplex* xc, size_t csc, SpectralOp op, RegParams rp, float rscale, double* sc,
+                      const Reduction& red, cudaStream_t st)
 {
     k_tl_finish<<<red.nblocks, kThreads, 0, st>>>(gf, reinterpret_cast<const float2*>(rf),
-                                                  reinterpret_cast<float2*>(zf), reinterpret_cast<const float2*>(zold),
-                                                  csf, gc, reinterpret_cast<const float2*>(xc), csc,
-                                                  static_cast<int>(op), rp, rscale, sc, red);
+                                                  reinterpret_cast<float2*>(zf), csf, gc,
+                                                  reinterpret_cast<const float2*>(xc), csc, static_cast<int>(op), rp,
+                                                  rscale, sc, red);
 }
 
 void launch_dot(const float* x, const float* y, size_t n, const Reduction& red, cudaStream_t st)
