@@ -381,12 +381,13 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3d_tc(const __nv_bfloat16*
     // staging: 16-byte pieces of the halo plane e = tid + 128 u < 360, piece e =
     // half e & 1 (8 channels) of slot e >> 1 = (sh * 10 + sw); the wrapped (h, w)
     // offsets are formed once, a plane costs one pointer step
-    uint32_t goff[3], soff[3];
+    size_t goff[3];  // a plane may hold 2^32 elements and more
+    uint32_t soff[3];
 #pragma unroll
     for (int u = 0; u < 3; ++u) {
         const int e = min(tid + u * kConvThreads, 2 * kTcPlaneSlots - 1);
         const int sl = e >> 1, hlf = e & 1, shh = sl / kTcHaloW, sw = sl - shh * kTcHaloW;
-        goff[u] = (static_cast<uint32_t>(wrapi(h0 + shh - 1, v.H)) * v.W + wrapi(w0 + sw - 1, v.W)) * Cxs + 8 * hlf;
+        goff[u] = (static_cast<size_t>(wrapi(h0 + shh - 1, v.H)) * v.W + wrapi(w0 + sw - 1, v.W)) * Cxs + 8 * hlf;
         soff[u] = hlf * sh.plane + sl * 16;
     }
     const bool third = tid + 2 * kConvThreads < 2 * kTcPlaneSlots;
@@ -734,7 +735,7 @@ __global__ void __launch_bounds__(kWgThreads) k_wgrad_tc(const __nv_bfloat16* __
                 for (int sb = 0; sb < wg.nsa; ++sb) {
                     const int d = wg.nsa == 3 ? wrapi(d0 + sb - 1, v.D) : d0;
                     const __nv_bfloat16* rowp = dY + (static_cast<size_t>(b) * v.D + d) * plane_y +
-                                                static_cast<uint32_t>(h0 + ja_r) * row_y +
+                                                static_cast<size_t>(h0 + ja_r) * row_y +
                                                 static_cast<uint32_t>(w0) * Cys + co0;
                     uint32_t dst = a_s + ja_r * albo + sb * cbn * 128;
                     if (tja <= nl) {
@@ -768,7 +769,7 @@ __global__ void __launch_bounds__(kWgThreads) k_wgrad_tc(const __nv_bfloat16* __
                         uint32_t dst = h_s + (sd * kTcHaloH + jx_r) * xrow_s + (wg.nkw == 1 ? x_q * 160 : x_q * 128) +
                                        x_sw * 16;
                         for (int sh = jx_r; sh < kTcHaloH; sh += rppx) {
-                            const __nv_bfloat16* src = plane + static_cast<uint32_t>(wrapi(h0 + sh - 1, v.H)) * row_x;
+                            const __nv_bfloat16* src = plane + static_cast<size_t>(wrapi(h0 + sh - 1, v.H)) * row_x;
                             if (wg.nkw == 1) {
                                 cp_async16(dst, src);
                             } else {

@@ -408,3 +408,30 @@ def test_invalid_shapes_are_rejected(env):
     y2 = torch.zeros((1, 8, 8, 6, 16), dtype=torch.bfloat16, device="cuda")
     with pytest.raises(net.NetError):
         net.conv3d(net.Act(x, 0, 16), w[:16], None, net.Act(y2, 0, 16), 0.1, 1, stream(torch))
+
+
+def test_tcgen05_layers_in_planes_of_more_than_2_to_32_elements(env):
+    """A 16-channel slice of a wide buffer whose (H, W) plane has 4.6e9 elements gives
+    the bits of the same slice stored by itself, forward and weight gradient: no
+    offset inside a plane is taken modulo 2^32."""
+    torch, net = env
+    B, D, H, W, c, stride = 1, 4, 4096, 4096, 16, 272
+    if torch.cuda.mem_get_info()[0] < 60 << 30:
+        pytest.skip("needs 60 GB of device memory")
+    g = torch.Generator(device="cuda").manual_seed(1)
+    x = torch.randn((B, D, H, W, c), device="cuda", generator=g, dtype=torch.bfloat16)
+    wide = torch.zeros((B, D, H, W, stride), dtype=torch.bfloat16, device="cuda")
+    wide[..., stride - c:] = x
+    w = torch.randn((c, 27, c), device="cuda", generator=g, dtype=torch.bfloat16)
+    chunks = net.wgrad_chunks(c, c, (B, D, H, W))
+    part, partb = torch.empty(chunks * c * 27 * c, device="cuda"), torch.empty(chunks * c, device="cuda")
+    got = []
+    for act in (net.Act(x, 0, c), net.Act(wide, stride - c, c)):
+        y = torch.empty((B, D, H, W, c), dtype=torch.bfloat16, device="cuda")
+        net.conv3d(act, w, None, net.Act(y, 0, c), 0.1, 1, stream(torch))
+        dw, db = torch.empty((c, 27, c), device="cuda"), torch.empty(c, device="cuda")
+        net.conv3d_wgrad(act, act, chunks, part, partb, dw, db, stream(torch))
+        got.append((y, dw, db))
+    for a, b in zip(*got):
+        assert torch.equal(a, b)
+    assert net.device_errors() == 0
