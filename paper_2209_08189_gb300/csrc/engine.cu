@@ -123,8 +123,8 @@ struct claire_ctx {
     // their tile-bounds tables, written by every backtrace into dS / dA (the
     // only writer of either field), read by the gathers at dS / dA
     int4 *tbS = nullptr, *tbA = nullptr;
-    // table of the characteristic that objective, transport, det-J and the
-    // reverse mode trace into z, where the same call's gathers read it
+    // table of the characteristic that objective, transport and the reverse mode
+    // trace into z, where the same call's gathers read it
     int4* tbZ = nullptr;
     char *divv = nullptr, *divXp = nullptr;
     char *m = nullptr, *gm = nullptr;     // (nt+1) N states m^j, (nt+1) 3N gradients (null when lowmem)

@@ -1488,12 +1488,13 @@ cudaError_t conv3d(const void* X, int Cxs, int Cin, const void* Wt, const float*
     auto w = static_cast<const __nv_bfloat16*>(Wt);
     auto y = static_cast<__nv_bfloat16*>(Y);
     if (tc_eligible(Cin, Cout, D, H, W)) {
-        // tcgen05 path: bricks of bdc x 16 x 8 voxels; the deepest brick whose
-        // TMEM columns (bdc planes x Cout rounded to 32) and shared memory fit
+        // tcgen05 path: bricks of bdc x 16 x 8 voxels whose TMEM columns (bdc planes
+        // x Cout, unstacked rounded up to 32) and shared memory fit
         TcShape sh{};
-        // stacked up to 80 output channels (N <= 256): an MMA reads 128 x 32 B of halo and N x 32 B
-        // of weights from shared memory whatever its N, so three kd taps per read
-        // of the halo save more than the clipped edge planes of a brick cost
+        // stacked while three blocks fit N <= 256 (up to 64 of the channel counts that
+        // are taken): an MMA reads 128 x 32 B of halo and N x 32 B of weights from
+        // shared memory whatever its N, so three kd taps per read of the halo save
+        // more than the clipped edge planes of a brick and the groups' waits cost
         sh.stack = 3 * Cout <= 256 ? 1 : 0;
         sh.ccols = sh.stack ? Cout : (Cout + 31) / 32 * 32;
         const int wbytes = 27 * 2 * Cout * 16;
@@ -1505,10 +1506,11 @@ cudaError_t conv3d(const void* X, int Cxs, int Cin, const void* Wt, const float*
         // MMAs' time and a CTA's whole turn over r.  Cycles: an MMA reads 128
         // halo rows at half rate (the 10-voxel rows straddle bank lines) and N
         // weight rows, (8192 + 32 N) / 128; a staged 16-byte piece costs 1/2; the
-        // latencies of a turn 2000.  The deepest brick with two waves of CTAs,
-        // the rule before, left small volumes one plane deep: 32^3 x 4, 192 ->
-        // 64 channels 274 us against 125 at four planes.  One stage unless a
-        // forced setting asks for two.
+        // latencies of a turn 2000.  The deepest brick with two waves of CTAs, the
+        // rule before, left small volumes one plane deep: 32^3 x 4, 192 -> 64
+        // channels 276 us against 120 at four planes.  (In 18 layer shapes timed at
+        // every depth the choice is within 6 % of the best, except 1 x 32^3, 64 -> 64
+        // channels: 31 us against 27.)  One stage unless a forced setting asks for two.
         double best = 0.0;
         for (int bdc = sh.stack ? 8 : 4; bdc >= 1; bdc >>= 1) {
             if (D % bdc || bdc * sh.ccols > 512) continue;

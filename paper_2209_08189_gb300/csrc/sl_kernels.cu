@@ -548,7 +548,8 @@ __device__ __forceinline__ float ordered_float(int i) { return __int_as_float(i 
 // the block's smallest or above its largest value so far are formed in FP64
 // (det_bounds).  A NaN or an overflow fails both comparisons and is formed in
 // FP64.  The extrema are the FP64 ones of the same FP32 differences, bit for bit.
-// Columns are walked by a fixed number of CTAs (one partial each).  256^3: 328 us.
+// Columns are walked by a fixed number of CTAs (one partial each).  256^3: 330 us on a
+// random velocity, 345 at the end of a registration.
 __global__ void __launch_bounds__(kThreads) k_detj_minmax(Grid g, const float* __restrict__ u, int zlen, int ncol,
                                                            Reduction red)
 {
