@@ -1509,8 +1509,8 @@ cudaError_t conv3d(const void* X, int Cxs, int Cin, const void* Wt, const float*
         // latencies of a turn 2000.  The deepest brick with two waves of CTAs, the
         // rule before, left small volumes one plane deep: 32^3 x 4, 192 -> 64
         // channels 276 us against 120 at four planes.  (In 18 layer shapes timed at
-        // every depth the choice is within 6 % of the best, except 1 x 32^3, 64 -> 64
-        // channels: 31 us against 27.)  One stage unless a forced setting asks for two.
+        // every depth the choice is within 6 % of the best, except 1 x 32^3 with 64
+        // output channels: 31 and 20 us against 27 and 18.)  One stage unless a forced setting asks for two.
         double best = 0.0;
         for (int bdc = sh.stack ? 8 : 4; bdc >= 1; bdc >>= 1) {
             if (D % bdc || bdc * sh.ccols > 512) continue;

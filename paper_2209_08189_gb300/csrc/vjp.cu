@@ -345,8 +345,10 @@ __device__ __forceinline__ void add_high(uint32_t hi, const FixedTerm& t, unsign
 // global atomics.  Integer sums do not depend on the order of additions, so
 // either path gives the same bits.
 //
-// Bound: the shared-memory atomics (128 per point, 2.3 wavefronts each).
-// 128^3, cubic: 326 us with 64-bit conversions and 64-bit shared atomics, 139 us.
+// Bound: instruction issue (68 % of the slots, 112 M warp instructions at 128^3) beside
+// the shared-memory data pipe (55 %: 128 atomics per point, 8.4 M warp
+// instructions of 2.8 wavefronts).  128^3, cubic: 326 us with 64-bit conversions
+// and 64-bit shared atomics, 139 us.
 constexpr int kST1 = 4, kST2 = 8, kST3 = 32;
 constexpr int kScatterCap = 6976;  // nodes of 8 B: four CTAs of 54.5 KB per SM
 
