@@ -10,6 +10,11 @@ namespace claire {
 // the output planes z = sd - kd that lie in the brick: nz planes from z0 on, whose
 // columns are adjacent, so one MMA covers them.  Block 0 of its B operand is
 // that of z0, i.e. of tap kd = sd - z0.
+//
+// The planes are issued in the order of sd, so that every output plane sums its depth
+// taps kd = 0, 1, 2 as the unstacked kernel does (the same bits; an order that
+// differs from plane to plane moves roundings, and with them the signs that the
+// leaky ReLU's backward pass reads).
 struct StackedPlane {
     int z0, nz;
 };
@@ -21,14 +26,20 @@ __host__ __device__ inline StackedPlane stacked_plane(int bdc, int sd)
 }
 
 // The order of two MMAs is defined only where they have the same accumulator and
-// the same shape, and planes one or two apart overlap in their columns with
-// other bases and, at the brick's edges, other widths.  So the planes are issued in
-// three groups, sd = g mod 3, whose members write disjoint columns; the issuing
-// thread waits for a group before it issues the next.  Group 0 writes every
-// column, so its first product of the first slice overwrites and all others add.
-// (One output plane: every MMA has the same accumulator and shape, no waits.)
-constexpr int kStackGroups = 3;
-
-__host__ __device__ inline bool stacked_wait(int bdc, int group) { return group > 0 && bdc > 1; }
+// the same shape, and neighbouring planes overlap in their columns with another
+// base or, at the brick's edges, another width: the issuing thread waits for
+// plane sd - 1 before it issues such a plane sd.  The waits are hidden where the
+// brick leaves room for four CTAs per SM and cost up to a sixth where it leaves
+// three: 128^3 x 4, 16 -> 16 channels, eight planes 302 us (257 without them), four
+// planes 373 either way; 64^3 x 4, 96 -> 32 channels 270 us (257).  Two interleaved
+// chains of four planes, whose waits overlap, need two planes more and took 319;
+// three groups of planes that do not overlap (two waits) took 266, but sum the depth taps
+// in orders that differ from plane to plane.
+__host__ __device__ inline bool stacked_wait(int bdc, int sd)
+{
+    if (sd == 0) return false;
+    const StackedPlane a = stacked_plane(bdc, sd - 1), b = stacked_plane(bdc, sd);
+    return a.z0 != b.z0 || a.nz != b.nz;
+}
 
 }  // namespace claire

@@ -236,8 +236,7 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3d(const __nv_bfloat16* __
 // core-matrix layout (8 rows x 16 bytes per core matrix, two 8-channel half
 // planes), then one elected thread issues tcgen05.mma.kind::f16 (M128 x N x
 // K16), 27 x BDc of them or, with the kd taps stacked along N (TcShape::stack),
-// 9 x (BDc + 2) in three groups (conv_schedule.cuh; 128^3 x 4, 16 -> 16 channels
-// 266 us, 257 without the two waits that keep overlapping MMAs apart): the A operand of a (plane, tap) pair is the halo at a
+// 9 x (BDc + 2) with a wait between planes (conv_schedule.cuh): the A operand of a (plane, tap) pair is the halo at a
 // shifted start address, because every core matrix is 8 consecutive voxels
 // along W and the next one is the next H row (a constant stride).  The halo
 // is shared by the BDc planes; with two stages the next slice is staged while
@@ -339,6 +338,14 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&q)[16])
     asm volatile("tcgen05.wait::ld.sync.aligned;");
 }
 
+// zeros in 16 consecutive TMEM columns of this warp's 32 lanes
+__device__ __forceinline__ void tmem_zero16(uint32_t taddr)
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1};" ::"r"(
+                     taddr),
+                 "r"(0));
+}
+
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
 
 template <int N>
@@ -364,7 +371,7 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3d_tc(const __nv_bfloat16*
                                                             TcShape sh, Vol v, int* __restrict__ err)
 {
     extern __shared__ __align__(128) unsigned char tc_smem[];
-    __shared__ __align__(8) uint64_t mbar, group, drain;
+    __shared__ __align__(8) uint64_t mbar, plane_bar, drain;
     __shared__ uint32_t tmem_slot;
     __shared__ int stall;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -376,7 +383,7 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3d_tc(const __nv_bfloat16*
     const int h0 = (r % nbh) * kTcBH; r /= nbh;
     const int d0 = (r % nbd) * bdc;
     const int b = r / nbd;
-    const uint32_t smem_s = smem_addr(tc_smem), mbar_s = smem_addr(&mbar), group_s = smem_addr(&group);
+    const uint32_t smem_s = smem_addr(tc_smem), mbar_s = smem_addr(&mbar), plane_s = smem_addr(&plane_bar);
     const int nchunks = Cin / 16;
     // staging: 16-byte pieces of the halo plane e = tid + 128 u < 360, piece e =
     // half e & 1 (8 channels) of slot e >> 1 = (sh * 10 + sw); the wrapped (h, w)
@@ -434,7 +441,7 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3d_tc(const __nv_bfloat16*
     const uint32_t drain_s = smem_addr(&drain);
     if (tid == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(mbar_s), "r"(1));
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(group_s), "r"(1));
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(plane_s), "r"(1));
         asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(drain_s), "r"(1));
         stall = g_tc_test_stall;
     }
@@ -442,6 +449,13 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3d_tc(const __nv_bfloat16*
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = tmem_slot;
+    // stacked accumulators start at zero: an MMA's planes would differ in whether
+    // they are written or added to (the barriers before the first MMA publish this)
+    if (sh.stack)
+        for (int c0 = 0; c0 < bdc * Cout; c0 += 16)
+            tmem_zero16(tmem + (static_cast<uint32_t>(32 * warp) << 16) + static_cast<uint32_t>(c0));
+    asm volatile("tcgen05.wait::st.sync.aligned;");
+    uint32_t plane_phase = 0;
     // failure-detection hook: a wait on phase 0 of mbar, which only the first
     // commit would complete, before any MMA is issued (it runs out)
     bool ok = true;
@@ -482,26 +496,24 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3d_tc(const __nv_bfloat16*
             bool issued = true;
             if (sh.stack) {
                 const uint32_t bstep = 6u * Cout;
-                for (int grp = 0; grp < kStackGroups && issued; ++grp) {
-                    if (stacked_wait(bdc, grp)) {
+                for (int sd = 0; sd < bdc + 2 && issued; ++sd) {
+                    if (stacked_wait(bdc, sd)) {
                         asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::
-                                         "r"(group_s)
+                                         "r"(plane_s)
                                      : "memory");
-                        // two phases per slice, waited for by this thread alone
-                        issued = mbar_wait(group_s, (grp - 1) & 1);
+                        issued = mbar_wait(plane_s, plane_phase);  // by this thread alone, every phase in turn
+                        plane_phase ^= 1u;
                         asm volatile("tcgen05.fence::after_thread_sync;");
+                        if (!issued) break;
                     }
-                    for (int sd = grp; sd < bdc + 2 && issued; sd += kStackGroups) {
-                        const StackedPlane sp = stacked_plane(bdc, sd);
-                        const uint32_t ap = a_lo + static_cast<uint32_t>(sd * kTcPlaneSlots);
-                        const uint32_t bp = b_lo + static_cast<uint32_t>((2 - (sd - sp.z0)) * Cout);
-                        const uint32_t dt = tmem + static_cast<uint32_t>(sp.z0 * Cout);
-                        const uint32_t id = idesc(sp.nz * Cout);
-                        umma(dt, ap, a_hi, bp, b_hi, id, c > 0 || grp > 0 ? 1u : 0u);
+                    const StackedPlane sp = stacked_plane(bdc, sd);
+                    const uint32_t ap = a_lo + static_cast<uint32_t>(sd * kTcPlaneSlots);
+                    const uint32_t bp = b_lo + static_cast<uint32_t>((2 - (sd - sp.z0)) * Cout);
+                    const uint32_t dt = tmem + static_cast<uint32_t>(sp.z0 * Cout);
+                    const uint32_t id = idesc(sp.nz * Cout);
 #pragma unroll
-                        for (int t = 1; t < 9; ++t)
-                            umma(dt, ap + (t / 3) * kTcHaloW + t % 3, a_hi, bp + t * bstep, b_hi, id, 1u);
-                    }
+                    for (int t = 0; t < 9; ++t)
+                        umma(dt, ap + (t / 3) * kTcHaloW + t % 3, a_hi, bp + t * bstep, b_hi, id, 1u);
                 }
             } else {
                 const uint32_t id = idesc(Cout), bstep = 2u * Cout;
@@ -518,7 +530,7 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3d_tc(const __nv_bfloat16*
                     }
                 }
             }
-            // a group that gave up leaves the phase open: every wait for it runs out
+            // a plane's wait that gave up leaves the phase open: every wait for it runs out
             if (issued)
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar_s)
                              : "memory");
@@ -1494,7 +1506,7 @@ cudaError_t conv3d(const void* X, int Cxs, int Cin, const void* Wt, const float*
         // stacked while three blocks fit N <= 256 (up to 64 of the channel counts that
         // are taken): an MMA reads 128 x 32 B of halo and N x 32 B of weights from
         // shared memory whatever its N, so three kd taps per read of the halo save
-        // more than the clipped edge planes of a brick and the groups' waits cost
+        // more than the clipped edge planes of a brick and the waits between planes cost
         sh.stack = 3 * Cout <= 256 ? 1 : 0;
         sh.ccols = sh.stack ? Cout : (Cout + 31) / 32 * 32;
         const int wbytes = 27 * 2 * Cout * 16;
@@ -1509,8 +1521,8 @@ cudaError_t conv3d(const void* X, int Cxs, int Cin, const void* Wt, const float*
         // latencies of a turn 2000.  The deepest brick with two waves of CTAs, the
         // rule before, left small volumes one plane deep: 32^3 x 4, 192 -> 64
         // channels 276 us against 120 at four planes.  (In 18 layer shapes timed at
-        // every depth the choice is within 6 % of the best, except 1 x 32^3 with 64
-        // output channels: 31 and 20 us against 27 and 18.)  One stage unless a forced setting asks for two.
+        // every depth the choice is within 6 % of the best, except 1 x 32^3, 64 -> 64
+        // channels: 30 us against 27.)  One stage unless a forced setting asks for two.
         double best = 0.0;
         for (int bdc = sh.stack ? 8 : 4; bdc >= 1; bdc >>= 1) {
             if (D % bdc || bdc * sh.ccols > 512) continue;

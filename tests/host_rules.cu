@@ -74,39 +74,27 @@ void scatter_boxes()
 
 // The stacked convolution: between two waits, MMAs that touch the same columns have
 // the same first column and the same width (only their order is defined); every
-// output plane gets its three depth taps once, and its first product overwrites.
+// output plane gets its depth taps 0, 1, 2 in that order.
 void conv_schedule()
 {
     struct Acc {
         int z0, nz;
     };
     for (int bdc : {1, 2, 4, 8}) {
-        std::vector<int> taps(bdc, 0);
+        std::vector<int> next(bdc, 0);
         std::vector<Acc> open;  // issued and not waited for
-        std::vector<bool> touched(bdc, false);
-        for (int slice = 0; slice < 2; ++slice) {
-            open.clear();  // a slice ends with a wait of the whole block
-            for (int grp = 0; grp < kStackGroups; ++grp) {
-                if (stacked_wait(bdc, grp)) open.clear();
-                for (int sd = grp; sd < bdc + 2; sd += kStackGroups) {
-                    const StackedPlane p = stacked_plane(bdc, sd);
-                    check(p.z0 >= 0 && p.nz >= 1 && p.nz <= 3 && p.z0 + p.nz <= bdc, "columns of the brick");
-                    for (const Acc& a : open) {
-                        const bool overlap = p.z0 < a.z0 + a.nz && a.z0 < p.z0 + p.nz;
-                        check(!overlap || (p.z0 == a.z0 && p.nz == a.nz), "overlapping MMAs of different shapes");
-                    }
-                    open.push_back({p.z0, p.nz});
-                    for (int z = p.z0; z < p.z0 + p.nz; ++z) {
-                        const int kd = sd - z;
-                        check(kd >= 0 && kd <= 2, "depth tap");
-                        if (slice == 0) taps[z] |= 1 << kd;
-                        check(touched[z] == (slice > 0 || grp > 0), "first product of a plane is in group 0");
-                        touched[z] = true;
-                    }
-                }
+        for (int sd = 0; sd < bdc + 2; ++sd) {
+            if (stacked_wait(bdc, sd)) open.clear();
+            const StackedPlane p = stacked_plane(bdc, sd);
+            check(p.z0 >= 0 && p.nz >= 1 && p.nz <= 3 && p.z0 + p.nz <= bdc, "columns of the brick");
+            for (const Acc& a : open) {
+                const bool overlap = p.z0 < a.z0 + a.nz && a.z0 < p.z0 + p.nz;
+                check(!overlap || (p.z0 == a.z0 && p.nz == a.nz), "overlapping MMAs of different shapes");
             }
+            open.push_back({p.z0, p.nz});
+            for (int z = p.z0; z < p.z0 + p.nz; ++z) check(sd - z == next[z]++, "depth taps in order");
         }
-        for (int z = 0; z < bdc; ++z) check(taps[z] == 7, "three depth taps");
+        for (int z = 0; z < bdc; ++z) check(next[z] == 3, "three depth taps");
     }
 }
 
