@@ -28,8 +28,8 @@ inline unsigned blocks_for(uint32_t n) { return (n + kThreads - 1) / kThreads; }
 // the predictor points of a tile share its bounds).  TBW: also write the
 // tile-bounds table of d (tile_index order), from the same FP32 values that
 // are stored, for the gathers at d.
-template <int ORDER, bool FULL, bool TBW>
-__global__ void __launch_bounds__(kTileThreads, tile_min_blocks<ORDER>())
+template <int ORDER, bool FULL, bool TBW, bool WIDE = false>
+__global__ void __launch_bounds__(kTileThreads, tile_min_blocks<ORDER, 4, WIDE>())
     k_backtrace_tiled(Grid g, const float* __restrict__ v, const float* __restrict__ vc, float dt, float sign,
                       float* __restrict__ d, int4* __restrict__ tb)
 {
@@ -128,11 +128,16 @@ template <int ORDER, bool FULL, bool TBW>
 void launch_backtrace_tiled_as(const Grid& g, const float* v, const float* vc, float dt, float sign, float* d,
                                int4* tb, cudaStream_t st)
 {
-    if (tiled_smem_bytes<ORDER>(g) > 48 * 1024)
-        cudaFuncSetAttribute(k_backtrace_tiled<ORDER, FULL, TBW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(tiled_smem_bytes<ORDER>(g)));
-    k_backtrace_tiled<ORDER, FULL, TBW><<<tiled_grid(g), kTileThreads, tiled_smem_bytes<ORDER>(g), st>>>(g, v, vc, dt, sign,
-                                                                                              d, tb);
+    const size_t smem = tiled_smem_bytes<ORDER>(g);
+    auto launch = [&](auto kernel) {
+        if (smem > 48 * 1024)
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+        kernel<<<tiled_grid(g), kTileThreads, smem, st>>>(g, v, vc, dt, sign, d, tb);
+    };
+    if constexpr (ORDER == 1) {
+        if (g.wide) return launch(k_backtrace_tiled<ORDER, FULL, TBW, true>);
+    }
+    launch(k_backtrace_tiled<ORDER, FULL, TBW>);
 }
 
 template <int ORDER>
@@ -656,29 +661,28 @@ void launch_interp(const Grid& g, int order, const void* f, const float* d, void
     });
 }
 
-template <int ORDER, bool FULL, bool MAP, bool WIDE>
+template <int ORDER, bool FULL, bool MAP>
 void launch_fields_tiles(const Grid& g, const float* f, int nf, const float* d, float* out, cudaStream_t st)
 {
     const size_t smem = tiled_smem_bytes<ORDER>(g);
-    if (smem > 48 * 1024)
-        cudaFuncSetAttribute(k_gather_tiled_fields<ORDER, FULL, MAP, WIDE>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    k_gather_tiled_fields<ORDER, FULL, MAP, WIDE><<<tiled_grid(g), kTileThreads, smem, st>>>(g, f, nf, d, out);
+    auto launch = [&](auto kernel) {
+        if (smem > 48 * 1024)
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+        kernel<<<tiled_grid(g), kTileThreads, smem, st>>>(g, f, nf, d, out);
+    };
+    if constexpr (ORDER == 1) {
+        if (g.wide) return launch(k_gather_tiled_fields<ORDER, FULL, MAP, true>);
+    }
+    launch(k_gather_tiled_fields<ORDER, FULL, MAP>);
 }
 
 template <int ORDER, bool MAP>
 void launch_fields_as(const Grid& g, const float* f, int nf, const float* d, float* out, cudaStream_t st)
 {
-    const bool full = tiles_cover_grid(g);
-    if constexpr (ORDER == 1) {
-        if (g.wide) {
-            full ? launch_fields_tiles<ORDER, true, MAP, true>(g, f, nf, d, out, st)
-                 : launch_fields_tiles<ORDER, false, MAP, true>(g, f, nf, d, out, st);
-            return;
-        }
-    }
-    full ? launch_fields_tiles<ORDER, true, MAP, false>(g, f, nf, d, out, st)
-         : launch_fields_tiles<ORDER, false, MAP, false>(g, f, nf, d, out, st);
+    if (tiles_cover_grid(g))
+        launch_fields_tiles<ORDER, true, MAP>(g, f, nf, d, out, st);
+    else
+        launch_fields_tiles<ORDER, false, MAP>(g, f, nf, d, out, st);
 }
 
 void launch_interp_fields(const Grid& g, int order, const float* f, int nf, const float* d, float* out,

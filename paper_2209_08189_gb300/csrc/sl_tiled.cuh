@@ -58,23 +58,27 @@ constexpr int kBoxCapFloats = CLAIRE_BOX_CAP;
 // The narrow box holds tiles whose cells spread over 5 nodes, the wide one 6, and a
 // tile that fits neither costs most where six CTAs leave the L1 28 KB.  So large
 // displacements (Grid::wide, set by the context where |v| dt is more than kWideCfl
-// cells somewhere) take the wide box.  Four steps at 512^3, modes up to 24, share
-// of tiles that overflow and time, narrow / wide: CFL 12: 13 % 5.3 ms / 1.4 % 5.6;
-// CFL 16: 42 % 7.6 / 14 % 6.4; CFL 24: 74 % 15.2 / 54 % 8.5; CFL 41: 91 % 29.4 /
-// 83 % 11.6.  Modes up to 6, CFL 12: 0.3 % 4.6 / 0 5.3; CFL 24: 19 % 5.7 / 7 % 5.9.
-// 320^3, up to 24, CFL 10: 16 % 1.44 / 1 % 1.45; CFL 15: 69 % 3.3 / 32 % 1.9.
-// Half boxes of 16 columns for the tiles that overflow: 1.3 to 1.9 times the
-// wide box's time.
+// cells somewhere) take the wide box and kernels compiled for its four CTAs.
+// Four steps at 512^3, modes up to 24, share of tiles that overflow and time,
+// narrow / wide: CFL 12: 13 % 5.3 ms / 1.4 % 5.2; CFL 16: 42 % 7.6 / 14 % 5.9;
+// CFL 24: 74 % 15.2 / 54 % 7.4; CFL 41: 91 % 29.4 / 83 % 9.5.  Modes up to 6,
+// CFL 12: 0.3 % 4.6 / 0 4.9; CFL 24: 19 % 5.7 / 7 % 5.4.  320^3, up to 24, CFL 10:
+// 16 % 1.44 narrow; CFL 13: 46 % 2.15 / 11 % 1.49; CFL 15: 69 % 3.3 / 32 % 1.7.
+// Half boxes of 16 columns for the tiles that overflow: 1.3 to 1.9 times the wide
+// box's time.
 constexpr int kBoxCapLinear = 9216;
 template <int ORDER, int ES = 4>
 __host__ __device__ __forceinline__ int box_cap(const Grid& g)
 {
     return ORDER == 1 && ES == 4 && !g.wide ? kBoxCapLinear : kBoxCapFloats;
 }
-template <int ORDER, int ES = 4>
+// WIDE: the kernel launched with the wide box, compiled for its four CTAs per SM (with
+// the registers of six, 512^3 interpolation at no displacement took 0.88 ms
+// instead of 0.75 behind the wide box).
+template <int ORDER, int ES = 4, bool WIDE = false>
 constexpr int tile_min_blocks()
 {
-    return ORDER == 1 && ES == 4 ? 6 : CLAIRE_TILE_MIN_BLOCKS;
+    return ORDER == 1 && ES == 4 && !WIDE ? 6 : CLAIRE_TILE_MIN_BLOCKS;
 }
 
 __device__ __forceinline__ void cp_async_f32(float* smem_dst, const float* gmem_src)
@@ -597,8 +601,8 @@ __device__ __forceinline__ float tile_eval(const float* box, const BoxPar& bp, i
 // block reduction.  Every point is checked against the box (in_box); if any
 // fails, which a table written with this d never causes, the tile takes the
 // global-memory path.
-template <int ORDER, class Epi, class S, bool FULL, bool TB = false>
-__global__ void __launch_bounds__(kTileThreads, tile_min_blocks<ORDER, sizeof(S)>())
+template <int ORDER, class Epi, class S, bool FULL, bool TB = false, bool WIDE = false>
+__global__ void __launch_bounds__(kTileThreads, tile_min_blocks<ORDER, sizeof(S), WIDE>())
     k_gather_tiled(Grid g, const S* __restrict__ f, const float* __restrict__ d, Epi epi,
                    const int4* __restrict__ tb = nullptr)
 {
@@ -709,12 +713,8 @@ __global__ void __launch_bounds__(kTileThreads, tile_min_blocks<ORDER, sizeof(S)
 // (X - x) in physical units, nf = 3.  It reads its 192 stencil values from the
 // box as the gathers do; the per-point kernel it replaced fetched them through
 // L1 (256^3, CFL 3.4: 0.80 ms per step; from the box 0.56 ms).
-// WIDE: the registers of four CTAs per SM, for the wide box (trilinear; the narrow
-// box has the registers of six).  With the narrow kernel's registers tiles that
-// overflow took 1.25 times as long (256^3, three fields, 30 cells per step: 659 us
-// against 540); small displacements: 214 us narrow, 239 wide.
-template <int ORDER, bool FULL, bool MAP, bool WIDE>
-__global__ void __launch_bounds__(kTileThreads, WIDE ? CLAIRE_TILE_MIN_BLOCKS : tile_min_blocks<ORDER>())
+template <int ORDER, bool FULL, bool MAP, bool WIDE = false>
+__global__ void __launch_bounds__(kTileThreads, tile_min_blocks<ORDER, 4, WIDE>())
     k_gather_tiled_fields(Grid g, const float* __restrict__ f, int nf, const float* __restrict__ d,
                           float* __restrict__ out)
 {
@@ -764,9 +764,12 @@ __global__ void __launch_bounds__(kTileThreads, WIDE ? CLAIRE_TILE_MIN_BLOCKS : 
     for (int fld = 0; fld < nf; ++fld) {
         // the weights and offsets of the four points are formed anew for each
         // field: kept across the loop they do not fit the 64 registers (the
-        // compiler then spilled 240 bytes per thread)
+        // compiler then spilled 240 bytes per thread), or the 40 of the narrow
+        // trilinear kernel; the wide one's 64 hold them
+        if constexpr (!(ORDER == 1 && WIDE)) {
 #pragma unroll
-        for (int q = 0; q < TILE1; ++q) asm volatile("" : "+f"(d1[q]), "+f"(d2[q]), "+f"(d3[q]));
+            for (int q = 0; q < TILE1; ++q) asm volatile("" : "+f"(d1[q]), "+f"(d2[q]), "+f"(d3[q]));
+        }
         tile_load_box<float>(g, f + fld * N, box, bp, lane, warp);
         cp_async_wait_all();
         __syncthreads();
@@ -799,10 +802,16 @@ size_t tiled_smem_bytes(const Grid& g)
 template <int ORDER, class Epi, class S, bool FULL, bool TB>
 inline void launch_tiled_as(const Grid& g, const S* f, const float* d, const Epi& e, cudaStream_t st, const int4* tb)
 {
-    if (tiled_smem_bytes<ORDER, sizeof(S)>(g) > 48 * 1024)
-        cudaFuncSetAttribute(k_gather_tiled<ORDER, Epi, S, FULL, TB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(tiled_smem_bytes<ORDER, sizeof(S)>(g)));
-    k_gather_tiled<ORDER, Epi, S, FULL, TB><<<tiled_grid(g), kTileThreads, tiled_smem_bytes<ORDER, sizeof(S)>(g), st>>>(g, f, d, e, tb);
+    const size_t smem = tiled_smem_bytes<ORDER, sizeof(S)>(g);
+    auto launch = [&](auto kernel) {
+        if (smem > 48 * 1024)
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+        kernel<<<tiled_grid(g), kTileThreads, smem, st>>>(g, f, d, e, tb);
+    };
+    if constexpr (ORDER == 1 && sizeof(S) == 4) {
+        if (g.wide) return launch(k_gather_tiled<ORDER, Epi, S, FULL, TB, true>);
+    }
+    launch(k_gather_tiled<ORDER, Epi, S, FULL, TB>);
 }
 
 template <int ORDER, class Epi, class S>
