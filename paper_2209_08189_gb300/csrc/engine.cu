@@ -1445,6 +1445,7 @@ claire_status claire_create(claire_ctx** out, const int grid[3], double beta_v, 
     g.ih1 = static_cast<float>(grid[0] / two_pi);
     g.ih2 = static_cast<float>(grid[1] / two_pi);
     g.ih3 = static_cast<float>(grid[2] / two_pi);
+    g.wide = 1;  // until a velocity is screened: displacements of any size may come
     c->hvol = (two_pi / grid[0]) * (two_pi / grid[1]) * (two_pi / grid[2]);
     c->rp.beta_v = static_cast<float>(beta_v);
     c->rp.beta_w = static_cast<float>(o.beta_w);
