@@ -313,6 +313,15 @@ struct ColumnMap {
     static constexpr int LPR = 64 / VPC;                             // threads per row
 };
 
+// Origin of the box wrapped into the grid.
+struct BoxOrigin {
+    int w1, w2, w3;
+    __device__ __forceinline__ BoxOrigin(const Grid& g, const BoxPar& bp)
+        : w1(wrap_index(bp.O1, g.n1)), w2(wrap_index(bp.O2, g.n2)), w3(wrap_index(bp.O3, g.n3))
+    {
+    }
+};
+
 // Box staging by columns: thread t owns box row t / LPR (and every
 // kTileThreads / LPR rows on) and chunk t % LPR (+ LPR) and copies that chunk
 // of each of the E1 planes in turn, so the wrapped x2 / x3 indices and the row
@@ -323,10 +332,11 @@ struct ColumnMap {
 // step from 171 to 111 us (the tile-bounds table included).
 template <class S, int BYTES>
 __device__ __forceinline__ void stage_box_columns(const Grid& g, const S* __restrict__ f, uint32_t dst0,
-                                                  const BoxPar& bp)
+                                                  const BoxPar& bp, const BoxOrigin* origin)
 {
     constexpr int VPC = ColumnMap<S, BYTES>::VPC, LPR = ColumnMap<S, BYTES>::LPR;
-    const int w1 = wrap_index(bp.O1, g.n1), w2 = wrap_index(bp.O2, g.n2), w3 = wrap_index(bp.O3, g.n3);
+    const BoxOrigin w = origin ? *origin : BoxOrigin(g, bp);
+    const int w1 = w.w1, w2 = w.w2, w3 = w.w3;
     const int nch = bp.E3 / VPC;
     const uint32_t row_bytes = static_cast<uint32_t>(bp.S3) * sizeof(S);
     const uint32_t plane_bytes = row_bytes * static_cast<uint32_t>(bp.E2);
@@ -382,18 +392,20 @@ __device__ __forceinline__ void widen_box_columns(const uint32_t* stage, float* 
 
 // Copy the (periodically wrapped) box of f into shared memory asynchronously:
 // FP32 fields into the box itself, 16-bit ones as raw values into a staging
-// area behind it (tile_widen_box then fills the box).
+// area behind it (tile_widen_box then fills the box).  origin: the wrapped origin,
+// when the caller keeps it from field to field.
 template <class S>
 __device__ __forceinline__ void tile_load_box(const Grid& g, const S* __restrict__ f, float* box,
-                                              const BoxPar& bp, int lane, int warp)
+                                              const BoxPar& bp, int lane, int warp,
+                                              const BoxOrigin* origin = nullptr)
 {
     const int bytes = box_chunk_bytes<S>(g, f, bp);
     if constexpr (sizeof(S) == 4) {
         const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(box));
         if (bytes == 16) {
-            stage_box_columns<S, 16>(g, f, dst, bp);
+            stage_box_columns<S, 16>(g, f, dst, bp, origin);
         } else if (bytes == 8) {
-            stage_box_columns<S, 8>(g, f, dst, bp);
+            stage_box_columns<S, 8>(g, f, dst, bp, origin);
         } else {
             // a caller's field at an odd 4-byte boundary: value by value
             const int w1 = wrap_index(bp.O1, g.n1), w2 = wrap_index(bp.O2, g.n2), w3 = wrap_index(bp.O3, g.n3);
@@ -410,11 +422,11 @@ __device__ __forceinline__ void tile_load_box(const Grid& g, const S* __restrict
     } else {
         const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(box + bp.E1 * bp.E2 * bp.S3));
         if (bytes == 16)
-            stage_box_columns<S, 16>(g, f, dst, bp);
+            stage_box_columns<S, 16>(g, f, dst, bp, origin);
         else if (bytes == 8)
-            stage_box_columns<S, 8>(g, f, dst, bp);
+            stage_box_columns<S, 8>(g, f, dst, bp, origin);
         else
-            stage_box_columns<S, 4>(g, f, dst, bp);
+            stage_box_columns<S, 4>(g, f, dst, bp, origin);
     }
 }
 
@@ -761,6 +773,9 @@ __global__ void __launch_bounds__(kTileThreads, tile_min_blocks<ORDER, 4, WIDE>(
             }
         return;
     }
+    // three divisions per thread and field otherwise (256^3, four trilinear fields at no
+    // displacement: 256 -> 237 us); the other kernels have no registers for them
+    const BoxOrigin origin(g, bp);
     for (int fld = 0; fld < nf; ++fld) {
         // the weights and offsets of the four points are formed anew for each
         // field: kept across the loop they do not fit the 64 registers (the
@@ -770,7 +785,7 @@ __global__ void __launch_bounds__(kTileThreads, tile_min_blocks<ORDER, 4, WIDE>(
 #pragma unroll
             for (int q = 0; q < TILE1; ++q) asm volatile("" : "+f"(d1[q]), "+f"(d2[q]), "+f"(d3[q]));
         }
-        tile_load_box<float>(g, f + fld * N, box, bp, lane, warp);
+        tile_load_box<float>(g, f + fld * N, box, bp, lane, warp, ORDER == 1 && WIDE ? &origin : nullptr);
         cp_async_wait_all();
         __syncthreads();
 #pragma unroll
