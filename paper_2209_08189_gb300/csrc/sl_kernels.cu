@@ -662,18 +662,14 @@ void launch_interp(const Grid& g, int order, const void* f, const float* d, void
 }
 
 template <int ORDER, bool FULL, bool MAP>
-void launch_fields_tiles(const Grid& g, const float* f, int nf, const float* d, float* out, cudaStream_t st)
+void launch_fields_tiles(Grid g, const float* f, int nf, const float* d, float* out, cudaStream_t st)
 {
+    g.wide = 1;
     const size_t smem = tiled_smem_bytes<ORDER>(g);
-    auto launch = [&](auto kernel) {
-        if (smem > 48 * 1024)
-            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-        kernel<<<tiled_grid(g), kTileThreads, smem, st>>>(g, f, nf, d, out);
-    };
-    if constexpr (ORDER == 1) {
-        if (g.wide) return launch(k_gather_tiled_fields<ORDER, FULL, MAP, true>);
-    }
-    launch(k_gather_tiled_fields<ORDER, FULL, MAP>);
+    if (smem > 48 * 1024)
+        cudaFuncSetAttribute(k_gather_tiled_fields<ORDER, FULL, MAP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(smem));
+    k_gather_tiled_fields<ORDER, FULL, MAP><<<tiled_grid(g), kTileThreads, smem, st>>>(g, f, nf, d, out);
 }
 
 template <int ORDER, bool MAP>

@@ -725,8 +725,10 @@ __global__ void __launch_bounds__(kTileThreads, tile_min_blocks<ORDER, sizeof(S)
 // (X - x) in physical units, nf = 3.  It reads its 192 stencil values from the
 // box as the gathers do; the per-point kernel it replaced fetched them through
 // L1 (256^3, CFL 3.4: 0.80 ms per step; from the box 0.56 ms).
-template <int ORDER, bool FULL, bool MAP, bool WIDE = false>
-__global__ void __launch_bounds__(kTileThreads, tile_min_blocks<ORDER, 4, WIDE>())
+// Every order takes the wide box here (set by the launch): the displacements and bounds
+// are read once for all fields, so that six CTAs gain nothing.
+template <int ORDER, bool FULL, bool MAP>
+__global__ void __launch_bounds__(kTileThreads, CLAIRE_TILE_MIN_BLOCKS)
     k_gather_tiled_fields(Grid g, const float* __restrict__ f, int nf, const float* __restrict__ d,
                           float* __restrict__ out)
 {
@@ -774,18 +776,18 @@ __global__ void __launch_bounds__(kTileThreads, tile_min_blocks<ORDER, 4, WIDE>(
         return;
     }
     // three divisions per thread and field otherwise (256^3, four trilinear fields at no
-    // displacement: 256 -> 237 us); the other kernels have no registers for them
+    // displacement: 255 -> 239 us); the other orders have no registers for them
     const BoxOrigin origin(g, bp);
     for (int fld = 0; fld < nf; ++fld) {
         // the weights and offsets of the four points are formed anew for each
         // field: kept across the loop they do not fit the 64 registers (the
-        // compiler then spilled 240 bytes per thread), or the 40 of the narrow
-        // trilinear kernel; the wide one's 64 hold them
-        if constexpr (!(ORDER == 1 && WIDE)) {
+        // compiler then spilled 240 bytes per thread; those of the trilinear
+        // stencil do)
+        if constexpr (ORDER != 1) {
 #pragma unroll
             for (int q = 0; q < TILE1; ++q) asm volatile("" : "+f"(d1[q]), "+f"(d2[q]), "+f"(d3[q]));
         }
-        tile_load_box<float>(g, f + fld * N, box, bp, lane, warp, ORDER == 1 && WIDE ? &origin : nullptr);
+        tile_load_box<float>(g, f + fld * N, box, bp, lane, warp, ORDER == 1 ? &origin : nullptr);
         cp_async_wait_all();
         __syncthreads();
 #pragma unroll
